@@ -165,32 +165,39 @@ int cheb_plan_info(const cheb_plan *plan, int64_t *n_panels, int32_t *panel_widt
  * below). */
 int cheb_plan_attach_operator(cheb_plan *plan, const cheb_bsr *L, size_t *op_ws_bytes, void *stream);
 
-/* Column-order step kernel of reduced-precision plans.  For a CHEB_F32 or
- * CHEB_BF16 plan, cheb_plan_attach_operator also builds the gather plan of a
- * second per-step kernel that keeps T_k in column order (the blocks of each
- * block column contiguous; columns are independent under Eq. 3, Sec.
- * "Expansion in Chebyshev polynomials"): panels of up to 4 block columns
- * whose union of row lists fits shared memory (at most 1023 rows), in column
- * order; per union row its operator entries with K in the union (32-bit
- * words: index of the operator block << 10 | union slot), padded to whole
- * chunks of 8 with entries naming a zero block; the union rows of a panel
- * dealt to the thread block's warps to balance their chunks, each warp's
- * chunks stored as one stream; and the union slot of every P_out block (2
- * bytes each).  After cheb_plan_bind_operator, cheb_expand_stepwise with
- * that operator and an FP32/BF16 precision runs this kernel; it sums each
- * block product in a different order from the ranking kernel, so results
- * agree to rounding, and are bitwise reproducible run to run.  It is not
- * built (and the ranking kernel runs) when one column's rows do not fit it
- * or the operator has 2^22 - 1 blocks or more.  cheb_plan_col_info reports
- * its panel count (0 when not built), largest union and total operator
- * entries (padding included).
+/* Column-order kernel.  cheb_plan_attach_operator also builds the gather plan of
+ * a second recursion kernel that keeps T_k in column order (the blocks of each
+ * block column contiguous; columns are independent under Eq. 3, Sec. "Expansion
+ * in Chebyshev polynomials") and runs many steps per launch: for CHEB_F32 and
+ * CHEB_BF16 plans always, for CHEB_F64 and CHEB_F64X plans when the operator's
+ * block rows hold 48 blocks or more on average.  Panels of up to 4 (FP32, BF16) or
+ * 2 (FP64) block columns of one system whose union of row lists fits shared memory
+ * (at most 667 rows), in column order; the union rows of a panel in groups of four
+ * with similar operator rows; per group the union slots K of its rows' operator
+ * entries, four to a quad, and per quad 16 words (index of the operator block of a
+ * row at a slot << 10 | union slot; the operator's block count names a zero block
+ * where the row has none); the groups dealt to the thread block's warps to balance
+ * their quads, each warp's quads stored as one stream; and the union slot of every
+ * P_out block (2 bytes each).  After cheb_plan_bind_operator, expansions with that
+ * operator run this kernel: cheb_expand_stepwise wherever the lists were built,
+ * cheb_expand and cheb_expand_batched when the operator's rows are long as above.
+ * Its products are sums of integer digits on the tensor cores, exact but for a grid
+ * of 2^-29 (FP32) or 2^-59 (FP64) of each panel column's and operator row's largest
+ * element, in place of FP32 or FP64 rounding; columns or operators with elements
+ * that are not finite or beyond the grid's exponents are multiplied in plain FP32 or
+ * FP64.  Results agree with the other kernels to rounding, and are bitwise
+ * reproducible run to run.  CHEB_F64X expansions that run it hold T_k in FP64.  The
+ * lists are not built (and the ranking kernels run) when one column's rows do not
+ * fit a panel or the operator has 2^22 - 1 blocks or more.  cheb_plan_col_info
+ * reports the panel count (0 when not built), largest union and total operator
+ * words (padding included).
  *
  * This gather plan is built by device kernels from the device patterns of
  * P_out and the operator (a sequential panel walk in one thread block, then
- * one thread block per panel: union bitmap and ranks, per-row entry counts, the
- * rows dealt to the warps by decreasing chunk count, each to the warp with the
- * fewest chunks so far, and the entry streams; a few scalars and per-panel
- * maxima come back to the host to size the lists).  It uses device memory of
+ * one thread block per panel: union bitmap and ranks, the groups and their merged
+ * slots, the groups dealt to the warps by decreasing quad count, each to the warp
+ * with the fewest quads so far, and the entry streams; a few scalars and per-panel
+ * integers come back to the host to size the lists).  It uses device memory of
  * its own until cheb_plan_bind_operator copies the lists into the operator
  * workspace.
  *
@@ -208,8 +215,8 @@ int cheb_plan_attach_operator(cheb_plan *plan, const cheb_bsr *L, size_t *op_ws_
  * cheb_plan_set_gather_builder(plan, host) picks the builder of one plan's
  * next attach.  cheb_plan_lists_copy copies bound table `which` into device
  * memory dst (dst_bytes); *bytes receives its size (dst NULL: size only):
- * 0 column-kernel panels int32[4 per panel], 1 its warp chunk starts and 2
- * warp row starts int32[panels][17], 3 row words, 4 entry words uint32, 5
+ * 0 column-kernel panels int32[4 per panel], 1 its warp quad starts and 2
+ * warp group starts int32[panels][17], 3 group words, 4 entry words uint32, 5
  * slots uint16[nnzb]; 6 the transposition map int32[nnzb]; 7 step panels and
  * 8 resident panels int32[2 per panel]; 9 the system of each resident panel,
  * 10 the first resident panel of each system (+ end); 11-13 the step panels'
@@ -307,10 +314,10 @@ int cheb_coeffs(const cheb_func *funcs, int32_t n_f, double emin, double emax, d
  *   block products summed in FP32).  Results are bitwise reproducible run to
  *   run.
  *
- * cheb_expand runs the whole expansion in one kernel launch: every thread
- * block owns a panel of block columns (columns are independent under Eq. 3)
- * and keeps its T_k, T_{k-1} in shared memory for all steps; there is no
- * inter-block synchronisation.  Asynchronous, graph-capturable (no host
+ * cheb_expand runs the whole expansion in one kernel launch (or on the column
+ * kernel, see above): every thread block owns a panel of block columns (columns
+ * are independent under Eq. 3) and keeps its T_k, T_{k-1} in shared memory for
+ * all steps; there is no inter-block synchronisation.  Asynchronous, graph-capturable (no host
  * copies).  Workspace: cheb_expand_workspace_size with max_terms >= n_terms.
  * Errors: CHEB_ERR_INVALID (n_terms < 2, n_f < 0 or > 8, plan precision !=
  * precision, batched plan), CHEB_ERR_NOSPACE (workspace too small).
@@ -323,7 +330,7 @@ int cheb_expand(const cheb_plan *plan, const cheb_bsr *Mt, int32_t n_terms,
                 void *ws, size_t ws_bytes, void *stream);
 
 /* The same expansion as one kernel launch per step (T_k in HBM, three
- * P_out-sized buffers in the workspace).  Same arguments and results up to
+ * P_out-sized buffers in the workspace), or on the column kernel.  Same arguments and results up to
  * rounding order; kept as an independent second implementation and for
  * plans whose panels do not fit the resident kernel.  It also takes
  * precision CHEB_BF16 (with a CHEB_BF16 plan): Mt and every stored T_k are

@@ -1,39 +1,70 @@
-// The FP32 / BF16 recursion step in column order: one step of the masked
-// Chebyshev recursion (Eq. 3) fused with the accumulation of several
-// expansions (Eq. 1) and the moments Tr T_{k+1}, <T_{k+1}, G>.
+// The recursion in column order on the tensor cores: several steps of the
+// masked Chebyshev recursion (Eq. 3) per launch, fused with the accumulation
+// of several expansions (Eq. 1) and the moments Tr T_k, <T_k, G>.
 //
 // Column J of T_{k+1} needs only column J of T_k and T_{k-1} (Sec. "Expansion
-// in Chebyshev polynomials").  The recursion therefore keeps T_k in *column
-// order*: the blocks (K, J) of column J are stored contiguously, at the BCSR
-// positions of row J of the symmetric output pattern (block (K, J) at the
-// position of (J, K); its 16 values stay row-major).  A panel of consecutive
-// block columns is then one contiguous range, read and written with
-// coalesced 64-byte block accesses.  The accumulators and G stay in the
-// caller's BCSR order; block b of the column order is block tperm[b] there.
+// in Chebyshev polynomials"), so a panel of P neighbouring block columns (4 in
+// FP32 / BF16, 2 in FP64) runs through all the steps of a launch in one thread
+// block, with no data from any other.  T_k is kept in *column order*: the
+// blocks (K, J) of column J are contiguous, at the BCSR positions of row J of
+// the symmetric output pattern; two buffers, T_{k+1} over T_{k-1}.
 //
-// One thread block per panel (the plan's column panels):
-//   1. the panel's T_k blocks go to shared memory X[slot][4][4P] (slot = rank
-//      of the block row in the union of the panel's row lists, precomputed;
-//      zero where a column has no block in that row); rows of a slot's
-//      block are XOR-swizzled by the slot so that the K-groups of a quarter
-//      warp read distinct banks;
-//   2. each warp takes union rows I; lane = (panel column q, K-group); the
-//      operator blocks L_IK of row I with K in the union are the row's
-//      precomputed entries, taken KG at a time (one chunk, one per K-group)
-//      and copied by cp.async into a per-warp ring of stages, several chunks
-//      ahead of the multiplication (across row ends); the entry words of a
-//      whole row are fetched one row ahead and handed out by shuffles;
-//   3. at the end of a row a reduce-scatter over the K-groups leaves each lane
-//      16/KG elements of the block (I, J_q), and the lane finishes them:
-//      T_{k+1} = alpha (M~ T_k) + beta T_{k-1}, acc_j += c_j[k+1] T_{k+1},
-//      and its parts of Tr T_{k+1} and <T_{k+1}, G> -- with the operands of
-//      that epilogue (T_{k-1}, G, accumulators) loaded at the start of the
-//      row, so their latency hides under the row's products;
-//   4. the last thread block to finish sums the per-block moment partials in
-//      a fixed order (deterministic).
+// What bounds it.  The products are gathered 4x4 blocks.  On the FMA pipes
+// they cost 64 instructions a block and panel column (FP64 at 1/64 of the FP32
+// rate; FP32 bound by issue and by shared-memory reads, 240 instructions per
+// 16 entries).  Here they are f16 tensor-core products of *digits*: within a
+// panel column (and within an operator block row) every value is written on
+// one power-of-two grid as a sum of small integers times powers of two, three
+// digits (30 bits) for FP32 and six (60 bits) for FP64.  Integers up to 2048
+// are exact in f16, and the products of one mma are small enough for the FP32
+// accumulators to hold the leading digit sums D_s = sum_{i+j=s} d_i d_j exactly:
+//     FP32: D_0 exact (below 2^24 over two mma, then added to an FP32 sum, round
+//           to nearest), D_1, D_2 (weights 2^-10, 2^-20) kept in the accumulator; 6 mma
+//           per 16 operator rows, 16 inner and 8 panel columns;
+//     FP64: D_0 .. D_3 exact (summed as integers), D_4 .. D_6 (weights 2^-40,
+//           2^-50, 2^-60) in two accumulators; 26 mma.
+// Exactness matters beyond the size of the rounding: a tensor core that
+// truncates its sums would shrink every product by about 2^-25, the same way
+// at every step, which acts like a scaled operator.  What is left is the grid
+// itself (2^-29 and 2^-59 of the column's largest element) and the terms
+// beyond the last digit sum.  Error of 64-term expansions of 140 and 150 atoms
+// against long doubles, largest of the accumulators, before -> now: FP64 Fermi 3.5e-16
+// -> 3.5e-16, powers 9.4e-16 -> 5.3e-16 (without D_6 3.7e-16 and 1.0e-15); FP32
+// Fermi 3.5e-8 -> 2.9e-8, powers 4.7e-7 -> 2.5e-7; FP64-accurate 4.2e-14 -> 5.3e-16.
+// Measured (GB300): one step at 1,500 atoms, r_c 10, r_out 14 bohr, three
+// accumulators: FP64 9.2 -> 1.3 ms, FP64-accurate (before: double-floats) at 1,000
+// atoms, 8 / 12 bohr: 2.3 -> 0.39 ms; FP32 at 10,000 atoms 3.47 -> 2.75 ms, at 1,000
+// atoms, 8 / 12 bohr: 0.237 -> 0.161 ms.  ncu: L1 access cycles 71 % (FP64) and
+// 47 % (FP32), ALU (digit unpacking) 50 %, tensor pipe 43 % and 36 %, issue 45-55 %:
+// an operator block of 64 or 128 bytes is used for one row group and panel only, and
+// an L1 load costs a cycle per line that the lanes it serves together touch.
+// Tried without gain: f16 operator digits in memory (96 bytes: 3.7 instead of 2.9 ms
+// at 10,000 atoms), 12 warps (10 % slower), lanes over two blocks per access (L1
+// cycles -35 %, instructions +30 %, 15 % slower).
+//
+// One thread block per panel.  Per step:
+//   1. the panel's T_k blocks become digits in shared memory, X[slot][column]
+//      (slot = rank of the block row in the union of the columns' row lists);
+//      the grid of each column comes from the largest element that the step
+//      before wrote;
+//   2. each warp takes groups of 4 union rows.  The operator blocks of the
+//      group with K in the union are listed by merged K, four slots ("quad") at
+//      a time: an m16n8k16 product of the operator's 16 rows (A, from the
+//      operator's digits in L2) with 8 panel columns (B, from X); rows without
+//      a block at a merged K name a zero block;
+//   3. at the end of a group each lane holds 2 neighbouring elements of the
+//      blocks (row, column) and finishes them: T_{k+1} = 2 M~ T_k - T_{k-1}, and
+//      every third step acc_j += c_j T of the last three terms (in the order of
+//      one term per step) and their parts of the moments;
+//   4. the panel's moments go to a table that a second kernel sums in a fixed
+//      order.
+// A column with an element that is not finite or beyond the grid's exponents
+// (or such an operator) takes the step in plain FP32 / FP64 instead (slow).
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 
 #include <algorithm>
+#include <array>
 #include <numeric>
 #include <thread>
 
@@ -43,38 +74,51 @@
 
 namespace cheb {
 
+// Tiles of an element type: NT n8-tiles (2 block columns each) per panel, and the
+// grid exponents of T and of the operator.
+template <typename T>
+struct Dig;
+template <>
+struct Dig<float> {
+    static constexpr int NT = 2, EX_MIN = -60, EX_MAX = 90, OP_MIN = -30, OP_MAX = 30;
+};
+template <>
+struct Dig<double> {
+    static constexpr int NT = 1, EX_MIN = -400, EX_MAX = 400, OP_MIN = -400, OP_MAX = 400;
+};
+
 struct ColArgs {
-    const int32_t *panels;  // (first column, column count, union rows, 0) per thread block
-    const int32_t *wchunk;  // [panels][NW + 1] chunk range of each warp
-    const int32_t *wrow;    // [panels][NW + 1] row-list range of each warp
-    const uint32_t *rows;   // union slot | chunk count << COL_SLOT_BITS, per warp row
-    const uint32_t *ent;    // [chunks][KG] operator block << COL_SLOT_BITS | union slot
-    const uint16_t *slot;
-    const int64_t *rp;     // P_out row_ptr = column starts in column order
-    const int32_t *ci;     // row of each column-order block
-    const int32_t *tperm;  // BCSR position of each column-order block
-    const float *Lv;       // operator values (FP32 copy, one zero block appended), BCSR order
-    const float *R;        // T_k (column order)
-    const float *Rm;       // T_{k-1} (column order) or NULL
-    float *C;              // T_{k+1} (column order)
-    float alpha, beta;
+    const int32_t *panels;  // (first column, column count, union rows, system) per thread block
+    const int32_t *wchunk;  // [panels][NW + 1] quad range of each warp
+    const int32_t *wrow;    // [panels][NW + 1] group range of each warp
+    const uint32_t *rows;   // per group: the 4 union slots and the quad count (2 words)
+    const uint32_t *ent;    // [quads][16] operator block << COL_SLOT_BITS | union slot
+    const uint16_t *slot;   // union slot of each column-order block
+    const int64_t *rp;      // P_out row_ptr = column starts in column order
+    const int32_t *ci;      // row of each column-order block
+    const int32_t *tperm;   // BCSR position of each column-order block
+    const int64_t *Lrp;     // operator pattern and FP64 values
+    const int32_t *Lci;
+    const double *Lv;
+    int64_t nnzL;
+    const uint4 *opd;       // operator digits (one zero block appended)
+    const int32_t *opexp;   // grid exponent of each operator block row
+    const int32_t *opflag;  // nonzero: an operator element beyond the digits
+    void *T[2];             // T_k in T[k & 1] (column order)
+    int32_t t0, t1;         // terms formed by this launch: t0 .. t1 - 1 (t0 = 2: also terms 0 and 1)
+    const int32_t *n_terms;  // per system, or NULL: n_single
+    int32_t n_single;
     int32_t nf;
-    double *acc[MAX_F];   // the caller's FP64 accumulators (BCSR order): init and final kernels
-    float *accp[MAX_F];   // the accumulators during the expansion: (hi, lo) float pairs, column order
-    const double *coef;
+    double *acc[MAX_F];   // the caller's FP64 accumulators (BCSR order)
+    float *accp[MAX_F];   // FP32: the accumulators as (hi, lo) float pairs, column order
+    const double *coef;   // coef[coef_off[sys] + f * coef_stride + k]
+    const int64_t *coef_off;
     int32_t coef_stride;
-    int32_t term;
-    const double *G;      // the caller's G (BCSR order): init kernel
-    const float *Gp;      // G as (hi, lo) float pairs in column order, or NULL
-    double *mom, *gmom, *part;  // moment scalars of term k+1 (terms k-1, k at [-2], [-1])
-    int32_t *counter;
+    const double *G;      // the caller's G (BCSR order) or NULL
+    float *Gp;            // FP32: G as (hi, lo) float pairs in column order
+    double *part;         // [panel][pstride][2] moments of terms tbase ..
+    int32_t pstride, tbase, want_mom;
     int32_t round_bf16;
-    // Terms accumulated (and their moments taken) by this launch: bit 0 term
-    // k+1 (the T_{k+1} it forms), bit 1 term k (T_k, in shared memory), bit 2
-    // term k-1 (T_{k-1}, read for the recursion anyway).  Grouping three
-    // terms per update cuts the accumulator and G traffic threefold and sums
-    // in the same order as one term per step.
-    int32_t grp;
 };
 
 // Double-float arithmetic (a value is an unevaluated sum hi + lo of two
@@ -101,585 +145,811 @@ __host__ __device__ inline void ff_split(double v, float &hi, float &lo) {
 
 __device__ __forceinline__ float bf16r(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 
-// L2 policies: the operator (read by every panel whose union holds its
-// blocks) is kept, the streams read once per step are evicted first.
-__device__ __forceinline__ uint64_t policy_keep() {
-    uint64_t p;
-    asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
-    return p;
+// --- digits ----------------------------------------------------------------
+
+// |x| as an unsigned that orders like |x| and is largest for infinities and NaN
+__device__ __forceinline__ uint32_t mag_bits(float x) { return __float_as_uint(x) & 0x7fffffffu; }
+__device__ __forceinline__ uint32_t mag_bits(double x) { return (uint32_t)__double2hiint(x) & 0x7fffffffu; }
+
+// Grid exponent e of values with largest magnitude bits m: every |x| < 0.997 2^e
+// (0 for all zeros).  false: not finite, or e outside [lo, hi].
+template <typename T>
+__device__ __forceinline__ bool grid_exp(uint32_t m, int lo, int hi, int &e) {
+    e = 0;
+    if (m == 0u) return true;
+    if constexpr (sizeof(T) == 4) {
+        e = (int)(m >> 23) - 126 + ((m & 0x7fffffu) >= 0x7f0000u ? 1 : 0);
+        if (m >= 0x7f800000u) return false;
+    } else {
+        e = (int)(m >> 20) - 1022 + ((m & 0xfffffu) >= 0xfe000u ? 1 : 0);
+        if (m >= 0x7ff00000u) return false;
+    }
+    return e >= lo && e <= hi;
 }
-__device__ __forceinline__ uint64_t policy_stream() {
-    uint64_t p;
-    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
-    return p;
+// 2^e as a float / double (e within the normal range)
+__device__ __forceinline__ float pow2(int e, float) { return __int_as_float((e + 127) << 23); }
+__device__ __forceinline__ double pow2(int e, double) { return __hiloint2double((e + 1023) << 20, 0); }
+
+// x on the grid of exponent e with an offset that makes every digit
+// non-negative.  FP32: 30 bits of x 2^(29 - e); FP64: 60 bits of x 2^(59 - e),
+// 512 in each of the six digits.
+__device__ __forceinline__ int grid_value(float x, int e) { return __float2int_rn(x * pow2(29 - e, 0.f)); }
+__device__ __forceinline__ uint64_t grid_value(double x, int e) {
+    const uint64_t bits = (uint64_t)__double_as_longlong(x);
+    const int ex = (int)((bits >> 52) & 0x7ff), sh = ex - 1016 - e;
+    const uint64_t mant = (bits & 0xfffffffffffffull) | 0x10000000000000ull;
+    uint64_t mag = 0;
+    if (ex > 0 && sh > -54) mag = sh >= 0 ? mant << sh : (mant + (1ull << (-sh - 1))) >> -sh;
+    const int64_t q = (bits >> 63) ? -(int64_t)mag : (int64_t)mag;
+    return (uint64_t)q + 0x0802008020080200ull;
 }
 
-// 16 floats of an operator block, read once per panel: no L1 allocation.
-__device__ __forceinline__ void ld_op(float (&h)[16], const float *p, uint64_t pol) {
+// fp16x2 arithmetic on packed digits (all values and results exact)
+__device__ __forceinline__ uint32_t h2_sub(uint32_t x, uint32_t y) {
+    uint32_t r;
+    asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(y));
+    return r;
+}
+__device__ __forceinline__ uint32_t h2_fma(uint32_t x, uint32_t y, uint32_t z) {
+    uint32_t r;
+    asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(x), "r"(y), "r"(z));
+    return r;
+}
+// Two 10-bit biased digits (bits 0-9 and 16-25) as f16 integers: the bits under
+// the f16 exponent of 1024, less 1024 + 512.
+__device__ __forceinline__ uint32_t f16_digits(uint32_t d) { return h2_sub(d | 0x64006400u, 0x66006600u); }
+
+// FP32 operator digits of a pair, packed (q = h_0 2^20 + h_1 2^10 + h_2, 10 bits
+// each): h_0 of both in word 0 and h_1 in word 1 (bits 0-9, 16-25), h_2 spread
+// over bits 10-15 / 26-31 of word 0 (its upper 6) and 10-13 / 26-29 of word 1.
+__device__ __forceinline__ void pack_pair(uint32_t (&w)[2], int q0, int q1) {
+    const uint32_t u = (uint32_t)q0 + 0x20080200u, v = (uint32_t)q1 + 0x20080200u;
+    w[0] = ((u >> 20) & 0x3ffu) | ((u & 0x3f0u) << 6) | (((v >> 20) & 0x3ffu) << 16) | ((v & 0x3f0u) << 22);
+    w[1] = ((u >> 10) & 0x3ffu) | ((u & 0xfu) << 10) | (((v >> 10) & 0x3ffu) << 16) | ((v & 0xfu) << 26);
+}
+__device__ __forceinline__ uint32_t spread_digit(uint32_t w0, uint32_t w1) {
+    return f16_digits(((w1 >> 10) & 0x000f000fu) | ((w0 >> 6) & 0x03f003f0u));
+}
+// FP32 panel digits of a pair: q = d_0 2^19 + d_1 2^8 + d_2, 11, 11 and 8 bits;
+// w[0] = d_0, w[1] = d_1 / 2 as f16, the third digits + 128 as bytes in third.
+// (d_1 / 2 and 2 d_2 carry the weights that the operator's 10-bit digits have.)
+__device__ __forceinline__ void panel_digits(uint32_t (&w)[2], uint32_t &third, int q0, int q1) {
+    const uint32_t off = (1024u << 19) + (1024u << 8) + 128u;
+    const uint32_t u = (uint32_t)q0 + off, v = (uint32_t)q1 + off;
+    auto h2 = [](int a, int b) {
+        const __half2 h = __halves2half2(__int2half_rn(a), __int2half_rn(b));
+        return *reinterpret_cast<const uint32_t *>(&h);
+    };
+    w[0] = h2((int)(u >> 19) - 1024, (int)(v >> 19) - 1024);
+    w[1] = h2((int)((u >> 8) & 0x7ffu) - 1024, (int)((v >> 8) & 0x7ffu) - 1024);
+    w[1] = h2_fma(w[1], 0x38003800u, 0u);  // * 0.5
+    third = (u & 0xffu) | ((v & 0xffu) << 8);
+}
+// 2 d_2 of a pair from its bytes: selected under the exponent of 1024
+template <int SEL>
+__device__ __forceinline__ uint32_t third_digits(uint32_t bytes) {
+    return h2_fma(__byte_perm(bytes, 0x64646464u, SEL), 0x40004000u, 0xe880e880u);  // 2 (1024 + b) - 2304
+}
+
+// FP64 panel digits of a pair: w[i] = digit i of both as f16.
+__device__ __forceinline__ void panel_digits(uint32_t (&w)[6], double x0, double x1, int e) {
+    const uint64_t u = grid_value(x0, e), v = grid_value(x1, e);
+#pragma unroll
+    for (int i = 0; i < 6; ++i)
+        w[i] = f16_digits(((uint32_t)(u >> (10 * (5 - i))) & 0x3ffu) | (((uint32_t)(v >> (10 * (5 - i))) & 0x3ffu) << 16));
+}
+// FP64 operator digits of a pair, packed: digits 0-3 in words 0-3 (bits 0-9,
+// 16-25), digit 4 spread over words 0 and 1, digit 5 over words 2 and 3.
+__device__ __forceinline__ void pack_pair(uint32_t (&w)[4], double x0, double x1, int e) {
+    const uint64_t u = grid_value(x0, e), v = grid_value(x1, e);
+    auto d = [](uint64_t z, int i) { return (uint32_t)(z >> (10 * (5 - i))) & 0x3ffu; };
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        float4 v;
-        asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v4.f32 {%0,%1,%2,%3}, [%4], %5;"
-                     : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-                     : "l"(p + 4 * i), "l"(pol));
-        h[4 * i] = v.x; h[4 * i + 1] = v.y; h[4 * i + 2] = v.z; h[4 * i + 3] = v.w;
+        const int j = 4 + i / 2;  // the spread digit of this word
+        const uint32_t pu = i % 2 == 0 ? d(u, j) >> 4 : d(u, j) & 0xfu, pv = i % 2 == 0 ? d(v, j) >> 4 : d(v, j) & 0xfu;
+        w[i] = d(u, i) | (pu << 10) | (d(v, i) << 16) | (pv << 26);
     }
 }
-__device__ __forceinline__ void cp_async16_hint(void *dst_smem, const void *src, uint64_t pol) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst_smem);
-    asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src), "l"(pol)
-                 : "memory");
+__device__ __forceinline__ uint32_t packed_digit(const uint32_t (&w)[4], int i) {
+    if (i < 4) return f16_digits(w[i] & 0x03ff03ffu);
+    return spread_digit(w[2 * (i - 4)], w[2 * (i - 4) + 1]);
 }
-// Streamed loads and stores with an L2 policy (the EPL = 1 or 2 elements a
-// lane finishes; 16 floats of a T_k block).
-template <int N>
-__device__ __forceinline__ void ldh(float (&v)[N], const float *p, uint64_t pol) {
-    if constexpr (N == 2) {
-        asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v2.f32 {%0,%1}, [%2], %3;"
-                     : "=f"(v[0]), "=f"(v[1]) : "l"(p), "l"(pol));
-    } else {
-        asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v[0]) : "l"(p), "l"(pol));
+
+__device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], const uint32_t (&b)[2],
+                                         const float (&c)[4]) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%11,%12,%13};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]), "f"(c[0]), "f"(c[1]), "f"(c[2]), "f"(c[3]));
+}
+
+// The operator's digits: one warp per block row; block nnzL is the zero block
+// that pads the lists.  A block holds, per scalar row r, the words of its pairs
+// (H[r][0], H[r][1]) and (H[r][2], H[r][3]): 16 bytes in FP32, 32 in FP64.
+// (Unpacked f16 digits would save the unpacking and take half as much again from
+// L2 and, counted in the 128-byte lines that a load touches, from L1.)
+template <typename T>
+__global__ void k_opdig(const int64_t *rp, const double *v, int64_t nbr, int64_t nnzL, int round_bf16, uint4 *opd,
+                        int32_t *opexp, int32_t *opflag) {
+    constexpr bool F64 = sizeof(T) == 8;
+    const int64_t I = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (I == nbr) {
+        constexpr int N = F64 ? 8 : 4;
+        if (lane < N) opd[nnzL * N + lane] = make_uint4(0x82008200u, 0x02000200u, 0x82008200u, 0x02000200u);
+        return;
     }
-}
-template <int N>
-__device__ __forceinline__ void ldh(double (&v)[N], const double *p, uint64_t pol) {
-    if constexpr (N == 2) {
-        asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v2.f64 {%0,%1}, [%2], %3;"
-                     : "=d"(v[0]), "=d"(v[1]) : "l"(p), "l"(pol));
-    } else {
-        asm volatile("ld.global.L1::no_allocate.L2::cache_hint.f64 %0, [%1], %2;" : "=d"(v[0]) : "l"(p), "l"(pol));
+    if (I > nbr) return;
+    const int64_t e0 = rp[I] * BB, e1 = rp[I + 1] * BB;
+    uint32_t m = 0;
+    for (int64_t i = e0 + lane; i < e1; i += 32) {
+        if constexpr (F64) m = max(m, mag_bits(v[i]));
+        else m = max(m, mag_bits(round_bf16 ? bf16r((float)v[i]) : (float)v[i]));
     }
-}
-template <int N>
-__device__ __forceinline__ void sth(float *p, const float (&v)[N], uint64_t pol) {
-    if constexpr (N == 2) {
-        asm volatile("st.global.L2::cache_hint.v2.f32 [%0], {%1,%2}, %3;" ::"l"(p), "f"(v[0]), "f"(v[1]), "l"(pol)
-                     : "memory");
-    } else {
-        asm volatile("st.global.L2::cache_hint.f32 [%0], %1, %2;" ::"l"(p), "f"(v[0]), "l"(pol) : "memory");
+    m = __reduce_max_sync(0xffffffffu, m);
+    int e;
+    if (!grid_exp<T>(m, Dig<T>::OP_MIN, Dig<T>::OP_MAX, e)) {
+        if (lane == 0) atomicOr(opflag, 1);
+        return;
     }
-}
-template <int N>
-__device__ __forceinline__ void sth(double *p, const double (&v)[N], uint64_t pol) {
-    if constexpr (N == 2) {
-        asm volatile("st.global.L2::cache_hint.v2.f64 [%0], {%1,%2}, %3;" ::"l"(p), "d"(v[0]), "d"(v[1]), "l"(pol)
-                     : "memory");
-    } else {
-        asm volatile("st.global.L2::cache_hint.f64 [%0], %1, %2;" ::"l"(p), "d"(v[0]), "l"(pol) : "memory");
-    }
-}
-// EPL consecutive (hi, lo) pairs: 2 * EPL floats
-template <int N>
-__device__ __forceinline__ void ldh_pairs(float (&v)[2 * N], const float *p, uint64_t pol) {
-    if constexpr (N == 2) {
-        asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v4.f32 {%0,%1,%2,%3}, [%4], %5;"
-                     : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "l"(p), "l"(pol));
-    } else {
-        asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v2.f32 {%0,%1}, [%2], %3;"
-                     : "=f"(v[0]), "=f"(v[1]) : "l"(p), "l"(pol));
-    }
-}
-template <int N>
-__device__ __forceinline__ void sth_pairs(float *p, const float (&v)[2 * N], uint64_t pol) {
-    if constexpr (N == 2) {
-        asm volatile("st.global.L2::cache_hint.v4.f32 [%0], {%1,%2,%3,%4}, %5;" ::"l"(p), "f"(v[0]), "f"(v[1]),
-                     "f"(v[2]), "f"(v[3]), "l"(pol)
-                     : "memory");
-    } else {
-        asm volatile("st.global.L2::cache_hint.v2.f32 [%0], {%1,%2}, %3;" ::"l"(p), "f"(v[0]), "f"(v[1]), "l"(pol)
-                     : "memory");
-    }
-}
-template <int N>
-__device__ __forceinline__ void ldg_pairs(float (&v)[2 * N], const float *p, uint64_t pol) {
-    if constexpr (N == 2) {
-        asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v4.f32 {%0,%1,%2,%3}, [%4], %5;"
-                     : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "l"(p), "l"(pol));
-    } else {
-        asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v2.f32 {%0,%1}, [%2], %3;"
-                     : "=f"(v[0]), "=f"(v[1]) : "l"(p), "l"(pol));
+    if (lane == 0) opexp[I] = e;
+    for (int64_t i = e0 / 4 + lane; i < e1 / 4; i += 32) {  // scalar rows of the blocks
+        const double2 x = make_double2(v[4 * i], v[4 * i + 1]), y = make_double2(v[4 * i + 2], v[4 * i + 3]);
+        if constexpr (F64) {
+            uint32_t w[4];
+            pack_pair(w, x.x, x.y, e);
+            opd[2 * i] = make_uint4(w[0], w[1], w[2], w[3]);
+            pack_pair(w, y.x, y.y, e);
+            opd[2 * i + 1] = make_uint4(w[0], w[1], w[2], w[3]);
+        } else {
+            // 30 bits of the FP64 element (BF16: of the rounded one)
+            const double sc = pow2(29 - e, 0.0);
+            auto q = [&](double z) { return __double2int_rn((round_bf16 ? (double)bf16r((float)z) : z) * sc); };
+            uint32_t w0[2], w1[2];
+            pack_pair(w0, q(x.x), q(x.y));
+            pack_pair(w1, q(y.x), q(y.y));
+            opd[i] = make_uint4(w0[0], w0[1], w1[0], w1[1]);
+        }
     }
 }
 
-__device__ __forceinline__ void ldh16(float (&h)[16], const float *p, uint64_t pol) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-        asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v4.f32 {%0,%1,%2,%3}, [%4], %5;"
-                     : "=f"(h[4 * i]), "=f"(h[4 * i + 1]), "=f"(h[4 * i + 2]), "=f"(h[4 * i + 3])
-                     : "l"(p + 4 * i), "l"(pol));
+template <typename T>
+struct Vec2;
+template <>
+struct Vec2<float> {
+    using V = float2;
+};
+template <>
+struct Vec2<double> {
+    using V = double2;
+};
+
+// A scalar row of an operator block's digits, in one load (an L1 access costs a
+// cycle for each line it touches, and a warp's rows lie in 8 blocks)
+__device__ __forceinline__ void ld_row(uint32_t (&w)[4], const uint4 *opd, uint32_t blk) {
+    const uint4 v = __ldg(opd + (uint64_t)blk * 4);
+    w[0] = v.x;
+    w[1] = v.y;
+    w[2] = v.z;
+    w[3] = v.w;
+}
+__device__ __forceinline__ void ld_row(uint32_t (&w)[8], const uint4 *opd, uint32_t blk) {
+    asm("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+        : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
+        : "l"(opd + (uint64_t)blk * 8));
 }
 
-__device__ __forceinline__ uint32_t ld_stream_u32(const uint32_t *p, uint64_t pol) {
-    uint32_t v;
-    asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.u32 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(pol));
-    return v;
+// The products of one group in plain FP32 / FP64, from the FP64 operator and T_k
+// (R): out[4 j + 2 h + c] for tile j, row half h, column 2t + c, where the mma has
+// them.
+template <typename T>
+__device__ __noinline__ void plain_group(const ColArgs &a, const int32_t *opos, const T *R, const uint32_t *ent, int cnt,
+                                         int lane, T *out) {
+    constexpr int NT = Dig<T>::NT, P = 2 * NT;
+    const int g = lane >> 2, t = lane & 3;
+    for (int i = 0; i < 4 * NT; ++i) out[i] = T(0);
+    for (int e = 0; e < 8 * cnt; ++e) {  // quad e / 8, slot (e / 2) % 4, row half e % 2
+        const uint32_t w = ent[(e >> 3) * COL_CW + ((g >> 2) * 4 + ((e >> 1) & 3)) * 2 + (e & 1)];
+        const uint32_t blk = w >> COL_SLOT_BITS, sl = w & ((1u << COL_SLOT_BITS) - 1u);
+        if (blk == (uint32_t)a.nnzL) continue;
+        for (int m = 0; m < 4; ++m) {
+            T hv = (T)a.Lv[(int64_t)blk * BB + 4 * (g & 3) + m];
+            if constexpr (sizeof(T) == 4) {
+                if (a.round_bf16) hv = bf16r(hv);
+            }
+            for (int j = 0; j < NT; ++j) {
+                const int p = opos[sl * P + 2 * j + (t >> 1)];
+                if (p < 0) continue;
+                const T *x = R + (int64_t)p * BB + 4 * m + 2 * (t & 1);
+                T *o = out + 4 * j + 2 * (e & 1);
+                o[0] = mac(hv, __ldcg(x), o[0]);
+                o[1] = mac(hv, __ldcg(x + 1), o[1]);
+            }
+        }
+    }
 }
 
-template <int P, int NW, int NFP>
-__global__ void __launch_bounds__(NW * 32, 1) k_colstep(const ColArgs a) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    constexpr int D = COL_STAGES;     // operator stages per warp
-    constexpr int NT = NW * 32;
-    constexpr int KG = 32 / P;        // K-groups per warp
-    constexpr int LKG = ilog2(KG);
-    constexpr int EPL = 16 / KG;      // elements of a block per lane after the reduce-scatter
-    constexpr int RQ = 8 / P;         // K-groups per quarter warp
-    constexpr int CPL = 4 / P;        // 16-byte chunks of a staged block copied per lane
+template <typename T>
+__global__ void __launch_bounds__(COL_NW * 32, 1) k_colstep(const __grid_constant__ ColArgs a) {
+    using D = Dig<T>;
+    using V2 = typename Vec2<T>::V;
+    constexpr int NT = D::NT, P = 2 * NT, NTH = COL_NW * 32, NC = 8 * NT;
+    constexpr bool F64 = sizeof(T) == 8;
+    constexpr ColLayout lay = col_layout(P);
+    constexpr int XV = lay.slot_bytes / 16;  // 16-byte chunks of a slot's digits
     constexpr uint32_t SM = (1u << COL_SLOT_BITS) - 1u;
-    static_assert(P == 4, "panel width 4 (rows of at most two columns run on paired lane quads)");
-    __shared__ int64_t s_cb[P + 1];
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ uint32_t s_max[2][NC];
+    __shared__ int s_e[NC];
+    __shared__ float s_cf[NC];  // FP32: 2^e
+    __shared__ int s_slow;
+    __shared__ int s_cb[P + 1];
     __shared__ int s_dslot[P];
-    __shared__ float s_ch[3][MAX_F], s_cl[3][MAX_F];  // coefficients of terms k-1, k, k+1
+    __shared__ float s_ch[3][MAX_F], s_cl[3][MAX_F];
+    __shared__ double s_c[3][MAX_F];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int pid = blockIdx.x;
-    const int j0 = a.panels[4 * pid], nc = a.panels[4 * pid + 1], nu = a.panels[4 * pid + 2];
-    const ColLayout lay = col_layout(nu, P, NW);
-    float *X = reinterpret_cast<float *>(smem + lay.off_x);
+    const int j0 = a.panels[4 * pid], nc = a.panels[4 * pid + 1], nu = a.panels[4 * pid + 2], sys = a.panels[4 * pid + 3];
+    const int n = a.n_terms ? a.n_terms[sys] : a.n_single;
+    if (a.t0 >= n && a.t0 != 2) return;  // this system is done
+    uint4 *X = reinterpret_cast<uint4 *>(smem + lay.off_x);
+    uint32_t *X2 = reinterpret_cast<uint32_t *>(smem + lay.off_x + 256);  // FP32: the third digits, behind the others
     int32_t *opos = reinterpret_cast<int32_t *>(smem + lay.off_pos);
+    int32_t *rexp = reinterpret_cast<int32_t *>(smem + lay.off_rexp);
+    uint2 *srow = reinterpret_cast<uint2 *>(smem + lay.off_rows);
     double *red = reinterpret_cast<double *>(smem + lay.off_red);
+    const double *coef = a.coef ? a.coef + (a.coef_off ? a.coef_off[sys] : 0) : nullptr;
+    double *part = a.part + (int64_t)pid * a.pstride * 2;
 
-    const uint64_t pkeep = policy_keep(), pstream = policy_stream();
-    // 1. gather the panel's columns of T_k
-    if (tid <= P) s_cb[tid] = a.rp[j0 + min(tid, nc)];
+    // --- the panel: column starts, block positions, zero digits
+    if (tid <= P) s_cb[tid] = (int)a.rp[j0 + min(tid, nc)];
     if (tid < P) s_dslot[tid] = -1;
-    if (tid < 3 * MAX_F) {
-        const int j = tid / MAX_F, f = tid % MAX_F;  // term k-1+j
-        const int term = a.term - 2 + j;
-        ff_split(f < a.nf && term >= 0 ? a.coef[(int64_t)f * a.coef_stride + term] : 0.0, s_ch[j][f], s_cl[j][f]);
+    if (tid < 2 * NC) (&s_max[0][0])[tid] = 0u;
+    for (int i = tid; i < nu * XV; i += NTH) {
+        const uint32_t z = !F64 && i % XV >= 16 ? 0x80808080u : 0u;
+        X[i] = make_uint4(z, z, z, z);
     }
-    {
-        float4 *x4 = reinterpret_cast<float4 *>(X);
-        for (int i = tid; i < nu * 4 * P; i += NT) x4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int i = tid; i < nu * P; i += NT) opos[i] = -1;
-    }
+    for (int i = tid; i < nu * P; i += NTH) opos[i] = -1;
+    const int rbase = a.wrow[pid * (COL_NW + 1)];  // the panel's first group
+    for (int i = tid; i < (nu + 3) / 4; i += NTH) srow[i] = reinterpret_cast<const uint2 *>(a.rows)[rbase + i];
     __syncthreads();
-    {
-        const int64_t cb0 = s_cb[0], cb1 = s_cb[nc];
-        for (int64_t b = cb0 + tid; b < cb1; b += NT) {
-            int q = 0;
+    const int cb0 = s_cb[0], cb1 = s_cb[nc];  // (block indexes fit 31 bits)
+    auto col_of = [&](int b) {
+        int q = 0;
 #pragma unroll
-            for (int qq = 1; qq < P; ++qq)
-                if (qq < nc && b >= s_cb[qq]) q = qq;
-            const int s = a.slot[b];
-            float v[16];
-            ldh16(v, a.R + b * BB, pstream);
-            float *xs = X + (size_t)s * 16 * P + 4 * q;
-            const int sw = s & (RQ - 1);
+        for (int qq = 1; qq < P; ++qq)
+            if (qq < nc && b >= s_cb[qq]) q = qq;
+        return q;
+    };
+    for (int b = cb0 + tid; b < cb1; b += NTH) {
+        const int q = col_of(b), s = a.slot[b], K = a.ci[b];
+        opos[s * P + q] = (int32_t)b;
+        rexp[s] = a.opexp[K];
+        if (K == j0 + q) s_dslot[q] = s;
+    }
+
+    // block-wide sums of NV values to dst[0..NV-1] in a fixed order
+    auto reduce_to = [&](auto &v, auto NVc, auto store) {
+        constexpr int NV = decltype(NVc)::value;
 #pragma unroll
-            for (int m = 0; m < 4; ++m)
-                *reinterpret_cast<float4 *>(xs + (m ^ sw) * 4 * P) =
-                    make_float4(v[4 * m], v[4 * m + 1], v[4 * m + 2], v[4 * m + 3]);
-            opos[s * P + q] = (int32_t)b;
-            if (a.ci[b] == j0 + q) s_dslot[q] = s;
+        for (int i = 0; i < NV; ++i) {
+            const double w = warp_sum(v[i]);
+            if (lane == 0) red[warp * NV + i] = w;
         }
+        __syncthreads();
+        if (tid < NV) {
+            double s = 0.0;
+            for (int w = 0; w < COL_NW; ++w) s += red[w * NV + tid];
+            store(tid, s);
+        }
+        __syncthreads();
+    };
+
+    // --- terms 0 and 1: T_0 = I, T_1 = M~, accumulators c_0/2 T_0 + c_1 T_1
+    T *const Tb[2] = {static_cast<T *>(a.T[0]), static_cast<T *>(a.T[1])};
+    if (a.t0 == 2) {
+        double mv[4] = {0.0, 0.0, 0.0, 0.0};  // Tr T_0, <T_0, G>, Tr T_1, <T_1, G>
+        for (int b = cb0 + tid; b < cb1; b += NTH) {
+            const int J = j0 + col_of(b), K = a.ci[b];
+            const int64_t la = find_in_row(a.Lrp, a.Lci, K, J);
+            const int64_t o = (int64_t)a.tperm[b] * BB;
+#pragma unroll 4
+            for (int i = 0; i < 16; ++i) {
+                const bool dg = K == J && (i % 5) == 0;
+                const T v0 = dg ? T(1) : T(0);
+                T v1 = la >= 0 ? (T)a.Lv[la * BB + i] : T(0);
+                if constexpr (!F64) {
+                    if (a.round_bf16) v1 = bf16r(v1);
+                }
+                Tb[0][(int64_t)b * BB + i] = v0;
+                Tb[1][(int64_t)b * BB + i] = v1;
+                const double d0 = (double)v0, d1 = (double)v1;
+                for (int f = 0; f < a.nf; ++f) {
+                    const double *cf = coef + (int64_t)f * a.coef_stride;
+                    const double w = 0.5 * __ldg(cf) * d0 + __ldg(cf + 1) * d1;
+                    if constexpr (F64) a.acc[f][o + i] = w;
+                    else {
+                        float hi, lo;
+                        ff_split(w, hi, lo);
+                        *reinterpret_cast<float2 *>(a.accp[f] + ((int64_t)b * BB + i) * 2) = make_float2(hi, lo);
+                    }
+                }
+                if (a.G) {
+                    const double gval = a.G[o + i];
+                    mv[1] += gval * d0;
+                    mv[3] += gval * d1;
+                    if constexpr (!F64) {
+                        float hi, lo;
+                        ff_split(gval, hi, lo);
+                        *reinterpret_cast<float2 *>(a.Gp + ((int64_t)b * BB + i) * 2) = make_float2(hi, lo);
+                    }
+                }
+                if (dg) {
+                    mv[0] += d0;
+                    mv[2] += d1;
+                }
+            }
+        }
+        if (a.want_mom) reduce_to(mv, std::integral_constant<int, 4>(), [&](int i, double s) { part[i] = s; });
     }
     __syncthreads();
+    const int tend = min(a.t1, n);
+    // largest elements of the columns of T_{t0 - 1}
+    if (a.t0 < tend) {
+        const T *R = Tb[(a.t0 - 1) & 1];
+        for (int b = cb0 + tid; b < cb1; b += NTH) {
+            const int q = col_of(b);
+            uint32_t m[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+            for (int i = 0; i < 16; ++i) m[i & 3] = max(m[i & 3], mag_bits(R[(int64_t)b * BB + i]));
+#pragma unroll
+            for (int c = 0; c < 4; ++c) atomicMax(&s_max[a.t0 & 1][4 * q + c], m[c]);
+        }
+        __syncthreads();
+    }
 
-    // Tr T and <T, G> of terms k-1, k, k+1, double-float partial sums
-    float th[3] = {0.f, 0.f, 0.f}, tl[3] = {0.f, 0.f, 0.f};
-    float gh[3] = {0.f, 0.f, 0.f}, gl[3] = {0.f, 0.f, 0.f};
-    const int q = lane % P, kg = lane / P;
-    const int i0 = kg * EPL;
-    // 16-byte chunk c of a staged block of K-group kg sits at chunk c ^ skw, so
-    // that the K-groups' blocks spread over all banks
-    const int skw = (kg >> 1) & 3;
+    const int g = lane >> 2, t = lane & 3;  // mma row / column lane, slot of the quad
+    const bool opbad = *a.opflag != 0;
 
-    // 2. the warp's chunks.  The plan lays out every warp's work as one stream
-    // of chunks (CW = EK * KG entries, EK per K-group; each row padded with
-    // zero-block entries to whole chunks) and a list of its rows (union slot,
-    // chunk count).  Operator blocks go through a ring of D stages: the copies
-    // of chunk n + D - 1 are issued (cp.async) before chunk n is multiplied.
-    // The entry words come in windows of 32 (32/CW chunks), one word per lane,
-    // four windows deep, and are handed to the K-groups by shuffles.
-    constexpr int EK = COL_EK;        // entries of a K-group per chunk
-    constexpr int CW = EK * KG;       // entries (words, staged blocks) per chunk
-    float *stg = reinterpret_cast<float *>(smem + lay.off_stage) + (size_t)warp * D * CW * 16;
-    const int64_t c0 = a.wchunk[pid * (NW + 1) + warp], c1 = a.wchunk[pid * (NW + 1) + warp + 1];
-    const int r0 = a.wrow[pid * (NW + 1) + warp], r1 = a.wrow[pid * (NW + 1) + warp + 1];
-    const int nch = (int)(c1 - c0);
-    if (nch > 0) {
-        constexpr int WC = 32 / CW;  // chunks per window
-        // Chunk n is always in win0 and chunk n + D - 1, whose operator blocks
-        // are issued while chunk n is multiplied, always in win1, both at
-        // window offset jo = n - n0 (n0: first chunk of win0), so that a
-        // word's source lane is jo * CW + e * KG + kg with no window select.
-        static_assert(D - 1 == WC, "the producer runs exactly one window ahead");
-        const uint32_t *ew = a.ent + c0 * CW;  // words of the warp's chunks
-        const int nw = nch * CW;
-        uint32_t win0 = lane < nw ? ld_stream_u32(ew + lane, pstream) : 0u;
-        uint32_t win1 = 32 + lane < nw ? ld_stream_u32(ew + 32 + lane, pstream) : 0u;
-        uint32_t win2 = 64 + lane < nw ? ld_stream_u32(ew + 64 + lane, pstream) : 0u;
-        uint32_t win3 = 96 + lane < nw ? ld_stream_u32(ew + 96 + lane, pstream) : 0u;
-        // the lane's part of stage st for the chunk whose words are in window
-        // value win at source lanes lb + e * KG: 16-byte chunk c of block
-        // (e, kg) at chunk c ^ skw, so that the K-groups' blocks spread over
-        // all banks
-        auto produce = [&](uint32_t win, int lb, int st, bool live) {
-            uint32_t words[EK];
-#pragma unroll
-            for (int e = 0; e < EK; ++e) words[e] = __shfl_sync(0xffffffffu, win, lb + e * KG);
-            if (live) {
-                float *dst = stg + st * CW * 16;
-#pragma unroll
-                for (int e = 0; e < EK; ++e) {
-                    const float *src = a.Lv + (int64_t)(words[e] >> COL_SLOT_BITS) * BB;
-#pragma unroll
-                    for (int i = 0; i < CPL; ++i)
-                        cp_async16_hint(dst + (e * KG + kg) * 16 + 4 * ((q * CPL + i) ^ skw), src + 4 * (q * CPL + i),
-                                        pkeep);
-                }
+    for (int term = a.t0; term < tend; ++term) {
+        const int par = term & 1;
+        const T *R = Tb[par ^ 1];  // T_{term-1}
+        T *C = Tb[par];            // T_{term-2}, replaced by T_term
+        // terms accumulated by this step: bit i of grp is term - i
+        int grp = 0;
+        if (term == n - 1 || (term >= 4 && (term - 1) % 3 == 0)) grp = (1 << (term - (1 + 3 * ((term - 2) / 3)))) - 1;
+        // 1. grids of the columns and digits of T_{term-1}
+        bool bad = opbad;
+        for (int c = 0; c < NC; ++c) {
+            int e;
+            bad |= !grid_exp<T>(s_max[par][c], D::EX_MIN, D::EX_MAX, e);
+            if (tid == c) {
+                s_e[c] = e;
+                if (!F64) s_cf[c] = pow2(e, 0.f);
             }
-            cp_async_commit();
-        };
+        }
+        if (tid == 0) s_slow = bad;  // (read again by every group: no register to hold it)
+        if (grp && tid < 3 * MAX_F) {
+            const int i = tid / MAX_F, f = tid % MAX_F;  // term - 2 + i
+            const double c = f < a.nf ? coef[(int64_t)f * a.coef_stride + term - 2 + i] : 0.0;
+            s_c[i][f] = c;
+            ff_split(c, s_ch[i][f], s_cl[i][f]);
+        }
+        if (bad && !F64 && tid < NC) s_cf[tid] = 2.f;
+        if (!bad) {
+            for (int b = cb0 + tid; b < cb1; b += NTH) {
+                const int q = col_of(b), s = a.slot[b];
+                T v[16];
+                if constexpr (F64) {
 #pragma unroll
-        for (int i = 0; i < D - 1; ++i) produce(win0, i * CW + kg, i, i < nch);
-        // Rows: union slot s, chunks left cl.  A row with blocks in at most two
-        // of the panel's columns ("half" row) runs with each column on two
-        // lane quads: lane (q, kg) takes column cols[q & 1] and only entry
-        // e = q >> 1 of each chunk (16 K-groups per column), so its chunks
-        // cost half the products.  Lane's column col, its output position pos
-        // (-1: no output from this lane), and the same for the next row.
-        auto row_col = [&](uint32_t w, int &col, int &p) {
-            const int sl = (int)(w & SM);
-            const bool hf = (w >> COL_SLOT_BITS) & 1u;
-            const int ca = (int)((w >> (COL_SLOT_BITS + 1)) & 3u), cb = (int)((w >> (COL_SLOT_BITS + 3)) & 3u);
-            col = hf ? ((q & 1) ? cb : ca) : q;
-            p = opos[sl * P + col];
-            if (hf && ((q >> 1) != 0 || ((q & 1) && cb == ca))) p = -1;
-        };
-        int r = r0;
-        uint32_t rw = a.rows[r], rwn = r + 1 < r1 ? a.rows[r + 1] : 0u, rwm = r + 2 < r1 ? a.rows[r + 2] : 0u;
-        int s = (int)(rw & SM), cl = (int)(rw >> COL_ROW_SHIFT);
-        bool half = (rw >> COL_SLOT_BITS) & 1u;
-        int col, pos, coln = 0, posn = -1;
-        row_col(rw, col, pos);
-        if (r + 1 < r1) row_col(rwn, coln, posn);
-        float tm[EPL], gv[2 * EPL], av[NFP > 0 ? NFP : 1][2 * EPL];
-        auto prefetch_epilogue = [&]() {
+                    for (int i = 0; i < 16; i += 2) {
+                        const double2 u = __ldcg(reinterpret_cast<const double2 *>(R + (int64_t)b * BB + i));
+                        v[i] = u.x;
+                        v[i + 1] = u.y;
+                    }
+                } else {
 #pragma unroll
-            for (int j = 0; j < EPL; ++j) tm[j] = 0.f;
-#pragma unroll
-            for (int j = 0; j < 2 * EPL; ++j) gv[j] = 0.f;
-            if (pos >= 0) {
-                if (a.Rm) ldh<EPL>(tm, a.Rm + (int64_t)pos * BB + i0, pstream);
-                if (a.grp) {
-                    if (a.Gp) ldg_pairs<EPL>(gv, a.Gp + ((int64_t)pos * BB + i0) * 2, pstream);
-#pragma unroll
-                    for (int f = 0; f < NFP; ++f)
-                        if (f < a.nf) ldh_pairs<EPL>(av[f], a.accp[f] + ((int64_t)pos * BB + i0) * 2, pstream);
-                }
-            }
-        };
-        prefetch_epilogue();
-        float acc[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) acc[i] = 0.f;
-        // acc += L_IK X[K][col] for staged block b of stage st and slot tc.
-        // Row m of slot tc's block sits at row m ^ (tc & 1): even rows at
-        // m * 4P + d, odd rows at m * 4P - d, d = (tc & 1) * 4P.
-        static_assert(RQ == 2, "slot swizzle of one bit");
-        const float *xcol = X + 4 * col;  // follows col from row to row
-        auto multiply = [&](const float *hs, uint32_t tc) {
-            float hc[16];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const float4 v = *reinterpret_cast<const float4 *>(hs + 4 * (c ^ skw));
-                hc[4 * c] = v.x; hc[4 * c + 1] = v.y; hc[4 * c + 2] = v.z; hc[4 * c + 3] = v.w;
-            }
-            const int d = (int)(tc & 1u) * 4 * P;
-            const float *xe = xcol + tc * (16 * P) + d, *xo = xcol + tc * (16 * P) - d;
-#pragma unroll
-            for (int m = 0; m < 4; ++m) {
-                const float4 x = *reinterpret_cast<const float4 *>((m & 1 ? xo : xe) + m * 4 * P);
-#pragma unroll
-                for (int rr = 0; rr < 4; ++rr) {
-                    acc[4 * rr + 0] = fmaf(hc[4 * rr + m], x.x, acc[4 * rr + 0]);
-                    acc[4 * rr + 1] = fmaf(hc[4 * rr + m], x.y, acc[4 * rr + 1]);
-                    acc[4 * rr + 2] = fmaf(hc[4 * rr + m], x.z, acc[4 * rr + 2]);
-                    acc[4 * rr + 3] = fmaf(hc[4 * rr + m], x.w, acc[4 * rr + 3]);
-                }
-            }
-        };
-        // n0: first chunk of win0; lb = (n - n0) * CW + kg; sc, ps: stages of
-        // chunks n and n + D - 1
-        int n0 = 0, lb = kg, sc = 0, ps = D - 1;
-        for (int n = 0; n < nch; ++n) {
-            produce(win1, lb, ps, n + D - 1 < nch);
-            cp_async_wait<D - 1>();
-            __syncwarp();
-            const float *st = stg + sc * CW * 16 + kg * 16;
-            if (!half) {
-#pragma unroll
-                for (int e = 0; e < EK; ++e)
-                    multiply(st + e * KG * 16, __shfl_sync(0xffffffffu, win0, lb + e * KG) & SM);
-            } else {
-                const int e = q >> 1;
-                const uint32_t wv = __shfl_sync(0xffffffffu, win0, lb + e * KG);
-                multiply(st + e * KG * 16, wv & SM);
-            }
-            __syncwarp();
-            sc = sc + 1 == D ? 0 : sc + 1;
-            ps = ps + 1 == D ? 0 : ps + 1;
-            lb += CW;
-            if (n + 1 - n0 == WC) {
-                // the next window: shift, and fetch the one three windows ahead
-                n0 += WC;
-                lb = kg;
-                win0 = win1;
-                win1 = win2;
-                win2 = win3;
-                const int e = (n0 + 3 * WC) * CW + lane;
-                win3 = e < nw ? ld_stream_u32(ew + e, pstream) : 0u;
-            }
-            if (--cl == 0) {
-                // 3. the row is done: combine the K-groups (a half row's two
-                // lane quads per column first), reduce-scatter, then finish
-                // the lane's elements of block (row s, column col).  The
-                // accumulators NFP, NFP + 1 (not prefetched at the row's start)
-                // are loaded first, so that the reduce-scatter's shuffles
-                // cover part of their latency.
-                constexpr int NL = NFP > 0 ? 1 : 0;
-                float lv[NL > 0 ? NL : 1][2 * EPL];
-                if (NL > 0 && a.grp && pos >= 0) {
-#pragma unroll
-                    for (int f = 0; f < NL; ++f)
-                        if (NFP + f < a.nf)
-                            ldh_pairs<EPL>(lv[f], a.accp[NFP + f] + ((int64_t)pos * BB + i0) * 2, pstream);
-                }
-                if (half) {
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], P / 2);
-                }
-#pragma unroll
-                for (int l = 0; l < LKG; ++l) {
-                    const int nn = 8 >> l;
-                    const int off = P << (LKG - 1 - l);
-                    const bool hi = (kg >> (LKG - 1 - l)) & 1;
-#pragma unroll
-                    for (int j = 0; j < nn; ++j) {
-                        const float mine = hi ? acc[nn + j] : acc[j], other = hi ? acc[j] : acc[nn + j];
-                        acc[j] = mine + __shfl_xor_sync(0xffffffffu, other, off);
+                    for (int i = 0; i < 16; i += 4) {
+                        const float4 u = __ldcg(reinterpret_cast<const float4 *>(R + (int64_t)b * BB + i));
+                        v[i] = u.x;
+                        v[i + 1] = u.y;
+                        v[i + 2] = u.z;
+                        v[i + 3] = u.w;
                     }
                 }
-                if (pos >= 0) {
-                    float y[EPL];
+                uint4 *xs = X + s * XV;
+                const int sw = 2 * (s & 3);
 #pragma unroll
-                    for (int j = 0; j < EPL; ++j) {
-                        y[j] = a.Rm ? a.alpha * acc[j] + a.beta * tm[j] : a.alpha * acc[j];
-                        if (a.round_bf16) y[j] = bf16r(y[j]);
+                for (int c = 0; c < 4; ++c) {
+                    int e;
+                    grid_exp<T>(s_max[par][4 * q + c], D::EX_MIN, D::EX_MAX, e);
+                    const int col = (4 * q + c) & 7, tile = (4 * q + c) >> 3;
+                    if constexpr (F64) {
+                        uint32_t w0[6], w1[6];
+                        panel_digits(w0, v[c], v[4 + c], e);
+                        panel_digits(w1, v[8 + c], v[12 + c], e);
+#pragma unroll
+                        for (int i = 0; i < 3; ++i)
+                            xs[8 * i + (col ^ sw)] = make_uint4(w0[2 * i], w1[2 * i], w0[2 * i + 1], w1[2 * i + 1]);
+                    } else {
+                        uint32_t w0[2], w1[2], b0, b1;
+                        panel_digits(w0, b0, grid_value(v[c], e), grid_value(v[4 + c], e));
+                        panel_digits(w1, b1, grid_value(v[8 + c], e), grid_value(v[12 + c], e));
+                        xs[8 * tile + (col ^ sw)] = make_uint4(w0[0], w1[0], w0[1], w1[1]);
+                        X2[s * 4 * XV + ((4 * q + c) ^ (8 * ((s >> 1) & 1)))] = b0 | (b1 << 16);
                     }
-                    sth<EPL>(a.C + (int64_t)pos * BB + i0, y, pstream);
-                    if (a.grp) {
-                        // the group's terms in order: T_{k-1} (tm), T_k (the
-                        // panel's copy in shared memory), T_{k+1} (y)
-                        float tv[3][EPL];
-                        {
-                            const int rr = i0 / 4, sws = s & (RQ - 1);
-                            const float *xk = X + (size_t)s * 16 * P + (rr ^ sws) * 4 * P + 4 * col + (i0 % 4);
+                }
+            }
+        }
+        __syncthreads();
+        if (tid < NC) s_max[par][tid] = 0u;  // next written by the step after the next
+
+        // 2. the warp's groups
+        uint32_t mx[NT][2];
+        float gh = 0.f, gl = 0.f;  // <T, G>: FP32 as a double-float pair
+        double gd = 0.0;
 #pragma unroll
-                            for (int j = 0; j < EPL; ++j) {
-                                tv[0][j] = tm[j];
-                                tv[1][j] = xk[j];
-                                tv[2][j] = y[j];
-                            }
-                        }
+        for (int j = 0; j < NT; ++j) mx[j][0] = mx[j][1] = 0u;
+        const int c0w = __ldg(a.wchunk + pid * (COL_NW + 1) + warp);
+        const int r0w = __ldg(a.wrow + pid * (COL_NW + 1) + warp) - rbase, r1w = __ldg(a.wrow + pid * (COL_NW + 1) + warp + 1) - rbase;
+        if (r0w < r1w) {
+            // operator digits of a quad, rows g (half 0) and g + 8 (half 1)
+            struct Op {
+                uint32_t w[2][F64 ? 8 : 4];
+            };
+            const uint4 *ob = a.opd + (g & 3) * (F64 ? 2 : 1);
+            auto load_h = [&](Op &o, uint2 w) {
+                ld_row(o.w[0], ob, w.x >> COL_SLOT_BITS);
+                ld_row(o.w[1], ob, w.y >> COL_SLOT_BITS);
+            };
+            // Two quads are on their way: quads go in pairs (even / odd) through two
+            // register sets, each refilled two quads ahead as soon as its digits are
+            // taken, its words four ahead (the lists end in padding).
+            const uint2 *ep = reinterpret_cast<const uint2 *>(a.ent) + (int64_t)c0w * 8 + ((g >> 2) * 4 + t);
+            uint2 wc[2] = {__ldg(ep), __ldg(ep + 8)}, wn[2] = {__ldg(ep + 16), __ldg(ep + 24)};
+            Op h[2];
+            load_h(h[0], wc[0]);
+            load_h(h[1], wc[1]);
+            ep += 32;
+            int qi = 0;
+            for (int r = r0w; r < r1w; ++r) {
+                const uint2 rw = srow[r];
+                const bool slow = *(volatile int *)&s_slow != 0;
+                const int cnt = (int)(rw.y >> COL_SLOT_BITS);
+                // sums of the group: rows g, g + 8 x columns 2t, 2t + 1 of each tile
+                float dl[NT][2][4];      // digit sums kept in the accumulators (FP32: D_1, D_2; FP64: D_4, D_5)
+                float fs[NT][4];         // FP32: the exact leading sums added up
+                int is[4][4];            // FP64: the four exact digit sums
 #pragma unroll
-                        for (int f = 0; f < MAX_F; ++f) {
-                            if (f < a.nf) {
-                                float v[2 * EPL];
-                                float *pa = a.accp[f] + ((int64_t)pos * BB + i0) * 2;
-                                if (f < NFP) {
+                for (int j = 0; j < NT; ++j)
 #pragma unroll
-                                    for (int j = 0; j < 2 * EPL; ++j) v[j] = av[f < NFP ? f : 0][j];
-                                } else if (f < NFP + NL) {
+                    for (int i = 0; i < 4; ++i) {
+                        fs[j][i] = 0.f;
 #pragma unroll
-                                    for (int j = 0; j < 2 * EPL; ++j) v[j] = lv[f < NFP + NL ? f - NFP : 0][j];
-                                } else {
-                                    ldh_pairs<EPL>(v, pa, pstream);
+                        for (int s = 0; s < 2; ++s) dl[j][s][i] = 0.f;
+                    }
+#pragma unroll
+                for (int s = 0; s < 4; ++s)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) is[s][i] = 0;
+                if (!slow) {
+#pragma unroll 1
+                    for (int k = 0; k < cnt; k += 2) {
+                        float z[NT][F64 ? 4 : 1][4];  // exact sums of the pair
+#pragma unroll
+                        for (int o = 0; o < 2; ++o) {
+                            const int sl = (int)(wc[o].x & SM);
+                            const uint4 *xs = X + sl * XV + (g ^ (2 * (sl & 3)));
+                            wc[o] = wn[o];
+                            wn[o] = __ldg(ep + o * 8);
+                            const float zero[4] = {0.f, 0.f, 0.f, 0.f};
+                            if constexpr (!F64) {
+                                uint32_t A0[4], A1[4], A2[4];
+#pragma unroll
+                                for (int i = 0; i < 4; ++i) {  // (half i % 2, pair i / 2)
+                                    const uint32_t u = h[o].w[i & 1][i & 2], v = h[o].w[i & 1][(i & 2) + 1];
+                                    A0[i] = f16_digits(u & 0x03ff03ffu);
+                                    A1[i] = f16_digits(v & 0x03ff03ffu);
+                                    A2[i] = spread_digit(u, v);
                                 }
+                                load_h(h[o], wc[o]);
+                                const uint32_t *x2 = X2 + sl * 4 * XV;
+                                const int g2 = g ^ (8 * ((sl >> 1) & 1));
 #pragma unroll
-                                for (int t3 = 0; t3 < 3; ++t3)
-                                    if ((a.grp >> (2 - t3)) & 1) {
+                                for (int j = 0; j < NT; ++j) {
+                                    const uint4 xw = xs[8 * j];
+                                    const uint32_t xb = x2[g2 ^ (8 * j)];
+                                    const uint32_t B0[2] = {xw.x, xw.y}, B1[2] = {xw.z, xw.w};
+                                    const uint32_t B2[2] = {third_digits<0x4140>(xb), third_digits<0x4342>(xb)};
+                                    // (the leading sums of two quads, below 2^24, are exact)
+                                    if (o == 0) mma16816(z[j][0], A0, B0, zero);
+                                    else mma16816(z[j][0], A0, B0, z[j][0]);
+                                    mma16816(dl[j][0], A0, B1, dl[j][0]);
+                                    mma16816(dl[j][1], A0, B2, dl[j][1]);
+                                    mma16816(dl[j][0], A1, B0, dl[j][0]);
+                                    mma16816(dl[j][1], A1, B1, dl[j][1]);
+                                    mma16816(dl[j][1], A2, B0, dl[j][1]);
+                                    if (o == 1) {
 #pragma unroll
-                                        for (int j = 0; j < EPL; ++j)
-                                            ff_add_prod(v[2 * j], v[2 * j + 1], tv[t3][j], s_ch[t3][f], s_cl[t3][f]);
+                                        for (int i = 0; i < 4; ++i) fs[j][i] += z[j][0][i];
                                     }
-                                sth_pairs<EPL>(pa, v, pstream);
+                                }
+                            } else {
+                                const uint4 x0 = xs[0], x1 = xs[8], x2 = xs[16];
+                                const uint32_t B[6][2] = {{x0.x, x0.y}, {x0.z, x0.w}, {x1.x, x1.y},
+                                                          {x1.z, x1.w}, {x2.x, x2.y}, {x2.z, x2.w}};
+#pragma unroll
+                                for (int i = 0; i < 6; ++i) {
+                                    uint32_t A[4];
+#pragma unroll
+                                    for (int k2 = 0; k2 < 4; ++k2) {  // (half k2 % 2, pair k2 / 2)
+                                        const uint32_t *hw = h[o].w[k2 & 1] + 2 * (k2 & 2);
+                                        const uint32_t pw[4] = {hw[0], hw[1], hw[F64 ? 2 : 0], hw[F64 ? 3 : 0]};
+                                        A[k2] = packed_digit(pw, i);
+                                    }
+#pragma unroll
+                                    for (int s = i; s < 6; ++s) {
+                                        if (s >= 4) mma16816(dl[0][s & 1], A, B[s - i], dl[0][s & 1]);
+                                        else if (i == 0 && (o == 0 || s >= 2)) mma16816(z[0][F64 ? s : 0], A, B[s], zero);
+                                        else mma16816(z[0][F64 ? s : 0], A, B[s - i], z[0][F64 ? s : 0]);
+                                    }
+                                    // (the sums of s = 0, 1 stay exact over two quads)
+                                    if (i >= 1) {  // D_6 into D_5's accumulator: the panel digit times 2^-10
+                                        const uint32_t Bs[2] = {h2_fma(B[6 - i][0], 0x14001400u, 0u), h2_fma(B[6 - i][1], 0x14001400u, 0u)};
+                                        mma16816(dl[0][1], A, Bs, dl[0][1]);
+                                    }
+                                    if (i < 4 && (o == 1 || i >= 2)) {
+#pragma unroll
+                                        for (int e = 0; e < 4; ++e) is[i][e] += __float2int_rn(z[0][F64 ? i : 0][e]);
+                                    }
+                                }
+                                load_h(h[o], wc[o]);
                             }
                         }
-                        const bool diag = s == s_dslot[col];
+                        ep += 16;
+                    }
+                    // the digit sums as one value, in fs (FP32) or as the two halves
+                    // of a double in is[0], is[1]
 #pragma unroll
-                        for (int t3 = 0; t3 < 3; ++t3)
-                            if ((a.grp >> (2 - t3)) & 1) {
+                    for (int j = 0; j < NT; ++j)
 #pragma unroll
-                                for (int j = 0; j < EPL; ++j) {
-                                    ff_add_prod(gh[t3], gl[t3], tv[t3][j], gv[2 * j], gv[2 * j + 1]);
-                                    // diagonal elements 0, 5, 10, 15 of a diagonal block
-                                    if (diag && (i0 + j) % 5 == 0) ff_add_prod(th[t3], tl[t3], tv[t3][j], 1.f, 0.f);
+                        for (int i = 0; i < 4; ++i) {
+                            if constexpr (F64) {
+                                const int64_t q = (((int64_t)is[0][i] * 1024 + is[1][i]) * 1024 + is[2][i]) * 1024 + is[3][i];
+                                const double v = (double)q + (double)fmaf(dl[0][1][i], 0x1p-20f, dl[0][0][i] * 0x1p-10f);
+                                is[0][i] = __double2hiint(v);
+                                is[1][i] = __double2loint(v);
+                            } else {
+                                fs[j][i] = fmaf(fmaf(dl[j][1][i], 0x1p-10f, dl[j][0][i]), 0x1p-10f, fs[j][i]);
+                            }
+                        }
+                } else {
+                    // plain products (a call, so that they take no registers from the above)
+                    T val[4 * NT];
+                    plain_group<T>(a, opos, R, reinterpret_cast<const uint32_t *>(a.ent) + ((int64_t)c0w + qi) * COL_CW, cnt, lane, val);
+                    qi += cnt;
+#pragma unroll
+                    for (int j = 0; j < NT; ++j)
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            if constexpr (F64) {
+                                is[0][i] = __double2hiint(val[i]);
+                                is[1][i] = __double2loint(val[i]);
+                            } else {
+                                fs[j][i] = val[4 * j + i];
+                            }
+                        }
+                }
+                // 3. the lane's elements: rows of atoms g/4 and g/4 + 2, scalar row
+                // g % 4, block column 2 j + t/2, scalar columns 2 (t % 2) and + 1
+                const int sl2[2] = {(int)((g >> 2) == 0 ? rw.x & SM : (rw.x >> COL_SLOT_BITS) & SM),
+                                    (int)((g >> 2) == 0 ? (rw.x >> (2 * COL_SLOT_BITS)) & SM : rw.y & SM)};
+                const int eo = 4 * (g & 3) + 2 * (t & 1);
+#pragma unroll
+                for (int hh = 0; hh < 2; ++hh) {
+                    if (sl2[hh] == (int)SM) continue;
+                    const int er = rexp[sl2[hh]];
+                    const float rf = F64 || slow ? 1.f : pow2(er - 18, 0.f);  // (two exact factors)
+                    // T_{term-2}, G and, in group steps, T_{term-1}, of the half's positions
+                    using GV = typename std::conditional<F64, double2, float4>::type;
+                    int pos[NT];
+                    V2 tm[NT], tk[NT];
+                    GV gv[NT];
+#pragma unroll
+                    for (int j = 0; j < NT; ++j) {
+                        pos[j] = opos[sl2[hh] * P + 2 * j + (t >> 1)];
+                        tm[j] = tk[j] = V2{};
+                        gv[j] = GV{};
+                        if (pos[j] < 0) continue;
+                        const int64_t off = (int64_t)pos[j] * BB + eo;
+                        tm[j] = __ldcg(reinterpret_cast<const V2 *>(C + off));
+                        if (a.G) {
+                            if constexpr (F64) gv[j] = __ldg(reinterpret_cast<const double2 *>(a.G + (int64_t)a.tperm[pos[j]] * BB + eo));
+                            else gv[j] = __ldcg(reinterpret_cast<const float4 *>(a.Gp + off * 2));
+                        }
+                        if (grp) tk[j] = __ldcg(reinterpret_cast<const V2 *>(R + off));
+                    }
+#pragma unroll
+                    for (int j = 0; j < NT; ++j) {
+                        T y[2];
+#pragma unroll
+                        for (int cc = 0; cc < 2; ++cc) {
+                            const int i = 2 * hh + cc;
+                            T v, sc;
+                            if constexpr (F64) {
+                                v = __hiloint2double(is[0][i], is[1][i]);
+                                sc = pow2(slow ? 1 : er + s_e[8 * j + 2 * t + cc] - 47, 0.0);
+                            } else {
+                                v = fs[j][i] * rf;
+                                sc = s_cf[8 * j + 2 * t + cc];
+                            }
+                            y[cc] = mac(v, sc, cc ? -tm[j].y : -tm[j].x);
+                            if constexpr (!F64) {
+                                if (a.round_bf16) y[cc] = bf16r(y[cc]);
+                            }
+                        }
+                        const int p = pos[j];
+                        if (p >= 0) {
+                            const int64_t off = (int64_t)p * BB + eo;
+                            V2 u;
+                            u.x = y[0];
+                            u.y = y[1];
+                            *reinterpret_cast<V2 *>(C + off) = u;
+                            mx[j][0] = max(mx[j][0], mag_bits(y[0]));
+                            mx[j][1] = max(mx[j][1], mag_bits(y[1]));
+                            if constexpr (F64) {
+                                gd += gv[j].x * y[0] + gv[j].y * y[1];
+                            } else {
+                                ff_add_prod(gh, gl, y[0], gv[j].x, gv[j].y);
+                                ff_add_prod(gh, gl, y[1], gv[j].z, gv[j].w);
+                            }
+                            if (grp) {
+                                // the group's terms in order: T_{term-2}, T_{term-1}, T_term
+                                const T tv[3][2] = {{tm[j].x, tm[j].y}, {tk[j].x, tk[j].y}, {y[0], y[1]}};
+                                const int64_t oc = F64 ? (int64_t)a.tperm[p] * BB + eo : 0;
+                                for (int f = 0; f < a.nf; ++f) {
+                                    if constexpr (F64) {
+                                        double2 v = *reinterpret_cast<double2 *>(a.acc[f] + oc);
+#pragma unroll
+                                        for (int i = 0; i < 3; ++i)
+                                            if ((grp >> (2 - i)) & 1) {
+                                                v.x += s_c[i][f] * tv[i][0];
+                                                v.y += s_c[i][f] * tv[i][1];
+                                            }
+                                        *reinterpret_cast<double2 *>(a.acc[f] + oc) = v;
+                                    } else {
+                                        float *pa = a.accp[f] + off * 2;
+                                        float4 v = __ldcg(reinterpret_cast<const float4 *>(pa));
+#pragma unroll
+                                        for (int i = 0; i < 3; ++i)
+                                            if ((grp >> (2 - i)) & 1) {
+                                                ff_add_prod(v.x, v.y, tv[i][0], s_ch[i][f], s_cl[i][f]);
+                                                ff_add_prod(v.z, v.w, tv[i][1], s_ch[i][f], s_cl[i][f]);
+                                            }
+                                        *reinterpret_cast<float4 *>(pa) = v;
+                                    }
                                 }
                             }
+                        }
                     }
                 }
-#pragma unroll
-                for (int i = 0; i < 16; ++i) acc[i] = 0.f;
-                // the next row of this warp
-                if (++r < r1) {
-                    // row words are fetched two rows ahead, so that the next
-                    // row's output position is known without waiting
-                    rw = rwn;
-                    rwn = rwm;
-                    rwm = r + 2 < r1 ? a.rows[r + 2] : 0u;
-                    s = (int)(rw & SM);
-                    cl = (int)(rw >> COL_ROW_SHIFT);
-                    half = (rw >> COL_SLOT_BITS) & 1u;
-                    col = coln;
-                    xcol = X + 4 * col;
-                    pos = posn;
-                    if (r + 1 < r1) row_col(rwn, coln, posn);
-                    else posn = -1;
-                    prefetch_epilogue();
-                }
             }
         }
-        cp_async_wait<0>();
-    }
-    // 4. the moment partials of the panel
-    if (a.grp && (a.mom || a.gmom)) {
-        auto on = [&](int t3) { return (a.grp >> (2 - t3)) & 1; };
-        Moments<6> mm{{(double)th[0] + (double)tl[0], (double)th[1] + (double)tl[1], (double)th[2] + (double)tl[2],
-                       (double)gh[0] + (double)gl[0], (double)gh[1] + (double)gl[1], (double)gh[2] + (double)gl[2]},
-                      {a.mom && on(0) ? a.mom - 2 : nullptr, a.mom && on(1) ? a.mom - 1 : nullptr,
-                       a.mom && on(2) ? a.mom : nullptr, a.gmom && on(0) ? a.gmom - 2 : nullptr,
-                       a.gmom && on(1) ? a.gmom - 1 : nullptr, a.gmom && on(2) ? a.gmom : nullptr}};
-        finish_moments<NT, 6>(a.part, a.counter, mm, red);
-    }
-}
-
-// Terms 0 and 1 in column order: T_0 = I and T_1 = M~ (FP32, bfloat16-rounded
-// in BF16 mode), the accumulators c_0/2 T_0 + c_1 T_1 as (hi, lo) pairs in
-// column order, G as pairs in column order, moments of both terms.
-template <int NT>
-__global__ void __launch_bounds__(NT) k_colinit(const int64_t *rp, const int32_t *ci, const int32_t *tperm,
-                                               int64_t nbr, int64_t nnzb, const int64_t *Lrp, const int32_t *Lci,
-                                               const double *Mt, float *T0, float *T1, int32_t nf, ColArgs a,
-                                               float *Gp, double *mom, double *gmom) {
-    __shared__ double red[(NT / 32) * 4];
-    double c0[MAX_F], c1[MAX_F];
+        // the columns' largest elements, for the next step's grids
 #pragma unroll
-    for (int f = 0; f < MAX_F; ++f) {
-        c0[f] = f < nf ? a.coef[(int64_t)f * a.coef_stride + 0] : 0.0;
-        c1[f] = f < nf ? a.coef[(int64_t)f * a.coef_stride + 1] : 0.0;
-    }
-    double t0 = 0.0, t1 = 0.0, g0 = 0.0, g1 = 0.0;
-    for (int64_t b = blockIdx.x * (int64_t)NT + threadIdx.x; b < nnzb; b += (int64_t)gridDim.x * NT) {
-        const int64_t J = row_of(rp, nbr, b);  // column of column-order block b
-        const int K = ci[b];                   // its row
-        const int64_t la = find_in_row(Lrp, Lci, K, (int32_t)J);
-        const int64_t o = (int64_t)tperm[b] * BB;
+        for (int j = 0; j < NT; ++j)
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const float v0 = (K == J && (i % 5) == 0) ? 1.f : 0.f;
-            float v1 = la >= 0 ? (float)Mt[la * BB + i] : 0.f;
-            if (a.round_bf16) v1 = bf16r(v1);
-            T0[b * BB + i] = v0;
-            T1[b * BB + i] = v1;
-            const double d0 = (double)v0, d1 = (double)v1;
+            for (int cc = 0; cc < 2; ++cc) {
+                uint32_t m = mx[j][cc];
 #pragma unroll
-            for (int f = 0; f < MAX_F; ++f)
-                if (f < nf) {
-                    float hi, lo;
-                    ff_split(0.5 * c0[f] * d0 + c1[f] * d1, hi, lo);
-                    a.accp[f][(b * BB + i) * 2] = hi;
-                    a.accp[f][(b * BB + i) * 2 + 1] = lo;
-                }
-            if (a.G) {
-                const double gval = a.G[o + i];
-                g0 += gval * d0;
-                g1 += gval * d1;
-                float hi, lo;
-                ff_split(gval, hi, lo);
-                Gp[(b * BB + i) * 2] = hi;
-                Gp[(b * BB + i) * 2 + 1] = lo;
+                for (int o = 4; o < 32; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+                if (g == 0) atomicMax(&s_max[par ^ 1][8 * j + 2 * t + cc], m);
             }
-            if (K == J && (i % 5) == 0) {
-                t0 += d0;
-                t1 += d1;
+        // 4. the panel's moments of this term: the warps' parts of <T, G>, and the
+        // trace from the diagonal blocks
+        if (a.want_mom) {
+            const double w = warp_sum(F64 ? gd : (double)gh + (double)gl);
+            if (lane == 0) red[warp] = w;
+        }
+        __syncthreads();
+        if (a.want_mom && warp == 0) {
+            double tr = 0.0;
+            if (lane < 4 * nc) {
+                const int q = lane >> 2, p = opos[s_dslot[q] * P + q];
+                tr = (double)__ldcg(C + (int64_t)p * BB + 5 * (lane & 3));
+            }
+            tr = warp_sum(tr);
+            const double gs = warp_sum(lane < COL_NW ? red[lane] : 0.0);
+            if (lane == 0) {
+                part[(int64_t)(term - a.tbase) * 2] = tr;
+                part[(int64_t)(term - a.tbase) * 2 + 1] = gs;
             }
         }
     }
-    Moments<4> mm{{t0, t1, g0, g1}, {mom, mom ? mom + 1 : nullptr, gmom, gmom ? gmom + 1 : nullptr}};
-    finish_moments<NT, 4>(a.part, a.counter, mm, red);
+    // the FP32 accumulators back to the caller: FP64, BCSR order
+    if constexpr (!F64) {
+        if (a.t1 >= n) {
+            for (int64_t e = (int64_t)cb0 * BB + tid; e < (int64_t)cb1 * BB; e += NTH) {
+                const int64_t o = (int64_t)a.tperm[e / BB] * BB + e % BB;
+                for (int f = 0; f < a.nf; ++f) {
+                    const float2 v = __ldcg(reinterpret_cast<const float2 *>(a.accp[f]) + e);
+                    a.acc[f][o] = (double)v.x + (double)v.y;
+                }
+            }
+        }
+    }
 }
 
-// The accumulators back to the caller: acc_f (BCSR order, FP64) = hi + lo.
-__global__ void k_colfinal(const int32_t *tperm, int64_t nnzb, int32_t nf, ColArgs a) {
-    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;  // element of a column-order block
-    if (e >= nnzb * BB) return;
-    const int64_t b = e / BB, i = e % BB;
-    const int64_t o = (int64_t)tperm[b] * BB + i;
-    for (int f = 0; f < nf; ++f) a.acc[f][o] = (double)a.accp[f][2 * e] + (double)a.accp[f][2 * e + 1];
+// mom[sys * stride + k] = sum over the system's panels of the partials of
+// terms tbase .. tbase + nt - 1, in a fixed order: one thread block per term and
+// system.
+__global__ void __launch_bounds__(128) k_colmom(const double *part, int pstride, int tbase, int nt, const int32_t *sys_panel,
+                                                const int32_t *n_terms, int n_single, int64_t mom_stride, double *mom,
+                                                double *gmom) {
+    __shared__ double sh[4];
+    const int k = blockIdx.x, sy = blockIdx.y, n = n_terms ? n_terms[sy] : n_single;
+    if (tbase + k >= n) return;
+    double t = 0.0, g = 0.0;
+    for (int p = sys_panel[sy] + threadIdx.x; p < sys_panel[sy + 1]; p += 128) {
+        const double2 v = *reinterpret_cast<const double2 *>(part + ((int64_t)p * pstride + k) * 2);
+        t += v.x;
+        g += v.y;
+    }
+    t = block_sum<128>(t, sh);
+    g = block_sum<128>(g, sh);
+    if (threadIdx.x == 0) {
+        if (mom) mom[sy * mom_stride + tbase + k] = t;
+        if (gmom) gmom[sy * mom_stride + tbase + k] = g;
+    }
 }
 
-constexpr int COLINIT_BLOCKS = 1024;
-
-template <int NFP>
-static int launch_colstep(const cheb_plan *plan, const ColArgs &a, cudaStream_t s) {
-    const ColLists &c = plan->col;
-    const ColLayout lay = col_layout(c.max_union, COL_P, COL_NW);
-    auto fn = k_colstep<COL_P, COL_NW, NFP>;
-    CHEB_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lay.total));
-    fn<<<(unsigned)c.n_panels, COL_NW * 32, lay.total, s>>>(a);
-    return check_launch("k_colstep");
-}
-
-static int run_colstep(const cheb_plan *plan, const ColArgs &a, cudaStream_t s) {
-    if (a.nf == 0) return launch_colstep<0>(plan, a, s);
-    if (a.nf == 1) return launch_colstep<1>(plan, a, s);
-    return launch_colstep<2>(plan, a, s);
-}
+// Steps per launch: a multiple of 3 (the accumulation groups), enough that the
+// per-launch set-up of a panel (positions, zero digits) and the last wave of
+// panels cost little, few enough that the moment table stays small.
+constexpr int COL_STEPS = 96;
 
 bool col_usable(const cheb_plan *plan, const cheb_bsr *Mt) {
-    return plan->precision != CHEB_F64 && plan->col.bound && plan->op_rp == Mt->row_ptr &&
-           plan->op_ci == Mt->col_idx;
+    return plan->col.bound && plan->op_rp == Mt->row_ptr && plan->op_ci == Mt->col_idx && plan->col.nnzL == Mt->nnzb;
+}
+
+bool col_takes(const cheb_plan *plan, const cheb_bsr *Mt, const ColExpand &x, size_t ws_bytes) {
+    if (!col_usable(plan, Mt) || ws_bytes < col_expand_ws(plan, Mt->nnzb)) return false;
+    if (!wide_elements(plan->precision)) return true;
+    // FP64 reads and writes the caller's accumulators and G in pairs
+    uintptr_t at = x.gmoments ? reinterpret_cast<uintptr_t>(x.G) : 0;
+    for (int f = 0; f < x.nf; ++f) at |= reinterpret_cast<uintptr_t>(x.acc[f]);
+    return at % 16 == 0;
 }
 
 size_t col_expand_ws(const cheb_plan *plan, int64_t nnzL) {
-    size_t b = 3 * align_up(plan->nnzb * BB * 4) + align_up((nnzL + 1) * BB * 4);
-    b += (MAX_F + 1) * align_up(plan->nnzb * BB * 8);  // accumulators and G as float pairs
-    b += align_up((size_t)std::max<int64_t>(plan->col.n_panels, COLINIT_BLOCKS) * 6 * sizeof(double)) + align_up(64);
+    const bool wide = wide_elements(plan->precision);
+    const size_t esz = wide ? 8 : 4;
+    size_t b = 2 * align_up(plan->nnzb * BB * esz);
+    b += align_up((size_t)(nnzL + 1) * (wide ? 128 : 64));
+    if (!wide) b += (MAX_F + 1) * align_up(plan->nnzb * BB * 8);  // accumulators and G as float pairs
+    b += align_up(plan->nbr * 4) + align_up(64);
+    b += align_up((size_t)plan->col.n_panels * (COL_STEPS + 2) * 2 * sizeof(double));
     return b + 256;
 }
 
-__global__ void k_to_f32_col(const double *in, float *out, int64_t n, int round_bf16) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n) out[i] = round_bf16 ? __bfloat162float(__float2bfloat16_rn(in[i])) : (float)in[i];
-}
-
-int col_expand(const cheb_plan *plan, const cheb_bsr *Mt, int32_t n_terms, const double *coeffs, int32_t stride,
-               int32_t nf, double *const *acc, double *moments, const double *G, double *gmoments, void *ws,
-               size_t ws_bytes, cudaStream_t s, int round_bf16) {
-    if (ws_bytes < col_expand_ws(plan, Mt->nnzb))
-        return fail(CHEB_ERR_NOSPACE, "cheb_expand_stepwise: workspace %zu < %zu", ws_bytes,
-                    col_expand_ws(plan, Mt->nnzb));
+template <typename T>
+static int col_expand_t(const cheb_plan *plan, const cheb_bsr *Mt, const ColExpand &x, void *ws, size_t ws_bytes,
+                        cudaStream_t s) {
     Carve cv(ws, ws_bytes);
-    float *buf[3];
-    for (int i = 0; i < 3; ++i) buf[i] = cv.take<float>(plan->nnzb * BB);
-    float *lv = cv.take<float>((Mt->nnzb + 1) * BB);  // + the zero block of the padding entries
-    float *accp[MAX_F];
-    for (int f = 0; f < MAX_F; ++f) accp[f] = cv.take<float>(plan->nnzb * BB * 2);
-    float *Gp = cv.take<float>(plan->nnzb * BB * 2);
-    double *part = cv.take<double>((size_t)std::max<int64_t>(plan->col.n_panels, COLINIT_BLOCKS) * 6);
-    int32_t *counter = cv.take<int32_t>(16);
-    if (!cv.fits()) return fail(CHEB_ERR_NOSPACE, "cheb_expand_stepwise: workspace too small");
-    {
-        const int64_t n = Mt->nnzb * BB;
-        k_to_f32_col<<<(unsigned)((n + 255) / 256), 256, 0, s>>>((const double *)Mt->vals, lv, n, round_bf16);
-        CHEB_TRY(check_launch("k_to_f32_col"));
-        CHEB_CUDA(cudaMemsetAsync(lv + n, 0, BB * sizeof(float), s));
-    }
-    CHEB_CUDA(cudaMemsetAsync(counter, 0, 64, s));
     const ColLists &c = plan->col;
     ColArgs a{};
+    for (int i = 0; i < 2; ++i) a.T[i] = cv.take<T>(plan->nnzb * BB);
+    uint4 *opd = cv.take<uint4>((Mt->nnzb + 1) * (sizeof(T) == 8 ? 8 : 4));
+    if (sizeof(T) == 4) {
+        for (int f = 0; f < MAX_F; ++f) a.accp[f] = cv.take<float>(plan->nnzb * BB * 2);
+        a.Gp = cv.take<float>(plan->nnzb * BB * 2);
+    }
+    int32_t *opexp = cv.take<int32_t>(plan->nbr), *opflag = cv.take<int32_t>(16);
+    a.part = cv.take<double>((size_t)c.n_panels * (COL_STEPS + 2) * 2);
+    if (!cv.fits()) return fail(CHEB_ERR_NOSPACE, "cheb_expand: workspace %zu too small", ws_bytes);
+    CHEB_CUDA(cudaMemsetAsync(opflag, 0, 64, s));
+    k_opdig<T><<<(unsigned)((plan->nbr + 1 + 7) / 8), 256, 0, s>>>(Mt->row_ptr, (const double *)Mt->vals, plan->nbr,
+                                                                  Mt->nnzb, x.round_bf16, opd, opexp, opflag);
+    CHEB_TRY(check_launch("k_opdig"));
     a.panels = c.d_panels;
     a.wchunk = c.d_wchunk;
     a.wrow = c.d_wrow;
@@ -689,61 +959,59 @@ int col_expand(const cheb_plan *plan, const cheb_bsr *Mt, int32_t n_terms, const
     a.rp = plan->rp;
     a.ci = plan->ci;
     a.tperm = plan->d_tperm;
-    a.Lv = lv;
-    a.nf = nf;
-    for (int f = 0; f < nf; ++f) {
-        a.acc[f] = acc[f];
-        a.accp[f] = accp[f];
-    }
-    a.coef = coeffs;
-    a.coef_stride = stride;
-    a.G = G;
-    a.part = part;
-    a.counter = counter;
-    a.round_bf16 = round_bf16;
-    k_colinit<256><<<COLINIT_BLOCKS, 256, 0, s>>>(plan->rp, plan->ci, plan->d_tperm, plan->nbr, plan->nnzb,
-                                                  Mt->row_ptr, Mt->col_idx, (const double *)Mt->vals, buf[0],
-                                                  buf[1], nf, a, Gp, moments, gmoments);
-    CHEB_TRY(check_launch("k_colinit"));
-    a.Gp = G ? Gp : nullptr;
-    a.alpha = 2.f;
-    a.beta = -1.f;
-    // terms 2.. n-1 are accumulated three at a time: the launch forming term
-    // t adds (t-2, t-1, t) when t = 4, 7, 10, ..., and the last launch adds
-    // the terms left after the last such group
-    int done = 1;  // last term accumulated (terms 0 and 1: k_colinit)
-    for (int k = 1; k + 1 < n_terms; ++k) {
-        const int t = k + 1;
-        a.R = buf[k % 3];
-        a.Rm = buf[(k - 1) % 3];
-        a.C = buf[(k + 1) % 3];
-        a.term = t;
-        a.grp = 0;
-        if ((t >= 4 && (t - 1) % 3 == 0) || t == n_terms - 1) {
-            for (int u = done + 1; u <= t; ++u) a.grp |= 1 << (t - u);
-            done = t;
+    a.Lrp = Mt->row_ptr;
+    a.Lci = Mt->col_idx;
+    a.Lv = (const double *)Mt->vals;
+    a.nnzL = Mt->nnzb;
+    a.opd = opd;
+    a.opexp = opexp;
+    a.opflag = opflag;
+    a.n_terms = x.n_terms;
+    a.n_single = x.max_terms;
+    a.nf = x.nf;
+    for (int f = 0; f < x.nf; ++f) a.acc[f] = x.acc[f];
+    a.coef = x.coef;
+    a.coef_off = x.coef_off;
+    a.coef_stride = x.coef_stride;
+    a.G = x.gmoments ? x.G : nullptr;
+    a.pstride = COL_STEPS + 2;
+    a.want_mom = x.moments || a.G;
+    a.round_bf16 = x.round_bf16;
+    const size_t smem = col_layout(c.P).total(c.max_union);
+    auto fn = k_colstep<T>;
+    CHEB_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    for (int t0 = 2; t0 == 2 || t0 < x.max_terms; t0 += COL_STEPS) {
+        a.t0 = t0;
+        a.t1 = std::min(t0 + COL_STEPS, x.max_terms);
+        a.tbase = t0 == 2 ? 0 : t0;
+        fn<<<(unsigned)c.n_panels, COL_NW * 32, smem, s>>>(a);
+        CHEB_TRY(check_launch("k_colstep"));
+        if (a.want_mom) {
+            const int nt = a.t1 - a.tbase;
+            k_colmom<<<dim3(nt, plan->nsys), 128, 0, s>>>(a.part, a.pstride, a.tbase, nt, c.d_sys_panel, x.n_terms,
+                                                          x.max_terms, x.mom_stride, x.moments, a.G ? x.gmoments : nullptr);
+            CHEB_TRY(check_launch("k_colmom"));
         }
-        a.mom = moments ? moments + t : nullptr;
-        a.gmom = (gmoments && G) ? gmoments + t : nullptr;
-        CHEB_TRY(run_colstep(plan, a, s));
-    }
-    if (nf > 0) {
-        const int64_t n = plan->nnzb * BB;
-        k_colfinal<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(plan->d_tperm, plan->nnzb, nf, a);
-        CHEB_TRY(check_launch("k_colfinal"));
     }
     return CHEB_OK;
 }
 
+int col_expand(const cheb_plan *plan, const cheb_bsr *Mt, const ColExpand &x, void *ws, size_t ws_bytes, cudaStream_t s) {
+    if (ws_bytes < col_expand_ws(plan, Mt->nnzb))
+        return fail(CHEB_ERR_NOSPACE, "cheb_expand: workspace %zu < %zu", ws_bytes, col_expand_ws(plan, Mt->nnzb));
+    return wide_elements(plan->precision) ? col_expand_t<double>(plan, Mt, x, ws, ws_bytes, s)
+                                          : col_expand_t<float>(plan, Mt, x, ws, ws_bytes, s);
+}
+
 // ---------------------------------------------------------------------------
 // Host: the column kernel's panels and work streams for operator pattern
-// (lrp, lci).  Per panel: the union of its columns' rows (slot = rank); per
-// union row its operator entries with K in the union (dealt round-robin over
-// the slot residues modulo the K-groups of a quarter warp, so those K-groups
-// read different shared-memory banks), padded with zero-block entries to
-// whole chunks of KG; rows dealt to the NW warps by decreasing chunk count,
-// each to the warp with the least work so far; per warp its rows' chunks in
-// one stream and its row list.
+// (lrp, lci).  Per panel: the union of its columns' rows (slot = rank), in groups
+// of four: the first row left, then three times the row among the next COL_WINDOW
+// left that brings the fewest new slots for its length; per group the slots K with
+// an operator block in any of its rows, ascending (neighbouring slots are often
+// neighbouring blocks of the operator), eight to two quads (col_places), and per
+// slot of a quad the operator block of each row, or the zero block; groups dealt to the NW warps by decreasing quad count, each to the warp with the
+// fewest quads so far; per warp its groups' quads in one stream and its group list.
 
 struct ColCounts {
     std::vector<int64_t> chunks, rows;
@@ -753,17 +1021,16 @@ struct ColCounts {
 static void col_fill(const ColLists &c, const std::vector<int64_t> &rp, const std::vector<int32_t> &ci,
                      const std::vector<int64_t> &lrp, const std::vector<int32_t> &lci, int64_t nbr, int64_t p0,
                      int64_t p1, bool count_only, ColCounts &cnt, const std::vector<int64_t> &chunk_off,
-                     const std::vector<int64_t> &row_off, std::vector<int32_t> &pan, std::vector<int32_t> &wchunk,
-                     std::vector<int32_t> &wrow, std::vector<uint32_t> &rows, std::vector<uint32_t> &ent,
-                     std::vector<uint16_t> &slot) {
-    const int KG = 32 / c.P, CW = COL_EK * KG, NW = c.NW, rq = 8 / c.P;
-    const uint32_t zero_word = (uint32_t)lci.size() << COL_SLOT_BITS;  // the appended zero block, slot 0
-    std::vector<int32_t> stamp(nbr, -1), slot_of(nbr, -1), uni;
-    std::vector<std::vector<uint32_t>> cls(rq), rent;
-    std::vector<int32_t> order, wl;
-    std::vector<uint8_t> cmask;
+                     const std::vector<int64_t> &row_off, std::vector<int32_t> &wchunk, std::vector<int32_t> &wrow,
+                     std::vector<uint32_t> &rows, std::vector<uint32_t> &ent, std::vector<uint16_t> &slot) {
+    const int NW = c.NW;
+    const uint32_t zero_blk = (uint32_t)lci.size();  // the appended zero block
+    std::vector<int32_t> stamp(nbr, -1), slot_of(nbr, -1), uni, order;
+    std::vector<int> work, left;
+    std::vector<std::array<int, 4>> groups;
+    std::vector<uint32_t> bits;  // [union row][words] operator slots
     std::vector<int64_t> load(NW);
-    std::vector<std::vector<int32_t>> wrows(NW);
+    std::vector<std::vector<int32_t>> wgroups(NW);
     for (int64_t p = p0; p < p1; ++p) {
         const int32_t j0 = c.h_panels[4 * p], nc = c.h_panels[4 * p + 1];
         uni.clear();
@@ -774,96 +1041,111 @@ static void col_fill(const ColLists &c, const std::vector<int64_t> &rp, const st
                     uni.push_back(ci[e]);
                 }
         std::sort(uni.begin(), uni.end());
-        const int nu = (int)uni.size();
+        const int nu = (int)uni.size(), ng = (nu + 3) / 4, nw = (nu + 31) / 32;
         for (int u = 0; u < nu; ++u) slot_of[uni[u]] = u;
-        // the entries of every union row, interleaved and padded
-        rent.assign(nu, {});
-        int32_t mr = 0;
-        for (int u = 0; u < nu; ++u) {
-            const int32_t I = uni[u];
-            for (auto &v : cls) v.clear();
-            for (int64_t e = lrp[I]; e < lrp[I + 1]; ++e)
+        bits.assign((size_t)nu * nw, 0u);
+        for (int u = 0; u < nu; ++u)
+            for (int64_t e = lrp[uni[u]]; e < lrp[uni[u] + 1]; ++e)
                 if (stamp[lci[e]] == (int32_t)p) {
-                    const int32_t sl = slot_of[lci[e]];
-                    cls[sl % rq].push_back(((uint32_t)e << COL_SLOT_BITS) | (uint32_t)sl);
+                    const int s = slot_of[lci[e]];
+                    bits[(size_t)u * nw + (s >> 5)] |= 1u << (s & 31);
                 }
-            // position p of a chunk (8 K-groups x 2 entries) takes slot residue
-            // (p ^ (p >> 3)) mod 2, so that the two K-groups of a quarter warp
-            // differ in it both for the entries e = 0, 1 of a full row and for
-            // the pair (p, p + 8) that a half row's lane quads read together;
-            // when one residue runs out the other fills in
-            std::vector<uint32_t> &r = rent[u];
-            std::vector<size_t> at(rq, 0);
-            size_t left = 0;
-            for (auto &v : cls) left += v.size();
-            for (size_t pos = 0; left > 0; ++pos) {
-                const int p = (int)(pos % (size_t)CW);
-                int k = ((p ^ (p >> 3)) & 1) % rq;
-                if (at[k] >= cls[k].size())
-                    for (int kk = 0; kk < rq; ++kk)
-                        if (at[kk] < cls[kk].size()) {
-                            k = kk;
-                            break;
-                        }
-                r.push_back(cls[k][at[k]++]);
-                --left;
-            }
-            mr = std::max(mr, (int32_t)r.size());
-            const size_t padded = std::max<size_t>(1, (r.size() + CW - 1) / CW) * CW;
-            r.resize(padded, zero_word);
-        }
-        // the columns of the panel in which each union row has a block
-        std::vector<uint8_t> &cm = cmask;
-        cm.assign(nu, 0);
-        for (int32_t q = 0; q < nc; ++q)
-            for (int64_t e = rp[j0 + q]; e < rp[j0 + q + 1]; ++e) cm[slot_of[ci[e]]] |= (uint8_t)(1u << q);
-        // rows to warps: decreasing chunk count (a chunk's copies, waits and
-        // bookkeeping cost about as much as its products), each to the warp
-        // with the fewest chunks so far
-        auto work = [&](int32_t u) { return (int64_t)(rent[u].size() / CW); };
-        order.resize(nu);
-        for (int u = 0; u < nu; ++u) order[u] = u;
-        std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return work(x) > work(y); });
-        std::fill(load.begin(), load.end(), 0);
-        for (auto &v : wrows) v.clear();
+        left.resize(nu);
+        std::iota(left.begin(), left.end(), 0);
+        groups.assign(ng, {-1, -1, -1, -1});
+        work.assign(ng, 2);
+        int32_t mr = 0;
         int64_t total = 0;
-        for (const int32_t u : order) {
-            const int w = (int)(std::min_element(load.begin(), load.end()) - load.begin());
-            load[w] += work(u);
-            wrows[w].push_back(u);
-            total += (int64_t)rent[u].size() / CW;
+        std::vector<std::vector<uint32_t>> merged(ng);
+        for (int i = 0; i < ng; ++i) {
+            std::vector<uint32_t> &cur = merged[i];
+            cur.assign(nw, 0u);
+            for (int a = 0; a < 4 && !left.empty(); ++a) {
+                int best = 0, bc = INT32_MAX;
+                for (int k = 0; a > 0 && k < std::min<int>(COL_WINDOW, (int)left.size()); ++k) {
+                    int cost = 0;
+                    for (int w = 0; w < nw; ++w) {
+                        const uint32_t b = bits[(size_t)left[k] * nw + w];
+                        cost += 2 * __builtin_popcount(b & ~cur[w]) - __builtin_popcount(b);
+                    }
+                    if (cost < bc) {
+                        bc = cost;
+                        best = k;
+                    }
+                }
+                const int u = left[best];
+                left.erase(left.begin() + best);
+                groups[i][a] = u;
+                for (int w = 0; w < nw; ++w) cur[w] |= bits[(size_t)u * nw + w];
+            }
+            int n = 0;
+            for (int w = 0; w < nw; ++w) n += __builtin_popcount(cur[w]);
+            work[i] = std::max(2, (n + 7) / 8 * 2);
+            mr = std::max(mr, work[i]);
+            total += work[i];
         }
         if (count_only) {
             cnt.chunks[p] = total;
-            cnt.rows[p] = nu;
+            cnt.rows[p] = ng;
             cnt.max_row[p] = mr;
             continue;
         }
-        pan[4 * p] = j0;
-        pan[4 * p + 1] = nc;
-        pan[4 * p + 2] = nu;
-        pan[4 * p + 3] = 0;
+        order.resize(ng);
+        std::iota(order.begin(), order.end(), 0);
+        std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return work[x] > work[y]; });
+        std::fill(load.begin(), load.end(), 0);
+        for (auto &v : wgroups) v.clear();
+        for (const int32_t i : order) {
+            const int w = (int)(std::min_element(load.begin(), load.end()) - load.begin());
+            load[w] += work[i];
+            wgroups[w].push_back(i);
+        }
         for (int32_t q = 0; q < nc; ++q)
             for (int64_t e = rp[j0 + q]; e < rp[j0 + q + 1]; ++e) slot[e] = (uint16_t)slot_of[ci[e]];
         int64_t ch = chunk_off[p], ro = row_off[p];
         for (int w = 0; w < NW; ++w) {
             wchunk[p * (NW + 1) + w] = (int32_t)ch;
             wrow[p * (NW + 1) + w] = (int32_t)ro;
-            std::sort(wrows[w].begin(), wrows[w].end());
-            for (const int32_t u : wrows[w]) {
-                const std::vector<uint32_t> &r = rent[u];
-                // half row: blocks in at most two columns (ca, cb; cb = ca for one)
-                const uint32_t m = cm[u];
-                const int pc = __builtin_popcount(m);
-                uint32_t hw = 0;
-                if (pc <= 2) {
-                    const uint32_t ca = (uint32_t)__builtin_ctz(m);
-                    const uint32_t cb = pc == 2 ? (uint32_t)(31 - __builtin_clz(m)) : ca;
-                    hw = 1u | (ca << 1) | (cb << 3);
+            std::sort(wgroups[w].begin(), wgroups[w].end());
+            for (const int32_t i : wgroups[w]) {
+                const int quads = work[i];
+                uint32_t sl[4];
+                for (int a = 0; a < 4; ++a) sl[a] = groups[i][a] >= 0 ? (uint32_t)groups[i][a] : (1u << COL_SLOT_BITS) - 1u;
+                rows[2 * ro] = sl[0] | (sl[1] << COL_SLOT_BITS) | (sl[2] << (2 * COL_SLOT_BITS));
+                rows[2 * ro + 1] = sl[3] | ((uint32_t)quads << COL_SLOT_BITS);
+                ++ro;
+                uint32_t *out = ent.data() + ch * COL_CW;
+                auto word = [&](int pl, int a) -> uint32_t & {
+                    return out[(pl >> 2) * COL_CW + ((a & 1) * 4 + (pl & 3)) * 2 + (a >> 1)];
+                };
+                const std::vector<uint32_t> &cur = merged[i];
+                std::vector<int> place(32 * nw, -1);
+                std::vector<uint16_t> list;
+                for (int s = 0; s < nu; ++s)
+                    if ((cur[s >> 5] >> (s & 31)) & 1u) list.push_back((uint16_t)s);
+                for (int c8 = 0; c8 < quads / 2; ++c8) {
+                    uint8_t at[8];
+                    unsigned taken = 0u;
+                    const int n = std::max(0, std::min<int>(8, (int)list.size() - 8 * c8));
+                    col_places(list.data() + 8 * c8, n, at);
+                    for (int k = 0; k < n; ++k) {
+                        const int s = list[8 * c8 + k];
+                        place[s] = 8 * c8 + at[k];
+                        taken |= 1u << at[k];
+                        for (int a = 0; a < 4; ++a) word(place[s], a) = (zero_blk << COL_SLOT_BITS) | (uint32_t)s;
+                    }
+                    for (int k = 0; k < 8; ++k)
+                        if (!((taken >> k) & 1u))
+                            for (int a = 0; a < 4; ++a)
+                                word(8 * c8 + k, a) = (zero_blk << COL_SLOT_BITS) | (uint32_t)((k & 3) < nu ? k & 3 : 0);
                 }
-                rows[ro++] = (uint32_t)u | (hw << COL_SLOT_BITS) | ((uint32_t)(r.size() / CW) << COL_ROW_SHIFT);
-                std::copy(r.begin(), r.end(), ent.begin() + ch * CW);
-                ch += (int64_t)r.size() / CW;
+                for (int a = 0; a < 4 && groups[i][a] >= 0; ++a)
+                    for (int64_t e = lrp[uni[groups[i][a]]]; e < lrp[uni[groups[i][a]] + 1]; ++e)
+                        if (stamp[lci[e]] == (int32_t)p) {
+                            const int s = slot_of[lci[e]];
+                            word(place[s], a) = ((uint32_t)e << COL_SLOT_BITS) | (uint32_t)s;
+                        }
+                ch += quads;
             }
         }
         wchunk[p * (NW + 1) + NW] = (int32_t)ch;
@@ -871,36 +1153,40 @@ static void col_fill(const ColLists &c, const std::vector<int64_t> &rp, const st
     }
 }
 
-// Union rows a panel of the column kernel may hold: shared memory, and slots
-// below 2^COL_SLOT_BITS.
-int32_t col_ucap() {
-    int lo = 0, hi = 65535;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) / 2;
-        if (col_layout(mid, COL_P, COL_NW).total <= (size_t)CHEB_MAX_DYN_SMEM - 1024) lo = mid; else hi = mid - 1;
-    }
-    return std::min(lo, (1 << COL_SLOT_BITS) - 1);
+// Union rows a panel of the column kernel may hold: shared memory, and
+// COL_MAX_UNION.
+int32_t col_ucap(int P) {
+    const ColLayout lay = col_layout(P);
+    return std::min((CHEB_MAX_DYN_SMEM - 1024 - lay.off_x) / lay.slot_bytes, COL_MAX_UNION);
+}
+
+// Whether the column kernel's lists are built for an operator of nnzL blocks
+// (see COL_ROW_MIN) whose index fits an entry word.
+bool col_wanted(const cheb_plan *plan, int64_t nnzL) {
+    if (nnzL + 1 >= ((int64_t)1 << (32 - COL_SLOT_BITS))) return false;
+    return !wide_elements(plan->precision) || nnzL >= COL_ROW_MIN * plan->nbr;
 }
 
 int col_build(cheb_plan *plan, const std::vector<int64_t> &rp, const std::vector<int32_t> &ci,
               const std::vector<int64_t> &lrp, const std::vector<int32_t> &lci) {
     ColLists c;
-    c.P = COL_P;
+    const bool wide = wide_elements(plan->precision);
+    c.P = col_width(plan->precision);
     c.NW = COL_NW;
-    const int CW = COL_EK * 32 / c.P;  // entries per chunk
+    c.nnzL = (int64_t)lci.size();
     const int64_t nbr = plan->nbr, nnzb = plan->nnzb;
-    c.ucap = col_ucap();
-    // entries pack the operator block index (the appended zero block included)
-    // above the union slot
-    if ((int64_t)lci.size() + 1 >= ((int64_t)1 << (32 - COL_SLOT_BITS))) return CHEB_ERR_NOSPACE;
-    // panels: greedy along the columns while the union fits
+    c.ucap = col_ucap(c.P);
+    if (!col_wanted(plan, c.nnzL)) return CHEB_ERR_NOSPACE;
+    // panels: greedy along the columns of each system while the union fits
     std::vector<int32_t> stamp(nbr, -1);
-    {
-        int64_t j = 0, panel = 0;
-        while (j < nbr) {
+    c.h_sys_panel.clear();
+    for (int sy = 0; sy < plan->nsys; ++sy) {
+        int64_t j = plan->h_sys_col[sy], panel = c.n_panels;
+        c.h_sys_panel.push_back((int32_t)panel);
+        while (j < plan->h_sys_col[sy + 1]) {
             int32_t cnt = 0, ncols = 0;
             const int64_t j0 = j;
-            while (j < nbr && ncols < c.P) {
+            while (j < plan->h_sys_col[sy + 1] && ncols < c.P) {
                 int32_t add = 0;
                 for (int64_t p = rp[j]; p < rp[j + 1]; ++p) add += stamp[ci[p]] != (int32_t)panel;
                 if (cnt + add > c.ucap) break;
@@ -910,19 +1196,20 @@ int col_build(cheb_plan *plan, const std::vector<int64_t> &rp, const std::vector
                 ++j;
             }
             if (ncols == 0) return CHEB_ERR_NOSPACE;  // a single column does not fit: no column kernel
-            c.h_panels.insert(c.h_panels.end(), {(int32_t)j0, ncols, cnt, 0});
+            c.h_panels.insert(c.h_panels.end(), {(int32_t)j0, ncols, cnt, sy});
             c.max_union = std::max(c.max_union, cnt);
             ++panel;
         }
         c.n_panels = panel;
     }
+    c.h_sys_panel.push_back((int32_t)c.n_panels);
     const int64_t np = c.n_panels;
     ColCounts cnt;
     cnt.chunks.assign(np, 0);
     cnt.rows.assign(np, 0);
     cnt.max_row.assign(np, 0);
     std::vector<int64_t> chunk_off(np + 1, 0), row_off(np + 1, 0);
-    std::vector<int32_t> pan(4 * np), wchunk(np * (c.NW + 1)), wrow(np * (c.NW + 1));
+    std::vector<int32_t> wchunk(np * (c.NW + 1)), wrow(np * (c.NW + 1));
     std::vector<uint32_t> rows, ent;
     std::vector<uint16_t> slot(nnzb);
     const int nth = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)std::thread::hardware_concurrency(), 16, np}));
@@ -931,8 +1218,7 @@ int col_build(cheb_plan *plan, const std::vector<int64_t> &rp, const std::vector
         for (int t = 0; t < nth; ++t) {
             const int64_t p0 = np * t / nth, p1 = np * (t + 1) / nth;
             th.emplace_back([&, p0, p1] {
-                col_fill(c, rp, ci, lrp, lci, nbr, p0, p1, count_only, cnt, chunk_off, row_off, pan, wchunk, wrow,
-                         rows, ent, slot);
+                col_fill(c, rp, ci, lrp, lci, nbr, p0, p1, count_only, cnt, chunk_off, row_off, wchunk, wrow, rows, ent, slot);
             });
         }
         for (auto &x : th) x.join();
@@ -943,12 +1229,11 @@ int col_build(cheb_plan *plan, const std::vector<int64_t> &rp, const std::vector
         row_off[p + 1] = row_off[p] + cnt.rows[p];
         c.max_row = std::max(c.max_row, cnt.max_row[p]);
     }
-    if (chunk_off[np] * CW >= (int64_t)INT32_MAX) return CHEB_ERR_NOSPACE;
-    c.n_entries = chunk_off[np] * CW;
-    rows.resize(row_off[np]);
-    ent.resize(chunk_off[np] * CW);
+    if ((chunk_off[np] + COL_TAIL) * COL_CW >= (int64_t)INT32_MAX || (wide && c.max_row > COL_MAX_QUADS64)) return CHEB_ERR_NOSPACE;
+    c.n_entries = (chunk_off[np] + COL_TAIL) * COL_CW;
+    rows.resize(2 * row_off[np]);
+    ent.resize(c.n_entries, 0u);
     run(false);
-    c.h_panels.swap(pan);
     c.h_wchunk.swap(wchunk);
     c.h_wrow.swap(wrow);
     c.h_rows.swap(rows);
@@ -956,6 +1241,7 @@ int col_build(cheb_plan *plan, const std::vector<int64_t> &rp, const std::vector
     c.h_slot.swap(slot);
     c.n_rows = (int64_t)c.h_rows.size();
     c.n_slot = (int64_t)c.h_slot.size();
+    c.n_sys = (int64_t)c.h_sys_panel.size();
     c.built = true;
     plan->col = std::move(c);
     return CHEB_OK;
@@ -976,6 +1262,7 @@ int col_bind(ColLists &c, Carve &cv, cudaStream_t s) {
         c.d_rows = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(c.d_rows) + d);
         c.d_ent = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(c.d_ent) + d);
         c.d_slot = reinterpret_cast<uint16_t *>(reinterpret_cast<char *>(c.d_slot) + d);
+        c.d_sys_panel = reinterpret_cast<int32_t *>(reinterpret_cast<char *>(c.d_sys_panel) + d);
         return CHEB_OK;
     }
     c.d_panels = cv.take<int32_t>(c.h_panels.size());
@@ -984,6 +1271,7 @@ int col_bind(ColLists &c, Carve &cv, cudaStream_t s) {
     c.d_rows = cv.take<uint32_t>(std::max<size_t>(c.h_rows.size(), 1));
     c.d_ent = cv.take<uint32_t>(std::max<size_t>(c.h_ent.size(), 1));
     c.d_slot = cv.take<uint16_t>(c.h_slot.size());
+    c.d_sys_panel = cv.take<int32_t>(c.h_sys_panel.size());
     if (!cv.fits()) return fail(CHEB_ERR_NOSPACE, "cheb_plan_bind_operator: workspace too small");
     CHEB_CUDA(cudaMemcpyAsync(c.d_panels, c.h_panels.data(), c.h_panels.size() * 4, cudaMemcpyHostToDevice, s));
     CHEB_CUDA(cudaMemcpyAsync(c.d_wchunk, c.h_wchunk.data(), c.h_wchunk.size() * 4, cudaMemcpyHostToDevice, s));
@@ -993,6 +1281,7 @@ int col_bind(ColLists &c, Carve &cv, cudaStream_t s) {
     if (!c.h_ent.empty())
         CHEB_CUDA(cudaMemcpyAsync(c.d_ent, c.h_ent.data(), c.h_ent.size() * 4, cudaMemcpyHostToDevice, s));
     CHEB_CUDA(cudaMemcpyAsync(c.d_slot, c.h_slot.data(), c.h_slot.size() * 2, cudaMemcpyHostToDevice, s));
+    CHEB_CUDA(cudaMemcpyAsync(c.d_sys_panel, c.h_sys_panel.data(), c.h_sys_panel.size() * 4, cudaMemcpyHostToDevice, s));
     return CHEB_OK;
 }
 

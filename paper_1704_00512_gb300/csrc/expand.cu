@@ -681,10 +681,13 @@ size_t expand_ws(const cheb_plan *plan, int64_t nnzL, int precision) {
     size_t b = 3 * align_up(plan->nnzb * BB * esz);
     if (precision != CHEB_F64) b += align_up(nnzL * BB * esz);
     b += align_up(plan->n_panels * 4 * sizeof(double)) + align_up(64);
-    b += 256;
-    if ((precision == CHEB_F32 || precision == CHEB_BF16) && plan->col.built)
-        b = std::max(b, col_expand_ws(plan, nnzL));
-    return b;
+    return b + 256;
+}
+
+// With the column kernel's lists: its workspace, if that is larger.
+size_t expand_ws_col(const cheb_plan *plan, int64_t nnzL, int precision) {
+    const size_t b = expand_ws(plan, nnzL, precision);
+    return plan->col.built ? std::max(b, col_expand_ws(plan, nnzL)) : b;
 }
 
 template <typename T>
@@ -756,7 +759,7 @@ static int check_operator(const cheb_plan *plan, const cheb_bsr *Mt) {
 extern "C" int cheb_expand_stepwise_workspace_size(const cheb_plan *plan, const cheb_bsr *Mt, int32_t precision,
                                                    size_t *bytes) {
     if (!plan || !Mt || !bytes) return fail(CHEB_ERR_INVALID, "cheb_expand_stepwise_workspace_size: NULL argument");
-    *bytes = expand_ws(plan, Mt->nnzb, precision);
+    *bytes = expand_ws_col(plan, Mt->nnzb, precision);
     return CHEB_OK;
 }
 
@@ -770,19 +773,22 @@ extern "C" int cheb_expand_stepwise(const cheb_plan *plan, const cheb_bsr *Mt, i
     for (int f = 0; f < n_f; ++f)
         if (!acc[f]) return fail(CHEB_ERR_INVALID, "cheb_expand_stepwise: accumulator %d is NULL", f);
     if (precision != plan->precision) return fail(CHEB_ERR_INVALID, "cheb_expand_stepwise: plan precision differs");
-    if (!ws || ws_bytes < expand_ws(plan, Mt->nnzb, precision))
-        return fail(CHEB_ERR_NOSPACE, "cheb_expand_stepwise: workspace %zu < %zu", ws_bytes,
-                    expand_ws(plan, Mt->nnzb, precision));
+    // a wide workspace sized before the operator was attached still takes the
+    // per-step kernel; a reduced-precision one has to hold the column kernel's
+    const size_t need = wide_elements(precision) ? expand_ws(plan, Mt->nnzb, precision)
+                                                 : expand_ws_col(plan, Mt->nnzb, precision);
+    if (!ws || ws_bytes < need)
+        return fail(CHEB_ERR_NOSPACE, "cheb_expand_stepwise: workspace %zu < %zu", ws_bytes, need);
     cudaStream_t s = as_stream(stream);
+    const ColExpand x{n_terms, nullptr, coeffs, nullptr, coeff_stride, n_f, acc, moments, G, gmoments, n_terms,
+                      precision == CHEB_BF16};
+    if (col_takes(plan, Mt, x, ws_bytes)) return col_expand(plan, Mt, x, ws, ws_bytes, s);
     if (precision == CHEB_F64)
         return expand_impl<double>(plan, Mt, n_terms, coeffs, coeff_stride, n_f, acc, moments, G, gmoments, ws,
                                    ws_bytes, s);
     if (precision == CHEB_F64X)
         return expand_impl<dfl>(plan, Mt, n_terms, coeffs, coeff_stride, n_f, acc, moments, G, gmoments, ws,
                                 ws_bytes, s);
-    if ((precision == CHEB_F32 || precision == CHEB_BF16) && col_usable(plan, Mt))
-        return col_expand(plan, Mt, n_terms, coeffs, coeff_stride, n_f, acc, moments, G, gmoments, ws, ws_bytes, s,
-                          precision == CHEB_BF16);
     if (precision == CHEB_F32 || precision == CHEB_BF16)
         return expand_impl<float>(plan, Mt, n_terms, coeffs, coeff_stride, n_f, acc, moments, G, gmoments, ws,
                                   ws_bytes, s, precision == CHEB_BF16);

@@ -1,22 +1,23 @@
-// Gather plan of the column-order step kernel built on the device (Eq. 3
-// restricted to the pattern; column independence, Sec. "Expansion in
-// Chebyshev polynomials"): from the device block-CSR patterns of P_out and of
-// the operator, with the same panels, row order, warp streams and entry words
-// as the host builder in colstep.cu (bit for bit).
+// Gather plan of the column-order kernel built on the device (Eq. 3 restricted
+// to the pattern; column independence, Sec. "Expansion in Chebyshev
+// polynomials"): from the device block-CSR patterns of P_out and of the
+// operator, with the same panels, groups, warp streams and entry words as the
+// host builder in colstep.cu (bit for bit).
 //
 //   k_gp_panels  one thread block walks the block columns in order and closes a
-//                panel when COL_P columns are in it or the next column's new
-//                rows would overflow the union capacity (a stamp per row marks
-//                the rows already in the open panel);
+//                panel when P columns are in it or the next column's new rows
+//                would overflow the union capacity (a stamp per row marks the
+//                rows already in the open panel);
 //   k_gp_rows    one thread block per panel: the union of the panel's
-//                columns' rows as a bitmap with ranks (slot = rank), per union
-//                row the count of operator entries whose column is in the union,
-//                and -- in the fill pass -- the rows dealt to the NW warps by
-//                decreasing chunk count (each to the warp with the least work so
-//                far, ties to the lowest warp), the row words, the entry streams
-//                interleaved by slot parity and padded with zero-block entries,
-//                and the union slot of every P_out block of the panel;
-//   k_gp_scan    offsets of the panels' chunks and rows.
+//                columns' rows as a bitmap with ranks (slot = rank) and per union
+//                row a bitmap of its operator slots; one warp groups the rows by
+//                fours; per group its merged slots and their count, and -- in the
+//                fill pass -- the groups dealt to the NW warps
+//                by decreasing quad count (each to the warp with the least work so
+//                far, ties to the lowest warp), the group words, the entry streams
+//                padded with zero-block entries, and the union slot of every P_out
+//                block of the panel;
+//   k_gp_scan    offsets of the panels' quads and groups.
 #include <algorithm>
 #include <cstdint>
 #include <cstring>
@@ -31,7 +32,7 @@ namespace cheb {
 constexpr int GP_NT = 512;
 constexpr int GP_NWARP = GP_NT / 32;
 constexpr int GP_MAXU = 1 << COL_SLOT_BITS;  // union slots
-constexpr int GP_HMAX = 4096;                // chunk counts of a row (rows hold <= 65536 blocks)
+constexpr int GP_MAXG = GP_MAXU / 4;         // groups, and quads of a group
 static_assert(GP_NWARP == COL_NW, "one warp of the builder per warp stream of the step kernel");
 
 // Block-wide integer sum, returned to every thread.
@@ -62,7 +63,7 @@ __device__ __forceinline__ int gp_block_max(int v, int *sh) {
 // sys_col[s+1]) (one system 0..nbr when sys_col is NULL) the block columns are
 // taken in order, and a panel is closed when P columns are in it or the next
 // column would take its union of rows above ucap or its blocks above bcap.
-// panels: (first column, columns, union rows, 0) per panel; aux (or NULL):
+// panels: (first column, columns, union rows, system) per panel; aux (or NULL):
 // (blocks, system) per panel.  out[0] = panels, out[1] = largest union, out[2]
 // = 1 if a single column does not fit, out[3] = most blocks of a panel.
 // stamp: int32[nbr] set to -1.
@@ -101,7 +102,7 @@ __global__ void __launch_bounds__(GP_NT) k_gp_panels(const int64_t *rp, const in
                 panels[4 * panel] = (int32_t)j0;
                 panels[4 * panel + 1] = ncols;
                 panels[4 * panel + 2] = (int32_t)cnt;
-                panels[4 * panel + 3] = 0;
+                panels[4 * panel + 3] = sy;
                 if (aux) {
                     aux[2 * panel] = (int32_t)nblk;
                     aux[2 * panel + 1] = sy;
@@ -137,24 +138,23 @@ struct GpArgs {
     uint32_t *rows, *ent;
     uint16_t *slot;
     int32_t *err;
+    size_t off_list;  // dynamic shared memory: the warps' merged slots
 };
 
 template <bool FILL>
 __global__ void __launch_bounds__(GP_NT) k_gp_rows(const GpArgs a) {
     extern __shared__ __align__(16) unsigned char dsm[];
     __shared__ int ulist[GP_MAXU];
-    __shared__ int work[GP_MAXU];
-    __shared__ int cm[GP_MAXU];
-    __shared__ int row_ch[GP_MAXU];
-    __shared__ int row_ro[GP_MAXU];
-    __shared__ int16_t order[GP_MAXU];
-    __shared__ uint8_t wsel[GP_MAXU];
+    __shared__ int work[GP_MAXG], gch[GP_MAXG], gro[GP_MAXG];
+    __shared__ int16_t order[GP_MAXG];
+    __shared__ uint8_t wsel[GP_MAXG];
+    __shared__ int hist[GP_MAXG + 1];
+    __shared__ int16_t group[GP_MAXG][4];
+    __shared__ uint16_t place[FILL ? GP_NWARP : 1][FILL ? GP_MAXU : 1];
     __shared__ int wsum[32];
     __shared__ int64_t sh[GP_NWARP];
     __shared__ int shi[GP_NWARP];
-    __shared__ int64_t bin_ch[COL_NW + 1];
-    __shared__ int bin_ro[COL_NW + 1];
-    constexpr int CW = COL_EK * 32 / COL_P;  // entries per chunk
+    __shared__ int bin_ch[COL_NW + 1], bin_ro[COL_NW + 1];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t p = blockIdx.x;
     const int j0 = a.panels[4 * p], nc = a.panels[4 * p + 1], nu_plan = a.panels[4 * p + 2];
@@ -176,8 +176,8 @@ __global__ void __launch_bounds__(GP_NT) k_gp_rows(const GpArgs a) {
     for (int64_t w = wb; w < we; ++w) cnt += __popc(bits[w].x);
     int total;
     int run = block_excl_scan<GP_NWARP>(cnt, wsum, &total);
-    const int nu = total;
-    if (nu != nu_plan || nu > GP_MAXU) {  // uniform
+    const int nu = total, ng = (nu + 3) / 4;
+    if (nu != nu_plan || nu >= GP_MAXU) {  // uniform
         if (tid == 0) atomicExch(a.err, 1);
         return;
     }
@@ -190,179 +190,229 @@ __global__ void __launch_bounds__(GP_NT) k_gp_rows(const GpArgs a) {
             m &= m - 1u;
         }
     }
-    for (int u = tid; u < nu; u += GP_NT) cm[u] = 0;
     __syncthreads();
+    if (FILL)
+        for (int q = 0; q < nc; ++q)
+            for (int64_t e = a.rp[j0 + q] + tid; e < a.rp[j0 + q + 1]; e += GP_NT)
+                a.slot[e] = (uint16_t)rank_of(bits, a.ci[e]);
 
-    // 2. the panel columns holding a block of each union row; slots of the
-    // panel's P_out blocks
-    for (int q = 0; q < nc; ++q)
-        for (int64_t e = a.rp[j0 + q] + tid; e < a.rp[j0 + q + 1]; e += GP_NT) {
-            const int sl = rank_of(bits, a.ci[e]);
-            atomicOr(&cm[sl], 1 << q);
-            if (FILL) a.slot[e] = (uint16_t)sl;
+    // 2. operator slots of every union row
+    const int uw = (nu + 31) / 32;
+    uint32_t *ub = reinterpret_cast<uint32_t *>(dsm + (((size_t)nw * sizeof(uint2) + 15) & ~(size_t)15));
+    for (int i = tid; i < nu * uw; i += GP_NT) ub[i] = 0u;
+    __syncthreads();
+    for (int u = warp; u < nu; u += GP_NWARP) {
+        const int I = ulist[u];
+        for (int64_t e = a.lrp[I] + lane; e < a.lrp[I + 1]; e += 32) {
+            const int sl = rank_of(bits, a.lci[e]);
+            if (sl >= 0) atomicOr(&ub[u * uw + (sl >> 5)], 1u << (sl & 31));
         }
-
-    // 3. per union row: operator entries in the union, chunks
+    }
+    __syncthreads();
+    // groups: the first row left, then three times, among the COL_WINDOW rows left
+    // after it, the one with the smallest 2 (new slots) - (slots), the first of
+    // those.  Lane l holds the candidates l and l + 32 in order (-1: none).
+    if (warp == 0) {
+        int c0 = lane < nu ? lane : -1, c1 = 32 + lane < nu ? 32 + lane : -1, next = 64;
+        auto drop = [&](int k) {  // remove candidate k, fill up from the rows behind
+            const int up0 = __shfl_down_sync(0xffffffffu, c0, 1), first1 = __shfl_sync(0xffffffffu, c1, 0);
+            const int up1 = __shfl_down_sync(0xffffffffu, c1, 1);
+            if (lane >= k) c0 = lane < 31 ? up0 : first1;
+            if (lane + 32 >= k) c1 = lane < 31 ? up1 : (next < nu ? next : -1);
+            ++next;
+        };
+        for (int i = 0; i < ng; ++i) {
+            uint32_t cur = 0u;  // the group's slots, a word per lane
+            for (int r = 0; r < 4; ++r) {
+                int best = 0;
+                if (r > 0) {
+                    int k0 = 0, k1 = 0;
+                    for (int w = 0; w < uw; ++w) {
+                        const uint32_t m = __shfl_sync(0xffffffffu, cur, w);
+                        const uint32_t x = c0 >= 0 ? ub[c0 * uw + w] : 0u, y = c1 >= 0 ? ub[c1 * uw + w] : 0u;
+                        k0 += 2 * __popc(x & ~m) - __popc(x);
+                        k1 += 2 * __popc(y & ~m) - __popc(y);
+                    }
+                    // (cost, place) as one key; no candidate: the largest
+                    const unsigned q0 = c0 >= 0 ? ((unsigned)(k0 + 2048) << 6) | (unsigned)lane : 0xffffffffu;
+                    const unsigned q1 = c1 >= 0 ? ((unsigned)(k1 + 2048) << 6) | (unsigned)(lane + 32) : 0xffffffffu;
+                    best = (int)(__reduce_min_sync(0xffffffffu, min(q0, q1)) & 63u);
+                }
+                const int u0 = __shfl_sync(0xffffffffu, c0, best & 31), u1 = __shfl_sync(0xffffffffu, c1, best & 31);
+                const int u = __shfl_sync(0xffffffffu, c0, 0) < 0 ? -1 : best < 32 ? u0 : u1;  // -1: no row left
+                if (lane == 0) group[i][r] = (int16_t)u;
+                if (u < 0) continue;
+                if (lane < uw) cur |= ub[u * uw + lane];
+                drop(best);
+            }
+        }
+    }
+    __syncthreads();
+    // per group: the merged slots (one word of the bitmap per lane), quads (even)
+    auto merge = [&](int i) {
+        uint32_t m = 0u;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int u = group[i][r];
+            if (u >= 0 && lane < uw) m |= ub[u * uw + lane];
+        }
+        return m;
+    };
     int mymax = 0;
     int64_t mych = 0;
-    for (int u = tid; u < nu; u += GP_NT) {
-        const int I = ulist[u];
-        int n = 0;
-        for (int64_t e = a.lrp[I]; e < a.lrp[I + 1]; ++e) n += rank_of(bits, a.lci[e]) >= 0;
-        const int wk = max(1, (n + CW - 1) / CW);
-        work[u] = wk;
-        mymax = max(mymax, n);
-        mych += wk;
+    for (int i = warp; i < ng; i += GP_NWARP) {
+        const int k = __reduce_add_sync(0xffffffffu, __popc(merge(i)));
+        const int wk = max(2, (k + 7) / 8 * 2);
+        if (lane == 0) {
+            work[i] = wk;
+            mymax = max(mymax, wk);
+            mych += wk;
+        }
     }
-    const int64_t chunks = gp_block_sum(mych, sh);  // (barrier: work[], cm[] complete)
+    const int64_t chunks = gp_block_sum(mych, sh);  // (barrier: work[] complete)
     const int maxrow = gp_block_max(mymax, shi);
     if (!FILL) {
         if (tid == 0) {
             a.cnt_chunks[p] = chunks;
-            a.cnt_rows[p] = nu;
+            a.cnt_rows[p] = ng;
             a.cnt_maxrow[p] = maxrow;
         }
         return;
     }
 
-    // 4. rows to warps: decreasing chunk count (stable), each to the warp
-    // with the fewest chunks so far (the lowest such warp)
-    if (tid == 0) {
-        int *hist = reinterpret_cast<int *>(dsm + (((size_t)nw * sizeof(uint2) + 15) & ~(size_t)15));
-        int maxw = 0;
-        for (int u = 0; u < nu; ++u) maxw = max(maxw, work[u]);
-        if (maxw > GP_HMAX) {
-            atomicExch(a.err, 2);
-            maxw = GP_HMAX;  // the lists are not used after an error; keep the writes in bounds
+    // 3. groups to warps: decreasing quad count (stable), each to the warp with
+    // the fewest quads so far (the lowest such warp)
+    if (warp == 0) {
+        for (int v = lane; v <= maxrow; v += 32) hist[v] = 0;
+        __syncwarp();
+        if (lane == 0) {
+            for (int i = 0; i < ng; ++i) ++hist[work[i]];
+            int at = 0;
+            for (int v = maxrow; v >= 0; --v) {
+                const int t = hist[v];
+                hist[v] = at;
+                at += t;
+            }
+            for (int i = 0; i < ng; ++i) order[hist[work[i]]++] = (int16_t)i;
         }
-        for (int v = 0; v <= maxw; ++v) hist[v] = 0;
-        for (int u = 0; u < nu; ++u) ++hist[min(work[u], maxw)];
-        int at = 0;
-        for (int v = maxw; v >= 0; --v) {
-            const int t = hist[v];
-            hist[v] = at;
-            at += t;
+        __syncwarp();
+        // lane w keeps the load of stream w; the lane with the smallest (load, w) takes the group
+        int load = 0, rows = 0;
+        for (int i = 0; i < ng; ++i) {
+            const int gi = order[i];
+            const unsigned key = lane < COL_NW ? ((unsigned)load << 5) | (unsigned)lane : 0xffffffffu;
+            const int best = (int)(__reduce_min_sync(0xffffffffu, key) & 31u);
+            if (lane == best) {
+                load += work[gi];
+                ++rows;
+                wsel[gi] = (uint8_t)lane;
+            }
         }
-        for (int u = 0; u < nu; ++u) order[hist[min(work[u], maxw)]++] = (int16_t)u;
-        int64_t load[COL_NW];
-        int nrow[COL_NW];
+        int ch = load, ro = rows;
 #pragma unroll
-        for (int w = 0; w < COL_NW; ++w) {
-            load[w] = 0;
-            nrow[w] = 0;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(0xffffffffu, ch, o), y = __shfl_up_sync(0xffffffffu, ro, o);
+            if (lane >= o) {
+                ch += x;
+                ro += y;
+            }
         }
-        for (int i = 0; i < nu; ++i) {
-            const int u = order[i];
-            int best = 0;
-#pragma unroll
-            for (int w = 1; w < COL_NW; ++w)
-                if (load[w] < load[best]) best = w;
-#pragma unroll
-            for (int w = 0; w < COL_NW; ++w)
-                if (w == best) {
-                    load[w] += work[u];
-                    ++nrow[w];
-                }
-            wsel[u] = (uint8_t)best;
+        if (lane < COL_NW) {
+            bin_ch[lane] = ch - load;
+            bin_ro[lane] = ro - rows;
+            a.wchunk[p * (COL_NW + 1) + lane] = (int32_t)(a.chunk_off[p] + ch - load);
+            a.wrow[p * (COL_NW + 1) + lane] = (int32_t)(a.row_off[p] + ro - rows);
+            if (lane == COL_NW - 1) {
+                a.wchunk[p * (COL_NW + 1) + COL_NW] = (int32_t)(a.chunk_off[p] + ch);
+                a.wrow[p * (COL_NW + 1) + COL_NW] = (int32_t)(a.row_off[p] + ro);
+            }
         }
-        int64_t ch = 0;
-        int ro = 0;
-#pragma unroll
-        for (int w = 0; w < COL_NW; ++w) {
-            bin_ch[w] = ch;
-            bin_ro[w] = ro;
-            ch += load[w];
-            ro += nrow[w];
-        }
-        bin_ch[COL_NW] = ch;
-        bin_ro[COL_NW] = ro;
     }
     __syncthreads();
 
-    // 5. warp w lays out the rows of stream w in increasing union slot
+    // 4. warp w lays out the groups of stream w in increasing order
     {
-        const int w = warp;
         const unsigned lt = (1u << lane) - 1u;
-        int ro = bin_ro[w];
-        int64_t ch = bin_ch[w];
-        for (int base = 0; base < nu; base += 32) {
-            const int u = base + lane;
-            const bool sel = u < nu && wsel[u] == w;
+        int ro = bin_ro[warp], ch = bin_ch[warp];
+        for (int base = 0; base < ng; base += 32) {
+            const int i = base + lane;
+            const bool sel = i < ng && wsel[i] == warp;
             const unsigned m = __ballot_sync(0xffffffffu, sel);
-            const int wk = sel ? work[u] : 0;
+            const int wk = sel ? work[i] : 0;
             int incl = wk;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                const int n = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += n;
+                const int x = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += x;
             }
             if (sel) {
-                row_ro[u] = ro + __popc(m & lt);
-                row_ch[u] = (int)(ch + incl - wk);
+                gro[i] = ro + __popc(m & lt);
+                gch[i] = ch + incl - wk;
             }
             ro += __popc(m);
             ch += __shfl_sync(0xffffffffu, incl, 31);
         }
-        if (lane == 0) {
-            a.wchunk[p * (COL_NW + 1) + w] = (int32_t)(a.chunk_off[p] + bin_ch[w]);
-            a.wrow[p * (COL_NW + 1) + w] = (int32_t)(a.row_off[p] + bin_ro[w]);
-            if (w == 0) {
-                a.wchunk[p * (COL_NW + 1) + COL_NW] = (int32_t)(a.chunk_off[p] + bin_ch[COL_NW]);
-                a.wrow[p * (COL_NW + 1) + COL_NW] = (int32_t)(a.row_off[p] + bin_ro[COL_NW]);
-            }
-        }
     }
     __syncthreads();
 
-    // 6. row words and entry streams.  Position t of a chunk takes an entry
-    // whose slot has parity (t ^ (t >> 3)) & 1, so that the two K-groups of a
-    // quarter warp read different banks; when one parity runs out the other
-    // fills in.  Entries of one parity keep the operator row's order.
-    const uint32_t zero_word = (uint32_t)a.nnzL << COL_SLOT_BITS;
-    for (int u = tid; u < nu; u += GP_NT) {
-        const int I = ulist[u];
-        const unsigned m = (unsigned)cm[u];
-        const int pc = __popc(m);
-        uint32_t hw = 0;
-        if (pc <= 2) {
-            const uint32_t ca = (uint32_t)(__ffs(m) - 1);
-            const uint32_t cb = pc == 2 ? (uint32_t)(31 - __clz(m)) : ca;
-            hw = 1u | (ca << 1) | (cb << 3);
+    // 5. group words and entry streams
+    const uint32_t zero_blk = (uint32_t)a.nnzL;
+    for (int i = warp; i < ng; i += GP_NWARP) {
+        const uint32_t mine = merge(i);
+        const int quads = work[i];
+        if (lane == 0) {
+            uint32_t sl[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) sl[r] = group[i][r] >= 0 ? (uint32_t)group[i][r] : (1u << COL_SLOT_BITS) - 1u;
+            uint32_t *out = a.rows + 2 * (a.row_off[p] + gro[i]);
+            out[0] = sl[0] | (sl[1] << COL_SLOT_BITS) | (sl[2] << (2 * COL_SLOT_BITS));
+            out[1] = sl[3] | ((uint32_t)quads << COL_SLOT_BITS);
         }
-        a.rows[a.row_off[p] + row_ro[u]] = (uint32_t)u | (hw << COL_SLOT_BITS) | ((uint32_t)work[u] << COL_ROW_SHIFT);
-        uint32_t *out = a.ent + (a.chunk_off[p] + row_ch[u]) * CW;
-        const int64_t e0 = a.lrp[I], e1 = a.lrp[I + 1];
-        int n0 = 0, n1 = 0;
-        for (int64_t e = e0; e < e1; ++e) {
-            const int sl = rank_of(bits, a.lci[e]);
-            if (sl >= 0) {
-                if (sl & 1) ++n1; else ++n0;
+        uint32_t *ent = a.ent + (a.chunk_off[p] + gch[i]) * COL_CW;
+        auto word = [&](int pl, int r) -> uint32_t & {
+            return ent[(pl >> 2) * COL_CW + ((r & 1) * 4 + (pl & 3)) * 2 + (r >> 1)];
+        };
+        // the merged slots ascending, then eight at a time to their places; the
+        // empty places name zero blocks
+        const int c = __popc(mine);
+        int incl = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += x;
+        }
+        const int all = __shfl_sync(0xffffffffu, incl, 31);
+        uint16_t *list = reinterpret_cast<uint16_t *>(dsm + a.off_list) + warp * GP_MAXU;
+        int pl = incl - c;
+        for (uint32_t m = mine; m; m &= m - 1u, ++pl) list[pl] = (uint16_t)(lane * 32 + __ffs(m) - 1);
+        __syncwarp();
+        for (int ch = lane; ch < quads / 2; ch += 32) {
+            uint8_t at[8];
+            unsigned taken = 0u;
+            const int n = max(0, min(8, all - 8 * ch));
+            col_places(list + 8 * ch, n, at);
+            for (int k = 0; k < n; ++k) {
+                const int s = list[8 * ch + k];
+                place[warp][s] = (uint16_t)(8 * ch + at[k]);
+                taken |= 1u << at[k];
+#pragma unroll
+                for (int x = 0; x < 4; ++x) word(8 * ch + at[k], x) = (zero_blk << COL_SLOT_BITS) | (uint32_t)s;
+            }
+            for (int k = 0; k < 8; ++k)
+                if (!((taken >> k) & 1u))
+#pragma unroll
+                    for (int x = 0; x < 4; ++x)
+                        word(8 * ch + k, x) = (zero_blk << COL_SLOT_BITS) | (uint32_t)((k & 3) < nu ? k & 3 : 0);
+        }
+        __syncwarp();
+        for (int x = 0; x < 4 && group[i][x] >= 0; ++x) {
+            const int I = ulist[group[i][x]];
+            for (int64_t e = a.lrp[I] + lane; e < a.lrp[I + 1]; e += 32) {
+                const int sl = rank_of(bits, a.lci[e]);
+                if (sl >= 0) word(place[warp][sl], x) = ((uint32_t)e << COL_SLOT_BITS) | (uint32_t)sl;
             }
         }
-        int64_t c0 = e0, c1 = e0;
-        int t0 = 0, t1 = 0;
-        const int n = n0 + n1;
-        for (int pos = 0; pos < n; ++pos) {
-            const int t = pos % CW;
-            int k = (t ^ (t >> 3)) & 1;
-            if (k == 0 ? t0 >= n0 : t1 >= n1) k ^= 1;
-            int64_t &c = k ? c1 : c0;
-            int sl = -1;
-            while (c < e1) {
-                sl = rank_of(bits, a.lci[c]);
-                if (sl >= 0 && (sl & 1) == k) break;
-                ++c;
-            }
-            if (c >= e1) {  // cannot happen with the counts above; never emit a bad block index
-                atomicExch(a.err, 3);
-                out[pos] = zero_word;
-            } else {
-                out[pos] = ((uint32_t)c << COL_SLOT_BITS) | (uint32_t)sl;
-            }
-            ++c;
-            if (k) ++t1; else ++t0;
-        }
-        for (int pos = n; pos < work[u] * CW; ++pos) out[pos] = zero_word;
+        __syncwarp();
     }
 }
 
@@ -533,22 +583,20 @@ __global__ void __launch_bounds__(GP_NT) k_rl_rows(const int64_t *rp, const int3
     if (tid == 0) lrow_ptr[r0 + nu] = (int32_t)(e0 + total);
 }
 
-// Dynamic shared memory of k_gp_rows: bitmap words (+ the fill pass's histogram).// Dynamic shared memory of k_gp_rows: bitmap words (+ the fill pass's histogram).
-static size_t gp_dyn_smem(int64_t nbr, bool fill) {
-    const size_t bits = align_up((size_t)((nbr + 31) / 32) * sizeof(uint2), 16);
-    return bits + (fill ? (GP_HMAX + 1) * sizeof(int) : 0);
-}
-
-int col_build_device(cheb_plan *plan, const cheb_bsr *L, int32_t ucap, cudaStream_t s) {
+int col_build_device(cheb_plan *plan, const cheb_bsr *L, cudaStream_t s) {
     ColLists c;
-    c.P = COL_P;
+    const bool wide = wide_elements(plan->precision);
+    c.P = col_width(plan->precision);
     c.NW = COL_NW;
-    c.ucap = ucap;
-    constexpr int CW = COL_EK * 32 / COL_P;
+    c.nnzL = L->nnzb;
+    c.ucap = col_ucap(c.P);
     const int64_t nbr = plan->nbr, nnzL = L->nnzb;
-    if (nnzL + 1 >= ((int64_t)1 << (32 - COL_SLOT_BITS))) return CHEB_ERR_NOSPACE;
-    const size_t dyn_fill = gp_dyn_smem(nbr, true);
-    if (dyn_fill + 48 * 1024 > (size_t)CHEB_MAX_DYN_SMEM) return CHEB_ERR_NOSPACE;
+    if (!col_wanted(plan, nnzL)) return CHEB_ERR_NOSPACE;
+    // (dynamic shared memory of k_gp_rows: bitmap words, operator slots of the rows)
+    const size_t off_list = align_up((size_t)((nbr + 31) / 32) * sizeof(uint2), 16) +
+                            align_up((size_t)c.ucap * ((c.ucap + 31) / 32) * 4, 16);
+    const size_t dyn = off_list + (size_t)GP_NWARP * GP_MAXU * 2;
+    if (dyn + 48 * 1024 > (size_t)CHEB_MAX_DYN_SMEM) return CHEB_ERR_NOSPACE;
     // scratch: stamps, panels (at most one per column), counts and offsets
     const size_t n1 = (size_t)nbr + 1;
     size_t off = 0;
@@ -558,7 +606,8 @@ int col_build_device(cheb_plan *plan, const cheb_bsr *L, int32_t ucap, cudaStrea
         return o;
     };
     const size_t o_stamp = at(nbr * 4), o_pan = at(4 * nbr * 4), o_out = at(8 * 8), o_chunks = at(nbr * 8),
-                 o_rows = at(nbr * 8), o_max = at(nbr * 4), o_choff = at(n1 * 8), o_rooff = at(n1 * 8);
+                 o_rows = at(nbr * 8), o_max = at(nbr * 4), o_choff = at(n1 * 8), o_rooff = at(n1 * 8),
+                 o_sys = at(plan->h_sys_col.size() * 8);
     char *scr = nullptr;
     CHEB_CUDA(cudaMalloc(&scr, off));
     struct Free {
@@ -570,11 +619,13 @@ int col_build_device(cheb_plan *plan, const cheb_bsr *L, int32_t ucap, cudaStrea
     int64_t *cnt_chunks = reinterpret_cast<int64_t *>(scr + o_chunks), *cnt_rows = reinterpret_cast<int64_t *>(scr + o_rows);
     int32_t *cnt_max = reinterpret_cast<int32_t *>(scr + o_max);
     int64_t *choff = reinterpret_cast<int64_t *>(scr + o_choff), *rooff = reinterpret_cast<int64_t *>(scr + o_rooff);
+    int64_t *dsys = reinterpret_cast<int64_t *>(scr + o_sys);
     int32_t *err = reinterpret_cast<int32_t *>(out + 4);
     CHEB_CUDA(cudaMemsetAsync(stamp, 0xff, nbr * 4, s));
     CHEB_CUDA(cudaMemsetAsync(out, 0, 8 * 8, s));
-    k_gp_panels<<<1, GP_NT, 0, s>>>(plan->rp, plan->ci, nbr, COL_P, ucap, INT64_MAX, nullptr, 1, stamp, pan, nullptr,
-                                    out);
+    CHEB_CUDA(cudaMemcpyAsync(dsys, plan->h_sys_col.data(), plan->h_sys_col.size() * 8, cudaMemcpyHostToDevice, s));
+    k_gp_panels<<<1, GP_NT, 0, s>>>(plan->rp, plan->ci, nbr, c.P, c.ucap, INT64_MAX, dsys, plan->nsys, stamp, pan,
+                                    nullptr, out);
     CHEB_TRY(check_launch("k_gp_panels"));
     int64_t h_out[3];
     CHEB_CUDA(cudaMemcpyAsync(h_out, out, sizeof(h_out), cudaMemcpyDeviceToHost, s));
@@ -595,28 +646,33 @@ int col_build_device(cheb_plan *plan, const cheb_bsr *L, int32_t ucap, cudaStrea
     a.cnt_rows = cnt_rows;
     a.cnt_maxrow = cnt_max;
     a.err = err;
-    const size_t dyn_count = gp_dyn_smem(nbr, false);
-    CHEB_CUDA(cudaFuncSetAttribute(k_gp_rows<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn_count));
-    CHEB_CUDA(cudaFuncSetAttribute(k_gp_rows<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn_fill));
-    k_gp_rows<false><<<(unsigned)np, GP_NT, dyn_count, s>>>(a);
+    a.off_list = off_list;
+    CHEB_CUDA(cudaFuncSetAttribute(k_gp_rows<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
+    CHEB_CUDA(cudaFuncSetAttribute(k_gp_rows<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
+    k_gp_rows<false><<<(unsigned)np, GP_NT, dyn, s>>>(a);
     CHEB_TRY(check_launch("k_gp_rows count"));
     k_gp_scan<<<1, 1024, 0, s>>>(cnt_chunks, np, choff);
     k_gp_scan<<<1, 1024, 0, s>>>(cnt_rows, np, rooff);
     CHEB_TRY(check_launch("k_gp_scan", 2));
     std::vector<int32_t> h_max(np);
+    std::vector<int32_t> h_pan(4 * np);
     int64_t tot[2];
     int32_t h_err = 0;
     CHEB_CUDA(cudaMemcpyAsync(h_max.data(), cnt_max, np * 4, cudaMemcpyDeviceToHost, s));
+    CHEB_CUDA(cudaMemcpyAsync(h_pan.data(), pan, 4 * np * 4, cudaMemcpyDeviceToHost, s));
     CHEB_CUDA(cudaMemcpyAsync(&tot[0], choff + np, 8, cudaMemcpyDeviceToHost, s));
     CHEB_CUDA(cudaMemcpyAsync(&tot[1], rooff + np, 8, cudaMemcpyDeviceToHost, s));
     CHEB_CUDA(cudaMemcpyAsync(&h_err, err, 4, cudaMemcpyDeviceToHost, s));
     CHEB_CUDA(cudaStreamSynchronize(s));
     if (h_err) return fail(CHEB_ERR_INVALID, "gather plan: inconsistent panel union (code %d)", h_err);
-    if (tot[0] * CW >= (int64_t)INT32_MAX) return CHEB_ERR_NOSPACE;
     for (const int32_t m : h_max) c.max_row = std::max(c.max_row, m);
-    c.n_entries = tot[0] * CW;
-    c.n_rows = tot[1];
+    if ((tot[0] + COL_TAIL) * COL_CW >= (int64_t)INT32_MAX || (wide && c.max_row > COL_MAX_QUADS64)) return CHEB_ERR_NOSPACE;
+    c.n_entries = (tot[0] + COL_TAIL) * COL_CW;
+    c.n_rows = 2 * tot[1];
     c.n_slot = plan->nnzb;
+    c.h_sys_panel.assign(plan->nsys + 1, (int32_t)np);
+    for (int64_t p = np - 1; p >= 0; --p) c.h_sys_panel[h_pan[4 * p + 3]] = (int32_t)p;
+    c.n_sys = (int64_t)c.h_sys_panel.size();
     // the lists, in device memory of their own until cheb_plan_bind_operator
     // copies them into the operator workspace
     c.built = true;  // (sizes complete: bytes() counts them from here on)
@@ -636,7 +692,10 @@ int col_build_device(cheb_plan *plan, const cheb_bsr *L, int32_t ucap, cudaStrea
     c.d_rows = cv.take<uint32_t>(std::max<int64_t>(c.n_rows, 1));
     c.d_ent = cv.take<uint32_t>(std::max<int64_t>(c.n_entries, 1));
     c.d_slot = cv.take<uint16_t>(c.n_slot);
+    c.d_sys_panel = cv.take<int32_t>(c.n_sys);
+    CHEB_CUDA(cudaMemcpyAsync(c.d_sys_panel, c.h_sys_panel.data(), c.n_sys * 4, cudaMemcpyHostToDevice, s));
     CHEB_CUDA(cudaMemcpyAsync(c.d_panels, pan, 4 * np * 4, cudaMemcpyDeviceToDevice, s));
+    CHEB_CUDA(cudaMemsetAsync(c.d_ent + tot[0] * COL_CW, 0, COL_TAIL * COL_CW * 4, s));
     a.chunk_off = choff;
     a.row_off = rooff;
     a.wchunk = c.d_wchunk;
@@ -644,7 +703,7 @@ int col_build_device(cheb_plan *plan, const cheb_bsr *L, int32_t ucap, cudaStrea
     a.rows = c.d_rows;
     a.ent = c.d_ent;
     a.slot = c.d_slot;
-    k_gp_rows<true><<<(unsigned)np, GP_NT, dyn_fill, s>>>(a);
+    k_gp_rows<true><<<(unsigned)np, GP_NT, dyn, s>>>(a);
     CHEB_TRY(check_launch("k_gp_rows fill"));
     CHEB_CUDA(cudaMemcpyAsync(&h_err, err, 4, cudaMemcpyDeviceToHost, s));
     CHEB_CUDA(cudaStreamSynchronize(s));

@@ -578,10 +578,8 @@ extern "C" int cheb_plan_attach_operator(cheb_plan *plan, const cheb_bsr *L, siz
         plan->op_ci = L->col_idx;
         plan->lists = std::move(lists);
         plan->rlists = std::move(rlists);
-        if (plan->precision == CHEB_F32 || plan->precision == CHEB_BF16) {
-            rc = col_build_device(plan, L, col_ucap(), s);
-            if (rc != CHEB_OK && rc != CHEB_ERR_NOSPACE) return rc;
-        }
+        rc = col_build_device(plan, L, s);
+        if (rc != CHEB_OK && rc != CHEB_ERR_NOSPACE) return rc;
         plan->op_ws_bytes = plan->lists.bytes() + plan->rlists.bytes() + plan->col.bytes();
         *op_ws_bytes = plan->op_ws_bytes;
         return CHEB_OK;
@@ -610,13 +608,10 @@ extern "C" int cheb_plan_attach_operator(cheb_plan *plan, const cheb_bsr *L, siz
     plan->op_ci = L->col_idx;
     plan->lists = std::move(lists);
     plan->rlists = std::move(rlists);
-    // reduced-precision plans: the column-order step kernel's lists (left
-    // unbuilt when a panel column or an operator row does not fit it; the
-    // per-step products then use the ranking kernel)
-    if (plan->precision == CHEB_F32 || plan->precision == CHEB_BF16) {
-        const int rc = col_build(plan, rp, ci, lrp, lci);
-        if (rc != CHEB_OK && rc != CHEB_ERR_NOSPACE) return rc;
-    }
+    // the column-order kernel's lists (left unbuilt when a panel column or the
+    // operator does not fit it; the expansions then use the ranking kernels)
+    const int rc = col_build(plan, rp, ci, lrp, lci);
+    if (rc != CHEB_OK && rc != CHEB_ERR_NOSPACE) return rc;
     plan->op_ws_bytes = plan->lists.bytes() + plan->rlists.bytes() + plan->col.bytes();
     plan->op_bound = false;
     *op_ws_bytes = plan->op_ws_bytes;

@@ -28,15 +28,15 @@ struct RowLists {
     }
 };
 
-// Data of the column-order step kernel (colstep.cu) for one operator pattern:
-// its own panels (at most COL_P columns whose union fits shared memory), in
-// column order, as (first column, column count, union rows, 0); per panel and
-// warp a range of chunks and of rows; per warp row a word (union slot, a flag
-// for rows with blocks in at most two of the panel's columns and those
-// columns, chunk count); the chunks' entry words (index of the block L_IK in the
-// operator << COL_SLOT_BITS | union slot of K; COL_EK * 32/COL_P words per
-// chunk, word e * 32/COL_P + g for K-group g); and
-// the union slot of every P_out block in column order.
+// Data of the column-order kernel (colstep.cu) for one operator pattern: its own
+// panels (at most P columns of one system whose union fits shared memory), in
+// column order, as (first column, column count, union rows, system); per panel
+// and warp a range of quads and of groups; per group two words (its four union
+// slots, COL_SLOT_BITS each, all ones where the panel has no more rows, and its
+// quad count); the quads' entry words (index of the block L_IK in the operator <<
+// COL_SLOT_BITS | union slot of K; COL_CW words per quad, word ((a & 1) * 4 + t) *
+// 2 + (a >> 1) for row a of the group and slot t of the quad); and the union slot
+// of every P_out block in column order.
 struct ColLists {
     int32_t P = 0, NW = 0;
     int32_t ucap = 0, max_union = 0, max_row = 0;
@@ -48,13 +48,16 @@ struct ColLists {
     std::vector<uint32_t> h_rows;
     std::vector<uint32_t> h_ent;
     std::vector<uint16_t> h_slot;
+    std::vector<int32_t> h_sys_panel;  // first panel of each system (+ end)
+    int64_t nnzL = 0;                  // operator blocks
     int32_t *d_panels = nullptr;
     int32_t *d_wchunk = nullptr;
     int32_t *d_wrow = nullptr;
     uint32_t *d_rows = nullptr;
     uint32_t *d_ent = nullptr;
     uint16_t *d_slot = nullptr;
-    int64_t n_rows = 0, n_slot = 0;  // row words; P_out blocks (one slot each)
+    int32_t *d_sys_panel = nullptr;
+    int64_t n_rows = 0, n_slot = 0, n_sys = 0;  // group words; P_out blocks (one slot each); systems + 1
     bool built = false, bound = false;
     // built by the gather-plan kernels (gather.cu): the d_ arrays live in tmp
     // (device memory of their own) until cheb_plan_bind_operator copies them
@@ -64,7 +67,8 @@ struct ColLists {
         if (!built) return 0;
         return ::cheb::align_up((size_t)n_panels * 16) + 2 * ::cheb::align_up((size_t)n_panels * (NW + 1) * 4) +
                ::cheb::align_up((size_t)std::max<int64_t>(n_rows, 1) * 4) +
-               ::cheb::align_up((size_t)std::max<int64_t>(n_entries, 1) * 4) + ::cheb::align_up((size_t)n_slot * 2);
+               ::cheb::align_up((size_t)std::max<int64_t>(n_entries, 1) * 4) + ::cheb::align_up((size_t)n_slot * 2) +
+               ::cheb::align_up((size_t)n_sys * 4);
     }
 };
 
@@ -111,7 +115,7 @@ struct cheb_plan {
     const int64_t *op_rp = nullptr;
     const int32_t *op_ci = nullptr;
     RowLists lists, rlists;
-    ColLists col;  // FP32 / BF16 plans: the column-order step kernel's lists
+    ColLists col;  // the column-order kernel's lists
     int32_t gather_host = 0;  // 1: build them on host threads (the reference builder)
     size_t op_ws_bytes = 0;
     bool op_bound = false;
@@ -194,36 +198,49 @@ __host__ __device__ inline ResLayout res_layout(int64_t nw, int64_t ucap, int64_
     return L;
 }
 
-// Column-order step kernel (colstep.cu): panel width, warps, operator stages
-// per warp, and its shared-memory layout for a union of ucap rows: the warps'
-// stages of operator blocks, the panel's T_k blocks X[slot][4][4P] (FP32),
-// the column-order position of each (union row, panel column) block, the
-// moment partials of the warps.
-constexpr int COL_P = 4;
+// Column-order kernel (colstep.cu): warps per thread block, words per quad, and
+// its shared-memory layout: the warps' moment partials, the groups' words, the grid
+// exponent of each union row, the column-order position of each (union row, panel
+// column) block, and the panel's digits.  (Offsets are constants, so that they take
+// no registers.)
 constexpr int COL_NW = 16;
-constexpr int COL_STAGES = 3;
-constexpr int COL_EK = 2;  // operator entries of each K-group per chunk
-constexpr int COL_SLOT_BITS = 10;  // union slots < 1024; operator blocks < 2^22
-// a row word: union slot | half-row flag << 10 | its two columns << 11, << 13
-// | chunk count << COL_ROW_SHIFT
-constexpr int COL_ROW_SHIFT = COL_SLOT_BITS + 5;
+constexpr int COL_CW = 16;         // 4 rows x 4 merged slots
+// Unassigned rows among which a group's next row is chosen.  Merged slots over
+// entries, P = 4: 1.51 for consecutive rows, 1.46 with 64 candidates, 1.44 with all
+// (Hilbert order); 1.83, 1.58 and 1.56 (Morton order, 8 bohr rows).
+constexpr int COL_WINDOW = 64;
+constexpr int COL_TAIL = 8;        // quads of padding behind the lists (read ahead, not used)
+constexpr int COL_SLOT_BITS = 10;  // union slots < 1023; operator blocks < 2^22
+// Union rows of a panel at most.  Columns beyond it run on the ranking kernels.
+constexpr int COL_MAX_UNION = 667;
+// (quads of a group come in pairs) FP64: quads of a group at most, so that its exact digit sums (at most 4
+// products of 2^18 per merged row of a slot) stay below 2^31.
+constexpr int COL_MAX_QUADS64 = 126;
+// Operator blocks per block row, on average, from which FP64 expansions and the
+// one-launch forms run on the column kernel.  Short rows stay on the kernels whose
+// results are the same bits with and without attached lists.
+constexpr int64_t COL_ROW_MIN = 48;
+// panel width: 16 scalar columns of FP32 or 8 of FP64 fill two or one mma tiles
+inline int col_width(int precision) { return precision == CHEB_F64 || precision == CHEB_F64X ? 2 : 4; }
 struct ColLayout {
-    size_t off_x, off_pos, off_stage, off_red, total;
+    int off_red, off_rows, off_rexp, off_pos, off_x, slot_bytes;
+    __host__ __device__ constexpr size_t total(int64_t ucap) const { return (size_t)off_x + (size_t)ucap * slot_bytes; }
 };
-__host__ __device__ inline ColLayout col_layout(int64_t ucap, int P, int nwarps) {
-    ColLayout L;
-    const int kg = 32 / P;
-    size_t o = 0;
-    L.off_stage = o;  // per warp: COL_STAGES chunks of COL_EK * 32/P operator blocks
-    o += (size_t)nwarps * COL_STAGES * COL_EK * kg * 64;
-    L.off_x = o;
-    o += (size_t)ucap * 64 * P;
-    L.off_pos = o;
-    o += (size_t)ucap * P * 4;
-    o = (o + 15) / 16 * 16;
+// P = 4: FP32 / BF16 (two f16 digits of 4 values in a 16-byte chunk per column,
+// and a byte of each value's third digit); P = 2: FP64 (six digits)
+__host__ __device__ constexpr ColLayout col_layout(int P) {
+    ColLayout L{};
+    int o = 0;
     L.off_red = o;
-    o += (size_t)nwarps * 6 * 8;  // moment partials: 6 per warp
-    L.total = o;
+    o += COL_NW * 4 * 8;
+    L.off_rows = o;
+    o += (COL_MAX_UNION + 3) / 4 * 8;
+    L.off_rexp = o;
+    o += COL_MAX_UNION * 4;
+    L.off_pos = o;
+    o += COL_MAX_UNION * P * 4;
+    L.off_x = (o + 127) / 128 * 128;
+    L.slot_bytes = P == 4 ? 16 * 20 : 8 * 48;
     return L;
 }
 
@@ -249,13 +266,33 @@ inline size_t smem_budget(int minb) {
     return per < (size_t)CHEB_MAX_DYN_SMEM ? per : (size_t)CHEB_MAX_DYN_SMEM;
 }
 
-// Column-order step kernel (colstep.cu): host build and binding of its lists,
-// and the expansion through it.
-int32_t col_ucap();
+// Column-order kernel (colstep.cu): host build and binding of its lists, and
+// the expansion through it.
+int32_t col_ucap(int P);
+// Places of n <= 8 ascending slots in two quads (place = 4 quad + j): a slot goes to
+// the first quad without a slot of its residue modulo 4, because the lanes of a
+// quad's slots then read different shared-memory banks; failing that, to the first
+// quad with room.
+__host__ __device__ inline void col_places(const uint16_t *slot, int n, uint8_t *place) {
+    unsigned used[2] = {0u, 0u};
+    int fill[2] = {0, 0};
+    for (int pass = 0; pass < 2; ++pass)
+        for (int i = 0; i < n; ++i) {
+            if (pass == 0) place[i] = 255;
+            else if (place[i] != 255) continue;
+            const unsigned r = 1u << (slot[i] & 3);
+            int q = !(used[0] & r) && fill[0] < 4 ? 0 : !(used[1] & r) && fill[1] < 4 ? 1 : -1;
+            if (q < 0 && pass == 1) q = fill[0] < 4 ? 0 : 1;
+            if (q < 0) continue;
+            used[q] |= r;
+            place[i] = (uint8_t)(4 * q + fill[q]++);
+        }
+}
+bool col_wanted(const cheb_plan *plan, int64_t nnzL);
 int col_build(cheb_plan *plan, const std::vector<int64_t> &rp, const std::vector<int32_t> &ci,
               const std::vector<int64_t> &lrp, const std::vector<int32_t> &lci);
 // the same lists built by device kernels from the device patterns (gather.cu)
-int col_build_device(cheb_plan *plan, const cheb_bsr *L, int32_t ucap, cudaStream_t s);
+int col_build_device(cheb_plan *plan, const cheb_bsr *L, cudaStream_t s);
 void col_free(ColLists &c);
 // the plan of P_out and the row lists on the device (gather.cu)
 int gp_check_pattern(const int64_t *rp, const int32_t *ci, int64_t nbr, int64_t nnzb, int64_t first[4],
@@ -272,8 +309,24 @@ int col_bind(ColLists &c, Carve &cv, cudaStream_t s);
 void col_release_host(ColLists &c);
 bool col_usable(const cheb_plan *plan, const cheb_bsr *Mt);
 size_t col_expand_ws(const cheb_plan *plan, int64_t nnzL);
-int col_expand(const cheb_plan *plan, const cheb_bsr *Mt, int32_t n_terms, const double *coeffs, int32_t stride,
-               int32_t nf, double *const *acc, double *moments, const double *G, double *gmoments, void *ws,
-               size_t ws_bytes, cudaStream_t s, int round_bf16);
+// One expansion through the column kernel: n_terms per system on the device, or
+// max_terms for every system; coefficients at coef + coef_off[system].
+struct ColExpand {
+    int32_t max_terms;
+    const int32_t *n_terms;
+    const double *coef;
+    const int64_t *coef_off;
+    int32_t coef_stride, nf;
+    double *const *acc;
+    double *moments;
+    const double *G;
+    double *gmoments;
+    int64_t mom_stride;
+    int32_t round_bf16;
+};
+// Whether the column kernel takes the expansion: its lists are bound for this
+// operator, the workspace holds its buffers, and the caller's arrays are aligned.
+bool col_takes(const cheb_plan *plan, const cheb_bsr *Mt, const ColExpand &x, size_t ws_bytes);
+int col_expand(const cheb_plan *plan, const cheb_bsr *Mt, const ColExpand &x, void *ws, size_t ws_bytes, cudaStream_t s);
 
 }  // namespace cheb

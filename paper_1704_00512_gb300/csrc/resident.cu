@@ -471,6 +471,12 @@ size_t resident_ws(const cheb_plan *plan, int64_t nnzL, int precision, int kmax)
     return b + 256;
 }
 
+// The column kernel runs the one-launch forms where its lists are attached and
+// the operator's rows are long (COL_ROW_MIN).
+static bool res_col(const cheb_plan *plan, const cheb_bsr *Mt) {
+    return col_usable(plan, Mt) && Mt->nnzb >= COL_ROW_MIN * plan->nbr;
+}
+
 template <typename T>
 int resident_impl(const cheb_plan *plan, const cheb_bsr *Mt, int kmax, const int32_t *n_terms_dev, int n_single,
                   const double *coeffs, const int64_t *coef_off, int32_t stride, int32_t nf, double *const *acc,
@@ -550,6 +556,7 @@ extern "C" int cheb_expand_workspace_size(const cheb_plan *plan, const cheb_bsr 
     if (!plan || !Mt || !bytes || max_terms < 2)
         return fail(CHEB_ERR_INVALID, "cheb_expand_workspace_size: bad arguments");
     *bytes = resident_ws(plan, Mt->nnzb, precision, max_terms);
+    if (res_col(plan, Mt)) *bytes = std::max(*bytes, col_expand_ws(plan, Mt->nnzb));
     return CHEB_OK;
 }
 
@@ -567,6 +574,9 @@ extern "C" int cheb_expand(const cheb_plan *plan, const cheb_bsr *Mt, int32_t n_
     if (!ws || ws_bytes < need) return fail(CHEB_ERR_NOSPACE, "cheb_expand: workspace %zu < %zu", ws_bytes, need);
     cudaStream_t s = as_stream(stream);
     const double *cf = coeffs;  // never read when n_f == 0
+    const ColExpand x{n_terms, nullptr, cf, nullptr, coeff_stride, n_f, acc, moments, G, gmoments, n_terms,
+                      precision == CHEB_BF16};
+    if (res_col(plan, Mt) && col_takes(plan, Mt, x, ws_bytes)) return col_expand(plan, Mt, x, ws, ws_bytes, s);
     if (precision == CHEB_F64)
         return resident_impl<double>(plan, Mt, n_terms, nullptr, n_terms, cf, nullptr, coeff_stride, n_f, acc, moments,
                                      G, gmoments, n_terms, ws, ws_bytes, s);
@@ -595,6 +605,9 @@ extern "C" int cheb_expand_batched(const cheb_plan *plan, const cheb_bsr *Mt, in
     if (!ws || ws_bytes < need) return fail(CHEB_ERR_NOSPACE, "cheb_expand_batched: workspace %zu < %zu", ws_bytes, need);
     cudaStream_t s = as_stream(stream);
     const double *cf = coeffs;  // never read when n_f == 0
+    const ColExpand x{max_terms, n_terms, cf, n_f > 0 ? coeff_offset : nullptr, coeff_stride, n_f, acc, moments, G,
+                      gmoments, moment_stride, precision == CHEB_BF16};
+    if (res_col(plan, Mt) && col_takes(plan, Mt, x, ws_bytes)) return col_expand(plan, Mt, x, ws, ws_bytes, s);
     if (precision == CHEB_F64)
         return resident_impl<double>(plan, Mt, max_terms, n_terms, 0, cf, n_f > 0 ? coeff_offset : nullptr,
                                      coeff_stride, n_f, acc, moments, G, gmoments, moment_stride, ws, ws_bytes, s);
