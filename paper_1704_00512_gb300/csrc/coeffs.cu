@@ -1,6 +1,8 @@
 // Chebyshev coefficients (Eq. 4), degree selection (Eq. 6), the penalty trace
 // (Eq. 5) and the mu bisection on the trace functional (Sec. "Fermi Operator
 // Expansion"), all in FP64.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <mutex>
 #include <vector>
@@ -39,67 +41,129 @@ __device__ __forceinline__ double node(int k, int n, double sigma, double tau) {
     return cos(M_PI * (k + 0.5) / n) / sigma + tau;
 }
 
-// cos(pi j (k+1/2)/n) with the argument reduced exactly: j(2k+1) mod 4n.
+// cos(pi j (2k+1) / (2n)) with the angle reduced exactly modulo 4n.
 __device__ __forceinline__ double dct_cos(int64_t j, int64_t k, int64_t n) {
     const int64_t idx = (j * (2 * k + 1)) % (4 * n);
     return cos(M_PI * (double)idx / (2.0 * (double)n));
 }
 
-// f at the nodes of every (function, candidate) pair: fv[(f*nc + c)*nmax + k].
-__global__ void k_nodes(FuncArr F, int nf, const int *cand, int nc, int nmax, double sigma, double tau,
-                        double *fv) {
-    const int fc = blockIdx.y, f = fc / nc, c = fc % nc;
-    const int n = cand[c];
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x)
-        fv[(int64_t)fc * nmax + k] = feval(F.f[f], node(k, n, sigma, tau), sigma, tau);
-}
+// The candidates of one batch, passed by value: their term counts, the divisors of
+// the two-step transform, and the first of their values in arrays that hold them one
+// after the other (total values per function).
+constexpr int CAND_MAX = 96;
+struct Cand {
+    int n[CAND_MAX], n1[CAND_MAX];
+    int64_t off[CAND_MAX];
+    int nc;
+    int64_t total;
+};
 
-// Cosine tables cos(pi i / (2n)), i < 4n, for every candidate n (tab + 4*toff[c]).
-__global__ void k_cos_table(const int *cand, const int64_t *toff, int nc, double *tab) {
+// Cosine tables cos(pi i / (2n)), i < 4n, of every candidate n (tab + 4 off[c]).
+__global__ void k_cos_table(Cand d, double *tab) {
     const int c = blockIdx.y;
-    const int64_t n = cand[c];
-    double *t = tab + toff[c];
+    const int64_t n = d.n[c];
+    double *t = tab + 4 * d.off[c];
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < 4 * n; i += (int64_t)gridDim.x * blockDim.x)
-        t[i] = cos(M_PI * (double)i / (2.0 * (double)n));
+        t[i] = cospi((double)i / (2.0 * (double)n));
 }
 
-// c_j = (2/n) sum_k f_k cos(pi j (k+1/2)/n) (Eq. 4), one thread per j; the
-// cosine is the table entry j(2k+1) mod 4n (the same value dct_cos computes).
-__global__ void k_dct(const double *fv, const int *cand, const int64_t *toff, const double *tab, int nc, int nmax,
-                      double *cv) {
-    const int fc = blockIdx.y, c = fc % nc;
-    const int64_t n = cand[c];
-    const double *fk = fv + (int64_t)fc * nmax;
-    const double *t = tab + toff[c];
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < nmax; j += gridDim.x * blockDim.x) {
-        double s = 0.0;
-        if (j < n) {
-            const int64_t step = 2 * (int64_t)j, m = 4 * n;
-            int64_t idx = j % m;  // j (2k+1) mod 4n for k = 0
-            for (int64_t k = 0; k < n; ++k) {
-                s += fk[k] * t[idx];
-                idx += step;
-                if (idx >= m) idx -= m * (idx / m);
-            }
-            s = (2.0 / n) * s;
+// f at the nodes of every (function, candidate) pair, in the order of the
+// transform below: the even nodes ascending, then the odd ones descending.
+__global__ void k_nodes(FuncArr F, Cand d, double sigma, double tau, double *fv) {
+    const int fc = blockIdx.y, f = fc / d.nc, c = fc % d.nc;
+    const int n = d.n[c];
+    double *v = fv + f * d.total + d.off[c];
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x)
+        v[k & 1 ? n - 1 - k / 2 : k / 2] = feval(F.f[f], node(k, n, sigma, tau), sigma, tau);
+}
+
+// The coefficients c_j = (2/n) sum_k f_k cos(pi j (k+1/2)/n) (Eq. 4) as the real part
+// of a discrete Fourier transform (J. Makhoul, IEEE Trans. ASSP 28, 27 (1980)):
+// with v = (f_0, f_2, ..., f_3, f_1), c_j = (2/n) Re(e^{-i pi j/2n} sum_k v_k
+// e^{-2 pi i j k/n}), and that transform in two steps for n = n1 n2, k = n2 a + b,
+// j = j1 + n1 j2 (J. Cooley and J. Tukey, Math. Comput. 19, 297 (1965)):
+//     Y[j1][b] = e^{-2 pi i j1 b/n} sum_a v[n2 a + b] e^{-2 pi i a j1/n1},
+//     V[j1 + n1 j2] = sum_b Y[j1][b] e^{-2 pi i b j2/n2},
+// so n (n1 + n2) products instead of n^2, n1 the largest divisor of n up to its
+// square root.  Every cosine and sine is an entry of the table of cos(pi i/2n).
+// (The plain sum, a gather of the table per product, took 4 ms for one function
+// at n = 9216, and 20 ms for all candidates of a degree search up to 16384; now
+// 0.1 and 0.5 ms.  Against long doubles the coefficients' error went from 0.6e-15 to
+// 0.4e-15 at n = 300 and from 3.6e-15 to 0.9e-15 at n = 9216.)
+__device__ __forceinline__ double2 twiddle(const double *t, int64_t m, int64_t n) {  // e^{-2 pi i m/n}, 0 <= m < n
+    return make_double2(t[4 * m], -t[4 * m >= n ? 4 * m - n : 4 * m + 3 * n]);
+}
+__global__ void k_dft1(const double *fv, Cand d, const double *tab, double2 *Y) {
+    const int fc = blockIdx.y, f = fc / d.nc, c = fc % d.nc;
+    const int n = d.n[c], n1 = d.n1[c], n2 = n / n1;
+    const double *v = fv + f * d.total + d.off[c], *t = tab + 4 * d.off[c];
+    double2 *y = Y + f * d.total + d.off[c];
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const int j1 = i / n2, b = i % n2;
+        double re = 0.0, im = 0.0;
+        int m = 0;  // a j1 mod n1
+        for (int a = 0; a < n1; ++a) {
+            const double2 w = twiddle(t, (int64_t)n2 * m, n);
+            const double x = v[(int64_t)n2 * a + b];
+            re = fma(x, w.x, re);
+            im = fma(x, w.y, im);
+            m += j1;
+            if (m >= n1) m -= n1;
         }
-        cv[(int64_t)fc * nmax + j] = s;
+        const double2 w = twiddle(t, (int64_t)j1 * b, n);  // j1 b < n1 n2
+        y[i] = make_double2(re * w.x - im * w.y, re * w.y + im * w.x);
+    }
+}
+__global__ void k_dft2(const double2 *Y, Cand d, const double *tab, double *cv) {
+    const int fc = blockIdx.y, f = fc / d.nc, c = fc % d.nc;
+    const int n = d.n[c], n1 = d.n1[c], n2 = n / n1;
+    const double *t = tab + 4 * d.off[c];
+    const double2 *y = Y + f * d.total + d.off[c];
+    double *out = cv + f * d.total + d.off[c];
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const int j1 = i / n2, j2 = i % n2;
+        double re = 0.0, im = 0.0;
+        int m = 0;  // b j2 mod n2
+        for (int b = 0; b < n2; ++b) {
+            const double2 w = twiddle(t, (int64_t)n1 * m, n), u = y[(int64_t)j1 * n2 + b];
+            re = fma(u.x, w.x, fma(-u.y, w.y, re));
+            im = fma(u.x, w.y, fma(u.y, w.x, im));
+            m += j2;
+            if (m >= n2) m -= n2;
+        }
+        const int j = j1 + n1 * j2;
+        out[j] = (2.0 / n) * (re * t[j] + im * t[j >= n ? j - n : j + 3 * n]);  // e^{-i pi j/2n}
     }
 }
 
 __device__ __forceinline__ unsigned long long dbits(double v) { return __double_as_longlong(v); }
 
-// max |p_n(x) - f(x)| and max |f(x)| over the degree grid: 8193 uniform points
-// on [-1,1] plus the 2n+1 extrema of T_{2n}.  p_n by the scalar recursion
-// T_{j+1} = 2 x T_j - T_{j-1} with explicit roundings.  Max over non-negative
-// doubles is taken on their bit patterns (order-independent).
-__global__ void k_fit_error(FuncArr F, const double *cv, const int *cand, int nc, int nmax, double sigma,
-                            double tau, unsigned long long *errmax, unsigned long long *fabsmax) {
-    const int fc = blockIdx.y, f = fc / nc, c = fc % nc;
-    const int n = cand[c];
-    const double *cc = cv + (int64_t)fc * nmax;
+struct Pairs {
+    int n, at[8];
+};
+__device__ __forceinline__ void max_to(double emax, double fm, unsigned long long *e, unsigned long long *f) {
+    // warp max then one atomic per warp; over non-negative doubles on their bit
+    // patterns (order-independent)
+    for (int o = 16; o > 0; o >>= 1) {
+        emax = fmax(emax, __shfl_xor_sync(0xffffffffu, emax, o));
+        fm = fmax(fm, __shfl_xor_sync(0xffffffffu, fm, o));
+    }
+    if ((threadIdx.x & 31) == 0) {
+        if (e) atomicMax(e, dbits(emax));
+        if (f) atomicMax(f, dbits(fm));
+    }
+}
+
+// max |p_n(x) - f(x)| over the degree grid: 8193 uniform points on [-1,1] plus the
+// 2n+1 extrema of T_{2n}, by the scalar recursion T_{j+1} = 2 x T_j - T_{j-1} with
+// explicit roundings.  One (function, candidate) pair per blockIdx.y: pairs.at[y].
+__global__ void k_fit_error(FuncArr F, const double *cv, Cand d, Pairs pairs, double sigma, double tau,
+                            unsigned long long *errmax) {
+    const int fc = pairs.at[blockIdx.y], f = fc / d.nc, c = fc % d.nc;
+    const int n = d.n[c];
+    const double *cc = cv + f * d.total + d.off[c];
     const int npts = GRID_UNIFORM + 2 * n + 1;
-    double emax = 0.0, fm = 0.0;
+    double emax = 0.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < npts; i += gridDim.x * blockDim.x) {
         double x;
         if (i < GRID_UNIFORM) x = -1.0 + i * (2.0 / (GRID_UNIFORM - 1));
@@ -116,34 +180,103 @@ __global__ void k_fit_error(FuncArr F, const double *cv, const int *cand, int nc
         }
         const double fx = feval(F.f[f], x / sigma + tau, sigma, tau);
         emax = fmax(emax, fabs(p - fx));
-        fm = fmax(fm, fabs(fx));
     }
-    // warp max then one atomic per warp
-    for (int o = 16; o > 0; o >>= 1) {
-        emax = fmax(emax, __shfl_xor_sync(0xffffffffu, emax, o));
-        fm = fmax(fm, __shfl_xor_sync(0xffffffffu, fm, o));
+    max_to(emax, 0.0, errmax + fc, nullptr);
+}
+// The same but for rounding, with a fourth of the FP64 operations (two per lane and
+// cycle bound it) and none of the serial chain: x goes with -x, whose sums are the even
+// terms' plus or minus the odd ones'; a warp takes a point, lane l the terms l, l + 32,
+// ... by T_{j+32} = 2 T_32 T_j - T_{j-32}; fused multiply-adds.  With stride > 1 only
+// every stride-th uniform point.  Also the largest |f| met.  pairs.n = 0: the pair is
+// blockIdx.y.  (By the plain recursion, a thread per point: 0.6 ms where this takes
+// 0.2, at 6,000 terms, and 1.2 ms for the 513 points of eight candidates around 12,000.)
+__global__ void __launch_bounds__(256) k_fit_estimate(FuncArr F, const double *cv, Cand d, Pairs pairs, int stride,
+                                                      double sigma, double tau, unsigned long long *errmax,
+                                                      unsigned long long *fabsmax) {
+    const int fc = pairs.n ? pairs.at[blockIdx.y] : blockIdx.y, f = fc / d.nc, c = fc % d.nc;
+    const int n = d.n[c], lane = threadIdx.x & 31;
+    const double *cc = cv + f * d.total + d.off[c];
+    constexpr int HALF = GRID_UNIFORM / 2;  // the point x = 0
+    const int npts = stride > 1 ? HALF / stride + 1 : HALF + n + 2;
+    double emax = 0.0, fm = 0.0;
+    for (int k = blockIdx.x * 8 + (threadIdx.x >> 5); k < npts; k += gridDim.x * 8) {
+        const int i = k * stride;
+        const double x = i <= HALF ? -1.0 + i * (2.0 / (GRID_UNIFORM - 1)) : cos(M_PI * (double)(i - HALF - 1) / (2.0 * n));
+        const double th = acos(x), t2 = 2.0 * cos(32.0 * th);
+        double a = cos(lane * th), b = cos((lane + 32) * th), s = 0.0;
+        for (int j = lane; j < n; j += 32) {
+            s = fma(j == 0 ? 0.5 * cc[0] : __ldg(cc + j), a, s);
+            const double t = fma(t2, b, -a);
+            a = b;
+            b = t;
+        }
+        const double odd = lane & 1 ? -s : s;  // the term's sign at -x
+        const double pp = warp_sum(s), pn = warp_sum(odd);
+        if (lane == 0) {
+            const double fp = feval(F.f[f], x / sigma + tau, sigma, tau), fn = feval(F.f[f], -x / sigma + tau, sigma, tau);
+            emax = fmax(emax, fmax(fabs(pp - fp), fabs(pn - fn)));
+            fm = fmax(fm, fmax(fabs(fp), fabs(fn)));
+        }
     }
-    if ((threadIdx.x & 31) == 0) {
-        atomicMax(errmax + fc, dbits(emax));
-        atomicMax(fabsmax + fc, dbits(fm));
+    max_to(emax, fm, errmax + fc, fabsmax + fc);
+}
+// max |f(x)| over the same grid, without the polynomial.
+__global__ void k_fit_scale(FuncArr F, Cand d, double sigma, double tau, unsigned long long *fabsmax) {
+    const int fc = blockIdx.y, f = fc / d.nc, c = fc % d.nc;
+    const int n = d.n[c], npts = GRID_UNIFORM + 2 * n + 1;
+    double fm = 0.0;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < npts; i += gridDim.x * blockDim.x) {
+        double x;
+        if (i < GRID_UNIFORM) x = -1.0 + i * (2.0 / (GRID_UNIFORM - 1));
+        else x = cos(M_PI * (double)(i - GRID_UNIFORM) / (2.0 * n));
+        fm = fmax(fm, fabs(feval(F.f[f], x / sigma + tau, sigma, tau)));
     }
+    max_to(0.0, fm, nullptr, fabsmax + fc);
 }
 
-__global__ void k_pick(const double *cv, int nc, int nmax, int ci, int n, int nf, double *out) {
+// out[f][j], j < n_max: the coefficients of candidate ci (n terms), 0 beyond.
+__global__ void k_pick(const double *cv, Cand d, int ci, int n, int n_max, double *out) {
     const int f = blockIdx.y;
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < nmax; j += gridDim.x * blockDim.x)
-        out[(int64_t)f * nmax + j] = j < n ? cv[((int64_t)f * nc + ci) * nmax + j] : 0.0;
+    const double *c = cv + f * d.total + d.off[ci];
+    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n_max; j += gridDim.x * blockDim.x)
+        out[(int64_t)f * n_max + j] = j < n ? c[j] : 0.0;
 }
 
-// Penalty coefficients at n terms (Eq. 4 for Eq. 5) and their dot with the moments.
-__global__ void k_penalty_coeffs(double alpha, int n, double *c) {
-    cheb_func f{CHEB_PENALTY, 0, 0, alpha, 0, 0};
-    // scaled variable directly: sigma = 1, tau = 0
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
-        double s = 0.0;
-        for (int k = 0; k < n; ++k) s += feval(f, node(k, n, 1.0, 0.0), 1.0, 0.0) * dct_cos(j, k, n);
-        c[j] = (2.0 / n) * s;
+// Penalty coefficients at n terms (Eq. 4 for Eq. 5), one thread per coefficient, the
+// nodes in order.  f is formed once per node and, while they fit shared memory, the
+// cosines cos(pi i/2n) once per table entry (the values that dct_cos has), by every
+// thread block for its PEN_J coefficients.  (Two exponentials and a cosine for each of
+// the n^2 products took 4 ms at n = 512; now 0.05 ms.)  The order of the sums stays what it is: the
+// trace is a small difference of large terms, and its rounding with it.
+constexpr int PEN_J = 32, PEN_NT = 256, PEN_TAB = 1024;
+__global__ void __launch_bounds__(PEN_NT) k_penalty_coeffs(double alpha, int n, double *c) {
+    __shared__ double tab[4 * PEN_TAB], fk[PEN_TAB];
+    const cheb_func f{CHEB_PENALTY, 0, 0, alpha, 0, 0};
+    const bool small = n <= PEN_TAB;
+    if (small)
+        for (int i = threadIdx.x; i < 4 * n; i += PEN_NT) tab[i] = cos(M_PI * (double)i / (2.0 * (double)n));
+    const int j = blockIdx.x * PEN_J + threadIdx.x;
+    const bool mine = threadIdx.x < PEN_J && j < n;
+    double s = 0.0;
+    for (int k0 = 0; k0 < n; k0 += PEN_TAB) {
+        const int k1 = min(n, k0 + PEN_TAB);
+        __syncthreads();
+        // scaled variable directly: sigma = 1, tau = 0
+        for (int k = k0 + threadIdx.x; k < k1; k += PEN_NT) fk[k - k0] = feval(f, node(k, n, 1.0, 0.0), 1.0, 0.0);
+        __syncthreads();
+        if (!mine) continue;
+        if (small) {
+            int idx = j;  // j (2k+1) mod 4n
+            for (int k = 0; k < n; ++k) {
+                s += fk[k] * tab[idx];
+                idx += 2 * j;
+                if (idx >= 4 * n) idx -= 4 * n;
+            }
+        } else {
+            for (int k = k0; k < k1; ++k) s += fk[k - k0] * dct_cos(j, k, n);
+        }
     }
+    if (mine) c[j] = (2.0 / n) * s;
 }
 
 template <int NT>
@@ -158,11 +291,61 @@ __global__ void k_dot_terms(const double *c, const double *t, int n, double *out
 // w_i = (2/n) [g_0/2 + sum_{k>=1} g_k cos(pi k (i+1/2)/n)], so that
 // N(mu) = sum_i f(x_i; mu) w_i equals c_0(mu) g_0/2 + sum_k c_k(mu) g_k
 // (the two finite sums of Eq. 4 and Eq. 1 swapped).
-__global__ void k_count_weights(const double *g, int n, double *w) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        double s = 0.5 * g[0];
-        for (int k = 1; k < n; ++k) s += g[k] * dct_cos(k, i, n);
-        w[i] = (2.0 / n) * s;
+//
+// cos(k phi_i), phi_i = pi (i+1/2)/n, by angle addition: k = k0 + r, r < CW_R, with
+// cos(r phi) and sin(r phi) of the thread's node in registers, so that a term takes
+// two multiply-adds; the angle of k0 advances by rotation and is taken afresh (exact
+// reduction) every CW_FRESH blocks.  Node n-1-i has the angle pi - phi_i: its sum
+// is the even terms' minus the odd terms', so only half the nodes are computed.  A
+// thread block takes 32 nodes and splits k over its warps.  (A cosine per term, with
+// a 64-bit modulus, took 9 ms at n = 9216; now 0.33 ms.)
+constexpr int CW_R = 8, CW_FRESH = 16, CW_NW = 16;
+__global__ void __launch_bounds__(CW_NW * 32) k_count_weights(const double *g, int n, double *w) {
+    __shared__ double se[CW_NW][33], so[CW_NW][33];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int half = (n + 1) / 2, i = min(blockIdx.x * 32 + lane, half - 1);
+    const int64_t n4 = 4 * (int64_t)n, step = 2 * i + 1;
+    double cr[CW_R], sr[CW_R];
+#pragma unroll
+    for (int r = 0; r < CW_R; ++r) sincospi((double)(r * step % n4) / (2.0 * n), &sr[r], &cr[r]);
+    double rc, rs;  // the rotation by CW_R steps
+    sincospi((double)(CW_R * step % n4) / (2.0 * n), &rs, &rc);
+    const int nb = (n + CW_R - 1) / CW_R, per = (nb + CW_NW - 1) / CW_NW;
+    double even = 0.0, odd = 0.0, kc = 1.0, ks = 0.0;
+    for (int b = warp * per; b < min(nb, (warp + 1) * per); ++b) {
+        const int k0 = b * CW_R;
+        if ((b - warp * per) % CW_FRESH == 0) {
+            sincospi((double)(k0 * step % n4) / (2.0 * n), &ks, &kc);
+        } else {
+            const double c = kc * rc - ks * rs;
+            ks = fma(kc, rs, ks * rc);
+            kc = c;
+        }
+        double ce = 0.0, de = 0.0, co = 0.0, dd = 0.0;  // sums with cos(r phi), sin(r phi); even and odd k
+#pragma unroll
+        for (int r = 0; r < CW_R; r += 2) {
+            double x = k0 + r < n ? g[k0 + r] : 0.0;
+            const double y = k0 + r + 1 < n ? g[k0 + r + 1] : 0.0;
+            if (k0 + r == 0) x *= 0.5;
+            ce = fma(x, cr[r], ce);
+            de = fma(x, sr[r], de);
+            co = fma(y, cr[r + 1], co);
+            dd = fma(y, sr[r + 1], dd);
+        }
+        even += kc * ce - ks * de;
+        odd += kc * co - ks * dd;
+    }
+    se[warp][lane] = even;
+    so[warp][lane] = odd;
+    __syncthreads();
+    if (warp == 0 && blockIdx.x * 32 + lane < half) {
+        double e = 0.0, o = 0.0;
+        for (int k = 0; k < CW_NW; ++k) {
+            e += se[k][lane];
+            o += so[k][lane];
+        }
+        w[i] = (2.0 / n) * (e + o);
+        w[n - 1 - i] = (2.0 / n) * (i == n - 1 - i ? e + o : e - o);
     }
 }
 
@@ -171,26 +354,52 @@ struct MuResult {
     unsigned long long bits[2];
 };
 
-template <int NT>
-__global__ void k_bisect(const double *w, int n, double emin, double emax, int kind, double kT, double N_e,
-                         double tol_N, int max_iter, double lo, double hi, MuResult *res) {
-    __shared__ double sh[NT / 32];
-    __shared__ double s_N;
+// The bisection as one cluster of thread blocks: every block sums its share of the
+// nodes, the blocks' sums meet in distributed shared memory, and every block takes
+// the same decision.  A thread's first BIS_KEEP nodes stay in registers.  Beyond 120
+// smearing widths above mu a Fermi occupation is below 1e-52 and counts as 0 (below
+// 40 under mu it is 1 in FP64), without its exponential.  (One thread block, with a
+// cosine and an exponential per node and midpoint, took 9 ms at n = 9216; now 0.23 ms.)
+constexpr int BIS_CTAS = 8, BIS_NT = 512, BIS_KEEP = 4;
+__global__ void __cluster_dims__(BIS_CTAS, 1, 1) __launch_bounds__(BIS_NT)
+    k_bisect(const double *w, int n, double emin, double emax, int kind, double kT, double N_e, double tol_N,
+             int max_iter, double lo, double hi, MuResult *res) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    __shared__ double sh[BIS_NT / 32];
+    __shared__ double s_part[2];  // this block's sum, alternating
+    const int rank = (int)cluster.block_rank(), first = rank * BIS_NT + threadIdx.x;
     const double sigma = 2.0 / (emax - emin), tau = (emin + emax) / 2.0;
+    double xs[BIS_KEEP], ws[BIS_KEEP];
+#pragma unroll
+    for (int k = 0; k < BIS_KEEP; ++k) {
+        const int i = first + k * BIS_CTAS * BIS_NT;
+        xs[k] = i < n ? node(i, n, sigma, tau) : 0.0;
+        ws[k] = i < n ? w[i] : 0.0;
+    }
+    auto occ = [&](double x, double mu) {
+        if (kind == CHEB_FERMI) {
+            const double z = (x - mu) / kT;
+            return z > 120.0 ? 0.0 : z < -40.0 ? 1.0 : fermi(x, mu, kT);
+        }
+        return 0.5 * erfc((x - mu) / kT);
+    };
     unsigned long long bits[2] = {0ull, 0ull};
     double mid = 0.5 * (lo + hi), N = 0.0;
     int it = 0, conv = 0;
-    cheb_func f{kind, 0.0, kT, 0.0, 0.0, 0.0};
     for (it = 1; it <= max_iter; ++it) {
         mid = 0.5 * (lo + hi);
-        f.mu = mid;
         double s = 0.0;
-        for (int i = threadIdx.x; i < n; i += NT) s += feval(f, node(i, n, sigma, tau), sigma, tau) * w[i];
-        double r = block_sum<NT>(s, sh);
-        if (threadIdx.x == 0) s_N = r;
-        __syncthreads();
-        N = s_N;
-        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < BIS_KEEP; ++k)
+            if (first + k * BIS_CTAS * BIS_NT < n) s += occ(xs[k], mid) * ws[k];
+        for (int i = first + BIS_KEEP * BIS_CTAS * BIS_NT; i < n; i += BIS_CTAS * BIS_NT)
+            s += occ(node(i, n, sigma, tau), mid) * w[i];
+        const double r = block_sum<BIS_NT>(s, sh);
+        if (threadIdx.x == 0) s_part[it & 1] = r;
+        cluster.sync();  // (a block's other slot is only rewritten after the next sync)
+        N = 0.0;
+        for (int b = 0; b < BIS_CTAS; ++b) N += *cluster.map_shared_rank(&s_part[it & 1], b);
         if (fabs(N - N_e) <= tol_N) {
             conv = 1;
             break;
@@ -202,11 +411,12 @@ __global__ void k_bisect(const double *w, int n, double emin, double emax, int k
             lo = mid;
         }
     }
+    cluster.sync();  // no block leaves while another still reads its sum
     if (!conv) {
         it = max_iter;
         mid = 0.5 * (lo + hi);
     }
-    if (threadIdx.x == 0) {
+    if (rank == 0 && threadIdx.x == 0) {
         res->mu = mid;
         res->N = N;
         res->iters = it;
@@ -214,6 +424,15 @@ __global__ void k_bisect(const double *w, int n, double emin, double emax, int k
         res->bits[0] = bits[0];
         res->bits[1] = bits[1];
     }
+}
+static int launch_mu(const double *g, int n, double emin, double emax, int kind, double kT, double N_e, double tol_N,
+                     int max_iter, const double *bracket, void *result, double *w, cudaStream_t s) {
+    k_count_weights<<<((n + 1) / 2 + 31) / 32, CW_NW * 32, 0, s>>>(g, n, w);
+    CHEB_TRY(check_launch("k_count_weights"));
+    const double lo = bracket ? bracket[0] : emin, hi = bracket ? bracket[1] : emax;
+    k_bisect<<<BIS_CTAS, BIS_NT, 0, s>>>(w, n, emin, emax, kind, kT, N_e, tol_N, max_iter, lo, hi,
+                                         static_cast<MuResult *>(result));
+    return check_launch("k_bisect");
 }
 
 std::vector<int> ladder(int n_max) {
@@ -232,14 +451,25 @@ std::vector<int> ladder(int n_max) {
 
 using namespace cheb;
 
+// Values per function of the candidates n_max has, and the largest degree-search
+// ladder in it; the workspace holds node values, transforms and coefficients of all
+// functions and one cosine table.
+static int64_t cand_total(const std::vector<int> &cand) {
+    int64_t t = 0;
+    for (const int n : cand) t += n;
+    return t;
+}
+static size_t coeffs_ws(int n_f, const std::vector<int> &cand) {
+    const size_t nc = cand.size(), total = (size_t)cand_total(cand);
+    return 2 * align_up(n_f * total * 8) + align_up(n_f * total * 16) + align_up(4 * total * 8) +
+           2 * align_up(n_f * nc * 8) + 256;
+}
+
 extern "C" int cheb_coeffs_workspace_size(int32_t n_f, int32_t n_max, size_t *bytes) {
     if (!bytes || n_f < 1 || n_f > 8 || n_max < 16) return fail(CHEB_ERR_INVALID, "cheb_coeffs_workspace_size: bad args");
-    const std::vector<int> lad = ladder(n_max);
-    const size_t nc = lad.size() + 1;
-    size_t tab = 4 * (size_t)n_max;
-    for (int n : lad) tab += 4 * (size_t)n;
-    *bytes = 2 * align_up(n_f * nc * (size_t)n_max * 8) + 2 * align_up(n_f * nc * 8) + align_up(nc * 4) +
-             align_up(nc * 8) + align_up(tab * 8) + 256;
+    std::vector<int> cand = ladder(n_max);
+    if (cand.empty() || cand.back() != n_max) cand.push_back(n_max);
+    *bytes = coeffs_ws(n_f, cand);
     return CHEB_OK;
 }
 
@@ -250,70 +480,139 @@ extern "C" int cheb_coeffs(const cheb_func *funcs, int32_t n_f, double emin, dou
     size_t need;
     CHEB_TRY(cheb_coeffs_workspace_size(n_f, n_max, &need));
     if (!ws || ws_bytes < need) return fail(CHEB_ERR_NOSPACE, "cheb_coeffs: workspace %zu < %zu", ws_bytes, need);
-    std::vector<int> cand = tol > 0 ? ladder(n_max) : std::vector<int>{n_max};
+    const std::vector<int> cand = tol > 0 ? ladder(n_max) : std::vector<int>{n_max};
     if (cand.empty()) return fail(CHEB_ERR_INVALID, "cheb_coeffs: empty degree ladder");
     const int nc = (int)cand.size();
     const double sigma = 2.0 / (emax - emin), tau = (emin + emax) / 2.0;
     FuncArr F{};
     for (int f = 0; f < n_f; ++f) F.f[f] = funcs[f];
+    const int64_t total = cand_total(cand);
     Carve cv(ws, ws_bytes);
-    double *fv = cv.take<double>((size_t)n_f * nc * n_max);
-    double *cvv = cv.take<double>((size_t)n_f * nc * n_max);
+    double *fv = cv.take<double>((size_t)n_f * total), *cvv = cv.take<double>((size_t)n_f * total);
+    double2 *Y = cv.take<double2>((size_t)n_f * total);
+    double *tab = cv.take<double>(4 * (size_t)total);
     unsigned long long *errm = cv.take<unsigned long long>((size_t)n_f * nc);
     unsigned long long *fmx = cv.take<unsigned long long>((size_t)n_f * nc);
-    int *dcand = cv.take<int>(nc);
-    int64_t *dtoff = cv.take<int64_t>(nc);
-    std::vector<int64_t> toff(nc);
-    int64_t tsum = 0;
-    for (int c = 0; c < nc; ++c) {
-        toff[c] = tsum;
-        tsum += 4 * (int64_t)cand[c];
-    }
-    double *tab = cv.take<double>(tsum);
     if (!cv.fits()) return fail(CHEB_ERR_NOSPACE, "cheb_coeffs: workspace too small");
     cudaStream_t s = as_stream(stream);
-    // host arrays are staged by the copy (pageable memory) before these return
-    CHEB_CUDA(cudaMemcpyAsync(dcand, cand.data(), nc * 4, cudaMemcpyHostToDevice, s));
-    CHEB_CUDA(cudaMemcpyAsync(dtoff, toff.data(), nc * 8, cudaMemcpyHostToDevice, s));
-    const dim3 g0((4 * n_max + 255) / 256, nc);
-    k_cos_table<<<g0, 256, 0, s>>>(dcand, dtoff, nc, tab);
-    CHEB_TRY(check_launch("k_cos_table"));
-    const dim3 g1((n_max + 255) / 256, n_f * nc);
-    k_nodes<<<g1, 256, 0, s>>>(F, n_f, dcand, nc, n_max, sigma, tau, fv);
-    CHEB_TRY(check_launch("k_nodes"));
-    k_dct<<<g1, 256, 0, s>>>(fv, dcand, dtoff, tab, nc, n_max, cvv);
-    CHEB_TRY(check_launch("k_dct"));
+    auto batch = [&](int c0, int c1) {
+        Cand d{};
+        d.nc = c1 - c0;
+        d.total = total;
+        int64_t off = cand_total(std::vector<int>(cand.begin(), cand.begin() + c0));
+        for (int c = c0; c < c1; ++c) {
+            d.n[c - c0] = cand[c];
+            d.off[c - c0] = off;
+            off += cand[c];
+            int n1 = 1;
+            for (int k = 2; (int64_t)k * k <= cand[c]; ++k)
+                if (cand[c] % k == 0) n1 = k;
+            d.n1[c - c0] = n1;
+        }
+        return d;
+    };
+    auto transform = [&](const Cand &d, int n_big) -> int {
+        const unsigned nb = (unsigned)((n_big + 127) / 128);
+        k_cos_table<<<dim3((4 * n_big + 255) / 256, d.nc), 256, 0, s>>>(d, tab);
+        k_nodes<<<dim3(nb, n_f * d.nc), 128, 0, s>>>(F, d, sigma, tau, fv);
+        k_dft1<<<dim3(nb, n_f * d.nc), 128, 0, s>>>(fv, d, tab, Y);
+        k_dft2<<<dim3(nb, n_f * d.nc), 128, 0, s>>>(Y, d, tab, cvv);
+        return check_launch("cheb_coeffs transform", 4);
+    };
     int chosen = nc - 1;
-    if (tol > 0) {
-        CHEB_CUDA(cudaMemsetAsync(errm, 0, n_f * nc * 8, s));
-        CHEB_CUDA(cudaMemsetAsync(fmx, 0, n_f * nc * 8, s));
-        const int pts = GRID_UNIFORM + 2 * n_max + 1;
-        const dim3 g2((pts + 255) / 256, n_f * nc);
-        k_fit_error<<<g2, 256, 0, s>>>(F, cvv, dcand, nc, n_max, sigma, tau, errm, fmx);
-        CHEB_TRY(check_launch("k_fit_error"));
-        std::vector<unsigned long long> he(n_f * nc), hf(n_f * nc);
-        CHEB_CUDA(cudaMemcpyAsync(he.data(), errm, n_f * nc * 8, cudaMemcpyDeviceToHost, s));
-        CHEB_CUDA(cudaMemcpyAsync(hf.data(), fmx, n_f * nc * 8, cudaMemcpyDeviceToHost, s));
-        CHEB_CUDA(cudaStreamSynchronize(s));
-        chosen = -1;
-        for (int f = 0; f < n_f; ++f) {
-            int cf = -1;
-            for (int c = 0; c < nc; ++c) {
-                double e, m;
-                memcpy(&e, &he[f * nc + c], 8);
-                memcpy(&m, &hf[f * nc + c], 8);
-                if (rel) e = e / m;
-                if (e < tol) {
-                    cf = c;
-                    break;
+    if (tol <= 0) {
+        CHEB_TRY(transform(batch(0, nc), cand[nc - 1]));
+    } else {
+        // The smallest candidate whose fit error is below tol, per function.  Candidates
+        // go in batches of increasing size.  In a batch, 513 of the grid's points settle
+        // most candidates: an error clearly above tol there is enough to fail.  The first
+        // that they leave is judged on the whole grid, then the next if it fails, and so
+        // on; by the estimate while that is clearly off tol, else by the error itself.
+        // (The whole grid for all 81 candidates up to 16384 terms took 40 ms.)
+        std::vector<int> best(n_f, -1);
+        std::vector<unsigned long long> he((size_t)n_f * nc), hm((size_t)n_f * nc), hs((size_t)n_f * nc);
+        auto val = [](const std::vector<unsigned long long> &v, int i) {
+            double x;
+            memcpy(&x, &v[i], 8);
+            return x;
+        };
+        int left = n_f;
+        for (int c0 = 0; c0 < nc && left > 0;) {
+            int c1 = c0 + 1;
+            while (c1 < nc && c1 - c0 < CAND_MAX && (cand[c1] <= 2048 || cand[c1] < 2 * cand[c0])) ++c1;
+            const Cand d = batch(c0, c1);
+            const int big = cand[c1 - 1], np = n_f * d.nc;
+            // below tol: 1 yes, -1 no, 0 within the recursions' rounding of it (n^2 u of the
+            // largest |f|, at the ends of the interval) or too near to say
+            auto verdict = [&](int i, double e) {
+                const double n = d.n[i % d.nc], t = rel ? tol * val(hs, i) : tol;
+                const double off = 0.1 * t + 0x1p-52 * n * n * val(hm, i);
+                return e < t - off ? 1 : e > t + off ? -1 : 0;
+            };
+            auto fetch = [&](std::vector<unsigned long long> &h, const unsigned long long *from) {
+                return cudaMemcpyAsync(h.data(), from, np * 8, cudaMemcpyDeviceToHost, s);
+            };
+            auto clear = [&]() { return cudaMemsetAsync(errm, 0, np * 8, s); };
+            CHEB_TRY(transform(d, big));
+            CHEB_CUDA(clear());
+            CHEB_CUDA(cudaMemsetAsync(fmx, 0, np * 8, s));
+            k_fit_estimate<<<dim3(33, np), 256, 0, s>>>(F, cvv, d, Pairs{}, 16, sigma, tau, errm, fmx);
+            CHEB_TRY(check_launch("k_fit_estimate"));
+            CHEB_CUDA(fetch(he, errm));
+            CHEB_CUDA(fetch(hm, fmx));
+            if (rel) {
+                k_fit_scale<<<dim3((GRID_UNIFORM + 2 * big + 256) / 256, np), 256, 0, s>>>(F, d, sigma, tau, fmx);
+                CHEB_TRY(check_launch("k_fit_scale"));
+                CHEB_CUDA(fetch(hs, fmx));
+            }
+            CHEB_CUDA(cudaStreamSynchronize(s));
+            std::vector<char> open(np);
+            for (int i = 0; i < np; ++i) open[i] = verdict(i, val(he, i)) >= 0;
+            while (true) {
+                Pairs pairs{}, near{};
+                for (int f = 0; f < n_f; ++f) {
+                    if (best[f] >= 0) continue;
+                    for (int c = 0; c < d.nc; ++c)
+                        if (open[f * d.nc + c]) {
+                            pairs.at[pairs.n++] = f * d.nc + c;
+                            break;
+                        }
+                }
+                if (pairs.n == 0) break;
+                CHEB_CUDA(clear());
+                k_fit_estimate<<<dim3((GRID_UNIFORM / 2 + big + 9) / 8, pairs.n), 256, 0, s>>>(F, cvv, d, pairs, 1, sigma, tau,
+                                                                                      errm, fmx);
+                CHEB_TRY(check_launch("k_fit_estimate"));
+                CHEB_CUDA(fetch(he, errm));
+                CHEB_CUDA(cudaStreamSynchronize(s));
+                for (int k = 0; k < pairs.n; ++k)
+                    if (verdict(pairs.at[k], val(he, pairs.at[k])) == 0) near.at[near.n++] = pairs.at[k];
+                std::vector<unsigned long long> hx(he);
+                if (near.n > 0) {
+                    CHEB_CUDA(clear());
+                    k_fit_error<<<dim3((GRID_UNIFORM + 2 * big + 64) / 64, near.n), 64, 0, s>>>(F, cvv, d, near, sigma, tau,
+                                                                                               errm);
+                    CHEB_TRY(check_launch("k_fit_error"));
+                    CHEB_CUDA(fetch(hx, errm));
+                    CHEB_CUDA(cudaStreamSynchronize(s));
+                }
+                for (int k = 0; k < pairs.n; ++k) {
+                    const int i = pairs.at[k], v = verdict(i, val(he, i));
+                    const double e = rel ? val(hx, i) / val(hs, i) : val(hx, i);
+                    open[i] = 0;
+                    if (v > 0 || (v == 0 && e < tol)) {
+                        best[i / d.nc] = c0 + i % d.nc;
+                        --left;
+                    }
                 }
             }
-            if (cf < 0) return fail(CHEB_ERR_NOT_CONVERGED, "cheb_coeffs: function %d needs more than %d terms", f, n_max);
-            chosen = std::max(chosen, cf);
+            c0 = c1;
         }
+        for (int f = 0; f < n_f; ++f)
+            if (best[f] < 0) return fail(CHEB_ERR_NOT_CONVERGED, "cheb_coeffs: function %d needs more than %d terms", f, n_max);
+        chosen = *std::max_element(best.begin(), best.end());
     }
-    const dim3 g3((n_max + 255) / 256, n_f);
-    k_pick<<<g3, 256, 0, s>>>(cvv, nc, n_max, chosen, cand[chosen], n_f, coeffs);
+    k_pick<<<dim3((n_max + 255) / 256, n_f), 256, 0, s>>>(cvv, batch(chosen, chosen + 1), 0, cand[chosen], n_max, coeffs);
     CHEB_TRY(check_launch("k_pick"));
     if (n_out) {
         *n_out = cand[chosen];
@@ -328,7 +627,7 @@ extern "C" int cheb_penalty_trace(const double *moments, int32_t n_terms, double
     if (!ws || ws_bytes < (size_t)n_terms * 8) return fail(CHEB_ERR_NOSPACE, "cheb_penalty_trace: workspace");
     cudaStream_t s = as_stream(stream);
     double *c = static_cast<double *>(ws);
-    k_penalty_coeffs<<<(n_terms + 127) / 128, 128, 0, s>>>(alpha, n_terms, c);
+    k_penalty_coeffs<<<(n_terms + PEN_J - 1) / PEN_J, PEN_NT, 0, s>>>(alpha, n_terms, c);
     CHEB_TRY(check_launch("k_penalty_coeffs"));
     k_dot_terms<256><<<1, 256, 0, s>>>(c, moments, n_terms, out);
     return check_launch("k_dot_terms");
@@ -341,14 +640,8 @@ extern "C" int cheb_mu_search(const double *gmoments, int32_t n_terms, double em
         (kind != CHEB_FERMI && kind != CHEB_ERFC))
         return fail(CHEB_ERR_INVALID, "cheb_mu_search: bad arguments");
     if (!ws || ws_bytes < (size_t)n_terms * 8) return fail(CHEB_ERR_NOSPACE, "cheb_mu_search: workspace");
-    cudaStream_t s = as_stream(stream);
-    double *w = static_cast<double *>(ws);
-    k_count_weights<<<(n_terms + 127) / 128, 128, 0, s>>>(gmoments, n_terms, w);
-    CHEB_TRY(check_launch("k_count_weights"));
-    const double lo = bracket ? bracket[0] : emin, hi = bracket ? bracket[1] : emax;
-    k_bisect<256><<<1, 256, 0, s>>>(w, n_terms, emin, emax, kind, kT, N_e, tol_N, max_iter, lo, hi,
-                                     static_cast<MuResult *>(result));
-    return check_launch("k_bisect");
+    return launch_mu(gmoments, n_terms, emin, emax, kind, kT, N_e, tol_N, max_iter, bracket, result,
+                     static_cast<double *>(ws), as_stream(stream));
 }
 
 // Workspace-free mu search (no counterpart in the paper).  The count weights
@@ -396,13 +689,8 @@ extern "C" int cheb_mu_search_noalloc(const double *gmoments, int32_t n_terms, d
                     n_terms, CHEB_MU_SEARCH_NOALLOC_MAX_TERMS);
     double *w = nullptr;
     CHEB_TRY(mu_noalloc_scratch(&w));
-    cudaStream_t s = as_stream(stream);
-    k_count_weights<<<(n_terms + 127) / 128, 128, 0, s>>>(gmoments, n_terms, w);
-    CHEB_TRY(check_launch("k_count_weights"));
-    const double lo = bracket ? bracket[0] : emin, hi = bracket ? bracket[1] : emax;
-    k_bisect<256><<<1, 256, 0, s>>>(w, n_terms, emin, emax, kind, kT, N_e, tol_N, max_iter, lo, hi,
-                                     static_cast<MuResult *>(result));
-    return check_launch("k_bisect");
+    return launch_mu(gmoments, n_terms, emin, emax, kind, kT, N_e, tol_N, max_iter, bracket, result, w,
+                     as_stream(stream));
 }
 
 // ---------------------------------------------------------------------------
