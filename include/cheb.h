@@ -598,7 +598,7 @@ int cheb_lagrange_weights(const double *nodes, int32_t n, double x, double *weig
  *   adam: one Adam step (beta1 0.9, beta2 0.999, eps 1e-8, step t >= 1).
  *   features: the 35 inputs from t_k = Tr T_k (device double[32]): t_k/n_rows,
  *     emin/10, emax/10, N_e/n_rows -> device float[35].
- * All asynchronous; reductions over the batch are sequential per thread
+ * All asynchronous; reductions over the batch run in a fixed order
  * (reproducible).
  */
 int cheb_mlp_param_count(void);

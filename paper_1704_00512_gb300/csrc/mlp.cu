@@ -2,8 +2,15 @@
 // in FP32 with hand-written forward, loss, backward and Adam kernels.
 //
 // Parameters are one flat vector: W1[128][35], b1[128], W2[128][128], b2[128],
-// W3[2][128], b3[2] (row-major, y = W x + b).  Every reduction over the batch is
-// a sequential loop in one thread (no atomics), so results are reproducible.
+// W3[2][128], b3[2] (row-major, y = W x + b).  Every reduction runs in a fixed order
+// (no atomics), so results are reproducible.
+//
+// At the training sets' few hundred samples everything is latency: what counts is how
+// many launches a step takes and how long the chain of dependent loads in each is.  So
+// a thread block takes four samples through all layers, a weight feeds all four, and
+// the sums over the batch are split over eight threads.  (A launch per layer, with one
+// serial loop per thread, took 233 us for a step at batch 346; now 58 us, of which the
+// device works 26.)
 #include "common.cuh"
 
 namespace cheb {
@@ -13,21 +20,64 @@ constexpr int OFF_W1 = 0, OFF_B1 = OFF_W1 + MLP_H * MLP_IN, OFF_W2 = OFF_B1 + ML
               OFF_B2 = OFF_W2 + MLP_H * MLP_H, OFF_W3 = OFF_B2 + MLP_H, OFF_B3 = OFF_W3 + MLP_OUT * MLP_H,
               MLP_NPARAMS = OFF_B3 + MLP_OUT;
 
-// pre[s][o] = b[o] + sum_i W[o][i] * in(s, i); in = relu(x) when relu_in.
-__global__ void k_dense(const float *__restrict__ W, const float *__restrict__ b, const float *__restrict__ x,
-                        int ldx, int B, int nin, int nout, int relu_in, float *__restrict__ pre, int ldp) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= B * nout) return;
-    const int s = idx / nout, o = idx % nout;
-    float acc = b[o];
-    const float *w = W + (size_t)o * nin;
-    const float *xs = x + (size_t)s * ldx;
-    for (int i = 0; i < nin; ++i) {
-        float v = xs[i];
-        if (relu_in) v = fmaxf(v, 0.f);
-        acc = fmaf(w[i], v, acc);
+constexpr int MLP_S = 4, MLP_NT = 512;  // samples and threads of a block
+
+// Rows o = warp, warp + 16, ... of y = W x + b for MLP_S samples (x = relu(xs) when
+// relu_in), a warp per row: the row's weights are one coalesced read, and four sums
+// over the lanes meet in six shuffles (lanes 8 s ... 8 s + 7 end with sample s).
+template <int NIN>
+__device__ __forceinline__ void dense_rows(const float *__restrict__ W, const float *__restrict__ b, int nout,
+                                           const float (*xs)[MLP_H], bool relu_in, float (*ys)[MLP_H]) {
+    constexpr int K = (NIN + 31) / 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float x[MLP_S][K];
+#pragma unroll
+    for (int s = 0; s < MLP_S; ++s)
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const int i = lane + 32 * k;
+            x[s][k] = i < NIN ? xs[s][i] : 0.f;
+            if (relu_in) x[s][k] = fmaxf(x[s][k], 0.f);
+        }
+#pragma unroll 8
+    for (int o = warp; o < nout; o += MLP_NT / 32) {
+        float v[MLP_S] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const int i = lane + 32 * k;
+            const float w = i < NIN ? W[o * NIN + i] : 0.f;
+#pragma unroll
+            for (int s = 0; s < MLP_S; ++s) v[s] = fmaf(w, x[s][k], v[s]);
+        }
+        const bool h16 = lane & 16, h8 = lane & 8;
+        const float p0 = (h16 ? v[2] : v[0]) + __shfl_xor_sync(0xffffffffu, h16 ? v[0] : v[2], 16);
+        const float p1 = (h16 ? v[3] : v[1]) + __shfl_xor_sync(0xffffffffu, h16 ? v[1] : v[3], 16);
+        float r = (h8 ? p1 : p0) + __shfl_xor_sync(0xffffffffu, h8 ? p0 : p1, 8);
+        r += __shfl_xor_sync(0xffffffffu, r, 4);
+        r += __shfl_xor_sync(0xffffffffu, r, 2);
+        r += __shfl_xor_sync(0xffffffffu, r, 1);
+        if ((lane & 7) == 0) ys[lane >> 3][o] = r + b[o];
     }
-    pre[(size_t)s * ldp + o] = acc;
+}
+
+// All three layers; act keeps the pre-activations of the hidden ones, a1 then a2.
+__global__ void __launch_bounds__(MLP_NT) k_mlp_forward(const float *__restrict__ theta, const float *__restrict__ X,
+                                                        int B, float *__restrict__ act, float *__restrict__ out) {
+    __shared__ float x[MLP_S][MLP_H], h1[MLP_S][MLP_H], h2[MLP_S][MLP_H], y[MLP_S][MLP_H];
+    const int64_t s0 = (int64_t)blockIdx.x * MLP_S;
+    const int s = threadIdx.x / MLP_H, i = threadIdx.x % MLP_H;
+    const bool in = s0 + s < B;
+    x[s][i] = in && i < MLP_IN ? X[(s0 + s) * MLP_IN + i] : 0.f;
+    __syncthreads();
+    dense_rows<MLP_IN>(theta + OFF_W1, theta + OFF_B1, MLP_H, x, false, h1);
+    __syncthreads();
+    if (in) act[(s0 + s) * MLP_H + i] = h1[s][i];
+    dense_rows<MLP_H>(theta + OFF_W2, theta + OFF_B2, MLP_H, h1, true, h2);
+    __syncthreads();
+    if (in) act[(B + s0 + s) * MLP_H + i] = h2[s][i];
+    dense_rows<MLP_H>(theta + OFF_W3, theta + OFF_B3, MLP_OUT, h2, true, y);
+    __syncthreads();
+    if (in && i < MLP_OUT) out[(s0 + s) * MLP_OUT + i] = y[s][i];
 }
 
 // Loss of the module docstring of the oracle: d = (xhat - xstar)/scale,
@@ -53,36 +103,93 @@ __global__ void k_mlp_loss(const float *out, const float *xstar, const float *sc
     if (threadIdx.x == 0 && loss) *loss = r / B;
 }
 
-// dprev[s][i] = (sum_o dy[s][o] W[o][i]) * [pre[s][i] > 0]
-__global__ void k_back_act(const float *__restrict__ W, const float *__restrict__ dy, int lddy, int nout,
-                           const float *__restrict__ pre, int ldp, int B, int nin, float *__restrict__ dprev,
-                           int ldd) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= B * nin) return;
-    const int s = idx / nin, i = idx % nin;
+// d2 = (dout W3) [a2 > 0] and d1 = (d2 W2) [a1 > 0], MLP_S samples per block; the sum
+// over the 128 rows of W2 is split over four threads.
+__global__ void __launch_bounds__(MLP_NT) k_mlp_back(const float *__restrict__ theta, const float *__restrict__ dout,
+                                                     const float *__restrict__ a1, const float *__restrict__ a2, int B,
+                                                     float *__restrict__ d1, float *__restrict__ d2) {
+    __shared__ float4 sd[MLP_H];  // d2 of the four samples
+    __shared__ float part[MLP_S][MLP_S][MLP_H];
+    static_assert(MLP_S == 4 && MLP_NT == MLP_S * MLP_H, "a thread per sample and unit; as many parts as samples");
+    const int64_t s0 = (int64_t)blockIdx.x * MLP_S;
+    const int q = threadIdx.x / MLP_H, i = threadIdx.x % MLP_H;  // q: the sample, or the part of the sum
+    const bool in = s0 + q < B;
+    const size_t at = (s0 + q) * MLP_H + i;
+    const float *W2 = theta + OFF_W2 + i, *W3 = theta + OFF_W3 + i;
+    float w[MLP_H / MLP_S];
+#pragma unroll
+    for (int o = 0; o < MLP_H / MLP_S; ++o) w[o] = W2[(q * (MLP_H / MLP_S) + o) * MLP_H];
     float acc = 0.f;
-    for (int o = 0; o < nout; ++o) acc = fmaf(dy[(size_t)s * lddy + o], W[(size_t)o * nin + i], acc);
-    dprev[(size_t)s * ldd + i] = pre[(size_t)s * ldp + i] > 0.f ? acc : 0.f;
+    if (in) {
+        acc = fmaf(dout[(s0 + q) * MLP_OUT], W3[0], acc);
+        acc = fmaf(dout[(s0 + q) * MLP_OUT + 1], W3[MLP_H], acc);
+        acc = a2[at] > 0.f ? acc : 0.f;
+        d2[at] = acc;
+    }
+    reinterpret_cast<float *>(&sd[i])[q] = acc;
+    __syncthreads();
+    float v[MLP_S] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int o = 0; o < MLP_H / MLP_S; ++o) {
+        const float4 d = sd[q * (MLP_H / MLP_S) + o];
+        v[0] = fmaf(d.x, w[o], v[0]);
+        v[1] = fmaf(d.y, w[o], v[1]);
+        v[2] = fmaf(d.z, w[o], v[2]);
+        v[3] = fmaf(d.w, w[o], v[3]);
+    }
+#pragma unroll
+    for (int s = 0; s < MLP_S; ++s) part[s][q][i] = v[s];
+    __syncthreads();
+    if (in) {
+        const float r = (part[q][0][i] + part[q][1][i]) + (part[q][2][i] + part[q][3][i]);
+        d1[at] = a1[at] > 0.f ? r : 0.f;
+    }
 }
 
-// gW[o][i] = sum_s dy[s][o] in(s, i), gb[o] = sum_s dy[s][o]; one thread per parameter.
-__global__ void k_wgrad(const float *__restrict__ dy, int lddy, const float *__restrict__ x, int ldx, int relu_in,
-                        int B, int nin, int nout, float *__restrict__ gW, float *__restrict__ gb) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx < nout * nin) {
-        const int o = idx / nin, i = idx % nin;
-        float acc = 0.f;
-        for (int s = 0; s < B; ++s) {
-            float v = x[(size_t)s * ldx + i];
-            if (relu_in) v = fmaxf(v, 0.f);
-            acc = fmaf(dy[(size_t)s * lddy + o], v, acc);
+// Every parameter's gradient: gW[o][i] = sum_s dy[s][o] in(s, i), gb[o] = sum_s dy[s][o].
+// A block takes 128 neighbouring parameters; the batch is split over WG_Q threads each.
+constexpr int WG_P = 128, WG_Q = 8;
+__global__ void __launch_bounds__(WG_P *WG_Q) k_mlp_wgrad(const float *__restrict__ X, const float *__restrict__ a1,
+                                                         const float *__restrict__ a2, const float *__restrict__ d1,
+                                                         const float *__restrict__ d2, const float *__restrict__ dout,
+                                                         int B, float *__restrict__ grad) {
+    __shared__ float part[WG_Q][WG_P];
+    const int lp = threadIdx.x % WG_P, q = threadIdx.x / WG_P, p = blockIdx.x * WG_P + lp;
+    float acc = 0.f;
+    if (p < MLP_NPARAMS) {
+        const float *dy, *x;
+        int ldy, ldx, nin, r;  // r: the parameter within its layer's weights and biases
+        bool relu = true;
+        if (p < OFF_W2) {
+            dy = d1, ldy = MLP_H, x = X, ldx = nin = MLP_IN, r = p, relu = false;
+        } else if (p < OFF_W3) {
+            dy = d2, ldy = MLP_H, x = a1, ldx = nin = MLP_H, r = p - OFF_W2;
+        } else {
+            dy = dout, ldy = MLP_OUT, x = a2, ldx = nin = MLP_H, r = p - OFF_W3;
         }
-        gW[idx] = acc;
-    } else if (idx < nout * nin + nout) {
-        const int o = idx - nout * nin;
-        float acc = 0.f;
-        for (int s = 0; s < B; ++s) acc += dy[(size_t)s * lddy + o];
-        gb[o] = acc;
+        const int nout = ldy;
+        if (r < nout * nin) {
+            dy += r / nin;
+            x += r % nin;
+#pragma unroll 8
+            for (int s = q; s < B; s += WG_Q) {
+                float v = x[(size_t)s * ldx];
+                if (relu) v = fmaxf(v, 0.f);
+                acc = fmaf(dy[(size_t)s * ldy], v, acc);
+            }
+        } else {
+            dy += r - nout * nin;
+#pragma unroll 8
+            for (int s = q; s < B; s += WG_Q) acc += dy[(size_t)s * ldy];
+        }
+    }
+    part[q][lp] = acc;
+    __syncthreads();
+    if (q == 0 && p < MLP_NPARAMS) {
+        float r = part[0][lp];
+#pragma unroll
+        for (int k = 1; k < WG_Q; ++k) r += part[k][lp];
+        grad[p] = r;
     }
 }
 
@@ -155,14 +262,8 @@ extern "C" int cheb_mlp_forward(const float *theta, const float *X, int32_t batc
                                 void *stream) {
     if (!theta || !X || !act || !out || batch < 1) return fail(CHEB_ERR_INVALID, "cheb_mlp_forward: bad arguments");
     cudaStream_t s = as_stream(stream);
-    float *a1 = act, *a2 = act + (size_t)batch * MLP_H;
-    k_dense<<<nb((int64_t)batch * MLP_H), 128, 0, s>>>(theta + OFF_W1, theta + OFF_B1, X, MLP_IN, batch, MLP_IN,
-                                                        MLP_H, 0, a1, MLP_H);
-    k_dense<<<nb((int64_t)batch * MLP_H), 128, 0, s>>>(theta + OFF_W2, theta + OFF_B2, a1, MLP_H, batch, MLP_H,
-                                                        MLP_H, 1, a2, MLP_H);
-    k_dense<<<nb((int64_t)batch * MLP_OUT), 128, 0, s>>>(theta + OFF_W3, theta + OFF_B3, a2, MLP_H, batch, MLP_H,
-                                                          MLP_OUT, 1, out, MLP_OUT);
-    return check_launch("cheb_mlp_forward", 3);
+    k_mlp_forward<<<nb(batch, MLP_S), MLP_NT, 0, s>>>(theta, X, batch, act, out);
+    return check_launch("k_mlp_forward");
 }
 
 extern "C" int cheb_mlp_loss(const float *out, const float *xstar, const float *scale, int32_t batch, float *dout,
@@ -179,17 +280,9 @@ extern "C" int cheb_mlp_backward(const float *theta, const float *X, int32_t bat
     cudaStream_t s = as_stream(stream);
     const float *a1 = act, *a2 = act + (size_t)batch * MLP_H;
     float *d2 = ws, *d1 = ws + (size_t)batch * MLP_H;
-    k_wgrad<<<nb(MLP_OUT * MLP_H + MLP_OUT), 128, 0, s>>>(dout, MLP_OUT, a2, MLP_H, 1, batch, MLP_H, MLP_OUT,
-                                                          grad + OFF_W3, grad + OFF_B3);
-    k_back_act<<<nb((int64_t)batch * MLP_H), 128, 0, s>>>(theta + OFF_W3, dout, MLP_OUT, MLP_OUT, a2, MLP_H, batch,
-                                                           MLP_H, d2, MLP_H);
-    k_wgrad<<<nb(MLP_H * MLP_H + MLP_H), 128, 0, s>>>(d2, MLP_H, a1, MLP_H, 1, batch, MLP_H, MLP_H, grad + OFF_W2,
-                                                      grad + OFF_B2);
-    k_back_act<<<nb((int64_t)batch * MLP_H), 128, 0, s>>>(theta + OFF_W2, d2, MLP_H, MLP_H, a1, MLP_H, batch, MLP_H,
-                                                           d1, MLP_H);
-    k_wgrad<<<nb(MLP_H * MLP_IN + MLP_H), 128, 0, s>>>(d1, MLP_H, X, MLP_IN, 0, batch, MLP_IN, MLP_H, grad + OFF_W1,
-                                                       grad + OFF_B1);
-    return check_launch("cheb_mlp_backward", 5);
+    k_mlp_back<<<nb(batch, MLP_S), MLP_NT, 0, s>>>(theta, dout, a1, a2, batch, d1, d2);
+    k_mlp_wgrad<<<nb(MLP_NPARAMS, WG_P), WG_P * WG_Q, 0, s>>>(X, a1, a2, d1, d2, dout, batch, grad);
+    return check_launch("cheb_mlp_backward", 2);
 }
 
 extern "C" int cheb_mlp_adam(float *theta, const float *grad, float *m, float *v, int32_t t, float lr, void *stream) {
