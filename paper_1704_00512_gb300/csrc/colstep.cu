@@ -88,7 +88,8 @@ struct Dig<double> {
 };
 
 struct ColArgs {
-    const int32_t *panels;  // (first column, column count, union rows, system) per thread block
+    const int32_t *panels;  // (first column, column count, union rows, system) per panel
+    const int32_t *order;   // panel of each thread block
     const int32_t *wchunk;  // [panels][NW + 1] quad range of each warp
     const int32_t *wrow;    // [panels][NW + 1] group range of each warp
     const uint32_t *rows;   // per group: the 4 union slots and the quad count (2 words)
@@ -387,7 +388,7 @@ __global__ void __launch_bounds__(COL_NW * 32, 1) k_colstep(const __grid_constan
     __shared__ float s_ch[3][MAX_F], s_cl[3][MAX_F];
     __shared__ double s_c[3][MAX_F];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int pid = blockIdx.x;
+    const int pid = a.order[blockIdx.x];
     const int j0 = a.panels[4 * pid], nc = a.panels[4 * pid + 1], nu = a.panels[4 * pid + 2], sys = a.panels[4 * pid + 3];
     const int n = a.n_terms ? a.n_terms[sys] : a.n_single;
     if (a.t0 >= n && a.t0 != 2) return;  // this system is done
@@ -951,6 +952,7 @@ static int col_expand_t(const cheb_plan *plan, const cheb_bsr *Mt, const ColExpa
                                                                   Mt->nnzb, x.round_bf16, opd, opexp, opflag);
     CHEB_TRY(check_launch("k_opdig"));
     a.panels = c.d_panels;
+    a.order = c.d_order;
     a.wchunk = c.d_wchunk;
     a.wrow = c.d_wrow;
     a.rows = c.d_rows;
@@ -1242,9 +1244,31 @@ int col_build(cheb_plan *plan, const std::vector<int64_t> &rp, const std::vector
     c.n_rows = (int64_t)c.h_rows.size();
     c.n_slot = (int64_t)c.h_slot.size();
     c.n_sys = (int64_t)c.h_sys_panel.size();
+    c.h_order = col_order(cnt.chunks);
     c.built = true;
     plan->col = std::move(c);
     return CHEB_OK;
+}
+
+// Thread blocks start in the order of their index, one per SM at a time, so the panels
+// that start last should be the short ones: the LAST panels with the fewest quads (two
+// per SM) go last, longest first, the others in their own order, in which neighbours
+// share operator rows in L2.  250 panels FP32: 10.1 -> 8.4 ms; 500 and 771 panels FP64:
+// 24.5 -> 22.2 and 91.0 -> 88.5 ms.  Beyond eight panels per SM all stay in their own
+// order: the last wave is a small part, and the short panels, far apart, miss L2 more
+// (2,502 panels FP32: 128.8 -> 131.7 ms).
+std::vector<int32_t> col_order(const std::vector<int64_t> &quads) {
+    constexpr size_t SMS = 152, LAST = 2 * SMS;
+    const size_t np = quads.size();
+    std::vector<int32_t> by(np), order;
+    std::iota(by.begin(), by.end(), 0);
+    if (np > 8 * SMS) return by;
+    std::stable_sort(by.begin(), by.end(), [&](int32_t x, int32_t y) { return quads[x] > quads[y]; });
+    const size_t first = np - std::min(np, LAST);
+    order.assign(by.begin(), by.begin() + first);
+    std::sort(order.begin(), order.end());
+    order.insert(order.end(), by.begin() + first, by.end());
+    return order;
 }
 
 int col_bind(ColLists &c, Carve &cv, cudaStream_t s) {
@@ -1263,6 +1287,7 @@ int col_bind(ColLists &c, Carve &cv, cudaStream_t s) {
         c.d_ent = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(c.d_ent) + d);
         c.d_slot = reinterpret_cast<uint16_t *>(reinterpret_cast<char *>(c.d_slot) + d);
         c.d_sys_panel = reinterpret_cast<int32_t *>(reinterpret_cast<char *>(c.d_sys_panel) + d);
+        c.d_order = reinterpret_cast<int32_t *>(reinterpret_cast<char *>(c.d_order) + d);
         return CHEB_OK;
     }
     c.d_panels = cv.take<int32_t>(c.h_panels.size());
@@ -1272,6 +1297,7 @@ int col_bind(ColLists &c, Carve &cv, cudaStream_t s) {
     c.d_ent = cv.take<uint32_t>(std::max<size_t>(c.h_ent.size(), 1));
     c.d_slot = cv.take<uint16_t>(c.h_slot.size());
     c.d_sys_panel = cv.take<int32_t>(c.h_sys_panel.size());
+    c.d_order = cv.take<int32_t>(c.h_order.size());
     if (!cv.fits()) return fail(CHEB_ERR_NOSPACE, "cheb_plan_bind_operator: workspace too small");
     CHEB_CUDA(cudaMemcpyAsync(c.d_panels, c.h_panels.data(), c.h_panels.size() * 4, cudaMemcpyHostToDevice, s));
     CHEB_CUDA(cudaMemcpyAsync(c.d_wchunk, c.h_wchunk.data(), c.h_wchunk.size() * 4, cudaMemcpyHostToDevice, s));
@@ -1282,6 +1308,7 @@ int col_bind(ColLists &c, Carve &cv, cudaStream_t s) {
         CHEB_CUDA(cudaMemcpyAsync(c.d_ent, c.h_ent.data(), c.h_ent.size() * 4, cudaMemcpyHostToDevice, s));
     CHEB_CUDA(cudaMemcpyAsync(c.d_slot, c.h_slot.data(), c.h_slot.size() * 2, cudaMemcpyHostToDevice, s));
     CHEB_CUDA(cudaMemcpyAsync(c.d_sys_panel, c.h_sys_panel.data(), c.h_sys_panel.size() * 4, cudaMemcpyHostToDevice, s));
+    CHEB_CUDA(cudaMemcpyAsync(c.d_order, c.h_order.data(), c.h_order.size() * 4, cudaMemcpyHostToDevice, s));
     return CHEB_OK;
 }
 

@@ -656,9 +656,11 @@ int col_build_device(cheb_plan *plan, const cheb_bsr *L, cudaStream_t s) {
     CHEB_TRY(check_launch("k_gp_scan", 2));
     std::vector<int32_t> h_max(np);
     std::vector<int32_t> h_pan(4 * np);
+    std::vector<int64_t> h_quads(np);
     int64_t tot[2];
     int32_t h_err = 0;
     CHEB_CUDA(cudaMemcpyAsync(h_max.data(), cnt_max, np * 4, cudaMemcpyDeviceToHost, s));
+    CHEB_CUDA(cudaMemcpyAsync(h_quads.data(), cnt_chunks, np * 8, cudaMemcpyDeviceToHost, s));
     CHEB_CUDA(cudaMemcpyAsync(h_pan.data(), pan, 4 * np * 4, cudaMemcpyDeviceToHost, s));
     CHEB_CUDA(cudaMemcpyAsync(&tot[0], choff + np, 8, cudaMemcpyDeviceToHost, s));
     CHEB_CUDA(cudaMemcpyAsync(&tot[1], rooff + np, 8, cudaMemcpyDeviceToHost, s));
@@ -673,6 +675,7 @@ int col_build_device(cheb_plan *plan, const cheb_bsr *L, cudaStream_t s) {
     c.h_sys_panel.assign(plan->nsys + 1, (int32_t)np);
     for (int64_t p = np - 1; p >= 0; --p) c.h_sys_panel[h_pan[4 * p + 3]] = (int32_t)p;
     c.n_sys = (int64_t)c.h_sys_panel.size();
+    c.h_order = col_order(h_quads);
     // the lists, in device memory of their own until cheb_plan_bind_operator
     // copies them into the operator workspace
     c.built = true;  // (sizes complete: bytes() counts them from here on)
@@ -693,7 +696,9 @@ int col_build_device(cheb_plan *plan, const cheb_bsr *L, cudaStream_t s) {
     c.d_ent = cv.take<uint32_t>(std::max<int64_t>(c.n_entries, 1));
     c.d_slot = cv.take<uint16_t>(c.n_slot);
     c.d_sys_panel = cv.take<int32_t>(c.n_sys);
+    c.d_order = cv.take<int32_t>(np);
     CHEB_CUDA(cudaMemcpyAsync(c.d_sys_panel, c.h_sys_panel.data(), c.n_sys * 4, cudaMemcpyHostToDevice, s));
+    CHEB_CUDA(cudaMemcpyAsync(c.d_order, c.h_order.data(), np * 4, cudaMemcpyHostToDevice, s));
     CHEB_CUDA(cudaMemcpyAsync(c.d_panels, pan, 4 * np * 4, cudaMemcpyDeviceToDevice, s));
     CHEB_CUDA(cudaMemsetAsync(c.d_ent + tot[0] * COL_CW, 0, COL_TAIL * COL_CW * 4, s));
     a.chunk_off = choff;

@@ -49,6 +49,7 @@ struct ColLists {
     std::vector<uint32_t> h_ent;
     std::vector<uint16_t> h_slot;
     std::vector<int32_t> h_sys_panel;  // first panel of each system (+ end)
+    std::vector<int32_t> h_order;      // panels in the order of their launch (col_order)
     int64_t nnzL = 0;                  // operator blocks
     int32_t *d_panels = nullptr;
     int32_t *d_wchunk = nullptr;
@@ -57,6 +58,7 @@ struct ColLists {
     uint32_t *d_ent = nullptr;
     uint16_t *d_slot = nullptr;
     int32_t *d_sys_panel = nullptr;
+    int32_t *d_order = nullptr;
     int64_t n_rows = 0, n_slot = 0, n_sys = 0;  // group words; P_out blocks (one slot each); systems + 1
     bool built = false, bound = false;
     // built by the gather-plan kernels (gather.cu): the d_ arrays live in tmp
@@ -68,7 +70,7 @@ struct ColLists {
         return ::cheb::align_up((size_t)n_panels * 16) + 2 * ::cheb::align_up((size_t)n_panels * (NW + 1) * 4) +
                ::cheb::align_up((size_t)std::max<int64_t>(n_rows, 1) * 4) +
                ::cheb::align_up((size_t)std::max<int64_t>(n_entries, 1) * 4) + ::cheb::align_up((size_t)n_slot * 2) +
-               ::cheb::align_up((size_t)n_sys * 4);
+               ::cheb::align_up((size_t)n_sys * 4) + ::cheb::align_up((size_t)n_panels * 4);
     }
 };
 
@@ -305,6 +307,8 @@ int gp_walk(const int64_t *rp, const int32_t *ci, int64_t nbr, int P, int64_t uc
 int gp_check_operator(const cheb_bsr *L, int64_t nbr, int64_t first[2], cudaStream_t s);
 int row_lists_device(const int64_t *rp, const int32_t *ci, int64_t nbr, const cheb_bsr *L, const int32_t *pairs,
                      int64_t np, int maxu, RowLists &out, cudaStream_t s);
+// The panels (quads of each) in the order of their launch.
+std::vector<int32_t> col_order(const std::vector<int64_t> &quads);
 int col_bind(ColLists &c, Carve &cv, cudaStream_t s);
 void col_release_host(ColLists &c);
 bool col_usable(const cheb_plan *plan, const cheb_bsr *Mt);

@@ -48,6 +48,7 @@ def run(plan, dM, n, c, G, nnzb, prec, stepwise=True):
     (150, 6, 2, True),     # a group and a rest
     (231, 99, 1, False),   # one term beyond the first launch's steps
     (230, 101, 3, True),   # ... and the next group's rest
+    (640, 5, 1, True),     # more panels (FP64) than the launch order sorts
 ])
 def test_digit_products_against_the_oracle(prec, n_atoms, n, nf, stepwise):
     Ht, P_out = system(n_atoms, 8.0, 3.0, 600 + n_atoms)
