@@ -33,8 +33,8 @@
 // Fermi 3.5e-8 -> 2.9e-8, powers 4.7e-7 -> 2.5e-7; FP64-accurate 4.2e-14 -> 5.3e-16.
 // Measured (GB300): one step at 1,500 atoms, r_c 10, r_out 14 bohr, three
 // accumulators: FP64 9.2 -> 1.3 ms, FP64-accurate (before: double-floats) at 1,000
-// atoms, 8 / 12 bohr: 2.3 -> 0.39 ms; FP32 at 10,000 atoms 3.47 -> 2.75 ms, at 1,000
-// atoms, 8 / 12 bohr: 0.237 -> 0.161 ms.  ncu: L1 access cycles 71 % (FP64) and
+// atoms, 8 / 12 bohr: 2.3 -> 0.35 ms; FP32 at 10,000 atoms 3.47 -> 2.7 ms, at 1,000
+// atoms, 8 / 12 bohr: 0.237 -> 0.131 ms, at 3,000 atoms with four functions 1.12 -> 0.88.  ncu: L1 access cycles 71 % (FP64) and
 // 47 % (FP32), ALU (digit unpacking) 50 %, tensor pipe 43 % and 36 %, issue 45-55 %:
 // an operator block of 64 or 128 bytes is used for one row group and panel only, and
 // an L1 load costs a cycle per line that the lanes it serves together touch.
@@ -655,24 +655,39 @@ __global__ void __launch_bounds__(COL_NW * 32, 1) k_colstep(const __grid_constan
                                 load_h(h[o], wc[o]);
                                 const uint32_t *x2 = X2 + sl * 4 * XV;
                                 const int g2 = g ^ (8 * ((sl >> 1) & 1));
+uint32_t B[NT][3][2];
 #pragma unroll
                                 for (int j = 0; j < NT; ++j) {
                                     const uint4 xw = xs[8 * j];
                                     const uint32_t xb = x2[g2 ^ (8 * j)];
-                                    const uint32_t B0[2] = {xw.x, xw.y}, B1[2] = {xw.z, xw.w};
-                                    const uint32_t B2[2] = {third_digits<0x4140>(xb), third_digits<0x4342>(xb)};
-                                    // (the leading sums of two quads, below 2^24, are exact)
-                                    if (o == 0) mma16816(z[j][0], A0, B0, zero);
-                                    else mma16816(z[j][0], A0, B0, z[j][0]);
-                                    mma16816(dl[j][0], A0, B1, dl[j][0]);
-                                    mma16816(dl[j][1], A0, B2, dl[j][1]);
-                                    mma16816(dl[j][0], A1, B0, dl[j][0]);
-                                    mma16816(dl[j][1], A1, B1, dl[j][1]);
-                                    mma16816(dl[j][1], A2, B0, dl[j][1]);
-                                    if (o == 1) {
+                                    B[j][0][0] = xw.x;
+                                    B[j][0][1] = xw.y;
+                                    B[j][1][0] = xw.z;
+                                    B[j][1][1] = xw.w;
+                                    B[j][2][0] = third_digits<0x4140>(xb);
+                                    B[j][2][1] = third_digits<0x4342>(xb);
+                                }
+                                // (the leading sums of two quads, below 2^24, are exact)
+#pragma unroll
+                                for (int j = 0; j < NT; ++j) {
+                                    if (o == 0) mma16816(z[j][0], A0, B[j][0], zero);
+                                    else mma16816(z[j][0], A0, B[j][0], z[j][0]);
+                                }
+#pragma unroll
+                                for (int j = 0; j < NT; ++j) mma16816(dl[j][0], A0, B[j][1], dl[j][0]);
+#pragma unroll
+                                for (int j = 0; j < NT; ++j) mma16816(dl[j][1], A0, B[j][2], dl[j][1]);
+#pragma unroll
+                                for (int j = 0; j < NT; ++j) mma16816(dl[j][0], A1, B[j][0], dl[j][0]);
+#pragma unroll
+                                for (int j = 0; j < NT; ++j) mma16816(dl[j][1], A1, B[j][1], dl[j][1]);
+#pragma unroll
+                                for (int j = 0; j < NT; ++j) mma16816(dl[j][1], A2, B[j][0], dl[j][1]);
+                                if (o == 1) {
+#pragma unroll
+                                    for (int j = 0; j < NT; ++j)
 #pragma unroll
                                         for (int i = 0; i < 4; ++i) fs[j][i] += z[j][0][i];
-                                    }
                                 }
                             } else {
                                 const uint4 x0 = xs[0], x1 = xs[8], x2 = xs[16];
@@ -687,6 +702,10 @@ __global__ void __launch_bounds__(COL_NW * 32, 1) k_colstep(const __grid_constan
                                         const uint32_t pw[4] = {hw[0], hw[1], hw[F64 ? 2 : 0], hw[F64 ? 3 : 0]};
                                         A[k2] = packed_digit(pw, i);
                                     }
+                                    if (i >= 1) {  // D_6 into D_5's accumulator: the panel digit times 2^-10
+                                        const uint32_t Bs[2] = {h2_fma(B[6 - i][0], 0x14001400u, 0u), h2_fma(B[6 - i][1], 0x14001400u, 0u)};
+                                        mma16816(dl[0][1], A, Bs, dl[0][1]);
+                                    }
 #pragma unroll
                                     for (int s = i; s < 6; ++s) {
                                         if (s >= 4) mma16816(dl[0][s & 1], A, B[s - i], dl[0][s & 1]);
@@ -694,10 +713,6 @@ __global__ void __launch_bounds__(COL_NW * 32, 1) k_colstep(const __grid_constan
                                         else mma16816(z[0][F64 ? s : 0], A, B[s - i], z[0][F64 ? s : 0]);
                                     }
                                     // (the sums of s = 0, 1 stay exact over two quads)
-                                    if (i >= 1) {  // D_6 into D_5's accumulator: the panel digit times 2^-10
-                                        const uint32_t Bs[2] = {h2_fma(B[6 - i][0], 0x14001400u, 0u), h2_fma(B[6 - i][1], 0x14001400u, 0u)};
-                                        mma16816(dl[0][1], A, Bs, dl[0][1]);
-                                    }
                                     if (i < 4 && (o == 1 || i >= 2)) {
 #pragma unroll
                                         for (int e = 0; e < 4; ++e) is[i][e] += __float2int_rn(z[0][F64 ? i : 0][e]);
@@ -745,15 +760,15 @@ __global__ void __launch_bounds__(COL_NW * 32, 1) k_colstep(const __grid_constan
                 const int sl2[2] = {(int)((g >> 2) == 0 ? rw.x & SM : (rw.x >> COL_SLOT_BITS) & SM),
                                     (int)((g >> 2) == 0 ? (rw.x >> (2 * COL_SLOT_BITS)) & SM : rw.y & SM)};
                 const int eo = 4 * (g & 3) + 2 * (t & 1);
+                using GV = typename std::conditional<F64, double2, float4>::type;
 #pragma unroll
                 for (int hh = 0; hh < 2; ++hh) {
                     if (sl2[hh] == (int)SM) continue;
                     const int er = rexp[sl2[hh]];
                     const float rf = F64 || slow ? 1.f : pow2(er - 18, 0.f);  // (two exact factors)
                     // T_{term-2}, G and, in group steps, T_{term-1}, of the half's positions
-                    using GV = typename std::conditional<F64, double2, float4>::type;
                     int pos[NT];
-                    V2 tm[NT], tk[NT];
+                    V2 tm[NT], tk[NT], y[NT];
                     GV gv[NT];
 #pragma unroll
                     for (int j = 0; j < NT; ++j) {
@@ -764,14 +779,14 @@ __global__ void __launch_bounds__(COL_NW * 32, 1) k_colstep(const __grid_constan
                         const int64_t off = (int64_t)pos[j] * BB + eo;
                         tm[j] = __ldcg(reinterpret_cast<const V2 *>(C + off));
                         if (a.G) {
-                            if constexpr (F64) gv[j] = __ldg(reinterpret_cast<const double2 *>(a.G + (int64_t)a.tperm[pos[j]] * BB + eo));
-                            else gv[j] = __ldcg(reinterpret_cast<const float4 *>(a.Gp + off * 2));
+                            if constexpr (F64) gv[j] = __ldg(reinterpret_cast<const GV *>(a.G + (int64_t)a.tperm[pos[j]] * BB + eo));
+                            else gv[j] = __ldcg(reinterpret_cast<const GV *>(a.Gp + off * 2));
                         }
                         if (grp) tk[j] = __ldcg(reinterpret_cast<const V2 *>(R + off));
                     }
 #pragma unroll
                     for (int j = 0; j < NT; ++j) {
-                        T y[2];
+                        T w[2];
 #pragma unroll
                         for (int cc = 0; cc < 2; ++cc) {
                             const int i = 2 * hh + cc;
@@ -783,52 +798,60 @@ __global__ void __launch_bounds__(COL_NW * 32, 1) k_colstep(const __grid_constan
                                 v = fs[j][i] * rf;
                                 sc = s_cf[8 * j + 2 * t + cc];
                             }
-                            y[cc] = mac(v, sc, cc ? -tm[j].y : -tm[j].x);
+                            w[cc] = mac(v, sc, cc ? -tm[j].y : -tm[j].x);
                             if constexpr (!F64) {
-                                if (a.round_bf16) y[cc] = bf16r(y[cc]);
+                                if (a.round_bf16) w[cc] = bf16r(w[cc]);
                             }
                         }
-                        const int p = pos[j];
-                        if (p >= 0) {
-                            const int64_t off = (int64_t)p * BB + eo;
-                            V2 u;
-                            u.x = y[0];
-                            u.y = y[1];
-                            *reinterpret_cast<V2 *>(C + off) = u;
-                            mx[j][0] = max(mx[j][0], mag_bits(y[0]));
-                            mx[j][1] = max(mx[j][1], mag_bits(y[1]));
-                            if constexpr (F64) {
-                                gd += gv[j].x * y[0] + gv[j].y * y[1];
-                            } else {
-                                ff_add_prod(gh, gl, y[0], gv[j].x, gv[j].y);
-                                ff_add_prod(gh, gl, y[1], gv[j].z, gv[j].w);
-                            }
+                        y[j].x = w[0];
+                        y[j].y = w[1];
+                        if (pos[j] < 0) continue;
+                        *reinterpret_cast<V2 *>(C + (int64_t)pos[j] * BB + eo) = y[j];
+                        mx[j][0] = max(mx[j][0], mag_bits(w[0]));
+                        mx[j][1] = max(mx[j][1], mag_bits(w[1]));
+                        if constexpr (F64) {
+                            gd += gv[j].x * w[0] + gv[j].y * w[1];
                             if (grp) {
                                 // the group's terms in order: T_{term-2}, T_{term-1}, T_term
-                                const T tv[3][2] = {{tm[j].x, tm[j].y}, {tk[j].x, tk[j].y}, {y[0], y[1]}};
-                                const int64_t oc = F64 ? (int64_t)a.tperm[p] * BB + eo : 0;
+                                const T tv[3][2] = {{tm[j].x, tm[j].y}, {tk[j].x, tk[j].y}, {w[0], w[1]}};
+                                const int64_t at = (int64_t)a.tperm[pos[j]] * BB + eo;
                                 for (int f = 0; f < a.nf; ++f) {
-                                    if constexpr (F64) {
-                                        double2 v = *reinterpret_cast<double2 *>(a.acc[f] + oc);
+                                    double2 v = *reinterpret_cast<double2 *>(a.acc[f] + at);
 #pragma unroll
-                                        for (int i = 0; i < 3; ++i)
-                                            if ((grp >> (2 - i)) & 1) {
-                                                v.x += s_c[i][f] * tv[i][0];
-                                                v.y += s_c[i][f] * tv[i][1];
-                                            }
-                                        *reinterpret_cast<double2 *>(a.acc[f] + oc) = v;
-                                    } else {
-                                        float *pa = a.accp[f] + off * 2;
-                                        float4 v = __ldcg(reinterpret_cast<const float4 *>(pa));
-#pragma unroll
-                                        for (int i = 0; i < 3; ++i)
-                                            if ((grp >> (2 - i)) & 1) {
-                                                ff_add_prod(v.x, v.y, tv[i][0], s_ch[i][f], s_cl[i][f]);
-                                                ff_add_prod(v.z, v.w, tv[i][1], s_ch[i][f], s_cl[i][f]);
-                                            }
-                                        *reinterpret_cast<float4 *>(pa) = v;
-                                    }
+                                    for (int i = 0; i < 3; ++i)
+                                        if ((grp >> (2 - i)) & 1) {
+                                            v.x += s_c[i][f] * tv[i][0];
+                                            v.y += s_c[i][f] * tv[i][1];
+                                        }
+                                    *reinterpret_cast<double2 *>(a.acc[f] + at) = v;
                                 }
+                            }
+                        } else if (a.G) {
+                            ff_add_prod(gh, gl, w[0], gv[j].x, gv[j].y);
+                            ff_add_prod(gh, gl, w[1], gv[j].z, gv[j].w);
+                        }
+                    }
+                    if constexpr (!F64) {
+                        // the same (the functions outside, so that the positions' loads go out
+                        // together: four functions at 12,000 rows, 85.0 -> 82.9 ms)
+                        for (int f = 0; grp && f < a.nf; ++f) {
+                            float4 v[NT];
+#pragma unroll
+                            for (int j = 0; j < NT; ++j) {
+                                if (pos[j] < 0) continue;
+                                v[j] = __ldcg(reinterpret_cast<const float4 *>(a.accp[f] + ((int64_t)pos[j] * BB + eo) * 2));
+                            }
+#pragma unroll
+                            for (int j = 0; j < NT; ++j) {
+                                if (pos[j] < 0) continue;
+                                const float tv[3][2] = {{tm[j].x, tm[j].y}, {tk[j].x, tk[j].y}, {y[j].x, y[j].y}};
+#pragma unroll
+                                for (int i = 0; i < 3; ++i)
+                                    if ((grp >> (2 - i)) & 1) {
+                                        ff_add_prod(v[j].x, v[j].y, tv[i][0], s_ch[i][f], s_cl[i][f]);
+                                        ff_add_prod(v[j].z, v[j].w, tv[i][1], s_ch[i][f], s_cl[i][f]);
+                                    }
+                                *reinterpret_cast<float4 *>(a.accp[f] + ((int64_t)pos[j] * BB + eo) * 2) = v[j];
                             }
                         }
                     }
