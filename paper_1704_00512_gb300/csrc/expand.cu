@@ -800,6 +800,8 @@ extern "C" int cheb_masked_product(const cheb_plan *plan, const cheb_bsr *L, con
     CHEB_TRY(check_operator(plan, L));
     if (plan->precision != CHEB_F64) return fail(CHEB_ERR_INVALID, "cheb_masked_product: needs an FP64 plan");
     if (!R || !C || C == R || (D && C == D)) return fail(CHEB_ERR_INVALID, "cheb_masked_product: bad pointers");
+    if (prod_takes(plan, L, R, D, C, as_stream(stream)))
+        return prod_run(plan, L, R, alpha, D, D ? beta : 0.0, C, as_stream(stream));
     StepArgs<double> a = base_args<double>(plan, L, (const double *)L->vals);
     a.R = R;
     a.Rm = D;

@@ -82,6 +82,7 @@ static int plan_create_device(cheb_plan *plan, const std::vector<int64_t> &sys_c
     CHEB_TRY(gp_tperm(plan->rp, plan->ci, nbr, nnzb, plan->tmp_tperm, &bad, s));
     if (bad < nnzb) return fail(CHEB_ERR_INVALID, "pattern not symmetric: block %lld has no transpose", (long long)bad);
     maxlen = std::max<int32_t>(maxlen, 1);
+    plan->max_row = maxlen;
     // step-kernel panels
     std::vector<int32_t> pan4, aux;
     int64_t out[4];
@@ -276,6 +277,7 @@ static int plan_create_impl(const cheb_bsr *P_out, int32_t precision, int32_t ti
     {
         int32_t maxlen = 1;
         for (int64_t j = 0; j < nbr; ++j) maxlen = std::max(maxlen, (int32_t)(rp[j + 1] - rp[j]));
+        plan->max_row = maxlen;
         auto bcap_for = [&](int64_t ucap) {
             int64_t lo = 0, hi = (int64_t)P * maxlen;
             while (lo < hi) {
@@ -415,6 +417,7 @@ extern "C" int cheb_plan_destroy(cheb_plan *plan) {
         free_row_lists(plan->lists);
         free_row_lists(plan->rlists);
         if (plan->tmp_tperm) cudaFree(plan->tmp_tperm);
+        if (plan->prod_done) cudaEventDestroy(plan->prod_done);
     }
     delete plan;
     return CHEB_OK;
@@ -580,7 +583,7 @@ extern "C" int cheb_plan_attach_operator(cheb_plan *plan, const cheb_bsr *L, siz
         plan->rlists = std::move(rlists);
         rc = col_build_device(plan, L, s);
         if (rc != CHEB_OK && rc != CHEB_ERR_NOSPACE) return rc;
-        plan->op_ws_bytes = plan->lists.bytes() + plan->rlists.bytes() + plan->col.bytes();
+        plan->op_ws_bytes = plan->lists.bytes() + plan->rlists.bytes() + plan->col.bytes() + prod_bytes(plan, nnzL);
         *op_ws_bytes = plan->op_ws_bytes;
         return CHEB_OK;
     }
@@ -612,7 +615,7 @@ extern "C" int cheb_plan_attach_operator(cheb_plan *plan, const cheb_bsr *L, siz
     // operator does not fit it; the expansions then use the ranking kernels)
     const int rc = col_build(plan, rp, ci, lrp, lci);
     if (rc != CHEB_OK && rc != CHEB_ERR_NOSPACE) return rc;
-    plan->op_ws_bytes = plan->lists.bytes() + plan->rlists.bytes() + plan->col.bytes();
+    plan->op_ws_bytes = plan->lists.bytes() + plan->rlists.bytes() + plan->col.bytes() + prod_bytes(plan, nnzL);
     plan->op_bound = false;
     *op_ws_bytes = plan->op_ws_bytes;
     return CHEB_OK;
@@ -652,6 +655,9 @@ extern "C" int cheb_plan_bind_operator(cheb_plan *plan, void *ws, size_t ws_byte
     CHEB_TRY(bind_row_lists(plan->lists, cv, s));
     CHEB_TRY(bind_row_lists(plan->rlists, cv, s));
     CHEB_TRY(col_bind(plan->col, cv, s));
+    const size_t pb = prod_bytes(plan, plan->col.nnzL);
+    plan->prod_ws = pb ? cv.take<char>(pb) : nullptr;
+    if (!cv.fits()) return fail(CHEB_ERR_NOSPACE, "cheb_plan_bind_operator: workspace too small");
     CHEB_CUDA(cudaStreamSynchronize(s));
     col_release_host(plan->col);
     free_row_lists(plan->lists);

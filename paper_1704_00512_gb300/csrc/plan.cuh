@@ -2,6 +2,7 @@
 #pragma once
 
 #include <algorithm>
+#include <mutex>
 #include <vector>
 
 #include "common.cuh"
@@ -121,6 +122,12 @@ struct cheb_plan {
     int32_t gather_host = 0;  // 1: build them on host threads (the reference builder)
     size_t op_ws_bytes = 0;
     bool op_bound = false;
+    // masked products by digits (product.cu): the left operand's digits, in the operator
+    // workspace; the event of their last use orders calls on different streams
+    int32_t max_row = 0;  // longest row of P_out
+    void *prod_ws = nullptr;
+    mutable std::mutex prod_mx;
+    mutable cudaEvent_t prod_done = nullptr;
 };
 
 namespace cheb {
@@ -310,6 +317,13 @@ int row_lists_device(const int64_t *rp, const int32_t *ci, int64_t nbr, const ch
 // The panels (quads of each) in the order of their launch.
 std::vector<int32_t> col_order(const std::vector<int64_t> &quads);
 int col_bind(ColLists &c, Carve &cv, cudaStream_t s);
+// Masked products by digits (product.cu): workspace for an operator of nnzL blocks (0:
+// not for this plan), whether a call is theirs, and the call.
+size_t prod_bytes(const cheb_plan *plan, int64_t nnzL);
+bool prod_takes(const cheb_plan *plan, const cheb_bsr *L, const double *R, const double *D, const double *C,
+                cudaStream_t s);
+int prod_run(const cheb_plan *plan, const cheb_bsr *L, const double *R, double alpha, const double *D, double beta,
+             double *C, cudaStream_t s);
 void col_release_host(ColLists &c);
 bool col_usable(const cheb_plan *plan, const cheb_bsr *Mt);
 size_t col_expand_ws(const cheb_plan *plan, int64_t nnzL);

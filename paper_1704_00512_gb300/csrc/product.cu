@@ -1,0 +1,417 @@
+// Masked products C = alpha P(A B) + beta D of FP64 plans with long rows (Eq. 3's
+// product by itself: orthogonalisation, post-processing and Newton-Schulz steps), on
+// the tensor cores by the digits of colstep.cu.
+//
+// What bounds it.  On the FP64 pipe (k_step) a 4x4 block product is 64 multiply-adds at
+// two per cycle and SM.  As digits it is 26 mma for 16 rows, 16 inner and 8 columns.
+// The left operand is often a matrix on the output pattern (an inverse root, a density
+// matrix), for which no quad lists are kept (the operator's are a few hundred MB
+// already at 6,000 rows), so a warp finds its quads itself: a table of its four rows
+// over the panel's union rows, from which it takes the fours of neighbouring union
+// rows that any of its rows has a block in.  That is a tenth of the work; neighbouring
+// union rows are often neighbours in space, so the fours are 60 % full.
+// Measured (GB300), orthogonalisation and post-processing at 1,500 atoms, 10 / 14 bohr
+// (one product with the operator on the left, three on the output pattern): 66.5 ms
+// on the FP64 pipe, 19.3 ms here.  Error against 64 bits 4.2e-16 -> 4.0e-16.
+//
+// One thread block per panel of two columns (one after the other where their union
+// does not fit): the union of their rows, the columns of B as packed digits in shared
+// memory, 32 bytes per union row and scalar column; a warp takes groups of four
+// neighbouring union rows.  The left operand's digits are formed once per call in the
+// plan's workspace; calls on other streams wait for it.
+#include <mutex>
+
+#include "common.cuh"
+#include "digits.cuh"
+#include "kernels.cuh"
+#include "plan.cuh"
+
+namespace cheb {
+
+constexpr int PR_NW = 16;
+// Quads whose exact digit sums (at most 2^24 a quad) stay below 2^31.
+constexpr int PR_CHUNK = 126;
+
+struct ProdArgs {
+    const int64_t *rp;
+    const int32_t *ci, *tperm, *panels;
+    const int64_t *Lrp;
+    const int32_t *Lci;
+    const double *Lv;
+    int64_t nnzL;
+    const uint4 *opd;
+    const int32_t *opexp, *opflag;
+    const double *R, *D;
+    double *C;
+    double alpha, beta;
+    int32_t cap;  // union rows that fit (a multiple of 4)
+};
+
+struct ProdLayout {
+    int off_pos, off_x, off_tab, off_q, total;
+};
+__host__ __device__ constexpr ProdLayout prod_layout(int cap) {
+    ProdLayout L{};
+    int o = cap * 4;  // union list
+    L.off_pos = o;    // block position of (union row, column)
+    o += cap * 8;
+    o = (o + 127) / 128 * 128;
+    L.off_x = o;  // packed digits: chunk (rows 0 1, rows 2 3) and column of each union row
+    o += (cap + 4) * 256;
+    L.off_tab = o;  // per warp: offset of the block (row of the group, union row) in its operator row
+    o += PR_NW * 4 * (cap + 4) * 2;
+    L.off_q = o;  // per warp: quads with a block
+    o += PR_NW * (cap / 4 + 4);
+    L.total = o;
+    return L;
+}
+constexpr int PR_CAP = 564;
+static_assert(prod_layout(PR_CAP).total + 1024 <= CHEB_MAX_DYN_SMEM, "shared memory");
+
+__device__ __forceinline__ int lower_of(const int32_t *v, int n, int x) {
+    int lo = 0, hi = n;
+    while (lo < hi) {
+        const int m = (lo + hi) >> 1;
+        if (v[m] < x) lo = m + 1; else hi = m;
+    }
+    return lo;
+}
+
+// The products of one group in plain FP64 (an element beyond the digits' grids).
+__device__ __noinline__ void prod_plain(const ProdArgs &a, const int32_t *opos, const uint16_t *tab, int ts, int nu,
+                                        const int64_t *base, int lane, double *out) {
+    const int g = lane >> 2, t = lane & 3;
+    for (int i = 0; i < 4; ++i) out[i] = 0.0;
+    for (int s = 0; s < nu; ++s) {
+        const int p = opos[2 * s + (t >> 1)];
+        if (p < 0) continue;
+        for (int h = 0; h < 2; ++h) {
+            const uint16_t id = tab[((g >> 2) + 2 * h) * ts + s];
+            if (id == 0xffffu) continue;
+            const double *hv = a.Lv + (base[h] + id) * BB + 4 * (g & 3);
+            const double *x = a.R + (int64_t)p * BB + 2 * (t & 1);
+            for (int m = 0; m < 4; ++m) {
+                out[2 * h] = fma(hv[m], x[4 * m], out[2 * h]);
+                out[2 * h + 1] = fma(hv[m], x[4 * m + 1], out[2 * h + 1]);
+            }
+        }
+    }
+}
+
+__global__ void __launch_bounds__(PR_NW * 32, 1) k_product(const __grid_constant__ ProdArgs a) {
+    using Dg = Dig<double>;
+    constexpr int NTH = PR_NW * 32;
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ uint32_t s_max[8];
+    __shared__ int s_e[8];
+    __shared__ int s_slow;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, cap = a.cap, ts = cap + 4;
+    const ProdLayout lay = prod_layout(cap);
+    int32_t *ulist = reinterpret_cast<int32_t *>(smem), *opos = reinterpret_cast<int32_t *>(smem + lay.off_pos);
+    uint4 *X = reinterpret_cast<uint4 *>(smem + lay.off_x);
+    uint16_t *pre = reinterpret_cast<uint16_t *>(smem + lay.off_tab);  // (before the groups)
+    uint16_t *tab = reinterpret_cast<uint16_t *>(smem + lay.off_tab) + warp * 4 * ts;
+    unsigned char *ql = smem + lay.off_q + warp * (cap / 4 + 4);
+    const unsigned lt = (1u << lane) - 1u;
+    const int j0 = a.panels[2 * blockIdx.x], nj = a.panels[2 * blockIdx.x + 1];
+    for (int q0 = 0, nc = 0; q0 < nj; q0 += nc) {
+        // 1. the union of the columns' rows.  pre[i]: blocks of column 0 before its i-th
+        // that column 1 has too; the rank in the union of column 0's i-th row, with l
+        // rows of column 1 before it, is i + l - pre[i], and the same the other way round
+        nc = min(2, nj - q0);
+        const int64_t r0 = a.rp[j0 + q0], r1 = a.rp[j0 + q0 + 1];
+        const int n0 = (int)(r1 - r0);
+        int n1 = nc == 2 ? (int)(a.rp[j0 + q0 + 2] - r1) : 0, nu = n0;
+        const int32_t *c0 = a.ci + r0, *c1 = a.ci + r1;
+        __syncthreads();  // (the pass before is done with shared memory)
+        if (nc == 2) {
+            for (int i = tid; i < n0; i += NTH) {
+                const int x = c0[i], l = lower_of(c1, n1, x);
+                pre[i] = l < n1 && c1[l] == x;
+            }
+            __syncthreads();
+            if (warp == 0) {
+                int run = 0;
+                for (int b = 0; b < n0; b += 32) {
+                    const int in = b + lane < n0 ? pre[b + lane] : 0;
+                    const unsigned m = __ballot_sync(0xffffffffu, in);
+                    if (b + lane < n0) pre[b + lane] = (uint16_t)(run + __popc(m & lt));
+                    run += __popc(m);
+                }
+                if (lane == 0) pre[n0] = (uint16_t)run;
+            }
+            __syncthreads();
+            nu = n0 + n1 - pre[n0];
+            if (nu > cap) {  // (every thread finds the same)
+                nc = 1;
+                n1 = 0;
+                nu = n0;
+            }
+        }
+        const int nu4 = (nu + 3) & ~3;
+        // 2. positions and the columns' largest elements, then their digits
+        for (int i = tid; i < (nu4 + 4) * 16; i += NTH) X[i] = make_uint4(0x82008200u, 0x02000200u, 0x82008200u, 0x02000200u);
+        for (int i = tid; i < 2 * nu; i += NTH) opos[i] = -1;
+        if (tid < 8) s_max[tid] = 0u;
+        if (tid == 0) s_slow = *a.opflag != 0;
+        __syncthreads();
+        for (int b = tid; b < n0 + n1; b += NTH) {
+            const int q = b >= n0, i = q ? b - n0 : b, K = q ? c1[i] : c0[i];
+            int s = i;
+            if (nc == 2) {
+                const int l = q ? lower_of(c0, n0, K) : lower_of(c1, n1, K);
+                s = i + l - pre[q ? l : i];
+            }
+            const int p = a.tperm[(q ? r1 : r0) + i];
+            ulist[s] = K;
+            opos[2 * s + q] = p;
+            uint32_t m[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+            for (int e = 0; e < 16; e += 2) {
+                const double2 v = *reinterpret_cast<const double2 *>(a.R + (int64_t)p * BB + e);
+                m[e & 3] = max(m[e & 3], mag_bits(v.x));
+                m[(e & 3) + 1] = max(m[(e & 3) + 1], mag_bits(v.y));
+            }
+#pragma unroll
+            for (int c = 0; c < 4; ++c) atomicMax(&s_max[4 * q + c], m[c]);
+        }
+        __syncthreads();
+        if (tid < 8) {
+            int e;
+            if (!grid_exp<double>(s_max[tid], Dg::EX_MIN, Dg::EX_MAX, e)) s_slow = 1;
+            s_e[tid] = e;
+        }
+        __syncthreads();
+        const bool slow = s_slow != 0;
+        if (!slow) {
+            for (int i = tid; i < 2 * nu; i += NTH) {
+                const int p = opos[i], s = i >> 1, q = i & 1, sw = 2 * (s & 3);
+                if (p < 0) continue;
+                double v[16];
+#pragma unroll
+                for (int e = 0; e < 16; e += 2) {
+                    const double2 u = *reinterpret_cast<const double2 *>(a.R + (int64_t)p * BB + e);
+                    v[e] = u.x;
+                    v[e + 1] = u.y;
+                }
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const int col = 4 * q + c, e = s_e[col];
+                    uint32_t w[4];
+                    pack_pair(w, v[c], v[4 + c], e);
+                    X[s * 16 + (col ^ sw)] = make_uint4(w[0], w[1], w[2], w[3]);
+                    pack_pair(w, v[8 + c], v[12 + c], e);
+                    X[s * 16 + 8 + (col ^ sw)] = make_uint4(w[0], w[1], w[2], w[3]);
+                }
+            }
+        }
+        __syncthreads();
+        // 3. the warp's groups of four union rows
+        const int g = lane >> 2, t = lane & 3;
+        const uint4 *ob = a.opd + (g & 3) * 2;
+        for (int gi = warp; 4 * gi < nu; gi += PR_NW) {
+            __syncwarp();
+            for (int i = lane; i < ts; i += 32) reinterpret_cast<uint64_t *>(tab)[i] = ~0ull;
+            __syncwarp();
+            for (int r = 0; r < 4 && 4 * gi + r < nu; ++r) {
+                const int64_t b = a.Lrp[ulist[4 * gi + r]];
+                const int len = (int)(a.Lrp[ulist[4 * gi + r] + 1] - b);
+                for (int i = lane; i < len; i += 32) {
+                    const int K = __ldg(a.Lci + b + i), s = lower_of(ulist, nu, K);
+                    if (s < nu && ulist[s] == K) tab[r * ts + s] = (uint16_t)i;
+                }
+            }
+            __syncwarp();
+            int64_t base[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int u = 4 * gi + (g >> 2) + 2 * h;
+                base[h] = u < nu ? a.Lrp[ulist[u]] : 0;
+            }
+            double val[4] = {0.0, 0.0, 0.0, 0.0};
+            if (slow) {
+                prod_plain(a, opos, tab, ts, nu, base, lane, val);
+            } else {
+                int cnt = 0;
+                for (int b = 0; b < nu4 / 4; b += 32) {
+                    const int q = b + lane;
+                    bool any = false;
+                    if (q < nu4 / 4) {
+                        uint64_t all = ~0ull;
+#pragma unroll
+                        for (int r = 0; r < 4; ++r) all &= *reinterpret_cast<const uint64_t *>(tab + r * ts + 4 * q);
+                        any = all != ~0ull;
+                    }
+                    const unsigned m = __ballot_sync(0xffffffffu, any);
+                    if (any) ql[cnt + __popc(m & lt)] = (unsigned char)q;
+                    cnt += __popc(m);
+                }
+                // quads go in pairs: an empty one (beyond the union) fills up the last
+                if (lane == 0) ql[cnt] = (unsigned char)(nu4 / 4);
+                cnt = (cnt + 1) & ~1;
+                __syncwarp();
+                struct Op {
+                    uint32_t w[2][8];
+                };
+                const uint32_t base0 = (uint32_t)base[0], base1 = (uint32_t)base[1], none = (uint32_t)a.nnzL;
+                const uint16_t *tl = tab + (g >> 2) * ts + t;
+                auto load_h = [&](Op &o, int k) {
+                    const int q = ql[min(k, cnt - 1)];
+                    const uint32_t i0 = tl[4 * q], i1 = tl[2 * ts + 4 * q];
+                    ld_row(o.w[0], ob, i0 == 0xffffu ? none : base0 + i0);
+                    ld_row(o.w[1], ob, i1 == 0xffffu ? none : base1 + i1);
+                };
+                Op h[2];
+                if (cnt > 0) {
+                    load_h(h[0], 0);
+                    load_h(h[1], 1);
+                }
+                for (int k0 = 0; k0 < cnt; k0 += PR_CHUNK) {
+                    const int k1 = min(cnt, k0 + PR_CHUNK);
+                    float dl[2][4];
+                    int is[4][4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        dl[0][i] = dl[1][i] = 0.f;
+#pragma unroll
+                        for (int s = 0; s < 4; ++s) is[s][i] = 0;
+                    }
+#pragma unroll 1
+                    for (int k = k0; k < k1; k += 2) {
+                        float z[4][4];
+#pragma unroll
+                        for (int o = 0; o < 2; ++o) {
+                            const uint4 *xs = X + (4 * ql[k + o] + t) * 16 + (g ^ (2 * t));
+                            const uint4 x0 = xs[0], x1 = xs[8];
+                            const uint32_t w0[4] = {x0.x, x0.y, x0.z, x0.w}, w1[4] = {x1.x, x1.y, x1.z, x1.w};
+                            uint32_t B[6][2];
+#pragma unroll
+                            for (int i = 0; i < 6; ++i) {
+                                B[i][0] = packed_digit(w0, i);
+                                B[i][1] = packed_digit(w1, i);
+                            }
+                            const float zero[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                            for (int i = 0; i < 6; ++i) {
+                                uint32_t A[4];
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) {  // (half e % 2, pair e / 2)
+                                    const uint32_t *hw = h[o].w[e & 1] + 2 * (e & 2);
+                                    const uint32_t pw[4] = {hw[0], hw[1], hw[2], hw[3]};
+                                    A[e] = packed_digit(pw, i);
+                                }
+#pragma unroll
+                                for (int s = i; s < 6; ++s) {
+                                    if (s >= 4) mma16816(dl[s & 1], A, B[s - i], dl[s & 1]);
+                                    else if (i == 0 && (o == 0 || s >= 2)) mma16816(z[s], A, B[s], zero);
+                                    else mma16816(z[s], A, B[s - i], z[s]);
+                                }
+                                // (the sums of s = 0, 1 stay exact over two quads)
+                                if (i >= 1) {  // D_6 into D_5's accumulator: the panel digit times 2^-10
+                                    const uint32_t Bs[2] = {h2_fma(B[6 - i][0], 0x14001400u, 0u), h2_fma(B[6 - i][1], 0x14001400u, 0u)};
+                                    mma16816(dl[1], A, Bs, dl[1]);
+                                }
+                                if (i < 4 && (o == 1 || i >= 2)) {
+#pragma unroll
+                                    for (int e = 0; e < 4; ++e) is[i][e] += __float2int_rn(z[i][e]);
+                                }
+                            }
+                            load_h(h[o], k + o + 2);
+                        }
+                    }
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int64_t q = (((int64_t)is[0][i] * 1024 + is[1][i]) * 1024 + is[2][i]) * 1024 + is[3][i];
+                        val[i] += (double)q + (double)fmaf(dl[1][i], 0x1p-20f, dl[0][i] * 0x1p-10f);
+                    }
+                }
+            }
+            // 4. the lane's elements (as in colstep.cu)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int u = 4 * gi + (g >> 2) + 2 * h;
+                if (u >= nu) continue;
+                const int p = opos[2 * u + (t >> 1)];
+                if (p < 0) continue;
+                double y[2];
+#pragma unroll
+                for (int c = 0; c < 2; ++c)
+                    y[c] = slow ? val[2 * h + c] : val[2 * h + c] * pow2(a.opexp[ulist[u]] + s_e[2 * t + c] - 48, 0.0);
+                const int64_t at = (int64_t)p * BB + 4 * (g & 3) + 2 * (t & 1);
+                double2 v = make_double2(a.alpha * y[0], a.alpha * y[1]);
+                if (a.D) {
+                    const double2 d = *reinterpret_cast<const double2 *>(a.D + at);
+                    v = make_double2(fma(a.alpha, y[0], a.beta * d.x), fma(a.alpha, y[1], a.beta * d.y));
+                }
+                *reinterpret_cast<double2 *>(a.C + at) = v;
+            }
+        }
+    }
+}
+
+size_t prod_bytes(const cheb_plan *plan, int64_t nnzL) {
+    if (plan->precision != CHEB_F64 || !plan->col.built || plan->max_row > PR_CAP || plan->nbr > 65535) return 0;
+    const int64_t n = std::max(nnzL, plan->nnzb);
+    return align_up((size_t)(n + 1) * 128) + align_up(plan->nbr * 4) + align_up(64);
+}
+
+// Long rows (those of the column kernel's lists: the FP64 pipe bounds them, and the
+// kernels for short rows keep their bits) of the operator or of a matrix on the output
+// pattern, in arrays aligned for the loads; not while the stream is captured, since a
+// graph's replays cannot be ordered with other calls' use of the digits.
+bool prod_takes(const cheb_plan *plan, const cheb_bsr *L, const double *R, const double *D, const double *C,
+                cudaStream_t s) {
+    if (!plan->prod_ws || !plan->op_bound) return false;
+    const bool op = L->row_ptr == plan->op_rp && L->col_idx == plan->op_ci && L->nnzb == plan->col.nnzL;
+    const bool out = L->row_ptr == plan->rp && L->col_idx == plan->ci && L->nnzb == plan->nnzb;
+    if (!op && !out) return false;
+    const uintptr_t at = reinterpret_cast<uintptr_t>(R) | reinterpret_cast<uintptr_t>(D) | reinterpret_cast<uintptr_t>(C);
+    if (at % 16) return false;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return st == cudaStreamCaptureStatusNone;
+}
+
+int prod_run(const cheb_plan *plan, const cheb_bsr *L, const double *R, double alpha, const double *D, double beta,
+             double *C, cudaStream_t s) {
+    const int64_t n = std::max(plan->col.nnzL, plan->nnzb);
+    Carve cv(plan->prod_ws, prod_bytes(plan, plan->col.nnzL));
+    ProdArgs a{};
+    uint4 *opd = cv.take<uint4>((n + 1) * 8);
+    int32_t *opexp = cv.take<int32_t>(plan->nbr), *flag = cv.take<int32_t>(16);
+    a.rp = plan->rp;
+    a.ci = plan->ci;
+    a.tperm = plan->d_tperm;
+    a.panels = plan->d_panels;
+    a.Lrp = L->row_ptr;
+    a.Lci = L->col_idx;
+    a.Lv = static_cast<const double *>(L->vals);
+    a.nnzL = L->nnzb;
+    a.opd = opd;
+    a.opexp = opexp;
+    a.opflag = flag;
+    a.R = R;
+    a.D = D;
+    a.C = C;
+    a.alpha = alpha;
+    a.beta = beta;
+    a.cap = std::min(PR_CAP, (plan->max_union + 3) & ~3);
+    const int smem = prod_layout(a.cap).total;
+    // one user of the digits at a time: this call waits, on its stream, for the last one
+    std::lock_guard<std::mutex> lock(plan->prod_mx);
+    if (!plan->prod_done) CHEB_CUDA(cudaEventCreateWithFlags(&plan->prod_done, cudaEventDisableTiming));
+    else CHEB_CUDA(cudaStreamWaitEvent(s, plan->prod_done, 0));
+    CHEB_CUDA(cudaMemsetAsync(flag, 0, 64, s));
+    k_opdig<double><<<(unsigned)((plan->nbr + 1 + 7) / 8), 256, 0, s>>>(L->row_ptr, a.Lv, plan->nbr, L->nnzb, 0, opd, opexp, flag);
+    CHEB_TRY(check_launch("k_opdig"));
+    CHEB_CUDA(cudaFuncSetAttribute(k_product, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    k_product<<<(unsigned)plan->n_panels, PR_NW * 32, smem, s>>>(a);
+    const int rc = check_launch("k_product");
+    CHEB_CUDA(cudaEventRecord(plan->prod_done, s));
+    return rc;
+}
+
+}  // namespace cheb
