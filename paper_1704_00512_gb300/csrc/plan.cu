@@ -94,6 +94,7 @@ static int plan_create_device(cheb_plan *plan, const std::vector<int64_t> &sys_c
     for (int64_t p = 0; p < out[0]; ++p) {
         plan->h_panels[2 * p] = pan4[4 * p];
         plan->h_panels[2 * p + 1] = pan4[4 * p + 1];
+        plan->h_union.push_back(pan4[4 * p + 2]);
     }
     // resident panels, as in the host builder
     const int64_t nw = (nbr + 31) / 32;
@@ -265,6 +266,7 @@ static int plan_create_impl(const cheb_bsr *P_out, int32_t precision, int32_t ti
             }
             plan->h_panels.push_back((int32_t)j0);
             plan->h_panels.push_back(ncols);
+            plan->h_union.push_back(cnt);
             max_union = std::max(max_union, cnt);
             ++panel;
         }
@@ -655,9 +657,8 @@ extern "C" int cheb_plan_bind_operator(cheb_plan *plan, void *ws, size_t ws_byte
     CHEB_TRY(bind_row_lists(plan->lists, cv, s));
     CHEB_TRY(bind_row_lists(plan->rlists, cv, s));
     CHEB_TRY(col_bind(plan->col, cv, s));
-    const size_t pb = prod_bytes(plan, plan->col.nnzL);
-    plan->prod_ws = pb ? cv.take<char>(pb) : nullptr;
-    if (!cv.fits()) return fail(CHEB_ERR_NOSPACE, "cheb_plan_bind_operator: workspace too small");
+    std::vector<int32_t> prod_panels;  // (outlives the copy)
+    CHEB_TRY(prod_bind(plan, cv, prod_panels, s));
     CHEB_CUDA(cudaStreamSynchronize(s));
     col_release_host(plan->col);
     free_row_lists(plan->lists);

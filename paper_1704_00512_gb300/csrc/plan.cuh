@@ -91,6 +91,7 @@ struct cheb_plan {
     std::vector<int32_t> h_tperm;   // slot of (J,I) for each slot (I,J)
     int32_t *tmp_tperm = nullptr;   // the same, built on the device, until cheb_plan_bind
     std::vector<int32_t> h_panels;  // pairs (first column, column count)
+    std::vector<int32_t> h_union;   // union rows of each
     // panels of the resident kernel (whole expansion per thread block); they
     // never straddle two systems of a block-diagonal batch
     int32_t nsys = 1;
@@ -318,8 +319,9 @@ int row_lists_device(const int64_t *rp, const int32_t *ci, int64_t nbr, const ch
 std::vector<int32_t> col_order(const std::vector<int64_t> &quads);
 int col_bind(ColLists &c, Carve &cv, cudaStream_t s);
 // Masked products by digits (product.cu): workspace for an operator of nnzL blocks (0:
-// not for this plan), whether a call is theirs, and the call.
+// not for this plan), its place, whether a call is theirs, and the call.
 size_t prod_bytes(const cheb_plan *plan, int64_t nnzL);
+int prod_bind(cheb_plan *plan, Carve &cv, std::vector<int32_t> &panels, cudaStream_t s);
 bool prod_takes(const cheb_plan *plan, const cheb_bsr *L, const double *R, const double *D, const double *C,
                 cudaStream_t s);
 int prod_run(const cheb_plan *plan, const cheb_bsr *L, const double *R, double alpha, const double *D, double beta,

@@ -12,7 +12,7 @@
 // union rows are often neighbours in space, so the fours are 60 % full.
 // Measured (GB300), orthogonalisation and post-processing at 1,500 atoms, 10 / 14 bohr
 // (one product with the operator on the left, three on the output pattern): 66.5 ms
-// on the FP64 pipe, 19.3 ms here.  Error against 64 bits 4.2e-16 -> 4.0e-16.
+// on the FP64 pipe, 14.4 ms here.  Error against 64 bits 4.2e-16 -> 4.0e-16.
 //
 // One thread block per panel of two columns (one after the other where their union
 // does not fit): the union of their rows, the columns of B as packed digits in shared
@@ -45,10 +45,11 @@ struct ProdArgs {
     double *C;
     double alpha, beta;
     int32_t cap;  // union rows that fit (a multiple of 4)
+    int32_t nw;   // words of the union's bitmap
 };
 
 struct ProdLayout {
-    int off_pos, off_x, off_tab, off_q, total;
+    int off_pos, off_x, off_tab, off_q, off_bits;
 };
 __host__ __device__ constexpr ProdLayout prod_layout(int cap) {
     ProdLayout L{};
@@ -62,19 +63,15 @@ __host__ __device__ constexpr ProdLayout prod_layout(int cap) {
     o += PR_NW * 4 * (cap + 4) * 2;
     L.off_q = o;  // per warp: quads with a block
     o += PR_NW * (cap / 4 + 4);
-    L.total = o;
+    L.off_bits = (o + 15) / 16 * 16;  // the union as a bitmap, 8 bytes a word of 32 block rows
     return L;
 }
-constexpr int PR_CAP = 564;
-static_assert(prod_layout(PR_CAP).total + 1024 <= CHEB_MAX_DYN_SMEM, "shared memory");
-
-__device__ __forceinline__ int lower_of(const int32_t *v, int n, int x) {
-    int lo = 0, hi = n;
-    while (lo < hi) {
-        const int m = (lo + hi) >> 1;
-        if (v[m] < x) lo = m + 1; else hi = m;
-    }
-    return lo;
+// Union rows that fit beside the bitmap (0: none).
+static int prod_cap(const cheb_plan *plan) {
+    const int64_t room = CHEB_MAX_DYN_SMEM - 1024 - (plan->nbr + 31) / 32 * 8;
+    int cap = (plan->max_union + 3) & ~3;
+    while (cap > 0 && prod_layout(cap).off_bits > room) cap -= 4;
+    return cap;
 }
 
 // The products of one group in plain FP64 (an element beyond the digits' grids).
@@ -104,49 +101,40 @@ __global__ void __launch_bounds__(PR_NW * 32, 1) k_product(const __grid_constant
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ uint32_t s_max[8];
     __shared__ int s_e[8];
-    __shared__ int s_slow;
+    __shared__ int s_slow, wsum[32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, cap = a.cap, ts = cap + 4;
     const ProdLayout lay = prod_layout(cap);
     int32_t *ulist = reinterpret_cast<int32_t *>(smem), *opos = reinterpret_cast<int32_t *>(smem + lay.off_pos);
     uint4 *X = reinterpret_cast<uint4 *>(smem + lay.off_x);
-    uint16_t *pre = reinterpret_cast<uint16_t *>(smem + lay.off_tab);  // (before the groups)
+    uint2 *bits = reinterpret_cast<uint2 *>(smem + lay.off_bits);
     uint16_t *tab = reinterpret_cast<uint16_t *>(smem + lay.off_tab) + warp * 4 * ts;
     unsigned char *ql = smem + lay.off_q + warp * (cap / 4 + 4);
     const unsigned lt = (1u << lane) - 1u;
     const int j0 = a.panels[2 * blockIdx.x], nj = a.panels[2 * blockIdx.x + 1];
     for (int q0 = 0, nc = 0; q0 < nj; q0 += nc) {
-        // 1. the union of the columns' rows.  pre[i]: blocks of column 0 before its i-th
-        // that column 1 has too; the rank in the union of column 0's i-th row, with l
-        // rows of column 1 before it, is i + l - pre[i], and the same the other way round
+        // 1. the union of the columns' rows as a bitmap with ranks, the second column only
+        // if it still fits
         nc = min(2, nj - q0);
-        const int64_t r0 = a.rp[j0 + q0], r1 = a.rp[j0 + q0 + 1];
-        const int n0 = (int)(r1 - r0);
-        int n1 = nc == 2 ? (int)(a.rp[j0 + q0 + 2] - r1) : 0, nu = n0;
-        const int32_t *c0 = a.ci + r0, *c1 = a.ci + r1;
-        __syncthreads();  // (the pass before is done with shared memory)
-        if (nc == 2) {
-            for (int i = tid; i < n0; i += NTH) {
-                const int x = c0[i], l = lower_of(c1, n1, x);
-                pre[i] = l < n1 && c1[l] == x;
-            }
+        const int64_t r0 = a.rp[j0 + q0], r1 = a.rp[j0 + q0 + 1], r2 = a.rp[j0 + q0 + nc];
+        int nu = 0;
+        int64_t re = r2;  // end of the blocks taken
+        while (true) {
+            __syncthreads();  // (the pass before is done with shared memory)
+            for (int w = tid; w < a.nw; w += NTH) bits[w] = make_uint2(0u, 0u);
             __syncthreads();
-            if (warp == 0) {
-                int run = 0;
-                for (int b = 0; b < n0; b += 32) {
-                    const int in = b + lane < n0 ? pre[b + lane] : 0;
-                    const unsigned m = __ballot_sync(0xffffffffu, in);
-                    if (b + lane < n0) pre[b + lane] = (uint16_t)(run + __popc(m & lt));
-                    run += __popc(m);
-                }
-                if (lane == 0) pre[n0] = (uint16_t)run;
-            }
+            for (int64_t b = r0 + tid; b < re; b += NTH) atomicOr(&bits[a.ci[b] >> 5].x, 1u << (a.ci[b] & 31));
             __syncthreads();
-            nu = n0 + n1 - pre[n0];
-            if (nu > cap) {  // (every thread finds the same)
-                nc = 1;
-                n1 = 0;
-                nu = n0;
+            const int per = (a.nw + NTH - 1) / NTH, w0 = min(a.nw, tid * per), w1 = min(a.nw, w0 + per);
+            int n = 0;
+            for (int w = w0; w < w1; ++w) n += __popc(bits[w].x);
+            int run = block_excl_scan<PR_NW>(n, wsum, &nu);
+            for (int w = w0; w < w1; ++w) {
+                bits[w].y = (unsigned)run;
+                run += __popc(bits[w].x);
             }
+            if (nu <= a.cap) break;  // (every thread finds the same; a single column fits)
+            nc = 1;
+            re = r1;
         }
         const int nu4 = (nu + 3) & ~3;
         // 2. positions and the columns' largest elements, then their digits
@@ -155,14 +143,9 @@ __global__ void __launch_bounds__(PR_NW * 32, 1) k_product(const __grid_constant
         if (tid < 8) s_max[tid] = 0u;
         if (tid == 0) s_slow = *a.opflag != 0;
         __syncthreads();
-        for (int b = tid; b < n0 + n1; b += NTH) {
-            const int q = b >= n0, i = q ? b - n0 : b, K = q ? c1[i] : c0[i];
-            int s = i;
-            if (nc == 2) {
-                const int l = q ? lower_of(c0, n0, K) : lower_of(c1, n1, K);
-                s = i + l - pre[q ? l : i];
-            }
-            const int p = a.tperm[(q ? r1 : r0) + i];
+        for (int64_t b = r0 + tid; b < re; b += NTH) {
+            const int q = b >= r1, K = a.ci[b], s = rank_of(bits, K);
+            const int p = a.tperm[b];
             ulist[s] = K;
             opos[2 * s + q] = p;
             uint32_t m[4] = {0u, 0u, 0u, 0u};
@@ -217,8 +200,8 @@ __global__ void __launch_bounds__(PR_NW * 32, 1) k_product(const __grid_constant
                 const int64_t b = a.Lrp[ulist[4 * gi + r]];
                 const int len = (int)(a.Lrp[ulist[4 * gi + r] + 1] - b);
                 for (int i = lane; i < len; i += 32) {
-                    const int K = __ldg(a.Lci + b + i), s = lower_of(ulist, nu, K);
-                    if (s < nu && ulist[s] == K) tab[r * ts + s] = (uint16_t)i;
+                    const int s = rank_of(bits, __ldg(a.Lci + b + i));
+                    if (s >= 0) tab[r * ts + s] = (uint16_t)i;
                 }
             }
             __syncwarp();
@@ -350,9 +333,24 @@ __global__ void __launch_bounds__(PR_NW * 32, 1) k_product(const __grid_constant
 }
 
 size_t prod_bytes(const cheb_plan *plan, int64_t nnzL) {
-    if (plan->precision != CHEB_F64 || !plan->col.built || plan->max_row > PR_CAP || plan->nbr > 65535) return 0;
+    if (plan->precision != CHEB_F64 || !plan->col.built || plan->nbr > 65535 || plan->max_row > prod_cap(plan)) return 0;
     const int64_t n = std::max(nnzL, plan->nnzb);
-    return align_up((size_t)(n + 1) * 128) + align_up(plan->nbr * 4) + align_up(64);
+    return align_up((size_t)(n + 1) * 128) + align_up(plan->nbr * 4) + align_up(64) + align_up(plan->n_panels * 8);
+}
+
+// The panels go to the device in the order of their launch: by the square of their
+// union, as the column kernel's by their quads.
+int prod_bind(cheb_plan *plan, Carve &cv, std::vector<int32_t> &panels, cudaStream_t s) {
+    const size_t bytes = prod_bytes(plan, plan->col.nnzL);
+    plan->prod_ws = bytes ? cv.take<char>(bytes) : nullptr;
+    if (!cv.fits()) return fail(CHEB_ERR_NOSPACE, "cheb_plan_bind_operator: workspace too small");
+    if (!bytes) return CHEB_OK;
+    std::vector<int64_t> work;
+    for (const int32_t u : plan->h_union) work.push_back((int64_t)u * u);
+    for (const int32_t p : col_order(work)) panels.insert(panels.end(), {plan->h_panels[2 * p], plan->h_panels[2 * p + 1]});
+    char *at = static_cast<char *>(plan->prod_ws) + bytes - align_up(plan->n_panels * 8);
+    CHEB_CUDA(cudaMemcpyAsync(at, panels.data(), panels.size() * 4, cudaMemcpyHostToDevice, s));
+    return CHEB_OK;
 }
 
 // Long rows (those of the column kernel's lists: the FP64 pipe bounds them, and the
@@ -382,10 +380,10 @@ int prod_run(const cheb_plan *plan, const cheb_bsr *L, const double *R, double a
     ProdArgs a{};
     uint4 *opd = cv.take<uint4>((n + 1) * 8);
     int32_t *opexp = cv.take<int32_t>(plan->nbr), *flag = cv.take<int32_t>(16);
+    a.panels = cv.take<int32_t>(2 * plan->n_panels);
     a.rp = plan->rp;
     a.ci = plan->ci;
     a.tperm = plan->d_tperm;
-    a.panels = plan->d_panels;
     a.Lrp = L->row_ptr;
     a.Lci = L->col_idx;
     a.Lv = static_cast<const double *>(L->vals);
@@ -398,8 +396,9 @@ int prod_run(const cheb_plan *plan, const cheb_bsr *L, const double *R, double a
     a.C = C;
     a.alpha = alpha;
     a.beta = beta;
-    a.cap = std::min(PR_CAP, (plan->max_union + 3) & ~3);
-    const int smem = prod_layout(a.cap).total;
+    a.cap = prod_cap(plan);
+    a.nw = (int32_t)((plan->nbr + 31) / 32);
+    const int smem = prod_layout(a.cap).off_bits + a.nw * 8;
     // one user of the digits at a time: this call waits, on its stream, for the last one
     std::lock_guard<std::mutex> lock(plan->prod_mx);
     if (!plan->prod_done) CHEB_CUDA(cudaEventCreateWithFlags(&plan->prod_done, cudaEventDisableTiming));
