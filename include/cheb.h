@@ -159,7 +159,7 @@ int cheb_plan_info(const cheb_plan *plan, int64_t *n_panels, int32_t *panel_widt
  * row_ptr/col_idx pointers reads its entries from the lists instead of
  * ranking the operator's rows at every step; other operators use the ranking
  * path.  Both paths multiply the same blocks in the same order, so results
- * are bit-identical.  Attaching again replaces the lists.  The lists are
+ * are bit-identical (the column-order kernel's, below, agree to rounding).  Attaching again replaces the lists.  The lists are
  * built by device kernels from the device arrays of P_out and L (the plan
  * must be bound first) unless the host builders were chosen (see "Builders"
  * below). */
@@ -193,8 +193,8 @@ int cheb_plan_attach_operator(cheb_plan *plan, const cheb_bsr *L, size_t *op_ws_
  * words (padding included).
  *
  * This gather plan is built by device kernels from the device patterns of
- * P_out and the operator (a sequential panel walk in one thread block, then
- * one thread block per panel: union bitmap and ranks, the groups and their merged
+ * P_out and the operator (where a panel starting at each column ends, the chain of
+ * starts, then one thread block per panel: union bitmap and ranks, the groups and their merged
  * slots, the groups dealt to the warps by decreasing quad count, each to the warp
  * with the fewest quads so far, and the entry streams; a few scalars and per-panel
  * integers come back to the host to size the lists).  It uses device memory of
@@ -375,6 +375,16 @@ int cheb_expand_batched(const cheb_plan *plan, const cheb_bsr *Mt, int32_t max_t
  * L: FP64 BCSR with nbr rows (any pattern); R, D, C: FP64 values on the plan's
  * P_out (BCSR order).  D may be NULL (beta ignored).  C must not alias R or D.
  * The plan must be an FP64 plan.  Asynchronous; no workspace.
+ *
+ * With the column kernel's lists bound (long operator rows) and L on the attached
+ * operator's pattern or on the plan's own (the same row_ptr / col_idx pointers), the
+ * product runs as that kernel's digit products, exact but for a grid of 2^-59 of each
+ * operator row's and each column's largest element.  It needs rows of P_out that fit
+ * shared memory (about 560 blocks), at most 65,535 block rows and 16-byte aligned R, D
+ * and C; otherwise, and while the stream is captured, it runs on the FP64 pipe, with
+ * results equal to rounding.  L's digits are kept in the operator workspace (128 bytes
+ * per block of the larger pattern, part of op_ws_bytes); calls with one plan on several
+ * streams or threads are put in order behind each other on the device.
  */
 int cheb_masked_product(const cheb_plan *plan, const cheb_bsr *L, const double *R, double alpha,
                         const double *D, double beta, double *C, void *stream);
