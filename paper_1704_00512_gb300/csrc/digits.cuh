@@ -96,7 +96,7 @@ __device__ __forceinline__ void panel_digits(uint32_t (&w)[2], uint32_t &third, 
     const uint32_t off = (1024u << 19) + (1024u << 8) + 128u;
     const uint32_t u = (uint32_t)q0 + off, v = (uint32_t)q1 + off;
     auto h2 = [](int a, int b) {
-        const __half2 h = __halves2half2(__int2half_rn(a), __int2half_rn(b));
+        const __half2 h = __floats2half2_rn((float)a, (float)b);  // (off the conversion unit)
         return *reinterpret_cast<const uint32_t *>(&h);
     };
     w[0] = h2((int)(u >> 19) - 1024, (int)(v >> 19) - 1024);
