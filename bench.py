@@ -40,8 +40,8 @@ import numpy as np  # noqa: E402
 METRIC = "density-matrix solves/s at <=1e-6 vs FP64 plain; masked SpGEMM HBM GB/s"
 UNIT = "solves/s"
 FALLBACK_HBM_GBS = 6800.0
-# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch of the
-# column-order step kernel, from one ncu capture of every k_colstep launch of a
+# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per step of the
+# column-order kernel, from one ncu capture of every k_colstep launch of a
 # 4-mu solve on 3,000 atoms (12,000 rows, r_c 10, r_out 14 bohr: 1,183,812
 # P_out blocks; kT 0.05 Ha, 960 terms: 478 pass-1 launches with moments only,
 # 958 pass-2 launches with four accumulators; grouped steps included; atoms in
@@ -98,7 +98,7 @@ WORKLOADS = {
     "powers_fp64_12k": dict(powers=True, n_atoms=3000, r_c=10.0, r_buf=4.0, tol=1e-10, precision="f64", n_mu=3,
                             exponents=(-1.0, 0.5, -0.5)),
     # The same powers with FP64-accurate double-float products on the FP32 pipe
-    # (CHEB_F64X), timed against the FP64 (DFMA) expansion in the same run.
+    # (CHEB_F64X), timed against the FP64 expansion in the same run.
     "powers_f64x_12k": dict(powers=True, n_atoms=3000, r_c=10.0, r_buf=4.0, tol=1e-10, precision="f64x", n_mu=3,
                             exponents=(-1.0, 0.5, -0.5)),
     # Batched: 64 independent systems of U{125..1500} atoms (seeds 0..63), 8 bohr
@@ -418,8 +418,8 @@ def run_cheb(args, rank: int, world: int, local: int):
         roof = {"bound": "alu", "achieved": round(tflops, 3), "peak": round(alu_peak, 3), "unit": "TFLOP/s",
                 "frac": round(tflops / alu_peak, 4), "traffic": traffic,
                 "peak_source": "FP32 FMA unit count: 152 SMs x 128 lanes x 2 flops x 2070 MHz",
-                "kernel": "k_colstep<4,16,*>", "algorithmic_flops_per_launch": flops,
-                "algorithmic_bytes_per_launch": int(alg_bytes), "avg_launch_ms": round(avg_ms, 5),
+                "kernel": "k_colstep<float>", "algorithmic_flops_per_step": flops,
+                "algorithmic_bytes_per_step": int(alg_bytes), "avg_step_ms": round(avg_ms, 5),
                 "hbm_gbs": round(gbs, 1), "hbm_frac": round(gbs / hbm_peak, 4),
                 "hbm_peak": hbm_peak, "hbm_peak_source": f"{hbm_src} copy bandwidth"}
     # ---- the plain FP64 GPU form on the same operator (time-to-solution)
@@ -543,8 +543,8 @@ def run_powers(args, rank: int, world: int, local: int):
     # coefficients included, so a lower bound on the kernel's rate)
     tflops = 2.0 * 64.0 * triples * (n_terms - 2) / (t_ms / args.steps / 1e3) / 1e12
     if prec == cg.F64X:
-        # the same step with FP64 (DFMA) products, timed here, and the distance
-        # between the two results
+        # the same step in FP64 mode, timed here, and the distance between the two
+        # results
         torch.cuda.synchronize()
         d0, d1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         d0.record()
@@ -555,29 +555,29 @@ def run_powers(args, rank: int, world: int, local: int):
         rel = max(float(torch.linalg.norm(a - b) / torch.linalg.norm(b)) for a, b in zip(out["acc"], o64["acc"]))
         alu_peak = SMS * FP32_LANES * 2 * MAX_SM_MHZ * 1e6 / 1e12
         roof = {"bound": "alu", "achieved": round(tflops, 4), "peak": round(alu_peak, 3), "unit": "TFLOP/s",
-                "frac": round(tflops / alu_peak, 4), "traffic": None, "kernel": "k_step<dfl,2,8>",
-                "peak_source": "FP32 FMA unit count: 152 SMs x 128 lanes x 2 flops x 2070 MHz (the pipe the "
-                               "double-float products run on; achieved counts FP64-accurate flops)",
+                "frac": round(tflops / alu_peak, 4), "traffic": None, "kernel": "k_colstep<double>",
+                "peak_source": "FP32 FMA unit count: 152 SMs x 128 lanes x 2 flops x 2070 MHz (for scale: the "
+                               "products are f16 tensor-core digits; achieved counts FP64-accurate flops)",
                 "vs_fp64_unit_peak": round(tflops / FP64_NOMINAL_TFLOPS, 3)}
-        vs_dfma = {"fp64_dfma_step_ms": round(ms64, 2), "f64x_step_ms": round(t_ms / args.steps, 2),
-                   "speedup": round(ms64 / (t_ms / args.steps), 3), "max_relF_vs_fp64": rel}
+        vs_f64 = {"f64_step_ms": round(ms64, 2), "f64x_step_ms": round(t_ms / args.steps, 2),
+                  "speedup": round(ms64 / (t_ms / args.steps), 3), "max_relF_vs_fp64": rel}
     else:
         roof = {"bound": "alu", "achieved": round(tflops, 4), "peak": FP64_NOMINAL_TFLOPS, "unit": "TFLOP/s",
                 "frac": round(tflops / FP64_NOMINAL_TFLOPS, 4), "traffic": None,
-                "kernel": "k_step<double,2,8>",
+                "kernel": "k_colstep<double>",
                 "peak_source": "FP64 unit count: 304 DFMA lanes per cycle x 2 flops x 2070 MHz"}
-        vs_dfma = None
+        vs_f64 = None
     res = {
         "metric": METRIC, "value": round(value, 4), "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": round(t_ms / args.steps, 2), "higher_is_better": True,
-        "scaling": "weak", "vs_baseline": None, "dtype": "f64" if prec == cg.F64 else "f32x2 (double-float)",
+        "scaling": "weak", "vs_baseline": None, "dtype": "f64" if prec == cg.F64 else "f64x (FP64-accurate)",
         "data": "synthetic",
         "config": {"workload": args.workload, "atoms_per_gpu": cfg["n_atoms"], "rows": 4 * cfg["n_atoms"],
                    "r_c": cfg["r_c"], "r_buf": cfg["r_buf"], "exponents": list(cfg["exponents"]), "n_terms": n_terms,
                    "fit_tol": cfg["tol"], "blocks_P_H": pb.P_H.nnzb, "blocks_P_out": pb.P_out.nnzb,
                    "triples": triples, "l2": "inputs larger than L2 (no flush)"},
         "roofline": roof,
-        "vs_fp64_dfma": vs_dfma,
+        "vs_f64": vs_f64,
         "e2e": None if args.e2e_steps == 0 else {
             "value": round(job_throughput(args.e2e_steps, world, te_ms), 4), "unit": UNIT,
             "h2d_bytes_per_step": int(h_S.numel() * 8), "d2h_bytes_per_step": int(sum(h.numel() for h in h_out) * 8)},
@@ -672,7 +672,7 @@ def run_batched(args, rank: int, world: int, local: int):
                    "blocks_P_out": bp.P_out.nnzb, "blocks_P_H": bp.P_H.nnzb, "tiles": out["tiles"],
                    "graphs": "expansions, post-processing and traces captured and replayed; bisections eager", "l2": "inputs larger than L2 (no flush)"},
         "roofline": {"bound": "alu", "achieved": round(tflops, 3), "peak": round(alu_peak, 3), "unit": "TFLOP/s",
-                     "frac": round(tflops / alu_peak, 4), "traffic": None, "kernel": "k_resident (batched)",
+                     "frac": round(tflops / alu_peak, 4), "traffic": None, "kernel": "k_colstep (batched), k_resident for short rows",
                      "peak_source": "FP32 FMA: 152 SMs x 128 lanes x 2 x 2070 MHz"},
         "pass_ms": round(statistics.mean(passes), 1),
         "e2e": {"value": round(e2e_value, 4), "unit": UNIT, "h2d_bytes_per_step": int(h_H.numel() * 8),

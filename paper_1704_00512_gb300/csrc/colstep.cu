@@ -33,11 +33,12 @@
 // Fermi 3.5e-8 -> 2.9e-8, powers 4.7e-7 -> 2.5e-7; FP64-accurate 4.2e-14 -> 5.3e-16.
 // Measured (GB300): one step at 1,500 atoms, r_c 10, r_out 14 bohr, three
 // accumulators: FP64 9.2 -> 1.3 ms, FP64-accurate (before: double-floats) at 1,000
-// atoms, 8 / 12 bohr: 2.3 -> 0.35 ms; FP32 at 10,000 atoms 3.47 -> 2.7 ms, at 1,000
-// atoms, 8 / 12 bohr: 0.237 -> 0.131 ms, at 3,000 atoms with four functions 1.12 -> 0.88.  ncu: L1 access cycles 71 % (FP64) and
-// 47 % (FP32), ALU (digit unpacking) 50 %, tensor pipe 43 % and 36 %, issue 45-55 %:
-// an operator block of 64 or 128 bytes is used for one row group and panel only, and
-// an L1 load costs a cycle per line that the lanes it serves together touch.
+// atoms, 8 / 12 bohr: 2.3 -> 0.35 ms; FP32 at 10,000 atoms 3.47 -> 2.65 ms, at 1,000
+// atoms, 8 / 12 bohr: 0.237 -> 0.128 ms, at 3,000 atoms with four functions 1.12 ->
+// 0.87 ms.  ncu: L1 access cycles 65 % (FP64) and 58 % (FP32), ALU (digit unpacking) 44 %
+// and 50 %, tensor pipe 48 % and 37 %: an operator block of 64 or 128 bytes is used for
+// one row group and panel only, and an L1 load costs a cycle per line that the lanes it
+// serves together touch.
 // Tried without gain: f16 operator digits in memory (96 bytes: 3.7 instead of 2.9 ms
 // at 10,000 atoms), 12 warps (10 % slower), lanes over two blocks per access (L1
 // cycles -35 %, instructions +30 %, 15 % slower).
