@@ -255,9 +255,10 @@ static int plan_create_impl(const cheb_bsr *P_out, int32_t precision, int32_t ti
                 for (int64_t p = rp[j]; p < rp[j + 1]; ++p) add += stamp[ci[p]] != (int32_t)panel;
                 if (ncols > 0 && cnt + add > plan->ucap) break;
                 if (cnt + add > plan->ucap) {
+                    const int32_t ucap = plan->ucap;
                     delete plan;
                     return fail(CHEB_ERR_NOSPACE, "column %lld has %d rows, shared-memory panel holds %d",
-                                (long long)j, add, plan->ucap);
+                                (long long)j, add, ucap);
                 }
                 for (int64_t p = rp[j]; p < rp[j + 1]; ++p) stamp[ci[p]] = (int32_t)panel;
                 cnt += add;
