@@ -487,7 +487,7 @@ extern "C" int cheb_coeffs(const cheb_func *funcs, int32_t n_f, double emin, dou
     FuncArr F{};
     for (int f = 0; f < n_f; ++f) F.f[f] = funcs[f];
     const int64_t total = cand_total(cand);
-    Carve cv(ws, ws_bytes);
+    Carve cv = carve_aligned(ws, ws_bytes);
     double *fv = cv.take<double>((size_t)n_f * total), *cvv = cv.take<double>((size_t)n_f * total);
     double2 *Y = cv.take<double2>((size_t)n_f * total);
     double *tab = cv.take<double>(4 * (size_t)total);

@@ -769,7 +769,7 @@ size_t col_expand_ws(const cheb_plan *plan, int64_t nnzL) {
 template <typename T>
 static int col_expand_t(const cheb_plan *plan, const cheb_bsr *Mt, const ColExpand &x, void *ws, size_t ws_bytes,
                         cudaStream_t s) {
-    Carve cv(ws, ws_bytes);
+    Carve cv = carve_aligned(ws, ws_bytes);
     const ColLists &c = plan->col;
     ColArgs a{};
     for (int i = 0; i < 2; ++i) a.T[i] = cv.take<T>(plan->nnzb * BB);

@@ -57,6 +57,14 @@ struct Carve {
     bool fits() const { return off <= cap; }
 };
 
+// The same from the first 256-byte boundary on, for kernels with loads of 16 or 32
+// bytes: callers may pass workspaces at any address, and the sizes they are told hold
+// 256 bytes to spare.
+inline Carve carve_aligned(void *b, size_t c) {
+    const size_t skip = (256 - reinterpret_cast<uintptr_t>(b) % 256) % 256;
+    return Carve(static_cast<char *>(b) + skip, c > skip ? c - skip : 0);
+}
+
 // ---------------------------------------------------------------------------
 // device helpers
 

@@ -338,9 +338,10 @@ extern "C" int cheb_bounds(const cheb_bsr *M, int32_t k, const double *v0, doubl
     CHEB_TRY(cheb_bounds_workspace_size(M->nbr, k, &need));
     if (!ws || ws_bytes < need) return fail(CHEB_ERR_NOSPACE, "cheb_bounds: workspace %zu < %zu", ws_bytes, need);
     const int64_t n = M->nbr * BS;
-    Carve cv(ws, ws_bytes);
+    Carve cv = carve_aligned(ws, ws_bytes);
     double *vm = cv.take<double>(n), *v = cv.take<double>(n), *w = cv.take<double>(n);
     LzState *st = cv.take<LzState>(1);
+    if (!cv.fits()) return fail(CHEB_ERR_NOSPACE, "cheb_bounds: workspace %zu too small", ws_bytes);
     cudaStream_t s = as_stream(stream);
     CHEB_CUDA(cudaMemsetAsync(st, 0, sizeof(LzState), s));
     const int kk = k;
