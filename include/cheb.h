@@ -181,11 +181,13 @@ int cheb_plan_attach_operator(cheb_plan *plan, const cheb_bsr *L, size_t *op_ws_
  * P_out block (2 bytes each).  After cheb_plan_bind_operator, expansions with that
  * operator run this kernel: cheb_expand_stepwise wherever the lists were built,
  * cheb_expand and cheb_expand_batched when the operator's rows are long as above.
- * Its products are sums of integer digits on the tensor cores, exact but for a grid
- * of 2^-29 (FP32) or 2^-59 (FP64) of each panel column's and operator row's largest
- * element, in place of FP32 or FP64 rounding; columns or operators with elements
- * that are not finite or beyond the grid's exponents are multiplied in plain FP32 or
- * FP64.  Results agree with the other kernels to rounding, and are bitwise
+ * Its products are sums of integer digits on the tensor cores: an element counts to
+ * 2^-30 (FP32) or 2^-60 (FP64) of the largest of its column of T_k or of its scalar row
+ * of the operator, in place of FP32 or FP64 rounding, so a product of K terms is off by
+ * at most K u max|row| max|column|, u = 2^-24 or 2^-53, and small elements of a row or
+ * column lose bits that floats of their own would keep; columns or operators with
+ * elements that are not finite or beyond the grid's exponents are multiplied in plain
+ * FP32 or FP64.  Results agree with the other kernels to rounding, and are bitwise
  * reproducible run to run.  CHEB_F64X expansions that run it hold T_k in FP64.  The
  * lists are not built (and the ranking kernels run) when one column's rows do not
  * fit a panel or the operator has 2^22 - 1 blocks or more.  cheb_plan_col_info

@@ -13,7 +13,7 @@
 // they cost 64 instructions a block and panel column (FP64 at 1/64 of the FP32
 // rate; FP32 bound by issue and by shared-memory reads, 240 instructions per
 // 16 entries).  Here they are f16 tensor-core products of *digits*: within a
-// panel column (and within an operator block row) every value is written on
+// panel column (and within a scalar row of the operator) every value is written on
 // one power-of-two grid as a sum of small integers times powers of two, three
 // digits (30 bits) for FP32 and six (60 bits) for FP64.  Integers up to 2048
 // are exact in f16, and the products of one mma are small enough for the FP32
@@ -89,7 +89,7 @@ struct ColArgs {
     const double *Lv;
     int64_t nnzL;
     const uint4 *opd;       // operator digits (one zero block appended)
-    const int32_t *opexp;   // grid exponent of each operator block row
+    const int32_t *opexp;   // grid exponents of the operator's scalar rows
     const int32_t *opflag;  // nonzero: an operator element beyond the digits
     void *T[2];             // T_k in T[k & 1] (column order)
     int32_t t0, t1;         // terms formed by this launch: t0 .. t1 - 1 (t0 = 2: also terms 0 and 1)
@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(COL_NW * 32, 1) k_colstep(const __grid_constan
     uint4 *X = reinterpret_cast<uint4 *>(smem + lay.off_x);
     uint32_t *X2 = reinterpret_cast<uint32_t *>(smem + lay.off_x + 256);  // FP32: the third digits, behind the others
     int32_t *opos = reinterpret_cast<int32_t *>(smem + lay.off_pos);
-    int32_t *rexp = reinterpret_cast<int32_t *>(smem + lay.off_rexp);
+    int8_t *rexp = reinterpret_cast<int8_t *>(smem + lay.off_rexp);  // of the union rows' scalar rows
     uint2 *srow = reinterpret_cast<uint2 *>(smem + lay.off_rows);
     double *red = reinterpret_cast<double *>(smem + lay.off_red);
     const double *coef = a.coef ? a.coef + (a.coef_off ? a.coef_off[sys] : 0) : nullptr;
@@ -233,7 +233,8 @@ __global__ void __launch_bounds__(COL_NW * 32, 1) k_colstep(const __grid_constan
     for (int b = cb0 + tid; b < cb1; b += NTH) {
         const int q = col_of(b), s = a.slot[b], K = a.ci[b];
         opos[s * P + q] = (int32_t)b;
-        rexp[s] = a.opexp[K];
+        const int4 e = *reinterpret_cast<const int4 *>(a.opexp + 4 * K);
+        *reinterpret_cast<char4 *>(rexp + 4 * s) = make_char4(e.x, e.y, e.z, e.w);
         if (K == j0 + q) s_dslot[q] = s;
     }
 
@@ -573,7 +574,7 @@ uint32_t B[NT][3][2];
 #pragma unroll
                 for (int hh = 0; hh < 2; ++hh) {
                     if (sl2[hh] == (int)SM) continue;
-                    const int er = rexp[sl2[hh]];
+                    const int er = rexp[4 * sl2[hh] + (g & 3)];
                     const float rf = F64 || slow ? 1.f : pow2(er - 18, 0.f);  // (two exact factors)
                     // T_{term-2}, G and, in group steps, T_{term-1}, of the half's positions
                     int pos[NT];
@@ -761,7 +762,7 @@ size_t col_expand_ws(const cheb_plan *plan, int64_t nnzL) {
     size_t b = 2 * align_up(plan->nnzb * BB * esz);
     b += align_up((size_t)(nnzL + 1) * (wide ? 128 : 64));
     if (!wide) b += (MAX_F + 1) * align_up(plan->nnzb * BB * 8);  // accumulators and G as float pairs
-    b += align_up(plan->nbr * 4) + align_up(64);
+    b += align_up(plan->nbr * 16) + align_up(64);
     b += align_up((size_t)plan->col.n_panels * (COL_STEPS + 2) * 2 * sizeof(double));
     return b + 256;
 }
@@ -778,12 +779,13 @@ static int col_expand_t(const cheb_plan *plan, const cheb_bsr *Mt, const ColExpa
         for (int f = 0; f < MAX_F; ++f) a.accp[f] = cv.take<float>(plan->nnzb * BB * 2);
         a.Gp = cv.take<float>(plan->nnzb * BB * 2);
     }
-    int32_t *opexp = cv.take<int32_t>(plan->nbr), *opflag = cv.take<int32_t>(16);
+    int32_t *opexp = cv.take<int32_t>(4 * plan->nbr), *opflag = cv.take<int32_t>(16);
     a.part = cv.take<double>((size_t)c.n_panels * (COL_STEPS + 2) * 2);
     if (!cv.fits()) return fail(CHEB_ERR_NOSPACE, "cheb_expand: workspace %zu too small", ws_bytes);
     CHEB_CUDA(cudaMemsetAsync(opflag, 0, 64, s));
     k_opdig<T><<<(unsigned)((plan->nbr + 1 + 7) / 8), 256, 0, s>>>(Mt->row_ptr, (const double *)Mt->vals, plan->nbr,
-                                                                  Mt->nnzb, x.round_bf16, opd, opexp, opflag);
+                                                                  Mt->nnzb, x.round_bf16, Dig<T>::OP_MIN, Dig<T>::OP_MAX,
+                                                                  opd, opexp, opflag);
     CHEB_TRY(check_launch("k_opdig"));
     a.panels = c.d_panels;
     a.order = c.d_order;

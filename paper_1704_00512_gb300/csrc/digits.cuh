@@ -10,16 +10,17 @@
 namespace cheb {
 
 // Tiles of an element type: NT n8-tiles (2 block columns each) per panel, and the
-// grid exponents of T and of the operator.
+// grid exponents that the recursion takes: of T's columns, and of the operator's
+// scalar rows (a byte each).
 template <typename T>
 struct Dig;
 template <>
 struct Dig<float> {
-    static constexpr int NT = 2, EX_MIN = -60, EX_MAX = 90, OP_MIN = -30, OP_MAX = 30;
+    static constexpr int NT = 2, EX_MIN = -60, EX_MAX = 90, OP_MIN = -80, OP_MAX = 30;
 };
 template <>
 struct Dig<double> {
-    static constexpr int NT = 1, EX_MIN = -400, EX_MAX = 400, OP_MIN = -400, OP_MAX = 400;
+    static constexpr int NT = 1, EX_MIN = -400, EX_MAX = 400, OP_MIN = -127, OP_MAX = 127;
 };
 
 __device__ __forceinline__ float bf16r(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
@@ -141,14 +142,15 @@ __device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], 
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]), "f"(c[0]), "f"(c[1]), "f"(c[2]), "f"(c[3]));
 }
 
-// The operator's digits: one warp per block row; block nnzL is the zero block
-// that pads the lists.  A block holds, per scalar row r, the words of its pairs
-// (H[r][0], H[r][1]) and (H[r][2], H[r][3]): 16 bytes in FP32, 32 in FP64.
+// The operator's digits, each scalar row on the grid of its largest element (exponent
+// opexp[4 block row + row], within [lo, hi]): one warp per block row; block nnzL is the
+// zero block that pads the lists.  A block holds, per scalar row r, the words of its
+// pairs (H[r][0], H[r][1]) and (H[r][2], H[r][3]): 16 bytes in FP32, 32 in FP64.
 // (Unpacked f16 digits would save the unpacking and take half as much again from
 // L2 and, counted in the 128-byte lines that a load touches, from L1.)
 template <typename T>
-__global__ void k_opdig(const int64_t *rp, const double *v, int64_t nbr, int64_t nnzL, int round_bf16, uint4 *opd,
-                        int32_t *opexp, int32_t *opflag) {
+__global__ void k_opdig(const int64_t *rp, const double *v, int64_t nbr, int64_t nnzL, int round_bf16, int lo, int hi,
+                        uint4 *opd, int32_t *opexp, int32_t *opflag) {
     constexpr bool F64 = sizeof(T) == 8;
     const int64_t I = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
@@ -159,19 +161,21 @@ __global__ void k_opdig(const int64_t *rp, const double *v, int64_t nbr, int64_t
     }
     if (I > nbr) return;
     const int64_t e0 = rp[I] * BB, e1 = rp[I + 1] * BB;
-    uint32_t m = 0;
+    uint32_t m = 0;  // of scalar row (lane / 4) % 4, whose elements the lane reads
     for (int64_t i = e0 + lane; i < e1; i += 32) {
         if constexpr (F64) m = max(m, mag_bits(v[i]));
         else m = max(m, mag_bits(round_bf16 ? bf16r((float)v[i]) : (float)v[i]));
     }
-    m = __reduce_max_sync(0xffffffffu, m);
+#pragma unroll
+    for (int o = 1; o < 32; o = o == 2 ? 16 : 2 * o) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
     int e;
-    if (!grid_exp<T>(m, Dig<T>::OP_MIN, Dig<T>::OP_MAX, e)) {
+    if (__any_sync(0xffffffffu, !grid_exp<T>(m, lo, hi, e))) {
         if (lane == 0) atomicOr(opflag, 1);
         return;
     }
-    if (lane == 0) opexp[I] = e;
-    for (int64_t i = e0 / 4 + lane; i < e1 / 4; i += 32) {  // scalar rows of the blocks
+    if (lane < 16 && (lane & 3) == 0) opexp[4 * I + (lane >> 2)] = e;
+    e = __shfl_sync(0xffffffffu, e, 4 * (lane & 3));
+    for (int64_t i = e0 / 4 + lane; i < e1 / 4; i += 32) {  // scalar rows (lane % 4) of the blocks
         const double2 x = make_double2(v[4 * i], v[4 * i + 1]), y = make_double2(v[4 * i + 2], v[4 * i + 3]);
         if constexpr (F64) {
             uint32_t w[4];

@@ -29,6 +29,8 @@
 namespace cheb {
 
 constexpr int PR_NW = 16;
+// Grid exponents that the products take, of either operand.
+constexpr int PR_EX = 400;
 // Quads whose exact digit sums (at most 2^24 a quad) stay below 2^31.
 constexpr int PR_CHUNK = 126;
 
@@ -96,7 +98,6 @@ __device__ __noinline__ void prod_plain(const ProdArgs &a, const int32_t *opos, 
 }
 
 __global__ void __launch_bounds__(PR_NW * 32, 1) k_product(const __grid_constant__ ProdArgs a) {
-    using Dg = Dig<double>;
     constexpr int NTH = PR_NW * 32;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ uint32_t s_max[8];
@@ -161,7 +162,7 @@ __global__ void __launch_bounds__(PR_NW * 32, 1) k_product(const __grid_constant
         __syncthreads();
         if (tid < 8) {
             int e;
-            if (!grid_exp<double>(s_max[tid], Dg::EX_MIN, Dg::EX_MAX, e)) s_slow = 1;
+            if (!grid_exp<double>(s_max[tid], -PR_EX, PR_EX, e)) s_slow = 1;
             s_e[tid] = e;
         }
         __syncthreads();
@@ -319,7 +320,7 @@ __global__ void __launch_bounds__(PR_NW * 32, 1) k_product(const __grid_constant
                 double y[2];
 #pragma unroll
                 for (int c = 0; c < 2; ++c)
-                    y[c] = slow ? val[2 * h + c] : val[2 * h + c] * pow2(a.opexp[ulist[u]] + s_e[2 * t + c] - 48, 0.0);
+                    y[c] = slow ? val[2 * h + c] : val[2 * h + c] * pow2(a.opexp[4 * ulist[u] + (g & 3)] + s_e[2 * t + c] - 48, 0.0);
                 const int64_t at = (int64_t)p * BB + 4 * (g & 3) + 2 * (t & 1);
                 double2 v = make_double2(a.alpha * y[0], a.alpha * y[1]);
                 if (a.D) {
@@ -335,7 +336,7 @@ __global__ void __launch_bounds__(PR_NW * 32, 1) k_product(const __grid_constant
 size_t prod_bytes(const cheb_plan *plan, int64_t nnzL) {
     if (plan->precision != CHEB_F64 || !plan->col.built || plan->nbr > 65535 || plan->max_row > prod_cap(plan)) return 0;
     const int64_t n = std::max(nnzL, plan->nnzb);
-    return align_up((size_t)(n + 1) * 128) + align_up(plan->nbr * 4) + align_up(64) + align_up(plan->n_panels * 8);
+    return align_up((size_t)(n + 1) * 128) + align_up(plan->nbr * 16) + align_up(64) + align_up(plan->n_panels * 8);
 }
 
 // The panels go to the device in the order of their launch: by the square of their
@@ -379,7 +380,7 @@ int prod_run(const cheb_plan *plan, const cheb_bsr *L, const double *R, double a
     Carve cv(plan->prod_ws, prod_bytes(plan, plan->col.nnzL));
     ProdArgs a{};
     uint4 *opd = cv.take<uint4>((n + 1) * 8);
-    int32_t *opexp = cv.take<int32_t>(plan->nbr), *flag = cv.take<int32_t>(16);
+    int32_t *opexp = cv.take<int32_t>(4 * plan->nbr), *flag = cv.take<int32_t>(16);
     a.panels = cv.take<int32_t>(2 * plan->n_panels);
     a.rp = plan->rp;
     a.ci = plan->ci;
@@ -404,7 +405,8 @@ int prod_run(const cheb_plan *plan, const cheb_bsr *L, const double *R, double a
     if (!plan->prod_done) CHEB_CUDA(cudaEventCreateWithFlags(&plan->prod_done, cudaEventDisableTiming));
     else CHEB_CUDA(cudaStreamWaitEvent(s, plan->prod_done, 0));
     CHEB_CUDA(cudaMemsetAsync(flag, 0, 64, s));
-    k_opdig<double><<<(unsigned)((plan->nbr + 1 + 7) / 8), 256, 0, s>>>(L->row_ptr, a.Lv, plan->nbr, L->nnzb, 0, opd, opexp, flag);
+    k_opdig<double><<<(unsigned)((plan->nbr + 1 + 7) / 8), 256, 0, s>>>(L->row_ptr, a.Lv, plan->nbr, L->nnzb, 0, -PR_EX, PR_EX, opd,
+                                                                      opexp, flag);
     CHEB_TRY(check_launch("k_opdig"));
     CHEB_CUDA(cudaFuncSetAttribute(k_product, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     k_product<<<(unsigned)plan->n_panels, PR_NW * 32, smem, s>>>(a);
