@@ -380,11 +380,17 @@ int cheb_expand_batched(const cheb_plan *plan, const cheb_bsr *Mt, int32_t max_t
  *
  * With the column kernel's lists bound (long operator rows) and L on the attached
  * operator's pattern or on the plan's own (the same row_ptr / col_idx pointers), the
- * product runs as that kernel's digit products, exact but for a grid of 2^-59 of each
- * operator row's and each column's largest element.  It needs rows of P_out that fit
- * shared memory (about 560 blocks), at most 65,535 block rows and 16-byte aligned R, D
- * and C; otherwise, and while the stream is captured, it runs on the FP64 pipe, with
- * results equal to rounding.  L's digits are kept in the operator workspace (128 bytes
+ * product runs as that kernel's digit products.  With K products per element, u = 2^-53,
+ * R_i the largest element of scalar row i of L and C_j that of column j of R, an element
+ * of L R is off by at most K u R_i C_j, and those of a column by at most 4 K u R_i s_j,
+ * s_j the largest over i of (sum_k |L_ik R_kj|) / R_i -- not by K u of the sum of its own
+ * |products|, which a small element beside large ones in its column would need.  Where
+ * the scales of rows and columns cancel, so that s_j is below 2^-6 C_j, the panel of
+ * column j is multiplied in plain FP64, as it is for elements that are not finite or
+ * beyond 2^+-400.  The digits need rows of P_out that fit shared memory (about 560
+ * blocks), at most 65,535 block rows and 16-byte aligned R, D and C; otherwise, and while
+ * the stream is captured, the product runs on the FP64 pipe.  The two agree within their
+ * errors, not to the bit.  L's digits are kept in the operator workspace (128 bytes
  * per block of the larger pattern, part of op_ws_bytes); calls with one plan on several
  * streams or threads are put in order behind each other on the device.
  */

@@ -76,25 +76,62 @@ static int prod_cap(const cheb_plan *plan) {
     return cap;
 }
 
-// The products of one group in plain FP64 (an element beyond the digits' grids).
+// The digits resolve a column when, for one of its rows, the sum of |products| is at
+// least 2^-PR_RESOLVE of the row's and the column's grids multiplied: the grids' error is
+// then at most K u of that sum, like that of FP64 sums.  Where none is -- the large
+// elements of the rows meet the small ones of the column, so that the scales cancel --
+// the panel is done once more in plain FP64.  A result of that size shows it for free; a
+// panel with a column of smaller ones gets its sums of |leading digits| formed (one mma
+// instead of 26; sums that cancel, as in the product of a density matrix with a column
+// that it nearly annihilates, are no reason to take FP64: 0.5 ms a panel at 800 rows).
+constexpr int PR_RESOLVE = 6;
+
+// The products of one group in plain FP64 (an element beyond the digits' grids, or a
+// column that they do not resolve).
 __device__ __noinline__ void prod_plain(const ProdArgs &a, const int32_t *opos, const uint16_t *tab, int ts, int nu,
                                         const int64_t *base, int lane, double *out) {
     const int g = lane >> 2, t = lane & 3;
     for (int i = 0; i < 4; ++i) out[i] = 0.0;
     for (int s = 0; s < nu; ++s) {
+        const uint32_t id[2] = {tab[(g >> 2) * ts + s], tab[((g >> 2) + 2) * ts + s]};
         const int p = opos[2 * s + (t >> 1)];
-        if (p < 0) continue;
+        if ((id[0] & id[1]) == 0xffffu || p < 0) continue;
+        double2 x[4];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) x[m] = __ldg(reinterpret_cast<const double2 *>(a.R + (int64_t)p * BB + 4 * m + 2 * (t & 1)));
+#pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const uint16_t id = tab[((g >> 2) + 2 * h) * ts + s];
-            if (id == 0xffffu) continue;
-            const double *hv = a.Lv + (base[h] + id) * BB + 4 * (g & 3);
-            const double *x = a.R + (int64_t)p * BB + 2 * (t & 1);
+            if (id[h] == 0xffffu) continue;
+            const double *hv = a.Lv + (base[h] + id[h]) * BB + 4 * (g & 3);
+#pragma unroll
             for (int m = 0; m < 4; ++m) {
-                out[2 * h] = fma(hv[m], x[4 * m], out[2 * h]);
-                out[2 * h + 1] = fma(hv[m], x[4 * m + 1], out[2 * h + 1]);
+                const double w = __ldg(hv + m);
+                out[2 * h] = fma(w, x[m].x, out[2 * h]);
+                out[2 * h + 1] = fma(w, x[m].y, out[2 * h + 1]);
             }
         }
     }
+}
+
+// The sums of |leading digits| of one group, where the mma has them (in units of 2^-18 of
+// the grids multiplied).
+__device__ __noinline__ void prod_scale(const uint4 *ob, const uint4 *X, const uint16_t *tl, int ts, const unsigned char *ql,
+                                        int cnt, uint32_t base0, uint32_t base1, uint32_t none, int g, int t, float *out) {
+    float z[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int k = 0; k < cnt; ++k) {
+        const int q = ql[k];
+        const uint32_t i0 = tl[4 * q], i1 = tl[2 * ts + 4 * q];
+        uint32_t w[2][8];
+        ld_row(w[0], ob, i0 == 0xffffu ? none : base0 + i0);
+        ld_row(w[1], ob, i1 == 0xffffu ? none : base1 + i1);
+        const uint4 *xs = X + (4 * q + t) * 16 + (g ^ (2 * t));
+        constexpr uint32_t D0 = 0x03ff03ffu, ABS = 0x7fff7fffu;
+        const uint32_t A[4] = {f16_digits(w[0][0] & D0) & ABS, f16_digits(w[1][0] & D0) & ABS,
+                               f16_digits(w[0][4] & D0) & ABS, f16_digits(w[1][4] & D0) & ABS};
+        const uint32_t B[2] = {f16_digits(xs[0].x & D0) & ABS, f16_digits(xs[8].x & D0) & ABS};
+        mma16816(z, A, B, z);
+    }
+    for (int i = 0; i < 4; ++i) out[i] = z[i];
 }
 
 __global__ void __launch_bounds__(PR_NW * 32, 1) k_product(const __grid_constant__ ProdArgs a) {
@@ -102,7 +139,7 @@ __global__ void __launch_bounds__(PR_NW * 32, 1) k_product(const __grid_constant
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ uint32_t s_max[8];
     __shared__ int s_e[8];
-    __shared__ int s_slow, wsum[32];
+    __shared__ int s_slow, s_big[8], wsum[32];  // s_big: columns that the digits resolve
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, cap = a.cap, ts = cap + 4;
     const ProdLayout lay = prod_layout(cap);
     int32_t *ulist = reinterpret_cast<int32_t *>(smem), *opos = reinterpret_cast<int32_t *>(smem + lay.off_pos);
@@ -164,10 +201,12 @@ __global__ void __launch_bounds__(PR_NW * 32, 1) k_product(const __grid_constant
             int e;
             if (!grid_exp<double>(s_max[tid], -PR_EX, PR_EX, e)) s_slow = 1;
             s_e[tid] = e;
+            s_big[tid] = 0;
         }
         __syncthreads();
-        const bool slow = s_slow != 0;
-        if (!slow) {
+        enum { DIGITS, SCALE, PLAIN };
+        int mode = s_slow != 0 ? PLAIN : DIGITS;
+        if (mode == DIGITS) {
             for (int i = tid; i < 2 * nu; i += NTH) {
                 const int p = opos[i], s = i >> 1, q = i & 1, sw = 2 * (s & 3);
                 if (p < 0) continue;
@@ -193,142 +232,166 @@ __global__ void __launch_bounds__(PR_NW * 32, 1) k_product(const __grid_constant
         // 3. the warp's groups of four union rows
         const int g = lane >> 2, t = lane & 3;
         const uint4 *ob = a.opd + (g & 3) * 2;
-        for (int gi = warp; 4 * gi < nu; gi += PR_NW) {
-            __syncwarp();
-            for (int i = lane; i < ts; i += 32) reinterpret_cast<uint64_t *>(tab)[i] = ~0ull;
-            __syncwarp();
-            for (int r = 0; r < 4 && 4 * gi + r < nu; ++r) {
-                const int64_t b = a.Lrp[ulist[4 * gi + r]];
-                const int len = (int)(a.Lrp[ulist[4 * gi + r] + 1] - b);
-                for (int i = lane; i < len; i += 32) {
-                    const int s = rank_of(bits, __ldg(a.Lci + b + i));
-                    if (s >= 0) tab[r * ts + s] = (uint16_t)i;
-                }
-            }
-            __syncwarp();
-            int64_t base[2];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int u = 4 * gi + (g >> 2) + 2 * h;
-                base[h] = u < nu ? a.Lrp[ulist[u]] : 0;
-            }
-            double val[4] = {0.0, 0.0, 0.0, 0.0};
-            if (slow) {
-                prod_plain(a, opos, tab, ts, nu, base, lane, val);
-            } else {
-                int cnt = 0;
-                for (int b = 0; b < nu4 / 4; b += 32) {
-                    const int q = b + lane;
-                    bool any = false;
-                    if (q < nu4 / 4) {
-                        uint64_t all = ~0ull;
-#pragma unroll
-                        for (int r = 0; r < 4; ++r) all &= *reinterpret_cast<const uint64_t *>(tab + r * ts + 4 * q);
-                        any = all != ~0ull;
-                    }
-                    const unsigned m = __ballot_sync(0xffffffffu, any);
-                    if (any) ql[cnt + __popc(m & lt)] = (unsigned char)q;
-                    cnt += __popc(m);
-                }
-                // quads go in pairs: an empty one (beyond the union) fills up the last
-                if (lane == 0) ql[cnt] = (unsigned char)(nu4 / 4);
-                cnt = (cnt + 1) & ~1;
+        while (true) {
+            for (int gi = warp; 4 * gi < nu; gi += PR_NW) {
                 __syncwarp();
-                struct Op {
-                    uint32_t w[2][8];
-                };
-                const uint32_t base0 = (uint32_t)base[0], base1 = (uint32_t)base[1], none = (uint32_t)a.nnzL;
-                const uint16_t *tl = tab + (g >> 2) * ts + t;
-                auto load_h = [&](Op &o, int k) {
-                    const int q = ql[min(k, cnt - 1)];
-                    const uint32_t i0 = tl[4 * q], i1 = tl[2 * ts + 4 * q];
-                    ld_row(o.w[0], ob, i0 == 0xffffu ? none : base0 + i0);
-                    ld_row(o.w[1], ob, i1 == 0xffffu ? none : base1 + i1);
-                };
-                Op h[2];
-                if (cnt > 0) {
-                    load_h(h[0], 0);
-                    load_h(h[1], 1);
-                }
-                for (int k0 = 0; k0 < cnt; k0 += PR_CHUNK) {
-                    const int k1 = min(cnt, k0 + PR_CHUNK);
-                    float dl[2][4];
-                    int is[4][4];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        dl[0][i] = dl[1][i] = 0.f;
-#pragma unroll
-                        for (int s = 0; s < 4; ++s) is[s][i] = 0;
+                for (int i = lane; i < ts; i += 32) reinterpret_cast<uint64_t *>(tab)[i] = ~0ull;
+                __syncwarp();
+                for (int r = 0; r < 4 && 4 * gi + r < nu; ++r) {
+                    const int64_t b = a.Lrp[ulist[4 * gi + r]];
+                    const int len = (int)(a.Lrp[ulist[4 * gi + r] + 1] - b);
+                    for (int i = lane; i < len; i += 32) {
+                        const int s = rank_of(bits, __ldg(a.Lci + b + i));
+                        if (s >= 0) tab[r * ts + s] = (uint16_t)i;
                     }
+                }
+                __syncwarp();
+                int64_t base[2];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int u = 4 * gi + (g >> 2) + 2 * h;
+                    base[h] = u < nu ? a.Lrp[ulist[u]] : 0;
+                }
+                double val[4] = {0.0, 0.0, 0.0, 0.0};
+                if (mode == PLAIN) {
+                    prod_plain(a, opos, tab, ts, nu, base, lane, val);
+                } else {
+                    int cnt = 0;
+                    for (int b = 0; b < nu4 / 4; b += 32) {
+                        const int q = b + lane;
+                        bool any = false;
+                        if (q < nu4 / 4) {
+                            uint64_t all = ~0ull;
+#pragma unroll
+                            for (int r = 0; r < 4; ++r) all &= *reinterpret_cast<const uint64_t *>(tab + r * ts + 4 * q);
+                            any = all != ~0ull;
+                        }
+                        const unsigned m = __ballot_sync(0xffffffffu, any);
+                        if (any) ql[cnt + __popc(m & lt)] = (unsigned char)q;
+                        cnt += __popc(m);
+                    }
+                    // quads go in pairs: an empty one (beyond the union) fills up the last
+                    if (lane == 0) ql[cnt] = (unsigned char)(nu4 / 4);
+                    cnt = (cnt + 1) & ~1;
+                    __syncwarp();
+                    struct Op {
+                        uint32_t w[2][8];
+                    };
+                    const uint32_t base0 = (uint32_t)base[0], base1 = (uint32_t)base[1], none = (uint32_t)a.nnzL;
+                    const uint16_t *tl = tab + (g >> 2) * ts + t;
+                    auto load_h = [&](Op &o, int k) {
+                        const int q = ql[min(k, cnt - 1)];
+                        const uint32_t i0 = tl[4 * q], i1 = tl[2 * ts + 4 * q];
+                        ld_row(o.w[0], ob, i0 == 0xffffu ? none : base0 + i0);
+                        ld_row(o.w[1], ob, i1 == 0xffffu ? none : base1 + i1);
+                    };
+                    if (mode == SCALE) {
+                        float z[4];
+                        prod_scale(ob, X, tl, ts, ql, cnt, base0, base1, none, g, t, z);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const int u = 4 * gi + (g >> 2) + 2 * (i >> 1);
+                            if (u < nu && opos[2 * u + (t >> 1)] >= 0 && z[i] >= (float)(1 << (18 - PR_RESOLVE)))
+                                s_big[2 * t + (i & 1)] = 1;
+                        }
+                        continue;
+                    }
+                    Op h[2];
+                    if (cnt > 0) {
+                        load_h(h[0], 0);
+                        load_h(h[1], 1);
+                    }
+                    for (int k0 = 0; k0 < cnt; k0 += PR_CHUNK) {
+                        const int k1 = min(cnt, k0 + PR_CHUNK);
+                        float dl[2][4];
+                        int is[4][4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            dl[0][i] = dl[1][i] = 0.f;
+#pragma unroll
+                            for (int s = 0; s < 4; ++s) is[s][i] = 0;
+                        }
 #pragma unroll 1
-                    for (int k = k0; k < k1; k += 2) {
-                        float z[4][4];
+                        for (int k = k0; k < k1; k += 2) {
+                            float z[4][4];
 #pragma unroll
-                        for (int o = 0; o < 2; ++o) {
-                            const uint4 *xs = X + (4 * ql[k + o] + t) * 16 + (g ^ (2 * t));
-                            const uint4 x0 = xs[0], x1 = xs[8];
-                            const uint32_t w0[4] = {x0.x, x0.y, x0.z, x0.w}, w1[4] = {x1.x, x1.y, x1.z, x1.w};
-                            uint32_t B[6][2];
+                            for (int o = 0; o < 2; ++o) {
+                                const uint4 *xs = X + (4 * ql[k + o] + t) * 16 + (g ^ (2 * t));
+                                const uint4 x0 = xs[0], x1 = xs[8];
+                                const uint32_t w0[4] = {x0.x, x0.y, x0.z, x0.w}, w1[4] = {x1.x, x1.y, x1.z, x1.w};
+                                uint32_t B[6][2];
 #pragma unroll
-                            for (int i = 0; i < 6; ++i) {
-                                B[i][0] = packed_digit(w0, i);
-                                B[i][1] = packed_digit(w1, i);
+                                for (int i = 0; i < 6; ++i) {
+                                    B[i][0] = packed_digit(w0, i);
+                                    B[i][1] = packed_digit(w1, i);
+                                }
+                                const float zero[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                                for (int i = 0; i < 6; ++i) {
+                                    uint32_t A[4];
+#pragma unroll
+                                    for (int e = 0; e < 4; ++e) {  // (half e % 2, pair e / 2)
+                                        const uint32_t *hw = h[o].w[e & 1] + 2 * (e & 2);
+                                        const uint32_t pw[4] = {hw[0], hw[1], hw[2], hw[3]};
+                                        A[e] = packed_digit(pw, i);
+                                    }
+#pragma unroll
+                                    for (int s = i; s < 6; ++s) {
+                                        if (s >= 4) mma16816(dl[s & 1], A, B[s - i], dl[s & 1]);
+                                        else if (i == 0 && (o == 0 || s >= 2)) mma16816(z[s], A, B[s], zero);
+                                        else mma16816(z[s], A, B[s - i], z[s]);
+                                    }
+                                    // (the sums of s = 0, 1 stay exact over two quads)
+                                    if (i >= 1) {  // D_6 into D_5's accumulator: the panel digit times 2^-10
+                                        const uint32_t Bs[2] = {h2_fma(B[6 - i][0], 0x14001400u, 0u), h2_fma(B[6 - i][1], 0x14001400u, 0u)};
+                                        mma16816(dl[1], A, Bs, dl[1]);
+                                    }
+                                    if (i < 4 && (o == 1 || i >= 2)) {
+#pragma unroll
+                                        for (int e = 0; e < 4; ++e) is[i][e] += __float2int_rn(z[i][e]);
+                                    }
+                                }
+                                load_h(h[o], k + o + 2);
                             }
-                            const float zero[4] = {0.f, 0.f, 0.f, 0.f};
+                        }
 #pragma unroll
-                            for (int i = 0; i < 6; ++i) {
-                                uint32_t A[4];
-#pragma unroll
-                                for (int e = 0; e < 4; ++e) {  // (half e % 2, pair e / 2)
-                                    const uint32_t *hw = h[o].w[e & 1] + 2 * (e & 2);
-                                    const uint32_t pw[4] = {hw[0], hw[1], hw[2], hw[3]};
-                                    A[e] = packed_digit(pw, i);
-                                }
-#pragma unroll
-                                for (int s = i; s < 6; ++s) {
-                                    if (s >= 4) mma16816(dl[s & 1], A, B[s - i], dl[s & 1]);
-                                    else if (i == 0 && (o == 0 || s >= 2)) mma16816(z[s], A, B[s], zero);
-                                    else mma16816(z[s], A, B[s - i], z[s]);
-                                }
-                                // (the sums of s = 0, 1 stay exact over two quads)
-                                if (i >= 1) {  // D_6 into D_5's accumulator: the panel digit times 2^-10
-                                    const uint32_t Bs[2] = {h2_fma(B[6 - i][0], 0x14001400u, 0u), h2_fma(B[6 - i][1], 0x14001400u, 0u)};
-                                    mma16816(dl[1], A, Bs, dl[1]);
-                                }
-                                if (i < 4 && (o == 1 || i >= 2)) {
-#pragma unroll
-                                    for (int e = 0; e < 4; ++e) is[i][e] += __float2int_rn(z[i][e]);
-                                }
-                            }
-                            load_h(h[o], k + o + 2);
+                        for (int i = 0; i < 4; ++i) {
+                            const int64_t q = (((int64_t)is[0][i] * 1024 + is[1][i]) * 1024 + is[2][i]) * 1024 + is[3][i];
+                            val[i] += (double)q + (double)fmaf(dl[1][i], 0x1p-20f, dl[0][i] * 0x1p-10f);
                         }
                     }
+                }
+                // 4. the lane's elements (as in colstep.cu)
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int64_t q = (((int64_t)is[0][i] * 1024 + is[1][i]) * 1024 + is[2][i]) * 1024 + is[3][i];
-                        val[i] += (double)q + (double)fmaf(dl[1][i], 0x1p-20f, dl[0][i] * 0x1p-10f);
+                for (int h = 0; h < 2; ++h) {
+                    const int u = 4 * gi + (g >> 2) + 2 * h;
+                    if (u >= nu) continue;
+                    const int p = opos[2 * u + (t >> 1)];
+                    if (p < 0) continue;
+                    double y[2];
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) {
+                        y[c] = val[2 * h + c];
+                        if (mode == PLAIN) continue;
+                        if (fabs(y[c]) >= (double)(1ll << (48 - PR_RESOLVE))) s_big[2 * t + c] = 1;
+                        y[c] *= pow2(a.opexp[4 * ulist[u] + (g & 3)] + s_e[2 * t + c] - 48, 0.0);
                     }
+                    const int64_t at = (int64_t)p * BB + 4 * (g & 3) + 2 * (t & 1);
+                    double2 v = make_double2(a.alpha * y[0], a.alpha * y[1]);
+                    if (a.D) {
+                        const double2 d = *reinterpret_cast<const double2 *>(a.D + at);
+                        v = make_double2(fma(a.alpha, y[0], a.beta * d.x), fma(a.alpha, y[1], a.beta * d.y));
+                    }
+                    *reinterpret_cast<double2 *>(a.C + at) = v;
                 }
             }
-            // 4. the lane's elements (as in colstep.cu)
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int u = 4 * gi + (g >> 2) + 2 * h;
-                if (u >= nu) continue;
-                const int p = opos[2 * u + (t >> 1)];
-                if (p < 0) continue;
-                double y[2];
-#pragma unroll
-                for (int c = 0; c < 2; ++c)
-                    y[c] = slow ? val[2 * h + c] : val[2 * h + c] * pow2(a.opexp[4 * ulist[u] + (g & 3)] + s_e[2 * t + c] - 48, 0.0);
-                const int64_t at = (int64_t)p * BB + 4 * (g & 3) + 2 * (t & 1);
-                double2 v = make_double2(a.alpha * y[0], a.alpha * y[1]);
-                if (a.D) {
-                    const double2 d = *reinterpret_cast<const double2 *>(a.D + at);
-                    v = make_double2(fma(a.alpha, y[0], a.beta * d.x), fma(a.alpha, y[1], a.beta * d.y));
-                }
-                *reinterpret_cast<double2 *>(a.C + at) = v;
-            }
+            if (mode == PLAIN) break;
+            __syncthreads();
+            bool done = true;
+            for (int c = 0; c < 8; ++c) done &= s_max[c] == 0u || s_big[c] != 0;
+            if (done) break;
+            ++mode;  // (every thread finds the same; a lane writes over its own results)
+            __syncthreads();
         }
     }
 }

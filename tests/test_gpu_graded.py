@@ -1,9 +1,11 @@
 """Digit products (csrc/colstep.cu, csrc/product.cu) of operands whose rows and columns
 have different scales: an operator element is held to 2^-60 (FP64) or 2^-30 (FP32) of its
-scalar row's largest, a column's of its own.
+scalar row's largest, a column's of its own, and a product column that the digits cannot
+resolve is multiplied in FP64.
 
 Bars, element by element: K products, each with both operands known to the working
-precision u of their row's or column's largest element: 4 K u max|row| max|column|."""
+precision u of their row's or column's largest element -- 4 K u max|row| max|column|; where
+the scales of rows and columns cancel within a product, K u of the sum of |products|."""
 import numpy as np
 import pytest
 import torch
@@ -67,6 +69,23 @@ def test_products_of_graded_rows_and_columns(shift):
         cg.masked_product(plan, cg.Bsr(Q[0], Q[1], A), B, C)
         DA, DB = dense(Q, A), dense(P, B)
         bar = 4 * (4 * 95) * 2.0 ** -53 * row_column_bar(DA, DB)
+        assert ((C - blocks(P, DA @ DB)).abs() <= blocks(P, bar)).all()
+
+
+@pytest.mark.parametrize("width", [24, 60])
+def test_products_whose_inner_scales_cancel(width):
+    # the large elements of every row meet the small ones of every column
+    L, P = band(181, 29), band(181, width)
+    plan = cg.Plan(cg.Bsr(*P), cg.F64).attach_operator(cg.Bsr(*L))
+    assert cg.plan_col_info(plan)[0] >= 1
+    d = SCALES.to(DEV)
+    for Q, A in ((L, rand(L, 1) / d[None, :]), (P, rand(P, 2) / d[None, :])):
+        B = rand(P, 3) * d[:, None]
+        B[:, :, 2] = 0.0  # (a zero column is exact by digits)
+        C = torch.full_like(B, 9.0)
+        cg.masked_product(plan, cg.Bsr(Q[0], Q[1], A), B, C)
+        DA, DB = dense(Q, A), dense(P, B)
+        bar = 2 * (4 * (2 * width + 1)) * 2.0 ** -53 * (DA.abs() @ DB.abs())
         assert ((C - blocks(P, DA @ DB)).abs() <= blocks(P, bar)).all()
 
 
