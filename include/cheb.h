@@ -185,9 +185,10 @@ int cheb_plan_attach_operator(cheb_plan *plan, const cheb_bsr *L, size_t *op_ws_
  * 2^-30 (FP32) or 2^-60 (FP64) of the largest of its column of T_k or of its scalar row
  * of the operator, in place of FP32 or FP64 rounding, so a product of K terms is off by
  * at most K u max|row| max|column|, u = 2^-24 or 2^-53, and small elements of a row or
- * column lose bits that floats of their own would keep; columns or operators with
- * elements that are not finite or beyond the grid's exponents are multiplied in plain
- * FP32 or FP64.  Results agree with the other kernels to rounding, and are bitwise
+ * column lose bits that floats of their own would keep; columns beyond the grid's
+ * exponents, and operators with such elements or ones that are not finite, are multiplied
+ * in plain FP32 or FP64.  Where a product meets an element of T_k that is not finite the
+ * result is NaN.  Results agree with the other kernels to rounding, and are bitwise
  * reproducible run to run.  CHEB_F64X expansions that run it hold T_k in FP64.  The
  * lists are not built (and the ranking kernels run) when one column's rows do not
  * fit a panel or the operator has 2^22 - 1 blocks or more.  cheb_plan_col_info

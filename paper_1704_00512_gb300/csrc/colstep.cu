@@ -59,8 +59,9 @@
 //      one term per step) and their parts of the moments;
 //   4. the panel's moments go to a table that a second kernel sums in a fixed
 //      order.
-// A column with an element that is not finite or beyond the grid's exponents
-// (or such an operator) takes the step in plain FP32 / FP64 instead (slow).
+// Elements that are not finite spread by a pass of their own (mark_not_finite).  A column
+// beyond the grid's exponents, or an operator with such elements or ones that are not
+// finite, takes the step in plain FP32 / FP64 instead (slow).
 #include <algorithm>
 #include <array>
 #include <numeric>
@@ -178,6 +179,65 @@ __device__ __noinline__ void plain_group(const ColArgs &a, const int32_t *opos, 
     }
 }
 
+// Before a step of a panel with elements of T_{term-1} (R) that are not finite: the largest
+// finite elements of its columns (into mx), and NaN in T_{term-2} (C) wherever a product
+// with one of the others goes.  T_term is then NaN there by its own sum, and the digits of
+// the finite elements do the rest: an expansion that leaves its interval, whose columns
+// overflow one after the other, goes on at the others' speed.  nf: the columns of each
+// union row's blocks with such an element, 16 bits.
+template <typename T>
+__device__ __noinline__ void mark_not_finite(const ColArgs &a, int par, uint32_t *mx) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    constexpr int NT = Dig<T>::NT, P = 2 * NT, NC = 8 * NT, NTH = COL_NW * 32;
+    constexpr uint32_t SM = (1u << COL_SLOT_BITS) - 1u;
+    constexpr ColLayout lay = col_layout(P);
+    const int32_t *opos = reinterpret_cast<const int32_t *>(smem + lay.off_pos);
+    const uint2 *srow = reinterpret_cast<const uint2 *>(smem + lay.off_rows);
+    uint32_t *nf = reinterpret_cast<uint32_t *>(smem + lay.off_nf);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int pid = a.order[blockIdx.x], nu = a.panels[4 * pid + 2];
+    const int32_t *wr = a.wrow + pid * (COL_NW + 1);
+    const T *R = static_cast<const T *>(a.T[par ^ 1]);
+    T *C = static_cast<T *>(a.T[par]);
+    __syncthreads();  // (every thread has read mx)
+    if (tid < NC) mx[tid] = 0u;
+    for (int i = tid; i < (nu + 1) / 2; i += NTH) nf[i] = 0u;
+    __syncthreads();
+    for (int i = tid; i < nu * P; i += NTH) {
+        const int p = opos[i], s = i / P, q = i % P;
+        if (p < 0) continue;
+        for (int e = 0; e < 16; ++e) {
+            const uint32_t m = mag_bits(__ldcg(R + (int64_t)p * BB + e));
+            const int c = 4 * q + (e & 3);
+            if (m >= NOT_FINITE<T>) atomicOr(&nf[s >> 1], (1u << c) << (16 * (s & 1)));
+            else if (m > mx[c]) atomicMax(&mx[c], m);
+        }
+    }
+    __syncthreads();
+    // the warp's groups: a lane has word (lane % 16) of every second quad, of row a
+    const int a4 = ((lane >> 3) & 1) | ((lane & 1) << 1);
+    const uint32_t *ent = a.ent + (int64_t)a.wchunk[pid * (COL_NW + 1) + warp] * COL_CW;
+    for (int r = wr[warp] - wr[0]; r < wr[warp + 1] - wr[0]; ++r) {
+        const uint2 rw = srow[r];
+        const int cnt = (int)(rw.y >> COL_SLOT_BITS);
+        uint32_t bits = 0u;
+        for (int k = lane; k < cnt * COL_CW; k += 32) {
+            const uint32_t w = __ldg(ent + k), s = w & SM;
+            if ((w >> COL_SLOT_BITS) != (uint32_t)a.nnzL) bits |= nf[s >> 1] >> (16 * (s & 1)) & 0xffffu;
+        }
+        ent += cnt * COL_CW;
+        for (int o = 2; o < 32; o = o == 4 ? 16 : 2 * o) bits |= __shfl_xor_sync(0xffffffffu, bits, o);
+        const uint32_t s = a4 == 3 ? rw.y & SM : (rw.x >> (a4 * COL_SLOT_BITS)) & SM;
+        // (the lanes of a row share its columns)
+        for (int q = 0; q < P && s != SM; ++q) {
+            const int p = opos[s * P + q], c = (lane >> 1) & 3;
+            if (p >= 0 && lane < 16 && (bits >> (4 * q + c)) & 1u)
+                for (int e = 0; e < 4; ++e) C[(int64_t)p * BB + 4 * e + c] = T(NAN);
+        }
+    }
+    // (the barrier before the products orders these stores before their loads)
+}
+
 template <typename T>
 __global__ void __launch_bounds__(COL_NW * 32, 1) k_colstep(const __grid_constant__ ColArgs a) {
     using D = Dig<T>;
@@ -190,8 +250,8 @@ __global__ void __launch_bounds__(COL_NW * 32, 1) k_colstep(const __grid_constan
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ uint32_t s_max[2][NC];
     __shared__ int s_e[NC];
-    __shared__ float s_cf[NC];  // FP32: 2^e
-    __shared__ int s_slow;
+    __shared__ float s_cf[NC];  // FP32: 2^(e - 1)
+    __shared__ int s_slow, s_marked;  // (shared, so that no register holds them)
     __shared__ int s_cb[P + 1];
     __shared__ int s_dslot[P];
     __shared__ float s_ch[3][MAX_F], s_cl[3][MAX_F];
@@ -213,6 +273,7 @@ __global__ void __launch_bounds__(COL_NW * 32, 1) k_colstep(const __grid_constan
     // --- the panel: column starts, block positions, zero digits
     if (tid <= P) s_cb[tid] = (int)a.rp[j0 + min(tid, nc)];
     if (tid < P) s_dslot[tid] = -1;
+    if (tid == 0) s_marked = 0;
     if (tid < 2 * NC) (&s_max[0][0])[tid] = 0u;
     for (int i = tid; i < nu * XV; i += NTH) {
         const uint32_t z = !F64 && i % XV >= 16 ? 0x80808080u : 0u;
@@ -329,23 +390,24 @@ __global__ void __launch_bounds__(COL_NW * 32, 1) k_colstep(const __grid_constan
         int grp = 0;
         if (term == n - 1 || (term >= 4 && (term - 1) % 3 == 0)) grp = (1 << (term - (1 + 3 * ((term - 2) / 3)))) - 1;
         // 1. grids of the columns and digits of T_{term-1}
-        bool bad = opbad;
-        for (int c = 0; c < NC; ++c) {
-            int e;
-            bad |= !grid_exp<T>(s_max[par][c], D::EX_MIN, D::EX_MAX, e);
-            if (tid == c) {
-                s_e[c] = e;
-                if (!F64) s_cf[c] = pow2(e, 0.f);
-            }
+        if (__any_sync(0xffffffffu, s_max[par][lane % NC] >= NOT_FINITE<T>)) {  // (the same in every warp)
+            mark_not_finite<T>(a, par, s_max[par]);
+            if (tid == 0) s_marked = 1;
+            __syncthreads();
         }
-        if (tid == 0) s_slow = bad;  // (read again by every group: no register to hold it)
+        int ec;  // of column lane % NC
+        const bool bad = opbad | __any_sync(0xffffffffu, !grid_exp<T>(s_max[par][lane % NC], D::EX_MIN, D::EX_MAX, ec));
+        if (tid < NC) {
+            s_e[tid] = ec;
+            if (!F64) s_cf[tid] = bad ? 2.f : pow2(ec - 1, 0.f);
+        }
+        if (tid == 0) s_slow = bad;
         if (grp && tid < 3 * MAX_F) {
             const int i = tid / MAX_F, f = tid % MAX_F;  // term - 2 + i
             const double c = f < a.nf ? coef[(int64_t)f * a.coef_stride + term - 2 + i] : 0.0;
             s_c[i][f] = c;
             ff_split(c, s_ch[i][f], s_cl[i][f]);
         }
-        if (bad && !F64 && tid < NC) s_cf[tid] = 2.f;
         if (!bad) {
             for (int b = cb0 + tid; b < cb1; b += NTH) {
                 const int q = col_of(b), s = a.slot[b];
@@ -366,6 +428,11 @@ __global__ void __launch_bounds__(COL_NW * 32, 1) k_colstep(const __grid_constan
                         v[i + 2] = u.z;
                         v[i + 3] = u.w;
                     }
+                }
+                if (*(volatile int *)&s_marked) {
+#pragma unroll
+                    for (int i = 0; i < 16; ++i)
+                        if (mag_bits(v[i]) >= NOT_FINITE<T>) v[i] = T(0);
                 }
                 uint4 *xs = X + s * XV;
                 const int sw = 2 * (s & 3);
@@ -393,6 +460,7 @@ __global__ void __launch_bounds__(COL_NW * 32, 1) k_colstep(const __grid_constan
         }
         __syncthreads();
         if (tid < NC) s_max[par][tid] = 0u;  // next written by the step after the next
+        if (tid == 0) s_marked = 0;
 
         // 2. the warp's groups
         uint32_t mx[NT][2];
@@ -575,7 +643,7 @@ uint32_t B[NT][3][2];
                 for (int hh = 0; hh < 2; ++hh) {
                     if (sl2[hh] == (int)SM) continue;
                     const int er = rexp[4 * sl2[hh] + (g & 3)];
-                    const float rf = F64 || slow ? 1.f : pow2(er - 18, 0.f);  // (two exact factors)
+                    const float rf = F64 || slow ? 1.f : pow2(er - 17, 0.f);  // (two exact factors)
                     // T_{term-2}, G and, in group steps, T_{term-1}, of the half's positions
                     int pos[NT];
                     V2 tm[NT], tk[NT], y[NT];
@@ -992,10 +1060,10 @@ static void col_fill(const ColLists &c, const std::vector<int64_t> &rp, const st
 }
 
 // Union rows a panel of the column kernel may hold: shared memory, and
-// COL_MAX_UNION.
+// col_max_union.
 int32_t col_ucap(int P) {
     const ColLayout lay = col_layout(P);
-    return std::min((CHEB_MAX_DYN_SMEM - 1024 - lay.off_x) / lay.slot_bytes, COL_MAX_UNION);
+    return std::min((CHEB_MAX_DYN_SMEM - 1024 - lay.off_x) / lay.slot_bytes, col_max_union(P));
 }
 
 // Whether the column kernel's lists are built for an operator of nnzL blocks

@@ -10,17 +10,18 @@
 namespace cheb {
 
 // Tiles of an element type: NT n8-tiles (2 block columns each) per panel, and the
-// grid exponents that the recursion takes: of T's columns, and of the operator's
-// scalar rows (a byte each).
+// grid exponents that the recursion takes: of T's columns, to the end of the finite
+// numbers, and of the operator's scalar rows (a byte each; FP64: OP_MAX + EX_MAX - 47 is
+// an exponent too).
 template <typename T>
 struct Dig;
 template <>
 struct Dig<float> {
-    static constexpr int NT = 2, EX_MIN = -60, EX_MAX = 90, OP_MIN = -80, OP_MAX = 30;
+    static constexpr int NT = 2, EX_MIN = -90, EX_MAX = 128, OP_MIN = -80, OP_MAX = 30;
 };
 template <>
 struct Dig<double> {
-    static constexpr int NT = 1, EX_MIN = -400, EX_MAX = 400, OP_MIN = -127, OP_MAX = 127;
+    static constexpr int NT = 1, EX_MIN = -400, EX_MAX = 1024, OP_MIN = -127, OP_MAX = 46;
 };
 
 __device__ __forceinline__ float bf16r(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
@@ -31,6 +32,10 @@ __device__ __forceinline__ float bf16r(float x) { return __bfloat162float(__floa
 __device__ __forceinline__ uint32_t mag_bits(float x) { return __float_as_uint(x) & 0x7fffffffu; }
 __device__ __forceinline__ uint32_t mag_bits(double x) { return (uint32_t)__double2hiint(x) & 0x7fffffffu; }
 
+// mag_bits of infinities and NaN and no others is at least this
+template <typename T>
+constexpr uint32_t NOT_FINITE = sizeof(T) == 4 ? 0x7f800000u : 0x7ff00000u;
+
 // Grid exponent e of values with largest magnitude bits m: every |x| < 0.997 2^e
 // (0 for all zeros).  false: not finite, or e outside [lo, hi].
 template <typename T>
@@ -39,12 +44,10 @@ __device__ __forceinline__ bool grid_exp(uint32_t m, int lo, int hi, int &e) {
     if (m == 0u) return true;
     if constexpr (sizeof(T) == 4) {
         e = (int)(m >> 23) - 126 + ((m & 0x7fffffu) >= 0x7f0000u ? 1 : 0);
-        if (m >= 0x7f800000u) return false;
     } else {
         e = (int)(m >> 20) - 1022 + ((m & 0xfffffu) >= 0xfe000u ? 1 : 0);
-        if (m >= 0x7ff00000u) return false;
     }
-    return e >= lo && e <= hi;
+    return m < NOT_FINITE<T> && e >= lo && e <= hi;
 }
 // 2^e as a float / double (e within the normal range)
 __device__ __forceinline__ float pow2(int e, float) { return __int_as_float((e + 127) << 23); }

@@ -210,9 +210,9 @@ __host__ __device__ inline ResLayout res_layout(int64_t nw, int64_t ucap, int64_
 
 // Column-order kernel (colstep.cu): warps per thread block, words per quad, and
 // its shared-memory layout: the warps' moment partials, the groups' words, the grid
-// exponent of each union row, the column-order position of each (union row, panel
-// column) block, and the panel's digits.  (Offsets are constants, so that they take
-// no registers.)
+// exponents of each union row, the column-order position of each (union row, panel
+// column) block, the marks of mark_not_finite, and the panel's digits.  (Offsets are
+// constants, so that they take no registers.)
 constexpr int COL_NW = 16;
 constexpr int COL_CW = 16;         // 4 rows x 4 merged slots
 // Unassigned rows among which a group's next row is chosen.  Merged slots over
@@ -221,8 +221,9 @@ constexpr int COL_CW = 16;         // 4 rows x 4 merged slots
 constexpr int COL_WINDOW = 64;
 constexpr int COL_TAIL = 8;        // quads of padding behind the lists (read ahead, not used)
 constexpr int COL_SLOT_BITS = 10;  // union slots < 1023; operator blocks < 2^22
-// Union rows of a panel at most.  Columns beyond it run on the ranking kernels.
-constexpr int COL_MAX_UNION = 667;
+// Union rows of a panel at most, of width 4 (FP32) and 2 (FP64).  Columns beyond it run on
+// the ranking kernels.
+__host__ __device__ constexpr int col_max_union(int P) { return P == 4 ? 667 : 576; }
 // (quads of a group come in pairs) FP64: quads of a group at most, so that its exact digit sums (at most 4
 // products of 2^18 per merged row of a slot) stay below 2^31.
 constexpr int COL_MAX_QUADS64 = 126;
@@ -233,7 +234,7 @@ constexpr int64_t COL_ROW_MIN = 48;
 // panel width: 16 scalar columns of FP32 or 8 of FP64 fill two or one mma tiles
 inline int col_width(int precision) { return precision == CHEB_F64 || precision == CHEB_F64X ? 2 : 4; }
 struct ColLayout {
-    int off_red, off_rows, off_rexp, off_pos, off_x, slot_bytes;
+    int off_red, off_rows, off_rexp, off_pos, off_nf, off_x, slot_bytes;
     __host__ __device__ constexpr size_t total(int64_t ucap) const { return (size_t)off_x + (size_t)ucap * slot_bytes; }
 };
 // P = 4: FP32 / BF16 (two f16 digits of 4 values in a 16-byte chunk per column,
@@ -244,11 +245,14 @@ __host__ __device__ constexpr ColLayout col_layout(int P) {
     L.off_red = o;
     o += COL_NW * 4 * 8;
     L.off_rows = o;
-    o += (COL_MAX_UNION + 3) / 4 * 8;
+    const int U = col_max_union(P);
+    o += (U + 3) / 4 * 8;
     L.off_rexp = o;
-    o += COL_MAX_UNION * 4;
+    o += U * 4;
     L.off_pos = o;
-    o += COL_MAX_UNION * P * 4;
+    o += U * P * 4;
+    L.off_nf = o;
+    o += (U + 1) / 2 * 4;
     L.off_x = (o + 127) / 128 * 128;
     L.slot_bytes = P == 4 ? 16 * 20 : 8 * 48;
     return L;
