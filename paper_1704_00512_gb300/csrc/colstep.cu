@@ -122,15 +122,9 @@ __device__ __forceinline__ void ff_add_prod(float &hi, float &lo, float y, float
     const float s = __fadd_rn(hi, p);
     const float bb = __fsub_rn(s, hi);
     const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(p, bb));
-    lo = __fadd_rn(lo, __fadd_rn(pe, e));
-    hi = s;
-}
-// hi back to the nearest float of the sum (the additions above leave lo a few units
-// of hi's last place, which costs its own last bits only)
-__device__ __forceinline__ void ff_norm(float &hi, float &lo) {
-    const float s = __fadd_rn(hi, lo);
-    lo = __fsub_rn(lo, __fsub_rn(s, hi));
-    hi = s;
+    const float t = __fadd_rn(__fadd_rn(lo, pe), e);
+    hi = __fadd_rn(s, t);
+    lo = __fsub_rn(t, __fsub_rn(hi, s));
 }
 __host__ __device__ inline void ff_split(double v, float &hi, float &lo) {
     hi = (float)v;
@@ -729,8 +723,6 @@ uint32_t B[NT][3][2];
                                         ff_add_prod(v[j].x, v[j].y, tv[i][0], s_ch[i][f], s_cl[i][f]);
                                         ff_add_prod(v[j].z, v[j].w, tv[i][1], s_ch[i][f], s_cl[i][f]);
                                     }
-                                ff_norm(v[j].x, v[j].y);
-                                ff_norm(v[j].z, v[j].w);
                                 *reinterpret_cast<float4 *>(a.accp[f] + ((int64_t)pos[j] * BB + eo) * 2) = v[j];
                             }
                         }
