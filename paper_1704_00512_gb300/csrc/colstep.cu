@@ -877,7 +877,7 @@ static int col_expand_t(const cheb_plan *plan, const cheb_bsr *Mt, const ColExpa
     a.round_bf16 = x.round_bf16;
     const size_t smem = col_layout(c.P).total(c.max_union);
     auto fn = k_colstep<T>;
-    CHEB_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CHEB_TRY(allow_shared(fn));
     for (int t0 = 2; t0 == 2 || t0 < x.max_terms; t0 += COL_STEPS) {
         a.t0 = t0;
         a.t1 = std::min(t0 + COL_STEPS, x.max_terms);

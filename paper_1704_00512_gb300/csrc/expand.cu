@@ -608,7 +608,7 @@ template <typename T, int P, int NW, int MINB>
 int launch_step(const cheb_plan *plan, const StepArgs<T> &a, cudaStream_t s) {
     const StepLayout lay = step_layout(a.nw, a.ucap, P, sizeof(T), NW);
     auto fn = k_step<T, P, NW, MINB>;
-    CHEB_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lay.total));
+    CHEB_TRY(allow_shared(fn));
     fn<<<(unsigned)plan->n_panels, NW * 32, lay.total, s>>>(a);
     return check_launch("k_step");
 }

@@ -685,8 +685,8 @@ int col_build_device(cheb_plan *plan, const cheb_bsr *L, cudaStream_t s) {
     a.cnt_maxrow = cnt_max;
     a.err = err;
     a.off_list = off_list;
-    CHEB_CUDA(cudaFuncSetAttribute(k_gp_rows<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
-    CHEB_CUDA(cudaFuncSetAttribute(k_gp_rows<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
+    CHEB_TRY(allow_shared(k_gp_rows<false>));
+    CHEB_TRY(allow_shared(k_gp_rows<true>));
     k_gp_rows<false><<<(unsigned)np, GP_NT, dyn, s>>>(a);
     CHEB_TRY(check_launch("k_gp_rows count"));
     k_gp_scan<<<1, 1024, 0, s>>>(cnt_chunks, np, choff);
@@ -854,8 +854,8 @@ int row_lists_device(const int64_t *rp, const int32_t *ci, int64_t nbr, const ch
     const size_t dyn = (((size_t)((nbr + 31) / 32) * sizeof(uint2) + 15) & ~(size_t)15) + (size_t)maxu * 4;
     if (dyn > (size_t)CHEB_MAX_DYN_SMEM - 2048)
         return fail(CHEB_ERR_NOSPACE, "cheb_plan_attach_operator: %zu bytes of panel bitmap and union", dyn);
-    CHEB_CUDA(cudaFuncSetAttribute(k_rl_rows<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
-    CHEB_CUDA(cudaFuncSetAttribute(k_rl_rows<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
+    CHEB_TRY(allow_shared(k_rl_rows<false>));
+    CHEB_TRY(allow_shared(k_rl_rows<true>));
     int64_t *scr = nullptr;  // cnt, nrow [np]; ent_off, row_base [np + 1]; error flag
     CHEB_CUDA(cudaMalloc(&scr, (4 * np + 3) * 8));
     struct Free {

@@ -133,6 +133,17 @@ struct cheb_plan {
 
 namespace cheb {
 
+// Lets launches of fn use all the dynamic shared memory there is beside its static part:
+// the same value for every plan, because the limit belongs to the function, and a thread
+// that set its own plan's size could lower it between another's setting and launch.
+template <typename F>
+int allow_shared(F fn) {
+    cudaFuncAttributes at;
+    CHEB_CUDA(cudaFuncGetAttributes(&at, fn));
+    CHEB_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, CHEB_MAX_DYN_SMEM - (int)at.sharedSizeBytes));
+    return CHEB_OK;
+}
+
 // Shared-memory layout of the step kernel for a panel of width P over a union of
 // ucap rows, element size esz, nw bitmap words, nwarps warps.
 // Operator blocks per staged batch of the step kernel: 16 for panels of two or

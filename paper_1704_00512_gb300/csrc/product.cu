@@ -463,6 +463,7 @@ int prod_run(const cheb_plan *plan, const cheb_bsr *L, const double *R, double a
     a.cap = prod_cap(plan);
     a.nw = (int32_t)((plan->nbr + 31) / 32);
     const int smem = prod_layout(a.cap).off_bits + a.nw * 8;
+    CHEB_TRY(allow_shared(k_product));
     // one user of the digits at a time: this call waits, on its stream, for the last one
     std::lock_guard<std::mutex> lock(plan->prod_mx);
     if (!plan->prod_done) CHEB_CUDA(cudaEventCreateWithFlags(&plan->prod_done, cudaEventDisableTiming));
@@ -471,7 +472,6 @@ int prod_run(const cheb_plan *plan, const cheb_bsr *L, const double *R, double a
     k_opdig<double><<<(unsigned)((plan->nbr + 1 + 7) / 8), 256, 0, s>>>(L->row_ptr, a.Lv, plan->nbr, L->nnzb, 0, -PR_EX, PR_EX, opd,
                                                                       opexp, flag);
     CHEB_TRY(check_launch("k_opdig"));
-    CHEB_CUDA(cudaFuncSetAttribute(k_product, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     k_product<<<(unsigned)plan->n_panels, PR_NW * 32, smem, s>>>(a);
     const int rc = check_launch("k_product");
     CHEB_CUDA(cudaEventRecord(plan->prod_done, s));

@@ -417,7 +417,7 @@ template <typename T, int P, int NW, int MINB>
 int launch_resident(const cheb_plan *plan, const ResArgs<T> &a, cudaStream_t s) {
     const ResLayout lay = res_layout(a.nw, a.ucap, a.bcap, P, sizeof(T), NW);
     auto fn = k_resident<T, P, NW, MINB>;
-    CHEB_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lay.total));
+    CHEB_TRY(allow_shared(fn));
     fn<<<(unsigned)plan->n_rpanels, NW * 32, lay.total, s>>>(a);
     return check_launch("k_resident");
 }
