@@ -254,13 +254,12 @@ __global__ void __launch_bounds__(64) k_tridiag(LzState *st, double margin_frac)
     }
     const double big = fmax(fabs(lo), fabs(hi));
     int e = 0;
-    if (big > 0.0 && big < 1e300) frexp(big, &e);
-    const double down = ldexp(1.0, -e), up2 = ldexp(1.0, e);
-    lo *= down;
-    hi *= down;
+    if (big > 0.0 && isfinite(big)) frexp(big, &e);
+    lo = ldexp(lo, -e);  // (2^-e need not be a double itself)
+    hi = ldexp(hi, -e);
     for (int i = threadIdx.x; i < k; i += 64) {
-        ab[0][i] = st->alpha[i] * down;
-        ab[1][i] = st->beta[i] * down;
+        ab[0][i] = ldexp(st->alpha[i], -e);
+        ab[1][i] = ldexp(st->beta[i], -e);
         ab[2][i] = ab[1][i] * ab[1][i];
     }
     __syncthreads();
@@ -290,7 +289,7 @@ __global__ void __launch_bounds__(64) k_tridiag(LzState *st, double margin_frac)
         }
         if (lane == 0) {
             const double t = which == 0 ? h : l;
-            th[which] = t * up2;
+            th[which] = ldexp(t, e);
             last[which] = last_component(a, b, k, t, scratch[which][0], scratch[which][1], scratch[which][2],
                                          scratch[which][3], piv[which]);
         }
