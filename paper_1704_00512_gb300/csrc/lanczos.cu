@@ -188,15 +188,18 @@ __device__ int sturm_count(const double *a, const double *b2, int k, double x) {
 // Last component of the unit eigenvector for eigenvalue th: inverse iteration, three
 // solves of (T - th I) y = y_prev with one factorisation by Gaussian elimination with
 // partial pivoting.  f: multipliers, rd: reciprocals of the pivots, du: superdiagonal
-// (a pivoted row i has b[i + 1] beyond it).
+// (a pivoted row i has b[i + 1] beyond it).  |a|, |b| <= 1.
 __device__ double last_component(const double *a, const double *b, int k, double th, double *f, double *rd, double *du,
                                  double *y, unsigned char *piv) {
     if (k == 1) return 1.0;
+    // the place of a pivot that is zero (th an eigenvalue to the last bit): small enough to
+    // leave the eigenvector alone, large enough for the squares of what it gives
+    constexpr double tiny = 1e-100;
     double d = a[0] - th, u = b[0];
     for (int i = 0; i < k - 1; ++i) {
         double dn = a[i + 1] - th, un = i < k - 2 ? b[i + 1] : 0.0;
         const bool p = fabs(d) < fabs(b[i]);
-        if (!p && d == 0.0) d = 1e-300;
+        if (!p && d == 0.0) d = tiny;
         rd[i] = 1.0 / (p ? b[i] : d);
         const double m = (p ? d : b[i]) * rd[i];
         if (p) {
@@ -212,7 +215,7 @@ __device__ double last_component(const double *a, const double *b, int k, double
         d = dn;
         u = un;
     }
-    rd[k - 1] = 1.0 / (d == 0.0 ? 1e-300 : d);
+    rd[k - 1] = 1.0 / (d == 0.0 ? tiny : d);
     for (int i = 0; i < k; ++i) y[i] = 1.0;
     for (int it = 0; it < 3; ++it) {
         double cur = y[0];

@@ -1,9 +1,13 @@
-"""Lanczos bounds (csrc/lanczos.cu) at the ends of the number range.
+"""Lanczos bounds (csrc/lanczos.cu) at the ends of the number range, and of a tridiagonal
+whose highest Ritz value is an eigenvalue to the last bit: then the last pivot of the
+inverse iteration is exactly zero, and the residual still counts.
 
 Bars: the recursion's rounding, 1e-12 of the interval; at subnormal scale one unit there."""
 import numpy as np
 import pytest
 import torch
+
+from oracle import ref
 
 pytestmark = pytest.mark.gpu
 
@@ -26,6 +30,19 @@ def test_a_multiple_of_the_identity_at_every_scale(c):
     unit = max(36 * 2.0 ** -52 * abs(c), 36 * 2.0 ** -1074)
     assert abs(th[0] - c) <= unit and abs(th[1] - c) <= unit
     assert e0 <= th[0] and e1 >= th[1] and np.isfinite([e0, e1]).all()
+
+
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** -400, 2.0 ** 400])
+def test_a_highest_ritz_value_that_is_exact(scale):
+    # v0 = e_1 gives T = [[0, 2], [2, 3]] after two steps: eigenvalues -1 and 4, the next
+    # beta 1, so the residuals are the last components 1/sqrt(5) and 2/sqrt(5)
+    M = np.array([[0.0, 2.0, 0.0, 0.0], [2.0, 3.0, 1.0, 0.0], [0.0, 1.0, 1.0, 1.0], [0.0, 0.0, 1.0, 2.0]]) * scale
+    v0 = torch.tensor([1.0, 0.0, 0.0, 0.0], dtype=torch.float64, device=DEV)
+    e0, e1, th = cg.bounds(diagonal(M[None]), 2, v0=v0)
+    want = np.array([-1.0 - 2.0 / 5 ** 0.5, 4.0 + 4.0 / 5 ** 0.5, -1.0, 4.0]) * scale
+    assert np.abs(np.array([e0, e1, *th]) - want).max() <= 1e-12 * 5 * scale
+    o0, o1, _, _ = ref.ritz_bounds(np.array([0.0, 3.0]), np.array([2.0, 1.0]))
+    assert abs(e0 / scale - o0) <= 1e-9 and abs(e1 / scale - o1) <= 1e-9
 
 
 def test_one_step_of_values_beyond_1e300():
