@@ -33,6 +33,7 @@ constexpr int GP_NT = 512;
 constexpr int GP_NWARP = GP_NT / 32;
 constexpr int GP_MAXU = 1 << COL_SLOT_BITS;  // union slots
 constexpr int GP_MAXG = GP_MAXU / 4;         // groups, and quads of a group
+constexpr int GP_STATIC = 12 * 1024;         // static shared memory of k_gp_rows at most
 static_assert(GP_NWARP == COL_NW, "one warp of the builder per warp stream of the step kernel");
 
 // Block-wide integer sum, returned to every thread.
@@ -176,7 +177,10 @@ struct GpArgs {
     uint32_t *rows, *ent;
     uint16_t *slot;
     int32_t *err;
-    size_t off_list;  // dynamic shared memory: the warps' merged slots
+    // dynamic shared memory: the union as a bitmap, the prefix count of each of its words,
+    // the operator slots of the union rows, and for each of the fill warps its group's
+    // merged slots and their places (ucap each)
+    int off_pre, off_ub, off_list, ucap, fill_warps;
 };
 
 template <bool FILL>
@@ -188,7 +192,6 @@ __global__ void __launch_bounds__(GP_NT) k_gp_rows(const GpArgs a) {
     __shared__ uint8_t wsel[GP_MAXG];
     __shared__ int hist[GP_MAXG + 1];
     __shared__ int16_t group[GP_MAXG][4];
-    __shared__ uint16_t place[FILL ? GP_NWARP : 1][FILL ? GP_MAXU : 1];
     __shared__ int wsum[32];
     __shared__ int64_t sh[GP_NWARP];
     __shared__ int shi[GP_NWARP];
@@ -197,21 +200,26 @@ __global__ void __launch_bounds__(GP_NT) k_gp_rows(const GpArgs a) {
     const int64_t p = blockIdx.x;
     const int j0 = a.panels[4 * p], nc = a.panels[4 * p + 1], nu_plan = a.panels[4 * p + 2];
     const int64_t nw = (a.nbr + 31) / 32;
-    uint2 *bits = reinterpret_cast<uint2 *>(dsm);
+    uint32_t *bits = reinterpret_cast<uint32_t *>(dsm);
+    uint16_t *pre = reinterpret_cast<uint16_t *>(dsm + a.off_pre);
+    auto rank = [&](int K) {  // union slot of block row K, or -1
+        const uint32_t w = bits[K >> 5], b = 1u << (K & 31);
+        return w & b ? (int)pre[K >> 5] + __popc(w & (b - 1u)) : -1;
+    };
 
     // 1. union bitmap of the panel's columns' rows, ranks, sorted union list
-    for (int64_t w = tid; w < nw; w += GP_NT) bits[w] = make_uint2(0u, 0u);
+    for (int64_t w = tid; w < nw; w += GP_NT) bits[w] = 0u;
     __syncthreads();
     for (int q = 0; q < nc; ++q)
         for (int64_t e = a.rp[j0 + q] + tid; e < a.rp[j0 + q + 1]; e += GP_NT) {
             const int K = a.ci[e];
-            atomicOr(&bits[K >> 5].x, 1u << (K & 31));
+            atomicOr(&bits[K >> 5], 1u << (K & 31));
         }
     __syncthreads();
     const int64_t chunk = (nw + GP_NT - 1) / GP_NT;
     const int64_t wb = min(nw, (int64_t)tid * chunk), we = min(nw, wb + chunk);
     int cnt = 0;
-    for (int64_t w = wb; w < we; ++w) cnt += __popc(bits[w].x);
+    for (int64_t w = wb; w < we; ++w) cnt += __popc(bits[w]);
     int total;
     int run = block_excl_scan<GP_NWARP>(cnt, wsum, &total);
     const int nu = total, ng = (nu + 3) / 4;
@@ -220,8 +228,8 @@ __global__ void __launch_bounds__(GP_NT) k_gp_rows(const GpArgs a) {
         return;
     }
     for (int64_t w = wb; w < we; ++w) {
-        unsigned m = bits[w].x;
-        bits[w].y = (unsigned)run;
+        unsigned m = bits[w];
+        pre[w] = (uint16_t)run;
         while (m) {
             const int b = __ffs(m) - 1;
             ulist[run++] = (int)(w * 32 + b);
@@ -232,17 +240,17 @@ __global__ void __launch_bounds__(GP_NT) k_gp_rows(const GpArgs a) {
     if (FILL)
         for (int q = 0; q < nc; ++q)
             for (int64_t e = a.rp[j0 + q] + tid; e < a.rp[j0 + q + 1]; e += GP_NT)
-                a.slot[e] = (uint16_t)rank_of(bits, a.ci[e]);
+                a.slot[e] = (uint16_t)rank(a.ci[e]);
 
     // 2. operator slots of every union row
     const int uw = (nu + 31) / 32;
-    uint32_t *ub = reinterpret_cast<uint32_t *>(dsm + (((size_t)nw * sizeof(uint2) + 15) & ~(size_t)15));
+    uint32_t *ub = reinterpret_cast<uint32_t *>(dsm + a.off_ub);
     for (int i = tid; i < nu * uw; i += GP_NT) ub[i] = 0u;
     __syncthreads();
     for (int u = warp; u < nu; u += GP_NWARP) {
         const int I = ulist[u];
         for (int64_t e = a.lrp[I] + lane; e < a.lrp[I + 1]; e += 32) {
-            const int sl = rank_of(bits, a.lci[e]);
+            const int sl = rank(a.lci[e]);
             if (sl >= 0) atomicOr(&ub[u * uw + (sl >> 5)], 1u << (sl & 31));
         }
     }
@@ -395,7 +403,9 @@ __global__ void __launch_bounds__(GP_NT) k_gp_rows(const GpArgs a) {
 
     // 5. group words and entry streams
     const uint32_t zero_blk = (uint32_t)a.nnzL;
-    for (int i = warp; i < ng; i += GP_NWARP) {
+    if (warp >= a.fill_warps) return;
+    uint16_t *list = reinterpret_cast<uint16_t *>(dsm + a.off_list) + 2 * warp * a.ucap, *place = list + a.ucap;
+    for (int i = warp; i < ng; i += a.fill_warps) {
         const uint32_t mine = merge(i);
         const int quads = work[i];
         if (lane == 0) {
@@ -420,7 +430,6 @@ __global__ void __launch_bounds__(GP_NT) k_gp_rows(const GpArgs a) {
             if (lane >= o) incl += x;
         }
         const int all = __shfl_sync(0xffffffffu, incl, 31);
-        uint16_t *list = reinterpret_cast<uint16_t *>(dsm + a.off_list) + warp * GP_MAXU;
         int pl = incl - c;
         for (uint32_t m = mine; m; m &= m - 1u, ++pl) list[pl] = (uint16_t)(lane * 32 + __ffs(m) - 1);
         __syncwarp();
@@ -431,7 +440,7 @@ __global__ void __launch_bounds__(GP_NT) k_gp_rows(const GpArgs a) {
             col_places(list + 8 * ch, n, at);
             for (int k = 0; k < n; ++k) {
                 const int s = list[8 * ch + k];
-                place[warp][s] = (uint16_t)(8 * ch + at[k]);
+                place[s] = (uint16_t)(8 * ch + at[k]);
                 taken |= 1u << at[k];
 #pragma unroll
                 for (int x = 0; x < 4; ++x) word(8 * ch + at[k], x) = (zero_blk << COL_SLOT_BITS) | (uint32_t)s;
@@ -446,8 +455,8 @@ __global__ void __launch_bounds__(GP_NT) k_gp_rows(const GpArgs a) {
         for (int x = 0; x < 4 && group[i][x] >= 0; ++x) {
             const int I = ulist[group[i][x]];
             for (int64_t e = a.lrp[I] + lane; e < a.lrp[I + 1]; e += 32) {
-                const int sl = rank_of(bits, a.lci[e]);
-                if (sl >= 0) word(place[warp][sl], x) = ((uint32_t)e << COL_SLOT_BITS) | (uint32_t)sl;
+                const int sl = rank(a.lci[e]);
+                if (sl >= 0) word(place[sl], x) = ((uint32_t)e << COL_SLOT_BITS) | (uint32_t)sl;
             }
         }
         __syncwarp();
@@ -630,11 +639,21 @@ int col_build_device(cheb_plan *plan, const cheb_bsr *L, cudaStream_t s) {
     c.ucap = col_ucap(c.P);
     const int64_t nbr = plan->nbr, nnzL = L->nnzb;
     if (!col_wanted(plan, nnzL)) return CHEB_ERR_NOSPACE;
-    // (dynamic shared memory of k_gp_rows: bitmap words, operator slots of the rows)
-    const size_t off_list = align_up((size_t)((nbr + 31) / 32) * sizeof(uint2), 16) +
-                            align_up((size_t)c.ucap * ((c.ucap + 31) / 32) * 4, 16);
-    const size_t dyn = off_list + (size_t)GP_NWARP * GP_MAXU * 2;
-    if (dyn + 48 * 1024 > (size_t)CHEB_MAX_DYN_SMEM) return CHEB_ERR_NOSPACE;
+    // dynamic shared memory of k_gp_rows; where it is short, fewer warps fill the lists
+    // (FP32: all 16 up to about 640,000 block rows, one at 860,000)
+    GpArgs a{};
+    const size_t nw = (size_t)((nbr + 31) / 32), o_pre = align_up(nw * 4, 16), o_ub = align_up(o_pre + nw * 2, 16),
+                 o_list = o_ub + align_up((size_t)c.ucap * ((c.ucap + 31) / 32) * 4, 16);
+    size_t dyn = 0;
+    for (a.fill_warps = GP_NWARP; a.fill_warps > 0; a.fill_warps /= 2) {
+        dyn = o_list + (size_t)a.fill_warps * c.ucap * 4;
+        if (dyn + GP_STATIC <= (size_t)CHEB_MAX_DYN_SMEM) break;
+    }
+    if (a.fill_warps == 0) return CHEB_ERR_NOSPACE;
+    a.off_pre = (int)o_pre;
+    a.off_ub = (int)o_ub;
+    a.off_list = (int)o_list;
+    a.ucap = c.ucap;
     // scratch: spans, panels (at most one per column), counts and offsets
     const size_t n1 = (size_t)nbr + 1;
     size_t off = 0;
@@ -672,7 +691,6 @@ int col_build_device(cheb_plan *plan, const cheb_bsr *L, cudaStream_t s) {
     const int64_t np = h_out[0];
     c.n_panels = np;
     c.max_union = (int32_t)h_out[1];
-    GpArgs a{};
     a.rp = plan->rp;
     a.ci = plan->ci;
     a.nbr = nbr;
@@ -684,7 +702,6 @@ int col_build_device(cheb_plan *plan, const cheb_bsr *L, cudaStream_t s) {
     a.cnt_rows = cnt_rows;
     a.cnt_maxrow = cnt_max;
     a.err = err;
-    a.off_list = off_list;
     CHEB_TRY(allow_shared(k_gp_rows<false>));
     CHEB_TRY(allow_shared(k_gp_rows<true>));
     k_gp_rows<false><<<(unsigned)np, GP_NT, dyn, s>>>(a);
