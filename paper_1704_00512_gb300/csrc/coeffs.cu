@@ -376,20 +376,24 @@ struct MuResult {
 // smearing widths above mu a Fermi occupation is below 1e-52 and counts as 0 (below
 // 40 under mu it is 1 in FP64), without its exponential.  (One thread block, with a
 // cosine and an exponential per node and midpoint, took 9 ms at n = 9216; now 0.23 ms.)
-constexpr int BIS_CTAS = 8, BIS_NT = 512, BIS_KEEP = 4;
-__global__ void __cluster_dims__(BIS_CTAS, 1, 1) __launch_bounds__(BIS_NT)
+//
+// Up to BIS_ONE nodes one thread block with a node per thread is faster than a cluster's
+// barriers: 128 midpoints 0.39 against 0.71 ms at 16 nodes, 0.55 against 0.87 at 256.
+constexpr int BIS_CTAS = 8, BIS_NT = 512, BIS_KEEP = 4, BIS_ONE = 256;
+template <int CTAS, int NT, int KEEP>
+__global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(NT)
     k_bisect(const double *w, int n, double emin, double emax, int kind, double kT, double N_e, double tol_N,
              int max_iter, double lo, double hi, MuResult *res) {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
-    __shared__ double sh[BIS_NT / 32];
+    __shared__ double sh[NT / 32];
     __shared__ double s_part[2];  // this block's sum, alternating
-    const int rank = (int)cluster.block_rank(), first = rank * BIS_NT + threadIdx.x;
+    const int rank = (int)cluster.block_rank(), first = rank * NT + threadIdx.x;
     const double sigma = 2.0 / (emax - emin), tau = (emin + emax) / 2.0;
-    double xs[BIS_KEEP], ws[BIS_KEEP];
+    double xs[KEEP], ws[KEEP];
 #pragma unroll
-    for (int k = 0; k < BIS_KEEP; ++k) {
-        const int i = first + k * BIS_CTAS * BIS_NT;
+    for (int k = 0; k < KEEP; ++k) {
+        const int i = first + k * CTAS * NT;
         xs[k] = i < n ? node(i, n, sigma, tau) : 0.0;
         ws[k] = i < n ? w[i] : 0.0;
     }
@@ -407,15 +411,17 @@ __global__ void __cluster_dims__(BIS_CTAS, 1, 1) __launch_bounds__(BIS_NT)
         mid = 0.5 * (lo + hi);
         double s = 0.0;
 #pragma unroll
-        for (int k = 0; k < BIS_KEEP; ++k)
-            if (first + k * BIS_CTAS * BIS_NT < n) s += occ(xs[k], mid) * ws[k];
-        for (int i = first + BIS_KEEP * BIS_CTAS * BIS_NT; i < n; i += BIS_CTAS * BIS_NT)
+        for (int k = 0; k < KEEP; ++k)
+            if (first + k * CTAS * NT < n) s += occ(xs[k], mid) * ws[k];
+        for (int i = first + KEEP * CTAS * NT; i < n; i += CTAS * NT)
             s += occ(node(i, n, sigma, tau), mid) * w[i];
-        const double r = block_sum<BIS_NT>(s, sh);
+        const double r = block_sum<NT>(s, sh);
         if (threadIdx.x == 0) s_part[it & 1] = r;
-        cluster.sync();  // (a block's other slot is only rewritten after the next sync)
+        // (a block's other slot is only rewritten after the next sync)
+        if constexpr (CTAS > 1) cluster.sync();
+        else __syncthreads();
         N = 0.0;
-        for (int b = 0; b < BIS_CTAS; ++b) N += *cluster.map_shared_rank(&s_part[it & 1], b);
+        for (int b = 0; b < CTAS; ++b) N += CTAS > 1 ? *cluster.map_shared_rank(&s_part[it & 1], b) : s_part[it & 1];
         if (fabs(N - N_e) <= tol_N) {
             conv = 1;
             break;
@@ -446,8 +452,12 @@ static int launch_mu(const double *g, int n, double emin, double emax, int kind,
     k_count_weights<<<((n + 1) / 2 + 31) / 32, CW_NW * 32, 0, s>>>(g, n, w);
     CHEB_TRY(check_launch("k_count_weights"));
     const double lo = bracket ? bracket[0] : emin, hi = bracket ? bracket[1] : emax;
-    k_bisect<<<BIS_CTAS, BIS_NT, 0, s>>>(w, n, emin, emax, kind, kT, N_e, tol_N, max_iter, lo, hi,
-                                         static_cast<MuResult *>(result));
+    MuResult *res = static_cast<MuResult *>(result);
+    if (n <= BIS_ONE)
+        k_bisect<1, BIS_ONE, 1><<<1, BIS_ONE, 0, s>>>(w, n, emin, emax, kind, kT, N_e, tol_N, max_iter, lo, hi, res);
+    else
+        k_bisect<BIS_CTAS, BIS_NT, BIS_KEEP><<<BIS_CTAS, BIS_NT, 0, s>>>(w, n, emin, emax, kind, kT, N_e, tol_N, max_iter, lo,
+                                                                        hi, res);
     return check_launch("k_bisect");
 }
 
