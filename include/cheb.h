@@ -191,8 +191,8 @@ int cheb_plan_attach_operator(cheb_plan *plan, const cheb_bsr *L, size_t *op_ws_
  * result is NaN.  Results agree with the other kernels to rounding, and are bitwise
  * reproducible run to run.  CHEB_F64X expansions that run it hold T_k in FP64.  The
  * lists are not built (and the ranking kernels run) when one column's rows do not
- * fit a panel, the operator has 2^22 - 1 blocks or more, or the pattern more than about
- * 800,000 block rows.  cheb_plan_col_info
+ * fit a panel, the operator has 2^22 - 1 blocks or more or rows whose columns do not
+ * strictly ascend, or the pattern more than about 800,000 block rows.  cheb_plan_col_info
  * reports the panel count (0 when not built), largest union and total operator
  * words (padding included).
  *

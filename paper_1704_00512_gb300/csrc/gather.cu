@@ -538,7 +538,8 @@ __global__ void k_pc_tperm(const int64_t *rp, const int32_t *ci, int64_t nbr, in
 }
 
 // Checks of an operator pattern (n blocks): first[0] rows decreasing or out of
-// [0, n] or longer than 65536 blocks; first[1] a column out of range.
+// [0, n] or longer than 65536 blocks; first[1] a column out of range; first[2] columns
+// that do not strictly ascend.
 __global__ void k_op_check(const int64_t *rp, const int32_t *ci, int64_t nbr, int64_t n, int64_t *first) {
     const int64_t I = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (I >= nbr) return;
@@ -547,11 +548,13 @@ __global__ void k_op_check(const int64_t *rp, const int32_t *ci, int64_t nbr, in
         atomicMin(reinterpret_cast<long long *>(first), (long long)I);
         return;
     }
-    for (int64_t p = a; p < b; ++p)
+    for (int64_t p = a; p < b; ++p) {
         if (ci[p] < 0 || ci[p] >= nbr) {
             atomicMin(reinterpret_cast<long long *>(first + 1), (long long)I);
             return;
         }
+        if (p > a && ci[p] <= ci[p - 1]) atomicMin(reinterpret_cast<long long *>(first + 2), (long long)I);
+    }
 }
 
 // Row lists of one panel set (the FP64 step kernel's and the resident
@@ -852,14 +855,14 @@ int gp_walk(const int64_t *rp, const int32_t *ci, int64_t nbr, int P, int64_t uc
     return CHEB_OK;
 }
 
-int gp_check_operator(const cheb_bsr *L, int64_t nbr, int64_t first[2], cudaStream_t s) {
+int gp_check_operator(const cheb_bsr *L, int64_t nbr, int64_t first[3], cudaStream_t s) {
     int64_t *d = nullptr;
-    CHEB_CUDA(cudaMallocAsync(&d, 2 * 8, s));
-    const int64_t init[2] = {nbr, nbr};
+    CHEB_CUDA(cudaMallocAsync(&d, 3 * 8, s));
+    const int64_t init[3] = {nbr, nbr, nbr};
     CHEB_CUDA(cudaMemcpyAsync(d, init, sizeof(init), cudaMemcpyHostToDevice, s));
     k_op_check<<<(unsigned)((nbr + 255) / 256), 256, 0, s>>>(L->row_ptr, L->col_idx, nbr, L->nnzb, d);
     const int rc = check_launch("k_op_check");
-    if (rc == CHEB_OK) CHEB_CUDA(cudaMemcpyAsync(first, d, 2 * 8, cudaMemcpyDeviceToHost, s));
+    if (rc == CHEB_OK) CHEB_CUDA(cudaMemcpyAsync(first, d, 3 * 8, cudaMemcpyDeviceToHost, s));
     CHEB_CUDA(cudaFreeAsync(d, s));
     CHEB_CUDA(cudaStreamSynchronize(s));
     return rc;

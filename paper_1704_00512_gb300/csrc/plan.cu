@@ -563,7 +563,7 @@ extern "C" int cheb_plan_attach_operator(cheb_plan *plan, const cheb_bsr *L, siz
         CHEB_CUDA(cudaMemcpyAsync(&ends[1], L->row_ptr + nbr, 8, cudaMemcpyDeviceToHost, s));
         CHEB_CUDA(cudaStreamSynchronize(s));
         if (ends[0] != 0 || ends[1] != nnzL) return fail(CHEB_ERR_INVALID, "cheb_plan_attach_operator: bad row_ptr");
-        int64_t first[2];
+        int64_t first[3];
         CHEB_TRY(gp_check_operator(L, nbr, first, s));
         if (first[0] < nbr)
             return fail(CHEB_ERR_INVALID, "cheb_plan_attach_operator: row_ptr decreasing or row longer than 65536 blocks at row %lld",
@@ -584,7 +584,9 @@ extern "C" int cheb_plan_attach_operator(cheb_plan *plan, const cheb_bsr *L, siz
         plan->op_ci = L->col_idx;
         plan->lists = std::move(lists);
         plan->rlists = std::move(rlists);
-        rc = col_build_device(plan, L, s);
+        // (the column kernel's lists have one place for a block; rows that name a column
+        // twice stay on the kernels that add them)
+        if (first[2] >= nbr) rc = col_build_device(plan, L, s);
         if (rc != CHEB_OK && rc != CHEB_ERR_NOSPACE) return rc;
         plan->op_ws_bytes = plan->lists.bytes() + plan->rlists.bytes() + plan->col.bytes() + prod_bytes(plan, nnzL);
         *op_ws_bytes = plan->op_ws_bytes;
@@ -598,13 +600,16 @@ extern "C" int cheb_plan_attach_operator(cheb_plan *plan, const cheb_bsr *L, siz
     CHEB_CUDA(cudaMemcpyAsync(lci.data(), L->col_idx, nnzL * 4, cudaMemcpyDeviceToHost, s));
     CHEB_CUDA(cudaStreamSynchronize(s));
     if (lrp[0] != 0 || lrp[nbr] != nnzL) return fail(CHEB_ERR_INVALID, "cheb_plan_attach_operator: bad row_ptr");
+    bool ascending = true;
     for (int64_t I = 0; I < nbr; ++I) {
         if (lrp[I + 1] < lrp[I] || lrp[I + 1] - lrp[I] > 65536)
             return fail(CHEB_ERR_INVALID, "cheb_plan_attach_operator: row_ptr decreasing or row longer than 65536 blocks at row %lld",
                         (long long)I);
-        for (int64_t a = lrp[I]; a < lrp[I + 1]; ++a)
+        for (int64_t a = lrp[I]; a < lrp[I + 1]; ++a) {
             if (lci[a] < 0 || lci[a] >= nbr)
                 return fail(CHEB_ERR_INVALID, "cheb_plan_attach_operator: column out of range in row %lld", (long long)I);
+            ascending &= a == lrp[I] || lci[a] > lci[a - 1];
+        }
     }
     RowLists lists, rlists;
     CHEB_TRY(make_row_lists(nbr, plan->h_panels, plan->n_panels, rp, ci, lrp, lci, lists));
@@ -615,8 +620,9 @@ extern "C" int cheb_plan_attach_operator(cheb_plan *plan, const cheb_bsr *L, siz
     plan->lists = std::move(lists);
     plan->rlists = std::move(rlists);
     // the column-order kernel's lists (left unbuilt when a panel column or the
-    // operator does not fit it; the expansions then use the ranking kernels)
-    const int rc = col_build(plan, rp, ci, lrp, lci);
+    // operator does not fit it or a row names a column twice; the expansions then use
+    // the ranking kernels)
+    const int rc = ascending ? col_build(plan, rp, ci, lrp, lci) : CHEB_ERR_NOSPACE;
     if (rc != CHEB_OK && rc != CHEB_ERR_NOSPACE) return rc;
     plan->op_ws_bytes = plan->lists.bytes() + plan->rlists.bytes() + plan->col.bytes() + prod_bytes(plan, nnzL);
     plan->op_bound = false;

@@ -327,7 +327,7 @@ int gp_tperm(const int64_t *rp, const int32_t *ci, int64_t nbr, int64_t nnzb, in
 int gp_walk(const int64_t *rp, const int32_t *ci, int64_t nbr, int P, int64_t ucap, int64_t bcap,
             const std::vector<int64_t> &sys_col, std::vector<int32_t> &panels4, std::vector<int32_t> &aux,
             int64_t out[4], cudaStream_t s);
-int gp_check_operator(const cheb_bsr *L, int64_t nbr, int64_t first[2], cudaStream_t s);
+int gp_check_operator(const cheb_bsr *L, int64_t nbr, int64_t first[3], cudaStream_t s);
 int row_lists_device(const int64_t *rp, const int32_t *ci, int64_t nbr, const cheb_bsr *L, const int32_t *pairs,
                      int64_t np, int maxu, RowLists &out, cudaStream_t s);
 // The panels (quads of each) in the order of their launch.
