@@ -10,6 +10,7 @@ from __future__ import annotations
 import concurrent.futures as cf
 import glob
 import os
+import re
 import subprocess
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -19,6 +20,40 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libcheb.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include")]
+
+# Sources whose kernels fill the register file (128 registers, 512 threads a block), and
+# the bytes of register spill that each kernel may have: those of the present code, which
+# lie outside the inner loops.  More would go unnoticed into the hot path, so it fails the
+# build.  Kernels not named here may have none.
+SPILL_LIMITS = {
+    "colstep.cu": {"k_colstepIfE": 12},
+    "product.cu": {"k_product": 64},
+}
+
+
+def spills(ptxas: str) -> dict[str, int]:
+    """Bytes of spill stores of every function in the output of ptxas -v."""
+    out, fn = {}, None
+    for line in ptxas.splitlines():
+        if m := re.search(r"Function properties for (\S+)", line):
+            fn = m.group(1)
+        elif (m := re.search(r"(\d+) bytes spill stores", line)) and fn:
+            out[fn] = int(m.group(1))
+    return out
+
+
+def check_spills(src: str, ptxas: str) -> None:
+    """Raise if a function of src spills more than its limit."""
+    limits = SPILL_LIMITS.get(os.path.basename(src))
+    if limits is None:
+        return
+    found = spills(ptxas)
+    if not found:
+        raise RuntimeError(f"{src}: ptxas reported no function")
+    for fn, n in found.items():
+        allowed = max([b for name, b in limits.items() if name in fn], default=0)
+        if n > allowed:
+            raise RuntimeError(f"{src}: {fn} spills {n} bytes of registers, {allowed} allowed")
 
 
 def _nvcc() -> str:
@@ -53,9 +88,12 @@ def build(force: bool = False, verbose: bool = False) -> str:
     def compile_one(src: str) -> str:
         obj = os.path.join(BUILD, os.path.basename(src)[:-3] + ".o")
         cmd = [nvcc, *ARCH, *FLAGS, "-c", src, "-o", obj]
+        if os.path.basename(src) in SPILL_LIMITS:
+            cmd += ["-Xptxas", "-v"]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"nvcc failed for {src}:\n{r.stdout}\n{r.stderr}")
+        check_spills(src, r.stderr)
         if verbose and r.stderr:
             print(r.stderr)
         return obj
