@@ -54,6 +54,10 @@ COL_KERNEL_END = "// Host: the column kernel's panels and work streams"
 COL_TRAFFIC = {"colstep_sha256": "154741e02d152208e90026c68cebafde56a0824781690b584981970ab666ee15",
                "blocks_P_out": 1183812, "pass1_bytes": 453.7e6, "pass2_4acc_bytes": 857.9e6, "order": "hilbert"}
 SMS, FP32_LANES, MAX_SM_MHZ = 152, 128, 2070.0
+# Dense f16 mma.sync rate measured with a register-only kernel (GB300, 2,070 MHz), and the
+# digit products that make one product of the column kernel.
+MMA_F16_TFLOPS = 604.0
+DIGIT_PRODUCTS = {"float": 6, "double": 26}
 
 WORKLOADS = {
     # The mixed-precision density matrix: 10,000 atoms x 4, 10 bohr cutoff,
@@ -412,13 +416,9 @@ def run_cheb(args, rank: int, world: int, local: int):
         alg_bytes = sum(b * l for b, l in zip(bytes_pass, launches_pass)) / n_launch
         tflops = flops / (avg_ms / 1e3) / 1e12
         gbs = alg_bytes / (avg_ms / 1e3) / 1e9
-        alu_peak = SMS * FP32_LANES * 2 * MAX_SM_MHZ * 1e6 / 1e12
         hbm_peak, hbm_src = measured_hbm_peak()
         traffic = col_traffic_per_launch(form, cfg["n_mu"], launches_pass, nnz_out, order=cfg.get("order"))
-        roof = {"bound": "alu", "achieved": round(tflops, 3), "peak": round(alu_peak, 3), "unit": "TFLOP/s",
-                "frac": round(tflops / alu_peak, 4), "traffic": traffic,
-                "peak_source": "FP32 FMA unit count: 152 SMs x 128 lanes x 2 flops x 2070 MHz",
-                "kernel": "k_colstep<float>", "algorithmic_flops_per_step": flops,
+        roof = {**step_roof(tflops, "f32", True), "traffic": traffic, "algorithmic_flops_per_step": flops,
                 "algorithmic_bytes_per_step": int(alg_bytes), "avg_step_ms": round(avg_ms, 5),
                 "hbm_gbs": round(gbs, 1), "hbm_frac": round(gbs / hbm_peak, 4),
                 "hbm_peak": hbm_peak, "hbm_peak_source": f"{hbm_src} copy bandwidth"}
@@ -478,6 +478,27 @@ def run_cheb(args, rank: int, world: int, local: int):
 
 # GB300 FP64: 304 DFMA lanes per cycle (152 SMs x 2, ncu peak_sustained) x 2 flops x 2070 MHz
 FP64_NOMINAL_TFLOPS = 1.26
+
+
+def step_roof(tflops: float, precision: str, column: bool) -> dict:
+    """Roofline of the recursion for tflops of useful block-triple FLOPs: of the f16 digit
+    products where the column kernel runs it, else of the FMA units (FP32 ones for the
+    double-floats of f64x).  The ratio to the FMA unit of the precision stands beside it."""
+    elem = "float" if precision == "f32" else "double"
+    fp32 = SMS * FP32_LANES * 2 * MAX_SM_MHZ * 1e6 / 1e12
+    unit = fp32 if precision == "f32" else FP64_NOMINAL_TFLOPS
+    if column:
+        n = DIGIT_PRODUCTS[elem]
+        bound, peak, kernel = "tensor", MMA_F16_TFLOPS / n, f"k_colstep<{elem}>"
+        src = f"f16 mma.sync, {MMA_F16_TFLOPS:.0f} TFLOP/s measured, over {n} digit products per product"
+    else:
+        bound, kernel = "alu", {"f32": "k_resident<float>", "f64": "k_step<double>", "f64x": "k_step<dfl>"}[precision]
+        peak = FP64_NOMINAL_TFLOPS if precision == "f64" else fp32
+        src = ("FP64 unit count: 304 DFMA lanes per cycle x 2 flops x 2070 MHz" if precision == "f64" else
+               "FP32 FMA unit count: 152 SMs x 128 lanes x 2 flops x 2070 MHz")
+    return {"bound": bound, "achieved": round(tflops, 3), "peak": round(peak, 3), "unit": "TFLOP/s",
+            "frac": round(tflops / peak, 4), "kernel": kernel, "peak_source": src,
+            f"vs_fp{32 if precision == 'f32' else 64}_unit_peak": round(tflops / unit, 4)}
 
 
 def run_powers(args, rank: int, world: int, local: int):
@@ -553,20 +574,13 @@ def run_powers(args, rank: int, world: int, local: int):
         torch.cuda.synchronize()
         ms64 = d0.elapsed_time(d1)
         rel = max(float(torch.linalg.norm(a - b) / torch.linalg.norm(b)) for a, b in zip(out["acc"], o64["acc"]))
-        alu_peak = SMS * FP32_LANES * 2 * MAX_SM_MHZ * 1e6 / 1e12
-        roof = {"bound": "alu", "achieved": round(tflops, 4), "peak": round(alu_peak, 3), "unit": "TFLOP/s",
-                "frac": round(tflops / alu_peak, 4), "traffic": None, "kernel": "k_colstep<double>",
-                "peak_source": "FP32 FMA unit count: 152 SMs x 128 lanes x 2 flops x 2070 MHz (for scale: the "
-                               "products are f16 tensor-core digits; achieved counts FP64-accurate flops)",
-                "vs_fp64_unit_peak": round(tflops / FP64_NOMINAL_TFLOPS, 3)}
         vs_f64 = {"f64_step_ms": round(ms64, 2), "f64x_step_ms": round(t_ms / args.steps, 2),
                   "speedup": round(ms64 / (t_ms / args.steps), 3), "max_relF_vs_fp64": rel}
     else:
-        roof = {"bound": "alu", "achieved": round(tflops, 4), "peak": FP64_NOMINAL_TFLOPS, "unit": "TFLOP/s",
-                "frac": round(tflops / FP64_NOMINAL_TFLOPS, 4), "traffic": None,
-                "kernel": "k_colstep<double>",
-                "peak_source": "FP64 unit count: 304 DFMA lanes per cycle x 2 flops x 2070 MHz"}
         vs_f64 = None
+    plan = pb.plan64 if prec == cg.F64 else pb.planX
+    column = cg.plan_col_info(plan)[0] > 0 and plan._op_pattern[0] is pb.S.row_ptr
+    roof = {**step_roof(tflops, cfg["precision"], column), "traffic": None}
     res = {
         "metric": METRIC, "value": round(value, 4), "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": round(t_ms / args.steps, 2), "higher_is_better": True,
@@ -654,14 +668,15 @@ def run_batched(args, rank: int, world: int, local: int):
     torch.cuda.synchronize()
     te_ms = max_over_ranks(f0.elapsed_time(f1), world, dev)
     e2e_value = job_throughput(args.e2e_steps * len(systems), world, te_ms)
-    # roofline of the batched launches (FP32 ALU): block triples of every system x terms
+    # roofline of the batched launches: block triples of every system x terms
     triples = [count_triples(bp.PH[i].row_ptr.cpu().numpy(), bp.PH[i].col_idx.cpu().numpy(),
                              bp.Pout[i].row_ptr.cpu().numpy(), bp.Pout[i].col_idx.cpu().numpy())
                for i in range(len(systems))]
     flops = sum(2.0 * 64.0 * t * 2 * (n - 2) for t, n in zip(triples, out["n_terms"]))
+    # (a batch runs on the column kernel from 48 operator blocks per block row on)
+    column = bp.P_H.nnzb >= 48 * bp.P_H.nbr
     pass_s = statistics.mean(passes) / 1e3
     tflops = flops / pass_s / 1e12
-    alu_peak = SMS * FP32_LANES * 2 * MAX_SM_MHZ * 1e6 / 1e12
     res = {
         "metric": METRIC, "value": round(value, 4), "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": round(t_ms / args.steps, 2), "higher_is_better": True,
@@ -671,9 +686,7 @@ def run_batched(args, rank: int, world: int, local: int):
                    "kT": cfg["kT"], "n_terms_range": [min(out["n_terms"]), max(out["n_terms"])],
                    "blocks_P_out": bp.P_out.nnzb, "blocks_P_H": bp.P_H.nnzb, "tiles": out["tiles"],
                    "graphs": "expansions, post-processing and traces captured and replayed; bisections eager", "l2": "inputs larger than L2 (no flush)"},
-        "roofline": {"bound": "alu", "achieved": round(tflops, 3), "peak": round(alu_peak, 3), "unit": "TFLOP/s",
-                     "frac": round(tflops / alu_peak, 4), "traffic": None, "kernel": "k_colstep (batched), k_resident for short rows",
-                     "peak_source": "FP32 FMA: 152 SMs x 128 lanes x 2 x 2070 MHz"},
+        "roofline": {**step_roof(tflops, cfg["precision"], column), "traffic": None},
         "pass_ms": round(statistics.mean(passes), 1),
         "e2e": {"value": round(e2e_value, 4), "unit": UNIT, "h2d_bytes_per_step": int(h_H.numel() * 8),
                 "d2h_bytes_per_step": int(h_F.numel() * 8)},
