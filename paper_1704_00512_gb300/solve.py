@@ -116,6 +116,9 @@ class Problem:
             self.plan64.attach_operator(self.P_H)
             if self.planX is not self.plan64:
                 self.planX.attach_operator(self.P_H)
+        # (called again: the plans' lists are used for matrices on the new pattern)
+        if hasattr(self, "S"):
+            self.S, self.H = self.P_H.with_vals(self.S.vals), self.P_H.with_vals(self.H.vals)
 
     @property
     def n_rows(self) -> int:
