@@ -191,7 +191,8 @@ int cheb_plan_attach_operator(cheb_plan *plan, const cheb_bsr *L, size_t *op_ws_
  * result is NaN.  Results agree with the other kernels to rounding, and are bitwise
  * reproducible run to run.  CHEB_F64X expansions that run it hold T_k in FP64.  The
  * lists are not built (and the ranking kernels run) when one column's rows do not
- * fit a panel, the operator has 2^22 - 1 blocks or more or rows whose columns do not
+ * fit a panel, an FP64 plan's group of rows merges more than 504 slots, the operator
+ * has 2^22 - 1 blocks or more or rows whose columns do not
  * strictly ascend, or the pattern more than about 800,000 block rows.  cheb_plan_col_info
  * reports the panel count (0 when not built), largest union and total operator
  * words (padding included).
@@ -358,8 +359,8 @@ int cheb_expand_stepwise(const cheb_plan *plan, const cheb_bsr *Mt, int32_t n_te
  * coefficients coeffs + coeff_offset[i] (device int64[nsys]; layout
  * [n_f][coeff_stride] per system); moments of system i go to
  * moments/gmoments + i*moment_stride.  acc / G are on the concatenated P_out.
- * One kernel launch for all systems and all steps (plus one moment reduction);
- * asynchronous and graph-capturable.
+ * One kernel launch for all systems and all steps (plus one moment reduction), or on the
+ * column kernel (see above) one for every 96 steps; asynchronous and graph-capturable.
  */
 int cheb_plan_create_batched(const cheb_bsr *P_out, int32_t precision, int32_t tile,
                              int32_t nsys, const int64_t *sys_row_start, cheb_plan **plan,
@@ -378,7 +379,7 @@ int cheb_expand_batched(const cheb_plan *plan, const cheb_bsr *Mt, int32_t max_t
  *   C = alpha P_out(L R) + beta D
  * L: FP64 BCSR with nbr rows (any pattern); R, D, C: FP64 values on the plan's
  * P_out (BCSR order).  D may be NULL (beta ignored).  C must not alias R or D.
- * The plan must be an FP64 plan.  Asynchronous; no workspace.
+ * The plan must be an FP64 plan.  Asynchronous; no workspace argument.
  *
  * With the column kernel's lists bound (long operator rows) and L on the attached
  * operator's pattern or on the plan's own (the same row_ptr / col_idx pointers), the

@@ -22,9 +22,9 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include")]
 
 # Sources whose kernels fill the register file (128 registers, 512 threads a block), and
-# the bytes of register spill that each kernel may have: those of the present code, which
-# lie outside the inner loops.  More would go unnoticed into the hot path, so it fails the
-# build.  Kernels not named here may have none.
+# the bytes of register spill that each kernel may have: those of the code whose times are
+# stated beside it.  More would go unnoticed into the hot path, so it fails the build.
+# Kernels not named here may have none.
 SPILL_LIMITS = {
     "colstep.cu": {"k_colstepIfE": 12},
     "product.cu": {"k_product": 64},

@@ -235,12 +235,14 @@ constexpr int COL_SLOT_BITS = 10;  // union slots < 1023; operator blocks < 2^22
 // Union rows of a panel at most, of width 4 (FP32) and 2 (FP64).  Columns beyond it run on
 // the ranking kernels.
 __host__ __device__ constexpr int col_max_union(int P) { return P == 4 ? 667 : 576; }
-// (quads of a group come in pairs) FP64: quads of a group at most, so that its exact digit sums (at most 4
-// products of 2^18 per merged row of a slot) stay below 2^31.
+// FP64: quads of a group at most, so that its exact digit sums (at most 4 products of 2^18
+// per merged row of a slot) stay below 2^31.  An operator with a larger group gets no lists.
 constexpr int COL_MAX_QUADS64 = 126;
 // Operator blocks per block row, on average, from which FP64 expansions and the
 // one-launch forms run on the column kernel.  Short rows stay on the kernels whose
-// results are the same bits with and without attached lists.
+// results are the same bits with and without attached lists.  (Not a crossing of times:
+// 100 FP64 terms at 50 atoms and 46 blocks a row take 10.7 ms on k_step, at 61 atoms and 60
+// blocks 2.1 ms on the column kernel and 15.2 ms on k_step.)
 constexpr int64_t COL_ROW_MIN = 48;
 // panel width: 16 scalar columns of FP32 or 8 of FP64 fill two or one mma tiles
 inline int col_width(int precision) { return precision == CHEB_F64 || precision == CHEB_F64X ? 2 : 4; }
