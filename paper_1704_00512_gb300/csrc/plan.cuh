@@ -234,7 +234,7 @@ constexpr int COL_TAIL = 8;        // quads of padding behind the lists (read ah
 constexpr int COL_SLOT_BITS = 10;  // union slots < 1023; operator blocks < 2^22
 // Union rows of a panel at most, of width 4 (FP32) and 2 (FP64).  Columns beyond it run on
 // the ranking kernels.
-__host__ __device__ constexpr int col_max_union(int P) { return P == 4 ? 667 : 576; }
+__host__ __device__ constexpr int col_max_union(int P) { return P == 4 ? 667 : 577; }
 // FP64: quads of a group at most, so that its exact digit sums (at most 4 products of 2^18
 // per merged row of a slot) stay below 2^31.  An operator with a larger group gets no lists.
 constexpr int COL_MAX_QUADS64 = 126;
