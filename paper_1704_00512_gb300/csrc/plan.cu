@@ -420,7 +420,8 @@ extern "C" int cheb_plan_destroy(cheb_plan *plan) {
         free_row_lists(plan->lists);
         free_row_lists(plan->rlists);
         if (plan->tmp_tperm) cudaFree(plan->tmp_tperm);
-        if (plan->prod_done) cudaEventDestroy(plan->prod_done);
+        for (const cheb_plan::ProdSlot &p : plan->prod_slot)
+            if (p.done) cudaEventDestroy(p.done);
     }
     delete plan;
     return CHEB_OK;

@@ -10,6 +10,9 @@
 // Largest dynamic shared memory a block may use on sm_100/sm_103 (227 KB).
 #define CHEB_MAX_DYN_SMEM 232448
 
+// Streams whose masked products may run side by side in one plan, at most (product.cu).
+constexpr int PROD_SLOTS = 8;
+
 // Operator row lists of one panel set (see cheb_plan).
 struct RowLists {
     std::vector<int64_t> h_base;  // [panels] first row pointer of each panel
@@ -124,11 +127,17 @@ struct cheb_plan {
     size_t op_ws_bytes = 0;
     bool op_bound = false;
     // masked products by digits (product.cu): the left operand's digits, in the operator
-    // workspace; the event of their last use orders calls on different streams
+    // workspace, a few of them where they are small; a stream keeps to one, and the event of
+    // its last use orders calls on streams that share one
     int32_t max_row = 0;  // longest row of P_out
     void *prod_ws = nullptr;
+    struct ProdSlot {
+        cudaEvent_t done = nullptr;
+        cudaStream_t stream = nullptr;
+    };
     mutable std::mutex prod_mx;
-    mutable cudaEvent_t prod_done = nullptr;
+    mutable ProdSlot prod_slot[PROD_SLOTS];
+    mutable int prod_next = 0;
 };
 
 namespace cheb {
