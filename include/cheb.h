@@ -394,7 +394,7 @@ int cheb_expand_batched(const cheb_plan *plan, const cheb_bsr *Mt, int32_t max_t
  * blocks), at most 65,535 block rows and 16-byte aligned R, D and C; otherwise, and while
  * the stream is captured, the product runs on the FP64 pipe.  The two agree within their
  * errors, not to the bit.  L's digits are kept in the operator workspace (128 bytes per
- * block of the larger pattern, part of op_ws_bytes; up to eight of them within 64 MB):
+ * block of the larger pattern, part of op_ws_bytes; up to eight of them within 24 MB):
  * calls on as many streams run side by side, beyond that they are put in order behind
  * each other on the device.
  */

@@ -399,13 +399,14 @@ __global__ void __launch_bounds__(PR_NW * 32, 1) k_product(const __grid_constant
 
 // The digits of one left operand, and how many of them a plan keeps: streams with their
 // own run side by side, which pays while a product leaves SMs idle (50 panels, eight
-// streams: 0.24 against 0.64 ms with one), so within 64 MB.
+// streams: 0.24 against 0.64 ms with one), so within 24 MB
+// (150 atoms; 300 atoms are 150 panels, and eight streams gain 6 %).
 static size_t prod_slot_bytes(const cheb_plan *plan, int64_t nnzL) {
     const int64_t n = std::max(nnzL, plan->nnzb);
     return align_up((size_t)(n + 1) * 128) + align_up(plan->nbr * 16) + align_up(64);
 }
 static int prod_slots(const cheb_plan *plan, int64_t nnzL) {
-    return (int)std::clamp<size_t>(((size_t)64 << 20) / prod_slot_bytes(plan, nnzL), 1, PROD_SLOTS);
+    return (int)std::clamp<size_t>(((size_t)24 << 20) / prod_slot_bytes(plan, nnzL), 1, PROD_SLOTS);
 }
 size_t prod_bytes(const cheb_plan *plan, int64_t nnzL) {
     if (plan->precision != CHEB_F64 || !plan->col.built || plan->nbr > 65535 || plan->max_row > prod_cap(plan)) return 0;
